@@ -36,66 +36,96 @@ std::vector<double> correction_axis(int n, int K, int J, double beta) {
     return s;
 }
 
+// The kernel as a function of r = 1 - (2t/J)^2, I0(beta sqrt(r)) / I0(beta),
+// by the series in r (entire in r, so it also continues the kernel past its
+// support), in arithmetic type A.
+template <typename A> struct KbSeries {
+    double beta;
+    A inv[400], norm;   // 1 / m^2, I0(beta)
+    explicit KbSeries(double b) : beta(b) {
+        for (int m = 1; m < 400; ++m) inv[m] = A(1) / ((A)m * m);
+        norm = sum(A(1));
+    }
+    A sum(A r) const {
+        const A q = A(0.25) * beta * beta * r;
+        A term = 1, s = 1;
+        for (int m = 1; m < 400; ++m) {
+            term *= q * inv[m];
+            const A s2 = s + term;
+            if (s2 == s && m > 4) break;
+            s = s2;
+        }
+        return s;
+    }
+    A tap(int J, int a, A phi) const {
+        const A t = phi + A(0.5) * J - 1 - a;
+        return sum(A(1) - (2 * t / J) * (2 * t / J)) / norm;
+    }
+};
+
 // Chebyshev interpolation of each tap's weight on z = 2 phi - 1 in [-1, 1],
-// converted to monomial coefficients for Horner evaluation.
+// converted to monomial coefficients for Horner evaluation, computed in A
+// and stored as C. The kernel is even in the offset: tap J-1-a at z equals
+// tap a at -z; the mirrored taps are stored as exact reflections (the middle
+// tap of an odd J as an even polynomial), so that the weights can be
+// evaluated from even and odd parts.
+template <typename A, typename C, int LD>
+static void fit_taps(const KbSeries<A>& kb, int J, int deg, C (&coef)[PURIFY_MAX_J][LD]) {
+    const int n = deg + 1;
+    const A pi = (A)3.14159265358979323846264338327950288L;
+    // monomial coefficients of T_0..T_deg, and cos(pi i / 2n)
+    std::vector<std::vector<A>> T(n, std::vector<A>(n, A(0)));
+    std::vector<A> cs(4 * n);
+    for (int i = 0; i < 4 * n; ++i) cs[i] = std::cos(pi * i / (2 * n));
+    T[0][0] = 1;
+    if (n > 1) T[1][1] = 1;
+    for (int k = 2; k < n; ++k)
+        for (int i = 0; i < n; ++i) T[k][i] = (i > 0 ? 2 * T[k - 1][i - 1] : A(0)) - T[k - 2][i];
+    for (int a = 0; a < (J + 1) / 2; ++a) {
+        std::vector<A> f(n), c(n, A(0));
+        for (int k = 0; k < n; ++k) f[k] = kb.tap(J, a, A(0.5) * (cs[2 * k + 1] + 1));
+        for (int j = 0; j < n; ++j) {
+            A acc = 0;
+            for (int k = 0; k < n; ++k) acc += f[k] * cs[j * (2 * k + 1) % (4 * n)];
+            c[j] = acc * 2 / n;
+        }
+        c[0] *= A(0.5);
+        for (int i = 0; i < n; ++i) {
+            A m = 0;
+            for (int j = 0; j < n; ++j) m += c[j] * T[j][i];
+            coef[a][i] = (2 * a + 1 == J && (i & 1)) ? C(0) : (C)m;
+            if (2 * a + 1 != J) coef[J - 1 - a][i] = (i & 1) ? -coef[a][i] : coef[a][i];
+        }
+    }
+}
+
 KbPoly fit_kb_poly(int J, double beta, int deg) {
     KbPoly kp;
     std::memset(&kp, 0, sizeof(kp));
     kp.J = J;
     kp.deg = deg;
-    const int n = deg + 1;
-    double i0b = bessel_i0_series(beta);
-    // monomial coefficients of T_0..T_deg
-    std::vector<std::vector<double>> T(n, std::vector<double>(n, 0.0));
-    T[0][0] = 1.0;
-    if (n > 1) T[1][1] = 1.0;
-    for (int k = 2; k < n; ++k) {
-        for (int i = 0; i < n; ++i) {
-            double v = -T[k - 2][i];
-            if (i > 0) v += 2.0 * T[k - 1][i - 1];
-            T[k][i] = v;
-        }
-    }
-    for (int a = 0; a < J; ++a) {
-        std::vector<double> f(n), c(n, 0.0);
-        for (int k = 0; k < n; ++k) {
-            double z = std::cos(kPi * (k + 0.5) / n);
-            double phi = 0.5 * (z + 1.0);
-            double t = phi + 0.5 * J - 1.0 - a;
-            double r = 1.0 - (2.0 * t / J) * (2.0 * t / J);
-            // the kernel is entire in t: continue I0(beta sqrt(r)) by its series in r
-            double q = 0.25 * beta * beta * r, term = 1.0, sum = 1.0;
-            for (int m = 1; m < 400; ++m) {
-                term *= q / ((double)m * (double)m);
-                double s2 = sum + term;
-                if (s2 == sum && std::fabs(term) < 1e-300 + 1e-18 * std::fabs(sum)) break;
-                sum = s2;
-            }
-            f[k] = sum / i0b;
-        }
-        for (int j = 0; j < n; ++j) {
-            double acc = 0.0;
-            for (int k = 0; k < n; ++k) acc += f[k] * std::cos(kPi * j * (k + 0.5) / n);
-            c[j] = acc * 2.0 / n;
-        }
-        c[0] *= 0.5;
-        for (int i = 0; i < n; ++i) {
-            double m = 0.0;
-            for (int j = 0; j < n; ++j) m += c[j] * T[j][i];
-            kp.coef[a][i] = (float)m;
-        }
-    }
-    // the kernel is even in the offset: tap J-1-a at z equals tap a at -z;
-    // store the mirrored taps as exact reflections (the middle tap of an odd
-    // J as an even polynomial), so that the weights can be evaluated from
-    // even and odd parts
+    fit_taps(KbSeries<double>(beta), J, deg, kp.coef);
+    return kp;
+}
+
+KbPolyD fit_kb_poly_d(int J, double beta) {
+    KbPolyD kp;
+    std::memset(&kp, 0, sizeof(kp));
+    kp.J = J;
+    kp.beta = beta;
+    kp.inv_i0beta = 1.0 / bessel_i0_series(beta);
+    const int deg = kb_poly_deg_d(J);
+    const KbSeries<long double> kb(beta);
+    fit_taps(kb, J, deg, kp.coef);
+    // a caller's beta may need a higher degree: compare with the definition
+    // between the nodes, to half a unit of double rounding at 1
+    kp.poly = 1;
     for (int a = 0; a < (J + 1) / 2; ++a)
-        for (int i = 0; i < n; ++i) {
-            if (2 * a + 1 == J) {
-                if (i & 1) kp.coef[a][i] = 0.0f;
-            } else {
-                kp.coef[J - 1 - a][i] = (i & 1) ? -kp.coef[a][i] : kp.coef[a][i];
-            }
+        for (int i = 0; i <= 24; ++i) {
+            const double z = -1.0 + i / 12.0;
+            double v = kp.coef[a][deg];
+            for (int k = deg - 1; k >= 0; --k) v = std::fma(v, z, kp.coef[a][k]);
+            if (!(std::fabs((long double)v - kb.tap(J, a, 0.5L * (z + 1.0L))) <= 2.5e-16L)) kp.poly = 0;
         }
     return kp;
 }

@@ -219,6 +219,7 @@ struct purify_plan {
     std::vector<int> bases;           // basis ids in dictionary order (0 = Dirac)
     purify::AxisConst ax, ay;
     purify::KbPoly kbp;
+    purify::KbPolyD kbpd;             // double plans
     purify::DevBuf sx, sy;            // per-axis correction (dtype)
     purify::DevBuf onesx, onesy;      // all-ones tables (transforms without the correction)
     purify::DevBuf twx, twy;          // twiddles (complex dtype)

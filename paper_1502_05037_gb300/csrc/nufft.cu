@@ -97,7 +97,7 @@ __device__ __forceinline__ int bits_int(double v) { return (int)__double_as_long
 template <typename T, int J, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32)
 k_grid_runs(const typename cplx_of<T>::type* __restrict__ yin, const T* __restrict__ us, const T* __restrict__ vs,
-            AxisConst ax, AxisConst ay, KbPoly kp, double beta, double inv_i0beta, const int* __restrict__ perm,
+            AxisConst ax, AxisConst ay, typename KbOf<T>::type kp, const int* __restrict__ perm,
             const int* __restrict__ sub_bin, const int* __restrict__ sub_off, const int* __restrict__ list, int tile,
             int tiles_x, int S, typename cplx_of<T>::type* __restrict__ grid, const int* __restrict__ skip) {
     pdl_wait();
@@ -142,13 +142,8 @@ k_grid_runs(const typename cplx_of<T>::type* __restrict__ yin, const T* __restri
                 split_coord(us[m], ax, J, kx0, phx);
                 split_coord(vs[m], ay, J, ky0, phy);
                 T wx[J], wy[J];
-                if constexpr (sizeof(T) == 4) {
-                    kb_weights<J>(kp, phx, wx);
-                    kb_weights<J>(kp, phy, wy);
-                } else {
-                    kb_weights<J>(beta, inv_i0beta, phx, wx);
-                    kb_weights<J>(beta, inv_i0beta, phy, wy);
-                }
+                kb_weights<J>(kp, phx, wx);
+                kb_weights<J>(kp, phy, wy);
                 const C yv = yin[perm ? perm[m] : m];
                 const int lx = (kx0 & (Kx - 1)) - ox, ly = (ky0 & (Ky - 1)) - oy;
                 if (lx >= 0 && lx < tile && ly >= 0 && ly < tile) {
@@ -316,17 +311,12 @@ __device__ __forceinline__ void ldg_row(const double2* __restrict__ row, int c0,
 // G^H G X needs no visibility vector. All J lanes of a group read the split
 // of the group's next record directly, one step ahead; the two warp
 // barriers of a step order every reuse of the single-buffered slots.
-template <int DEG> __device__ __forceinline__ float kb_tap_poly(const float (&c)[DEG + 1], float phi) {
-    const float z = fmaf(2.0f, phi, -1.0f);
-    float acc = c[DEG];
+template <typename T, int DEG> __device__ __forceinline__ T kb_tap_poly(const T (&c)[DEG + 1], T phi) {
+    const T z = fma(T(2), phi, T(-1));
+    T acc = c[DEG];
 #pragma unroll
-    for (int i = DEG - 1; i >= 0; --i) acc = fmaf(acc, z, c[i]);
+    for (int i = DEG - 1; i >= 0; --i) acc = fma(acc, z, c[i]);
     return acc;
-}
-__device__ __forceinline__ double kb_tap_exact(int J, int a, double beta, double inv_i0beta, double phi) {
-    const double t = phi + (0.5 * J - 1.0 - a);
-    const double r = 1.0 - (2.0 * t / J) * (2.0 * t / J);
-    return r > 0.0 ? bessel_i0_series(beta * sqrt(r)) * inv_i0beta : (r == 0.0 ? inv_i0beta : 0.0);
 }
 
 template <typename T, int J, int WARPS, bool FUSED>
@@ -334,12 +324,12 @@ __global__ void __launch_bounds__(WARPS * 32)
 k_grid_sets(const typename cplx_of<T>::type* __restrict__ yin, const typename cplx_of<T>::type* __restrict__ X,
             const typename RunRecOf<T>::type* __restrict__ recs, const int* __restrict__ run_cell,
             const int* __restrict__ run_start, const int* __restrict__ run_len, int nsets,
-            const int* __restrict__ perm, KbPoly kp, double beta, double inv_i0beta, int Kx, int Ky,
+            const int* __restrict__ perm, typename KbOf<T>::type kp, int Kx, int Ky,
             typename cplx_of<T>::type* __restrict__ out, const int* __restrict__ skip) {
     using C = typename cplx_of<T>::type;
     using Rec = typename RunRecOf<T>::type;
     constexpr int G = 32 / J;
-    constexpr int DEG = kb_poly_deg(J);
+    constexpr int DEG = sizeof(T) == 4 ? kb_poly_deg(J) : kb_poly_deg_d(J);
     pdl_wait();
     if (skip && *skip) return;
     const int lane = threadIdx.x & 31;
@@ -361,7 +351,7 @@ k_grid_sets(const typename cplx_of<T>::type* __restrict__ yin, const typename cp
     T (*sw)[GS][SWS] = s_w[threadIdx.x >> 5];
     C (*st)[STS] = s_t[FUSED ? (threadIdx.x >> 5) : 0];
     auto set_of = [&](int i) { return i * W + ((i & 1) ? W - 1 - wg : wg); };
-    float cf[DEG + 1];
+    T cf[DEG + 1];
 #pragma unroll
     for (int i = 0; i <= DEG; ++i) cf[i] = kp.coef[b][i];
     struct Meta { int len, lmax, start; unsigned cell; };
@@ -453,12 +443,14 @@ k_grid_sets(const typename cplx_of<T>::type* __restrict__ yin, const typename cp
             }
             const bool valid = k < cur.len;
             T wxb, wyb;
-            if constexpr (sizeof(T) == 4) {
-                wxb = kb_tap_poly<DEG>(cf, phx);
-                wyb = kb_tap_poly<DEG>(cf, phy);
-            } else {
-                wxb = kb_tap_exact(J, b, beta, inv_i0beta, phx);
-                wyb = kb_tap_exact(J, b, beta, inv_i0beta, phy);
+            bool poly = true;
+            if constexpr (sizeof(T) == 8) poly = kp.poly != 0;
+            if (poly) {
+                wxb = kb_tap_poly<T, DEG>(cf, phx);
+                wyb = kb_tap_poly<T, DEG>(cf, phy);
+            } else if constexpr (sizeof(T) == 8) {
+                wxb = kb_tap_exact(J, b, kp.beta, kp.inv_i0beta, phx);
+                wyb = kb_tap_exact(J, b, kp.beta, kp.inv_i0beta, phy);
             }
             const int par = NPAR == 1 ? 0 : (k & 1);
             sw[par][g][b] = wxb;
@@ -864,7 +856,7 @@ k_lane_gather(const float2* __restrict__ P, int64_t dstride, const int* __restri
 template <typename T, int J>
 __global__ void __launch_bounds__(128)
 k_degrid_tile(const typename cplx_of<T>::type* __restrict__ grid, const T* __restrict__ us, const T* __restrict__ vs,
-              AxisConst ax, AxisConst ay, KbPoly kp, double beta, double inv_i0beta, const int* __restrict__ perm,
+              AxisConst ax, AxisConst ay, typename KbOf<T>::type kp, const int* __restrict__ perm,
               const int* __restrict__ sub_bin, const int* __restrict__ sub_off, const int* __restrict__ list,
               int tile, int tiles_x, typename cplx_of<T>::type* __restrict__ y, const int* __restrict__ skip) {
     pdl_wait();
@@ -890,13 +882,8 @@ k_degrid_tile(const typename cplx_of<T>::type* __restrict__ grid, const T* __res
         split_coord(us[m], ax, J, kx0, phx);
         split_coord(vs[m], ay, J, ky0, phy);
         T wx[J], wy[J];
-        if constexpr (sizeof(T) == 4) {
-            kb_weights<J>(kp, phx, wx);
-            kb_weights<J>(kp, phy, wy);
-        } else {
-            kb_weights<J>(beta, inv_i0beta, phx, wx);
-            kb_weights<J>(beta, inv_i0beta, phy, wy);
-        }
+        kb_weights<J>(kp, phx, wx);
+        kb_weights<J>(kp, phy, wy);
         int lx = (kx0 & (Kx - 1)) - ox, ly = (ky0 & (Ky - 1)) - oy;
         T accx = 0, accy = 0;
         if (lx >= 0 && lx < tile && ly >= 0 && ly < tile) {
@@ -959,6 +946,12 @@ static int blocks_per_sm(std::atomic<int> (&cache)[64], K kernel, int threads, s
 }
 
 
+// the plan's kernel polynomials in precision T
+template <typename T> static const typename KbOf<T>::type& kb_table(const purify_plan* p) {
+    if constexpr (sizeof(T) == 4) return p->kbp;
+    else return p->kbpd;
+}
+
 template <typename T, int J> static void degrid_tj(purify_plan* p, void* y, bool caller_order, const int* skip) {
     using C = typename cplx_of<T>::type;
     const GridWork& w = p->dwork;
@@ -968,7 +961,7 @@ template <typename T, int J> static void degrid_tj(purify_plan* p, void* y, bool
     set_smem(k_degrid_tile<T, J>, sm);
     Launch L(p, "degrid");
     launch_dependent(k_degrid_tile<T, J>, w.nsub, 128, sm, p->stream, 
-        p->grid.as<C>(), p->us.as<T>(), p->vs.as<T>(), p->ax, p->ay, p->kbp, p->beta, 1.0 / p->i0beta,
+        p->grid.as<C>(), p->us.as<T>(), p->vs.as<T>(), p->ax, p->ay, kb_table<T>(p),
         caller_order ? p->perm.as<int>() : nullptr, w.sub_bin.as<int>(), w.sub_off.as<int>(), w.list.as<int>(),
         tile, w.tiles_x, (C*)y, skip);
     L.done();
@@ -1002,7 +995,7 @@ static void grid_tj(purify_plan* p, const void* y, bool caller_order, const int*
     set_smem(k_grid_runs<T, J, W>, sm);
     Launch L(p, "grid");
     launch_dependent(k_grid_runs<T, J, W>, p->work.nsub, W * 32, sm, p->stream, 
-        (const C*)y, p->us.as<T>(), p->vs.as<T>(), p->ax, p->ay, p->kbp, p->beta, 1.0 / p->i0beta,
+        (const C*)y, p->us.as<T>(), p->vs.as<T>(), p->ax, p->ay, kb_table<T>(p),
         caller_order ? p->perm.as<int>() : nullptr, p->work.sub_bin.as<int>(), p->work.sub_off.as<int>(),
         p->work.list.as<int>(), tile, p->work.tiles_x, S, p->gacc.as<C>(), skip);
     L.done();
@@ -1051,8 +1044,8 @@ static void grid_sets_tj(purify_plan* p, const void* y, bool caller_order, const
     Launch L(p, FUSED ? "normal_gg" : "grid");
     launch_dependent(k_grid_sets<T, J, W, FUSED>, blocks, W * 32, 0, p->stream,
         (const C*)y, p->grid.as<C>(), rw.rec.as<typename RunRecOf<T>::type>(), rw.cell.as<int>(),
-        rw.start.as<int>(), rw.len.as<int>(), rw.nsets, caller_order ? p->perm.as<int>() : nullptr, p->kbp,
-        p->beta, 1.0 / p->i0beta, p->Kx, p->Ky, p->gacc.as<C>(), skip);
+        rw.start.as<int>(), rw.len.as<int>(), rw.nsets, caller_order ? p->perm.as<int>() : nullptr,
+        kb_table<T>(p), p->Kx, p->Ky, p->gacc.as<C>(), skip);
     L.done();
 }
 // Lane-per-run launches (kind 3: one lane per run, 4: two lanes per run,

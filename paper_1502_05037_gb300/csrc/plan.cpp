@@ -739,6 +739,7 @@ purify_plan* create_plan(const purify_plan_desc* d) {
         p->ax = AxisConst{(int)Kx, (float)cx, (float)(cx - (double)(float)cx), cx};
         p->ay = AxisConst{(int)Ky, (float)cy, (float)(cy - (double)(float)cy), cy};
         p->kbp = fit_kb_poly(p->J, p->beta, kb_poly_degree(p->J));
+        if (p->dtype == PURIFY_F64) p->kbpd = fit_kb_poly_d(p->J, p->beta);
         if (p->dtype == PURIFY_F32) finish_plan<float>(p); else finish_plan<double>(p);
         p->desc.u = p->desc.v = nullptr;
         p->desc.block_offsets = nullptr;

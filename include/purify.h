@@ -115,9 +115,10 @@ typedef struct {
     int32_t grid_mode;             /* the G^H decomposition in use: 1 tile subproblems, 2 runs,
                                       3..5 lanes, 6 deterministic lanes (as grid_mode of the
                                       description) */
-    int32_t degrid_mode;           /* the G decomposition in use: 1 tile subproblems, 3..5 lanes */
+    int32_t degrid_mode;           /* the G decomposition in use: 1 tile subproblems, 3..5 lanes,
+                                      8 visibilities sorted by cell (autotuned plans) */
     int32_t normal_mode;           /* the fused G^H G of the CG normal operator: 2 runs, 3..5 lanes,
-                                      6 deterministic lanes */
+                                      6 deterministic lanes, 7 a stencil on the grid (autotuned plans) */
     int32_t lane_tile;             /* grid tile edge grouping the runs of normal_mode 5 (else 0) */
     int32_t fft_rows_per_block;    /* FFT launch shape in use: row transforms per block, */
     int32_t fft_cols_per_block;    /* column transforms per block, */

@@ -204,11 +204,12 @@ purify_status purify_phi_normal(purify_plan* p, const void* x, void* out) {
         Staged xs = stage_in(p, x, rb * p->N, p->stage_in);
         Staged os = stage_out(p, out, rb * p->N, p->stage_out);
         // the forward row pass clears the accumulator that G^H G adds into
-        launch_scale_pad_rows(p, xs.dev, 1.0, nullptr, true, true);
-        launch_cols_fwd(p, nullptr);
-        launch_normal_gg(p, nullptr, true);
-        launch_cols_inv(p, nullptr);
-        launch_rows_inv_crop(p, os.dev, 1.0, 1, nullptr, 0.0, nullptr);
+        const bool half = normal_half(p);
+        launch_scale_pad_rows(p, xs.dev, 1.0, nullptr, true, true, nullptr, half);
+        launch_cols_fwd(p, nullptr, half);
+        launch_normal_gg(p, nullptr, true, half);
+        launch_cols_inv(p, nullptr, nullptr, half);
+        launch_rows_inv_crop(p, os.dev, 1.0, 1, nullptr, 0.0, nullptr, nullptr, true, half);
         finish_out(p, os, out, rb * p->N);
     });
 }

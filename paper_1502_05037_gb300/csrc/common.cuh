@@ -112,16 +112,19 @@ PURIFY_HD void split_coord(double coord, const AxisConst& ax, int J, int& k0, do
 // 3e-8 of it on [0, 1), below half an FP32 unit at 1.
 PURIFY_HD constexpr int kb_poly_deg(int J) { return J <= 3 ? 10 : (J == 4 ? 9 : 8); }
 
+// z = 2 phi - 1 of an offset phi in [0, 1), the polynomials' variable
+PURIFY_HD float kb_z(float phi) { return fmaf(2.0f, phi, -1.0f); }
+PURIFY_HD double kb_z(double phi) { return fma(2.0, phi, -1.0); }
+
 // Float weights of one axis from the per-tap polynomials (Horner in z).
 // The kernel is even in the tap offset, so tap J-1-a at z is tap a at -z
 // (the host table holds p_{J-1-a}(z) = p_a(-z) exactly): each mirrored pair
 // comes from the even and odd parts of p_a, p_a(+-z) = E(z^2) +- z O(z^2),
 // Horner in z^2 (the middle tap of an odd J is even).
 template <int J>
-__device__ __forceinline__ void kb_weights(const KbPoly& kp, float phi, float (&w)[J]) {
+__device__ __forceinline__ void kb_weights_z(const KbPoly& kp, float z, float (&w)[J]) {
     constexpr int DEG = kb_poly_deg(J);
     constexpr int DE = DEG & ~1, DO = (DEG & 1) ? DEG : DEG - 1;   // top even / odd degree
-    const float z = fmaf(2.0f, phi, -1.0f);
     const float z2 = z * z;
 #pragma unroll
     for (int a = 0; a < (J + 1) / 2; ++a) {
@@ -141,6 +144,11 @@ __device__ __forceinline__ void kb_weights(const KbPoly& kp, float phi, float (&
     }
 }
 
+template <int J>
+__device__ __forceinline__ void kb_weights(const KbPoly& kp, float phi, float (&w)[J]) {
+    kb_weights_z<J>(kp, kb_z(phi), w);
+}
+
 // Modified Bessel function I0 by its power series sum_k ((x/2)^2)^k / (k!)^2
 // (all terms positive; stops once a term no longer changes the sum).
 PURIFY_HD double bessel_i0_series(double x) {
@@ -155,10 +163,10 @@ PURIFY_HD double bessel_i0_series(double x) {
     return sum;
 }
 
-// Tap a's weight straight from the kernel definition
+// Tap a's weight at z straight from the kernel definition
 // g(t) = I0(beta sqrt(1 - (2t/J)^2)), normalised by I0(beta).
-__device__ __forceinline__ double kb_tap_exact(int J, int a, double beta, double inv_i0beta, double phi) {
-    const double t = phi + (0.5 * J - 1.0 - a);
+__device__ __forceinline__ double kb_tap_exact(int J, int a, double beta, double inv_i0beta, double z) {
+    const double t = 0.5 * z + (0.5 * J - 0.5 - a);
     const double r = 1.0 - (2.0 * t / J) * (2.0 * t / J);
     return r > 0.0 ? bessel_i0_series(beta * sqrt(r)) * inv_i0beta : (r == 0.0 ? inv_i0beta : 0.0);
 }
@@ -174,11 +182,11 @@ PURIFY_HD constexpr int kb_poly_deg_d(int J) { return J <= 2 ? 18 : (J <= 4 ? 17
 // it replaces about 25 terms with a division each (two SDMM iterations of the
 // 64 x 64 double problem, 8192 visibilities, J = 4: 8364 -> 1899 us).
 template <int J>
-__device__ __forceinline__ void kb_weights(const KbPolyD& kp, double phi, double (&w)[J]) {
+__device__ __forceinline__ void kb_weights_z(const KbPolyD& kp, double z, double (&w)[J]) {
     if (!kp.poly) {
 #pragma unroll 1
         for (int a = 0; a < J; ++a) {
-            const double v = kb_tap_exact(J, a, kp.beta, kp.inv_i0beta, phi);
+            const double v = kb_tap_exact(J, a, kp.beta, kp.inv_i0beta, z);
 #pragma unroll
             for (int b = 0; b < J; ++b) w[b] = b == a ? v : w[b];
         }
@@ -186,7 +194,6 @@ __device__ __forceinline__ void kb_weights(const KbPolyD& kp, double phi, double
     }
     constexpr int DEG = kb_poly_deg_d(J);
     constexpr int DE = DEG & ~1, DO = (DEG & 1) ? DEG : DEG - 1;
-    const double z = fma(2.0, phi, -1.0);
     const double z2 = z * z;
 #pragma unroll
     for (int a = 0; a < (J + 1) / 2; ++a) {
@@ -204,6 +211,10 @@ __device__ __forceinline__ void kb_weights(const KbPolyD& kp, double phi, double
             w[J - 1 - a] = e - oz;
         }
     }
+}
+template <int J>
+__device__ __forceinline__ void kb_weights(const KbPolyD& kp, double phi, double (&w)[J]) {
+    kb_weights_z<J>(kp, kb_z(phi), w);
 }
 
 }  // namespace purify

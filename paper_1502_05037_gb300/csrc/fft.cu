@@ -10,6 +10,11 @@
 //   rows_inv : inverse row transforms fused with Z^T (crop) and S, and in a
 //              CG step with the step's dot products and decision;
 // plus the plain in-place 2-D transform (purify_fft2).
+// Images are real, so the oversampled grid is Hermitian and the solver's
+// adjoint needs only the real part: the half-plane forms of the row passes
+// transform two image rows as one complex row and keep the HalfPlane columns
+// only; the column passes then run over those columns. (The adjoint's complex
+// image, purify_phi_adj, takes the whole plane.)
 //
 // Each transform is a length-N (N = 2^LOGN, 16 <= N <= 8192) Stockham
 // autosort FFT run by N / 8 threads holding eight values each; the length is
@@ -375,11 +380,75 @@ template <int N8> __device__ __forceinline__ void row_thread(int rb, int& i, int
     i = blockIdx.x * rb + f;
 }
 
+// The CG state a forward row pass works on (see CgFold): whether the pass has
+// anything to do, and the input pixel after the step's update.
+template <typename T> struct RowFold {
+    T *x, *r, *s, *p;
+    const T *u, *add;
+    bool on, first, pending;
+    T alpha, beta;
+    // false: the solve stopped at an earlier step (block 0 of this pass may
+    // set the flag meanwhile: each block reads it once)
+    __device__ __forceinline__ bool start(const CgFold& f, const int* skip) {
+        on = f.x != nullptr;
+        first = on && f.step == 0;
+        x = static_cast<T*>(f.x);
+        r = static_cast<T*>(f.r);
+        s = static_cast<T*>(f.s);
+        p = static_cast<T*>(f.p);
+        u = static_cast<const T*>(f.u);
+        add = static_cast<const T*>(f.add);
+        pending = false;
+        alpha = beta = T(0);
+        if (block_flag(first ? nullptr : skip)) return false;
+        if (on && !first) {
+            // the previous step's update (it did not stop the solve: checked above)
+            double al, be;
+            if (!cg_pending(f, al, be)) return false;
+            pending = true;
+            alpha = (T)al;
+            beta = (T)be;
+        }
+        if (first && blockIdx.x == 0 && threadIdx.x == 0) f.flags[F_CGDONE] = 0;   // the next kernels read it
+        return true;
+    }
+    // Chronopoulos-Gear update of pixel idx, then the new r
+    __device__ __forceinline__ T pixel(size_t idx) const {
+        T rv = r[idx];
+        if (first) {
+            if (add) {
+                rv += add[idx];
+                r[idx] = rv;
+            }
+            p[idx] = T(0);
+            s[idx] = T(0);
+        } else if (pending) {
+            const T pv = rv + beta * p[idx];
+            const T sv = u[idx] + beta * s[idx];
+            p[idx] = pv;
+            s[idx] = sv;
+            x[idx] += alpha * pv;
+            rv = rv - alpha * sv;
+            r[idx] = rv;
+        }
+        return rv;
+    }
+};
+
+// Block b clears rows [b Ky/gridDim, (b+1) Ky/gridDim) of a Ky x ld grid of
+// C (Ky is a multiple of the block count) in 16-byte stores.
+template <typename C> __device__ __forceinline__ void clear_rows(C* grid, int Ky, int ld) {
+    const int per = Ky / gridDim.x;
+    float4* g = reinterpret_cast<float4*>(grid + (size_t)blockIdx.x * per * ld);
+    const int n16 = per * ld * (int)sizeof(C) / 16;
+    for (int t = threadIdx.x; t < n16; t += blockDim.x) g[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 // S Z and the forward row FFT: rows [i0, i0+rb) of the image to rows[i][0..Kx).
 // With a CG fold (fold.x set) the input is the residual r after the step's
-// update (see CgFold), not x. When zero_grid != null block b also clears rows
-// [b Ky/gridDim, (b+1) Ky/gridDim) of that Ky x Kx complex grid (the gridding
-// accumulator of the same CG step, or of the adjoint that follows Phi).
+// update (see CgFold), not x. When zero_grid != null the pass also clears
+// that Ky x Kx complex grid (the gridding accumulator of the same CG step, or
+// of the adjoint that follows Phi).
 template <typename T, int LX>
 __global__ void __launch_bounds__(1024) k_rows_fwd(const T* __restrict__ x, typename cplx_of<T>::type* __restrict__ rows,
                            const T* __restrict__ sx, const T* __restrict__ sy,
@@ -389,38 +458,10 @@ __global__ void __launch_bounds__(1024) k_rows_fwd(const T* __restrict__ x, type
     using C = typename cplx_of<T>::type;
     constexpr int Kx = 1 << LX, N8 = Kx >> 3;
     pdl_wait();
-    // step 0 starts the solve; later steps first apply the previous step's
-    // update unless it met the stop test (see CgFold)
-    const bool first = fold.x && fold.step == 0;
-    T* const fx = static_cast<T*>(fold.x);
-    T* const fr = static_cast<T*>(fold.r);
-    T* const fs = static_cast<T*>(fold.s);
-    T* const pdir = static_cast<T*>(fold.p);
-    const T* const fu = static_cast<const T*>(fold.u);
-    const T* const fadd = static_cast<const T*>(fold.add);
-    // stopped at an earlier step (block 0 of this pass may set the flag
-    // meanwhile: each block reads it once)
-    if (block_flag(first ? nullptr : skip)) return;
-    bool pending = false;
-    T alpha = T(0), cbeta = T(0);
-    if (fold.x && !first) {
-        // the previous step's update (it did not stop the solve: checked above)
-        double al, be;
-        if (!cg_pending(fold, al, be)) return;
-        pending = true;
-        alpha = (T)al;
-        cbeta = (T)be;
-    }
-    if (first && blockIdx.x == 0 && threadIdx.x == 0) fold.flags[F_CGDONE] = 0;   // the next kernels read it
+    RowFold<T> cg;
+    if (!cg.start(fold, skip)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (zero_grid) {
-        // whole rows per block (Ky is a multiple of the block count), in
-        // 16-byte stores
-        const int per = Ky / gridDim.x;
-        float4* g = reinterpret_cast<float4*>(zero_grid + (size_t)blockIdx.x * per * Kx);
-        const int n16 = per * Kx * (int)sizeof(C) / 16;
-        for (int t = threadIdx.x; t < n16; t += blockDim.x) g[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    if (zero_grid) clear_rows(zero_grid, Ky, Kx);
     int i0, t, f;
     row_thread<N8>(rb, i0, t, f);
     // S Z of pixel p1 of image row i (p1 < Kx/2 exactly when k < 4)
@@ -429,31 +470,7 @@ __global__ void __launch_bounds__(1024) k_rows_fwd(const T* __restrict__ x, type
         const int j = (k < 4 ? p1 : p1 - Kx) + nx / 2;
         if (j < 0 || j >= nx) return T(0);
         const size_t idx = (size_t)i * nx + j;
-        T xv;
-        if (fold.x) {
-            // Chronopoulos-Gear update, then the transform of the new r
-            T rv = fr[idx];
-            if (first) {
-                if (fadd) {
-                    rv += fadd[idx];
-                    fr[idx] = rv;
-                }
-                pdir[idx] = T(0);
-                fs[idx] = T(0);
-            } else if (pending) {
-                const T pv = rv + cbeta * pdir[idx];
-                const T sv = fu[idx] + cbeta * fs[idx];
-                pdir[idx] = pv;
-                fs[idx] = sv;
-                fx[idx] += alpha * pv;
-                rv = rv - alpha * sv;
-                fr[idx] = rv;
-            }
-            xv = rv;
-        } else {
-            xv = x[idx];
-        }
-        return xv * sx[j] * (sy[i] * scale);
+        return (cg.on ? cg.pixel(idx) : x[idx]) * sx[j] * (sy[i] * scale);
     };
     C* buf = reinterpret_cast<C*>(smem_raw) + f * fft_padded(Kx);
     C* const out = rows + (size_t)i0 * Kx;
@@ -463,13 +480,64 @@ __global__ void __launch_bounds__(1024) k_rows_fwd(const T* __restrict__ x, type
     pdl_trigger();
 }
 
+// The half-plane form: image rows 2i and 2i + 1 (both real) as the real and
+// imaginary part of one transform Z; their spectra are
+//   R_2i[k] = (Z[k] + conj Z[-k]) / 2,  R_2i+1[k] = (Z[k] - conj Z[-k]) / 2i,
+// of which columns k = j - hp.off, j < hp.W, are written (rows[i][j]). A block
+// holds rb pairs. Half the transforms and half the columns of k_rows_fwd; the
+// passes are bound by latency and L2, so both count (1024 x 1024: 18 -> 13 us).
+template <typename T, int LX>
+__global__ void __launch_bounds__(1024) k_rows_fwd_half(const T* __restrict__ x,
+                           typename cplx_of<T>::type* __restrict__ rows, const T* __restrict__ sx,
+                           const T* __restrict__ sy, const typename cplx_of<T>::type* __restrict__ tw, int nx,
+                           int rb, int alt, T scale, const int* __restrict__ skip,
+                           typename cplx_of<T>::type* __restrict__ zero_grid, int Ky, CgFold fold, HalfPlane hp) {
+    using C = typename cplx_of<T>::type;
+    constexpr int Kx = 1 << LX, N8 = Kx >> 3;
+    pdl_wait();
+    RowFold<T> cg;
+    if (!cg.start(fold, skip)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (zero_grid) clear_rows(zero_grid, Ky, hp.W);
+    int i, t, f;
+    row_thread<N8>(rb, i, t, f);
+    auto pix = [&](int row, int k, int p1) -> T {
+        const int j = (k < 4 ? p1 : p1 - Kx) + nx / 2;
+        if (j < 0 || j >= nx) return T(0);
+        const size_t idx = (size_t)row * nx + j;
+        return (cg.on ? cg.pixel(idx) : x[idx]) * sx[j] * (sy[row] * scale);
+    };
+    C* const buf = reinterpret_cast<C*>(smem_raw) + f * fft_padded(Kx);
+    // the transform's output goes back to shared memory: the buffer its last
+    // stage does not read (see fft_core), or the only one after a barrier
+    constexpr int NST = (LX - (LX % 3 == 0 ? 3 : LX % 3)) / 3;
+    C* const z = (alt && NST % 2 == 1) ? buf + alt : buf;
+    auto load = [&](int k, int p1) -> C { return cmake<C>(pix(2 * i, k, p1), pix(2 * i + 1, k, p1)); };
+    auto store = [&](int q, int k, C v) {
+        if (q == 0 && !alt) __syncthreads();
+        z[fft_pad(k)] = v;
+    };
+    fft_core<C, false, LX>(t, tw, load, store, FftSlots<C>{buf, 1, alt});
+    __syncthreads();
+    C* const r0 = rows + (size_t)(2 * i) * hp.W;
+    C* const r1 = r0 + hp.W;
+    for (int j = t; j < hp.W; j += N8) {
+        const int k = (j - hp.off) & (Kx - 1);
+        const C a = z[fft_pad(k)], b = z[fft_pad((Kx - k) & (Kx - 1))];
+        r0[j] = cmake<C>(T(0.5) * (a.x + b.x), T(0.5) * (a.y - b.y));
+        r1[j] = cmake<C>(T(0.5) * (a.y + b.y), T(0.5) * (b.x - a.x));
+    }
+    pdl_trigger();
+}
+
 // Column kernels: a block holds cb adjacent columns of length Ky = 2^LY.
 // With W = 1 thread (t, f) = (tid / cb, tid mod cb) runs column f, element
 // n in shared slot pad(n) * cb + f; with W = 2 (FP32) thread
 // (t, f) = (tid / (cb/2), tid mod (cb/2)) runs columns 2f and 2f + 1 as one
 // pair with 16-byte global accesses, element n in float4 slot
 // pad(n) * (cb/2) + f. A warp's global accesses cover consecutive cells of
-// each row. The second buffer (alt > 0) follows the first.
+// each row (`ld` cells: the whole plane or the half plane's columns). The
+// second buffer (alt > 0) follows the first.
 template <int W> __device__ __forceinline__ void col_thread(int cb, int& c0, int& t, int& f) {
     const int cp = cb / W;
     t = threadIdx.x / cp;
@@ -482,7 +550,7 @@ template <int W> __device__ __forceinline__ void col_thread(int cb, int& c0, int
 template <typename T, int LY, int W>
 __global__ void __launch_bounds__(1024) k_cols_fwd(const typename cplx_of<T>::type* __restrict__ rows,
                            typename cplx_of<T>::type* __restrict__ grid,
-                           const typename cplx_of<T>::type* __restrict__ tw, int ny, int Kx,
+                           const typename cplx_of<T>::type* __restrict__ tw, int ny, int ld,
                            int cb, int alt, const int* __restrict__ skip) {
     using C = typename cplx_of<T>::type;
     constexpr int Ky = 1 << LY;
@@ -500,20 +568,20 @@ __global__ void __launch_bounds__(1024) k_cols_fwd(const typename cplx_of<T>::ty
         C* buf = reinterpret_cast<C*>(smem_raw);
         auto load = [&](int k, int n) -> C {
             const int i = src_row(k, n);
-            return i >= 0 ? rows[(size_t)i * Kx + c] : cmake<C>(T(0), T(0));
+            return i >= 0 ? rows[(size_t)i * ld + c] : cmake<C>(T(0), T(0));
         };
-        auto store = [&](int, int k, C v) { grid[(size_t)k * Kx + c] = v; };
+        auto store = [&](int, int k, C v) { grid[(size_t)k * ld + c] = v; };
         fft_core<C, false, LY>(t, tw, load, store, FftSlots<C>{buf + f, cb, alt});
     } else {
         float4* buf = reinterpret_cast<float4*>(smem_raw);
         auto load = [&](int k, int n) -> P2 {
             const int i = src_row(k, n);
             if (i < 0) return P2{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-            const float4 q = *reinterpret_cast<const float4*>(rows + (size_t)i * Kx + c);
+            const float4 q = *reinterpret_cast<const float4*>(rows + (size_t)i * ld + c);
             return P2{make_float2(q.x, q.z), make_float2(q.y, q.w)};
         };
         auto store = [&](int, int k, P2 v) {
-            *reinterpret_cast<float4*>(grid + (size_t)k * Kx + c) = make_float4(v.re.x, v.im.x, v.re.y, v.im.y);
+            *reinterpret_cast<float4*>(grid + (size_t)k * ld + c) = make_float4(v.re.x, v.im.x, v.re.y, v.im.y);
         };
         fft_core2<false, LY>(t, tw, load, store, FftSlots2{buf + f, cb / 2, alt / 2});
     }
@@ -525,7 +593,7 @@ __global__ void __launch_bounds__(1024) k_cols_fwd(const typename cplx_of<T>::ty
 template <typename T, int LY, int W>
 __global__ void __launch_bounds__(1024) k_cols_inv(const typename cplx_of<T>::type* __restrict__ grid,
                            typename cplx_of<T>::type* __restrict__ rows,
-                           const typename cplx_of<T>::type* __restrict__ tw, int ny, int Kx,
+                           const typename cplx_of<T>::type* __restrict__ tw, int ny, int ld,
                            int cb, int alt, const int* __restrict__ skip, const T* __restrict__ mult) {
     using C = typename cplx_of<T>::type;
     constexpr int Ky = 1 << LY;
@@ -542,20 +610,20 @@ __global__ void __launch_bounds__(1024) k_cols_inv(const typename cplx_of<T>::ty
     if constexpr (W == 1) {
         C* buf = reinterpret_cast<C*>(smem_raw);
         auto load = [&](int, int k) -> C {
-            const size_t g = (size_t)k * Kx + c;
+            const size_t g = (size_t)k * ld + c;
             C v = grid[g];
             if (mult) v = cscale(v, mult[g]);
             return v;
         };
         auto store = [&](int, int p2, C v) {
             const int i = dst_row(p2);
-            if (i >= 0) rows[(size_t)i * Kx + c] = v;
+            if (i >= 0) rows[(size_t)i * ld + c] = v;
         };
         fft_core<C, true, LY>(t, tw, load, store, FftSlots<C>{buf + f, cb, alt});
     } else {
         float4* buf = reinterpret_cast<float4*>(smem_raw);
         auto load = [&](int, int k) -> P2 {
-            const size_t g = (size_t)k * Kx + c;
+            const size_t g = (size_t)k * ld + c;
             float4 q = *reinterpret_cast<const float4*>(grid + g);
             if (mult) {
                 const float2 m = *reinterpret_cast<const float2*>(mult + g);
@@ -566,11 +634,27 @@ __global__ void __launch_bounds__(1024) k_cols_inv(const typename cplx_of<T>::ty
         auto store = [&](int, int p2, P2 v) {
             const int i = dst_row(p2);
             if (i >= 0)
-                *reinterpret_cast<float4*>(rows + (size_t)i * Kx + c) = make_float4(v.re.x, v.im.x, v.re.y, v.im.y);
+                *reinterpret_cast<float4*>(rows + (size_t)i * ld + c) = make_float4(v.re.x, v.im.x, v.re.y, v.im.y);
         };
         fft_core2<true, LY>(t, tw, load, store, FftSlots2{buf + f, cb / 2, alt / 2});
     }
     pdl_trigger();
+}
+
+// Chronopoulos-Gear partials of an inverse row pass (see CgFold): the block's
+// sums of gamma = r.r and delta = r.A r; the last block reduces them all and
+// decides the step.
+template <typename T> __device__ __forceinline__ void cg_partials(const CgFold& cgf, T gam, T del) {
+    const double b0 = block_sum_t(gam);
+    const double b1 = block_sum_t(del);
+    if (threadIdx.x == 0) {
+        cgf.part[2 * blockIdx.x] = b0;
+        cgf.part[2 * blockIdx.x + 1] = b1;
+    }
+    if (arrive_last(cgf.counter)) {
+        cg_decide(cgf, cgf.step, gridDim.x);
+        if (threadIdx.x == 0) *cgf.counter = 0;
+    }
 }
 
 // Inverse row FFT of image rows [i0, i0+rb), then Z^T and S:
@@ -618,20 +702,65 @@ __global__ void __launch_bounds__(MAXT) k_rows_inv(const typename cplx_of<T>::ty
     auto load = [&](int, int k) -> C { return in[k]; };
     auto store = [&](int, int p1, C v) { emit(i0, p1, v.x, v.y); };
     fft_core<C, true, LX>(t, tw, load, store, FftSlots<C>{buf, 1, alt});
-    if (cg) {
-        // Chronopoulos-Gear partials (see CgFold): gamma = r.r, delta = r.A r;
-        // the consumer of this step's scalars reduces them
-        const double b0 = block_sum_t(gacc2);
-        const double b1 = block_sum_t(dacc);
-        if (threadIdx.x == 0) {
-            cgf.part[2 * blockIdx.x] = b0;
-            cgf.part[2 * blockIdx.x + 1] = b1;
+    if (cg) cg_partials(cgf, gacc2, dacc);
+    pdl_trigger();
+}
+
+// The half-plane form of k_rows_inv for a real image (out_mode 1): the real
+// part of the inverse transform of row i's stored columns r_i is the inverse
+// transform of their Hermitian part h_i[k] = (r_i[k] + conj r_i[-k]) / 2
+// (column k held at j = k + off, and also at j = k - Kx + off where the
+// stored columns pass 0), and two rows share one complex transform,
+// h_2i + i h_2i+1.
+template <typename T, int LX, int MAXT>
+__global__ void __launch_bounds__(MAXT) k_rows_inv_half(const typename cplx_of<T>::type* __restrict__ rows,
+                           T* __restrict__ out, const T* __restrict__ sx, const T* __restrict__ sy,
+                           const typename cplx_of<T>::type* __restrict__ tw, int nx, int rb, int alt, T scale,
+                           const T* __restrict__ add, T add_coef, const int* __restrict__ skip, CgFold cgf,
+                           HalfPlane hp) {
+    using C = typename cplx_of<T>::type;
+    constexpr int Kx = 1 << LX, N8 = Kx >> 3;
+    pdl_wait();
+    if (skip && *skip) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int i, t, f;
+    row_thread<N8>(rb, i, t, f);
+    T dacc = 0, gacc2 = 0;   // add.out, and with the folded CG add.add (add = r, out = A r)
+    const bool cg = cgf.part != nullptr;
+    auto emit = [&](int row, int j, T v) {
+        const size_t idx = (size_t)row * nx + j;
+        T r = v * (sx[j] * (sy[row] * scale));
+        if (add) {
+            const T a = add[idx];
+            r += add_coef * a;
+            dacc += a * r;
+            if (cg) gacc2 += a * a;
         }
-        if (arrive_last(cgf.counter)) {
-            cg_decide(cgf, cgf.step, gridDim.x);
-            if (threadIdx.x == 0) *cgf.counter = 0;
-        }
-    }
+        out[idx] = r;
+    };
+    const C* const r0 = rows + (size_t)(2 * i) * hp.W;
+    const C* const r1 = r0 + hp.W;
+    auto column = [&](const C* r, int k) -> C {
+        C v = cmake<C>(T(0), T(0));
+        const int j = k + hp.off;
+        if (j < hp.W0) v = r[j];
+        if (j >= Kx) v = cadd(v, r[j - Kx]);
+        return v;
+    };
+    auto load = [&](int, int k) -> C {
+        const int m = (Kx - k) & (Kx - 1);
+        const C a = column(r0, k), am = column(r0, m), b = column(r1, k), bm = column(r1, m);
+        return cmake<C>(T(0.5) * ((a.x + am.x) - (b.y - bm.y)), T(0.5) * ((a.y - am.y) + (b.x + bm.x)));
+    };
+    auto store = [&](int, int p1, C v) {
+        const int j = (p1 + nx / 2) & (Kx - 1);
+        if (j >= nx) return;
+        emit(2 * i, j, v.x);
+        emit(2 * i + 1, j, v.y);
+    };
+    C* buf = reinterpret_cast<C*>(smem_raw) + f * fft_padded(Kx);
+    fft_core<C, true, LX>(t, tw, load, store, FftSlots<C>{buf, 1, alt});
+    if (cg) cg_partials(cgf, gacc2, dacc);
     pdl_trigger();
 }
 
@@ -744,9 +873,17 @@ template <typename T> static int plan_rows_per_block(const purify_plan* p) {
     while (p->ny % rb) rb >>= 1;
     return rb;
 }
+// row pairs per block of the half-plane passes
+template <typename T> static int plan_pairs_per_block(const purify_plan* p) {
+    int rb = p->fft_rb > 0 ? p->fft_rb : rows_per_block<T>(p->ny / 2, p->Kx);
+    while ((p->ny / 2) % rb) rb >>= 1;
+    return rb;
+}
 template <typename T> static int plan_cols_per_block(const purify_plan* p) {
     return p->fft_cb > 0 ? p->fft_cb : cols_per_block<T>(p->Ky, p->Kx);
 }
+// row stride and number of columns of the grid a column pass runs over
+static int plan_cols(const purify_plan* p, bool half) { return half ? p->half.W : p->Kx; }
 // columns per thread: the tuned choice, else two (packed) for FP32 blocks of
 // an even number of columns
 template <typename T> static int col_lanes(int cb, int tuned) {
@@ -756,25 +893,36 @@ template <typename T> static int col_lanes(int cb, int tuned) {
 
 template <typename T>
 static void rows_fwd_t(purify_plan* p, const void* x, double scale, const int* skip, bool corr, bool zero_acc,
-                       const CgFold* fold) {
+                       const CgFold* fold, bool half) {
     using C = typename cplx_of<T>::type;
-    const int rb = plan_rows_per_block<T>(p);
+    const int rb = half ? plan_pairs_per_block<T>(p) : plan_rows_per_block<T>(p);
     const int alt = fft_alt(rb, p->Kx, sizeof(C));
     const size_t sm = fft_smem(rb, p->Kx, sizeof(C), alt);
     with_log2(p->Kx, [&](auto lg) {
-        auto kern = k_rows_fwd<T, decltype(lg)::value>;
-        set_fft_smem(kern, sm);
-        Launch L(p, "fft_rows_fwd");
-        launch_dependent(kern, p->ny / rb, rb * (p->Kx / 8), sm, p->stream,
-            (const T*)x, p->rows.as<C>(), corr ? p->sx.as<T>() : p->onesx.as<T>(),
-            corr ? p->sy.as<T>() : p->onesy.as<T>(), p->twx.as<C>(), p->nx, p->ny,
-            rb, alt, (T)scale, skip, zero_acc ? p->gacc.as<C>() : nullptr, p->Ky,
-            fold ? *fold : CgFold());
-        L.done();
+        constexpr int LX = decltype(lg)::value;
+        const T* sx = corr ? p->sx.as<T>() : p->onesx.as<T>();
+        const T* sy = corr ? p->sy.as<T>() : p->onesy.as<T>();
+        C* acc = zero_acc ? p->gacc.as<C>() : nullptr;
+        const CgFold cg = fold ? *fold : CgFold();
+        if (half) {
+            auto kern = k_rows_fwd_half<T, LX>;
+            set_fft_smem(kern, sm);
+            Launch L(p, "fft_rows_fwd");
+            launch_dependent(kern, p->ny / 2 / rb, rb * (p->Kx / 8), sm, p->stream, (const T*)x, p->rows.as<C>(), sx,
+                             sy, p->twx.as<C>(), p->nx, rb, alt, (T)scale, skip, acc, p->Ky, cg, p->half);
+            L.done();
+        } else {
+            auto kern = k_rows_fwd<T, LX>;
+            set_fft_smem(kern, sm);
+            Launch L(p, "fft_rows_fwd");
+            launch_dependent(kern, p->ny / rb, rb * (p->Kx / 8), sm, p->stream, (const T*)x, p->rows.as<C>(), sx, sy,
+                             p->twx.as<C>(), p->nx, p->ny, rb, alt, (T)scale, skip, acc, p->Ky, cg);
+            L.done();
+        }
     });
 }
 
-template <typename T> static void cols_fwd_t(purify_plan* p, const int* skip) {
+template <typename T> static void cols_fwd_t(purify_plan* p, const int* skip, bool half) {
     using C = typename cplx_of<T>::type;
     const int cb = plan_cols_per_block<T>(p);
     const int alt = fft_alt(cb, p->Ky, sizeof(C));
@@ -786,13 +934,13 @@ template <typename T> static void cols_fwd_t(purify_plan* p, const int* skip) {
         if constexpr (sizeof(T) == 4) { if (w == 2) kern = k_cols_fwd<T, LY, 2>; }
         set_fft_smem(kern, sm);
         Launch L(p, "fft_cols_fwd");
-        launch_dependent(kern, p->Kx / cb, cb / w * (p->Ky / 8), sm, p->stream, p->rows.as<C>(), p->grid.as<C>(),
-                         p->twy.as<C>(), p->ny, p->Kx, cb, alt, skip);
+        launch_dependent(kern, plan_cols(p, half) / cb, cb / w * (p->Ky / 8), sm, p->stream, p->rows.as<C>(),
+                         p->grid.as<C>(), p->twy.as<C>(), p->ny, plan_cols(p, half), cb, alt, skip);
         L.done();
     });
 }
 
-template <typename T> static void cols_inv_t(purify_plan* p, const int* skip, const void* mult) {
+template <typename T> static void cols_inv_t(purify_plan* p, const int* skip, const void* mult, bool half) {
     using C = typename cplx_of<T>::type;
     const int cb = plan_cols_per_block<T>(p);
     const int alt = fft_alt(cb, p->Ky, sizeof(C));
@@ -806,31 +954,42 @@ template <typename T> static void cols_inv_t(purify_plan* p, const int* skip, co
         if constexpr (sizeof(T) == 4) { if (w == 2) kern = k_cols_inv<T, LY, 2>; }
         set_fft_smem(kern, sm);
         Launch L(p, "fft_cols_inv");
-        launch_dependent(kern, p->Kx / cb, cb / w * (p->Ky / 8), sm, p->stream, src, p->rows.as<C>(),
-                         p->twy.as<C>(), p->ny, p->Kx, cb, alt, skip, (const T*)mult);
+        launch_dependent(kern, plan_cols(p, half) / cb, cb / w * (p->Ky / 8), sm, p->stream, src, p->rows.as<C>(),
+                         p->twy.as<C>(), p->ny, plan_cols(p, half), cb, alt, skip, (const T*)mult);
         L.done();
     });
 }
 
 template <typename T>
 static void rows_inv_t(purify_plan* p, void* out, double scale, int out_mode, const void* add, double add_coef,
-                       const int* skip, const CgFold* cg, bool corr) {
+                       const int* skip, const CgFold* cg, bool corr, bool half) {
     using C = typename cplx_of<T>::type;
-    const int rb = plan_rows_per_block<T>(p);
+    const int rb = half ? plan_pairs_per_block<T>(p) : plan_rows_per_block<T>(p);
     const int alt = fft_alt(rb, p->Kx, sizeof(C));
     const size_t sm = fft_smem(rb, p->Kx, sizeof(C), alt);
     const int nt = rb * (p->Kx / 8);
     with_log2(p->Kx, [&](auto lg) {
         constexpr int LX = decltype(lg)::value;
+        const T* sx = corr ? p->sx.as<T>() : p->onesx.as<T>();
+        const T* sy = corr ? p->sy.as<T>() : p->onesy.as<T>();
+        const CgFold fold = cg ? *cg : CgFold();
         // blocks of at most 512 threads may take more than 64 registers
-        auto kern = nt <= 512 ? k_rows_inv<T, LX, 512> : k_rows_inv<T, LX, 1024>;
-        set_fft_smem(kern, sm);
-        Launch L(p, "fft_rows_inv");
-        launch_dependent(kern, p->ny / rb, nt, sm, p->stream, p->rows.as<C>(), out,
-                         corr ? p->sx.as<T>() : p->onesx.as<T>(), corr ? p->sy.as<T>() : p->onesy.as<T>(),
-                         p->twx.as<C>(), p->nx, p->ny, rb, alt, (T)scale, out_mode, (const T*)add,
-                         (T)add_coef, skip, cg ? *cg : CgFold());
-        L.done();
+        if (half) {
+            auto kern = nt <= 512 ? k_rows_inv_half<T, LX, 512> : k_rows_inv_half<T, LX, 1024>;
+            set_fft_smem(kern, sm);
+            Launch L(p, "fft_rows_inv");
+            launch_dependent(kern, p->ny / 2 / rb, nt, sm, p->stream, p->rows.as<C>(), (T*)out, sx, sy,
+                             p->twx.as<C>(), p->nx, rb, alt, (T)scale, (const T*)add, (T)add_coef, skip, fold,
+                             p->half);
+            L.done();
+        } else {
+            auto kern = nt <= 512 ? k_rows_inv<T, LX, 512> : k_rows_inv<T, LX, 1024>;
+            set_fft_smem(kern, sm);
+            Launch L(p, "fft_rows_inv");
+            launch_dependent(kern, p->ny / rb, nt, sm, p->stream, p->rows.as<C>(), out, sx, sy, p->twx.as<C>(), p->nx,
+                             p->ny, rb, alt, (T)scale, out_mode, (const T*)add, (T)add_coef, skip, fold);
+            L.done();
+        }
     });
 }
 
@@ -846,26 +1005,22 @@ void fft_launch_shape(const purify_plan* p, int& rb, int& cb, int& cw) {
     }
 }
 
-int rows_inv_blocks(purify_plan* p) {
-    const int rb = p->dtype == PURIFY_F32 ? plan_rows_per_block<float>(p) : plan_rows_per_block<double>(p);
-    return p->ny / rb;
-}
-
 void launch_scale_pad_rows(purify_plan* p, const void* x, double scale, const int* skip, bool corr, bool zero_acc,
-                           const CgFold* fold) {
-    if (p->dtype == PURIFY_F32) rows_fwd_t<float>(p, x, scale, skip, corr, zero_acc, fold);
-    else rows_fwd_t<double>(p, x, scale, skip, corr, zero_acc, fold);
+                           const CgFold* fold, bool half) {
+    if (p->dtype == PURIFY_F32) rows_fwd_t<float>(p, x, scale, skip, corr, zero_acc, fold, half);
+    else rows_fwd_t<double>(p, x, scale, skip, corr, zero_acc, fold, half);
 }
-void launch_cols_fwd(purify_plan* p, const int* skip) {
-    if (p->dtype == PURIFY_F32) cols_fwd_t<float>(p, skip); else cols_fwd_t<double>(p, skip);
+void launch_cols_fwd(purify_plan* p, const int* skip, bool half) {
+    if (p->dtype == PURIFY_F32) cols_fwd_t<float>(p, skip, half); else cols_fwd_t<double>(p, skip, half);
 }
-void launch_cols_inv(purify_plan* p, const int* skip, const void* mult) {
-    if (p->dtype == PURIFY_F32) cols_inv_t<float>(p, skip, mult); else cols_inv_t<double>(p, skip, mult);
+void launch_cols_inv(purify_plan* p, const int* skip, const void* mult, bool half) {
+    if (p->dtype == PURIFY_F32) cols_inv_t<float>(p, skip, mult, half);
+    else cols_inv_t<double>(p, skip, mult, half);
 }
 void launch_rows_inv_crop(purify_plan* p, void* out, double scale, int out_mode, const void* add, double add_coef,
-                          const int* skip, const CgFold* cg, bool corr) {
-    if (p->dtype == PURIFY_F32) rows_inv_t<float>(p, out, scale, out_mode, add, add_coef, skip, cg, corr);
-    else rows_inv_t<double>(p, out, scale, out_mode, add, add_coef, skip, cg, corr);
+                          const int* skip, const CgFold* cg, bool corr, bool half) {
+    if (p->dtype == PURIFY_F32) rows_inv_t<float>(p, out, scale, out_mode, add, add_coef, skip, cg, corr, half);
+    else rows_inv_t<double>(p, out, scale, out_mode, add, add_coef, skip, cg, corr, half);
 }
 
 template <typename T, bool INV> static void fft2_dir(purify_plan* p, void* grid) {

@@ -84,15 +84,15 @@ struct RunWork {
     DevBuf rec, cell, start, len;
 };
 
-// Lane-per-run work (FP32 plans, J <= 6): the same runs, `width` per warp
+// Lane-per-run work (FP32 plans, J <= 6; the half-plane's for every plan, in
+// its precision): the same runs, `width` per warp
 // set (32 / lanes per run). Set s holds record rows [row0, row0 + lmax) with
 // lmax its longest run; the record of run width s + r at step k is in
-// record row row0 + k: with width 32 the float2 (phx, phy) at
-// rec[(row0 + k) * 32 + r], with width 16 (a lane pair per run) phx at
-// float (row0 + k) * 32 + r and phy at float (row0 + k) * 32 + 16 + r, so
-// one step of a warp reads one record row (8 bytes per run), each lane of a
-// pair its own axis. Records past a run's end are padding (zero offsets,
-// index -1). run_cl[width s + r] = (cell, len), the cell packed as
+// record row row0 + k and holds z = 2 phi - 1 of both axes: with width 32 the
+// pair (zx, zy) at rec[(row0 + k) * 32 + r], with width 16 (a lane pair per
+// run) zx at scalar (row0 + k) * 32 + r and zy at scalar (row0 + k) * 32 + 16
+// + r, so one step of a warp reads one record row, each lane of a pair its
+// own axis. Records past a run's end are padding (zero offsets, index -1). run_cl[width s + r] = (cell, len), the cell packed as
 // (cy << 16) | cx; idx / idx_caller give each record's visibility in
 // internal / caller order. Set order: runs sorted by length (longest
 // first), or with tile > 0 grouped by grid tile of that edge (tiles in
@@ -124,6 +124,39 @@ struct LaneWork {
         cstart.release();
         clist.release();
     }
+};
+
+// Columns of the half-plane grid. A real image's visibility at (-u, -v) is
+// the conjugate of the one at (u, v), so Phi, the real part of its adjoint and
+// the normal operator can move every visibility whose first-tap column lies in
+// the upper half (cx >= Kx / 2) to its mirrored footprint: first tap
+// (Kx - cx - J + 1, Ky - cy - J + 1), offsets z = 2 phi - 1 negated (the
+// mirrored taps have the same weights, exactly), value conjugated. All taps
+// then lie in columns k = -(J - 2) .. Kx / 2 + J - 2, stored at j = k + off
+// without wrapping, W0 of them (row stride W, a multiple of 16 cells with at
+// least eight unused columns past W0). Half the columns to transform and to keep in L2,
+// and twice the visibilities per first-tap cell.
+struct HalfPlane {
+    int off = 0, W0 = 0, W = 0;
+};
+// index code of a lane record: the visibility, folded ones as -2 - m, -1 padding
+PURIFY_HD int fold_index(int m) { return -2 - m; }
+
+// The folded visibilities in the order of their first-tap cells (row * W +
+// column), `per` of a cell to an entry (a cell's last entry padded with code
+// -1): per entry the cell ((row << 16) | column), per visibility the offsets z
+// of both axes and its index code in internal and caller order.
+struct SortedWork {
+    int64_t n = 0;
+    int per = 1;
+    DevBuf z, cell, idx, idx_caller;
+};
+
+// G^H G as a stencil on the half plane (stencil.cu): the coefficients, and a
+// byte per block that has any.
+struct Stencil {
+    bool on = false;
+    DevBuf coef, used;
 };
 
 // Block groups of the stochastic block-subset iterations: block i belongs to
@@ -234,14 +267,21 @@ struct purify_plan {
     purify::RunWork runs;             // run-ordered work of the fused normal operator
     purify::LaneWork lanes[3];        // lane-per-run forms of the same runs (FP32, J <= 6): one lane
                                       // per run; two lanes per run; two, sets grouped by tile
+    bool half_on = false;             // the half-plane path is built (autotuned plans)
+    purify::HalfPlane half;
+    purify::LaneWork half_lanes;      // lane pairs of the folded visibilities (any dtype, J;
+                                      // internal order only)
+    purify::SortedWork half_sorted;   // the same visibilities sorted by cell
+    purify::Stencil stencil;          // G^H G of the half plane as a stencil, where it is the faster form
     purify::DevBuf det_patch;         // run patches of the deterministic lane form (float2)
-    int normal_kind = 2;              // G^H G: 2 run sets, 3..5 lanes (as lanes[kind - 3]), 6 the
-                                      // deterministic lane pairs (lanes[1]); autotuned or forced
+    int normal_kind = 2;              // G^H G: 2 run sets, 3..5 lanes (as lanes[kind - 3]; on the half plane
+                                      // half_lanes), 6 the deterministic lane pairs (lanes[1]), 7 the
+                                      // half plane's stencil
     int group_count = 0;              // G of group_lanes / group_chunks (0: not built)
     std::vector<purify::LaneWork> group_lanes;
     std::vector<purify::GroupChunks> group_chunks;
     int grid_kind = 1;                // G^H: 1 tile subproblems, 2 run sets, 3..5 lanes, 6 deterministic
-    int degrid_kind = 1;              // G: 1 tile subproblems, 3..5 lanes; autotuned
+    int degrid_kind = 1;              // G: 1 tile subproblems, 3..5 lanes, 8 sorted (half plane)
     int fft_rb = 0, fft_cb = 0;       // FFT rows / columns per block (0: heuristic)
     int fft_cw = 0;                   // FFT columns per thread, 1 or 2 (0: 2 where the shape allows)
     // workspaces
@@ -284,9 +324,6 @@ struct CgFold {
     int* flags = nullptr;
     int step = 0;
 };
-// blocks of the inverse row pass (the number of CG partials it writes)
-int rows_inv_blocks(purify_plan* p);
-
 // ----------------------------------------------------------- operator steps
 // Phi: x real [ny][nx] (internal pointer) -> y complex [M]. If perm != null
 // the output is written in caller order through perm. `scale` multiplies S.
@@ -299,29 +336,33 @@ void launch_phi(purify_plan* p, const void* x, void* y, bool caller_order, doubl
 void launch_phi_adj(purify_plan* p, const void* y, void* out, bool caller_order, double scale,
                     int out_mode, const void* add, bool acc_zeroed = false);
 void launch_fft2(purify_plan* p, void* grid, bool inverse);
-// Phi stages used by the solver's fused forms
+// Phi stages used by the solver's fused forms; half: on the half-plane grid
+// (a real image in, or the real part out: out_mode 1)
 // zero_acc: the same launch clears the gridding accumulator (gacc); fold:
 // apply the pending CG update first (see CgFold)
 void launch_scale_pad_rows(purify_plan* p, const void* x, double scale, const int* skip_flag, bool corr = true,
-                           bool zero_acc = false, const CgFold* fold = nullptr);
-void launch_cols_fwd(purify_plan* p, const int* skip_flag);
-void launch_degrid(purify_plan* p, void* y, bool caller_order, const int* skip_flag);
-void launch_grid(purify_plan* p, const void* y, bool caller_order, const int* skip_flag, bool zeroed = false);
+                           bool zero_acc = false, const CgFold* fold = nullptr, bool half = false);
+void launch_cols_fwd(purify_plan* p, const int* skip_flag, bool half = false);
+void launch_degrid(purify_plan* p, void* y, bool caller_order, const int* skip_flag, bool half = false);
+void launch_grid(purify_plan* p, const void* y, bool caller_order, const int* skip_flag, bool zeroed = false,
+                 bool half = false);
 // inverse column pass: reads the gridding output (gacc), or with `mult` the
 // forward grid multiplied elementwise by mult
-void launch_cols_inv(purify_plan* p, const int* skip_flag, const void* mult = nullptr);
+void launch_cols_inv(purify_plan* p, const int* skip_flag, const void* mult = nullptr, bool half = false);
 // G^H G of the grid (the oversampled image after F Z S): for every
 // visibility the J x J interpolation of the forward grid spread back with the
 // same weights, into gacc (the visibility values are never stored)
-// (zeroed: gacc was cleared by this step's forward row pass, no memset)
-void launch_normal_gg(purify_plan* p, const int* skip_flag, bool zeroed = false);
+// (zeroed: gacc was cleared by this step's forward row pass, no memset; half:
+// on the half-plane grid, for a real image whose real part is wanted)
+void launch_normal_gg(purify_plan* p, const int* skip_flag, bool zeroed = false, bool half = false);
 // G^H by runs (same output as launch_grid)
 void launch_grid_sets(purify_plan* p, const void* y, bool caller_order, const int* skip_flag, bool zeroed = false);
 // cg: a CG step (out = A r, add = r): per-block partials of r.r and r.A r
 // (2 per block, in cg->part), reduced and decided by the last block (see
 // CgFold); cg->step is the step
 void launch_rows_inv_crop(purify_plan* p, void* out, double scale, int out_mode, const void* add,
-                          double add_coef, const int* skip_flag, const CgFold* cg = nullptr, bool corr = true);
+                          double add_coef, const int* skip_flag, const CgFold* cg = nullptr, bool corr = true,
+                          bool half = false);
 
 // Psi / Psi^dagger
 void launch_psi_adj(purify_plan* p, const void* x, void* c);
@@ -373,6 +414,32 @@ void add_launches(int64_t n);
 bool timing_enabled(const purify_plan* p);
 void reweight(purify_plan* p, const void* x, double rho, void* w);
 double coef_std(purify_plan* p, const void* x);
+
+// the normal operator runs on the half plane (its lane form is FP32 only)
+inline bool normal_half(const purify_plan* p) { return p->half_on && (p->stencil.on || p->dtype == PURIFY_F32); }
+// G^H G as a stencil (stencil.cu): bytes of the coefficients; the build from
+// the half-plane lane work (cells: the runs' first-tap cells, row * W +
+// column); the application, which writes all of gacc
+int64_t stencil_bytes(const purify_plan* p);
+void build_stencil(purify_plan* p, const std::vector<int>& cells);
+void launch_stencil(purify_plan* p, const int* skip);
+#define PURIFY_J_DISPATCH(J, FN, ...)                                     \
+    switch (J) {                                                          \
+        case 2: FN<2>(__VA_ARGS__); break;                                \
+        case 3: FN<3>(__VA_ARGS__); break;                                \
+        case 4: FN<4>(__VA_ARGS__); break;                                \
+        case 5: FN<5>(__VA_ARGS__); break;                                \
+        case 6: FN<6>(__VA_ARGS__); break;                                \
+        case 7: FN<7>(__VA_ARGS__); break;                                \
+        case 8: FN<8>(__VA_ARGS__); break;                                \
+        default: throw Error{PURIFY_EINVAL, "kb_width out of range"};     \
+    }
+
+// the plan's kernel polynomials in precision T
+template <typename T> inline const typename KbOf<T>::type& kb_table(const purify_plan* p) {
+    if constexpr (sizeof(T) == 4) return p->kbp;
+    else return p->kbpd;
+}
 
 int max_grid_tile(int dtype, int J);
 // the lane-per-run kernels apply to this plan (FP32, J <= kLaneMaxJ)

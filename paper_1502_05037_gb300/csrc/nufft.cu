@@ -34,7 +34,7 @@ __device__ __forceinline__ void atomic_add_c(double2* a, double2 v) {
 }
 
 // Adds the J complex values (ar[a], ai[a]) to row[c0 .. c0 + J) of a grid row
-// of Kx cells (periodic): where the segment does not wrap, two cells at a
+// of Kx cells (periodic; on the half plane no segment wraps): where the segment does not wrap, two cells at a
 // time with 16-byte vector reductions (one L2 operation for two cells), the
 // odd cells at the ends with 8-byte ones.
 template <int J>
@@ -61,8 +61,9 @@ __device__ __forceinline__ void red_row(float2* row, int c0, int Kx, const float
 }
 template <int J>
 __device__ __forceinline__ void red_row(double2* row, int c0, int Kx, const double (&ar)[J], const double (&ai)[J]) {
+    const int wrap = c0 + J <= Kx ? ~0 : Kx - 1;
 #pragma unroll
-    for (int k = 0; k < J; ++k) atomic_add_c(row + ((c0 + k) & (Kx - 1)), make_double2(ar[k], ai[k]));
+    for (int k = 0; k < J; ++k) atomic_add_c(row + ((c0 + k) & wrap), make_double2(ar[k], ai[k]));
 }
 
 // G^H by cell runs. A block owns one subproblem: a grid tile and an explicit
@@ -312,7 +313,7 @@ __device__ __forceinline__ void ldg_row(const double2* __restrict__ row, int c0,
 // of the group's next record directly, one step ahead; the two warp
 // barriers of a step order every reuse of the single-buffered slots.
 template <typename T, int DEG> __device__ __forceinline__ T kb_tap_poly(const T (&c)[DEG + 1], T phi) {
-    const T z = fma(T(2), phi, T(-1));
+    const T z = kb_z(phi);
     T acc = c[DEG];
 #pragma unroll
     for (int i = DEG - 1; i >= 0; --i) acc = fma(acc, z, c[i]);
@@ -449,8 +450,8 @@ k_grid_sets(const typename cplx_of<T>::type* __restrict__ yin, const typename cp
                 wxb = kb_tap_poly<T, DEG>(cf, phx);
                 wyb = kb_tap_poly<T, DEG>(cf, phy);
             } else if constexpr (sizeof(T) == 8) {
-                wxb = kb_tap_exact(J, b, kp.beta, kp.inv_i0beta, phx);
-                wyb = kb_tap_exact(J, b, kp.beta, kp.inv_i0beta, phy);
+                wxb = kb_tap_exact(J, b, kp.beta, kp.inv_i0beta, kb_z(phx));
+                wyb = kb_tap_exact(J, b, kp.beta, kp.inv_i0beta, kb_z(phy));
             }
             const int par = NPAR == 1 ? 0 : (k & 1);
             sw[par][g][b] = wxb;
@@ -493,7 +494,7 @@ k_grid_sets(const typename cplx_of<T>::type* __restrict__ yin, const typename cp
     pdl_trigger();
 }
 
-// Lane-per-run forms of G^H G, G^H and G (FP32, J <= 6; see LaneWork). A
+// Lane-per-run forms of G^H G, G^H and G (see LaneWork). A
 // warp takes a set of 32 / H runs (sets w, 2W - 1 - w, 2W + w, ... for warp
 // w of W, which balances the length-sorted sets); the H lanes r, r + 32 / H,
 // ... own run r of the set, lane h of them rows [h RH, (h + 1) RH) of the
@@ -509,64 +510,140 @@ k_grid_sets(const typename cplx_of<T>::type* __restrict__ yin, const typename cp
 //   G    : yout[idx] = sum_b wy[b] sum_a wx[a] X[b][a]
 // One step of the warp reads 32 / H consecutive records, three steps ahead
 // (with H = 2 each lane only its own axis offset); padding records (past a
-// run's end) get zero weights. The accumulators are flushed with vector
-// reductions after the set.
+// run's end) add nothing. The accumulators are flushed with vector reductions
+// after the set. On the half plane (HalfPlane; `ld` its row stride, `xm` all
+// ones: no wrapping along x) a folded visibility's value is conjugated where
+// it is read or written.
 enum { LANE_GG = 0, LANE_GRID = 1, LANE_DEGRID = 2 };
 
-// Shared staging of the lane kernels: per warp two buffers (current and next
-// set) of each lane's RH x J patch of X, lane stride RH J + 1 complex values
-// (odd, so the 8-byte accesses of a half-warp fall on distinct banks).
-template <int J, int H> struct LaneStage {
-    static constexpr int RH = (J + H - 1) / H;
-    static constexpr int LS = RH * J + 1;
-    static constexpr size_t bytes_per_warp = 2 * 32 * LS * sizeof(float2);
+// Shared staging of the lane kernels, per warp and buffer [run][row][GW]
+// cells. A lane copies its rows of the next run's grid patch there cell by
+// cell. G^H adds the accumulated patches of a set to the grid from there, a row
+// at a time by GL neighbouring lanes in 16-byte accesses (the row's cells from
+// the even column at or below its first one: GW cells), 32 / GL rows per
+// instruction: a lane adding its own rows touches a cache line per lane and
+// access (512 x 512 channel, 786 433 visibilities, J = 6: 37.5 -> 34.5 us). In
+// G^H G, which has no registers to spare, both that and copying the patches
+// in the same way cost more than they gave (34 -> 35 and 37 us). The stride RS
+// of a run keeps 16-byte alignment and spreads the runs over the banks.
+template <typename T, int J, int H> struct LaneStage {
+    static constexpr int WID = 32 / H;                     // runs per set
+    static constexpr int RH = (J + H - 1) / H;             // patch rows per lane
+    static constexpr int CV = 16 / sizeof(typename cplx_of<T>::type);   // cells per 16-byte access
+    static constexpr int GL = CV == 2 ? (J + 2) / 2 : J;   // lanes per row
+    static constexpr int GW = CV * GL;
+    static constexpr int RS = CV == 2 ? (J * GW + 13) / 16 * 16 + 2 : (J * GW) | 1;
+    static constexpr int IPI = 32 / GL;                    // rows per instruction
+    static constexpr int NIT = (WID * J + IPI - 1) / IPI;
+    static constexpr size_t buffer_bytes = (size_t)WID * RS * sizeof(typename cplx_of<T>::type);
+    // buffers of a mode: two where patches are read ahead, one to add them back
+    static constexpr int buffers(int mode, bool det) { return mode != 1 ? 2 : (det ? 0 : 1); }
+    static constexpr size_t smem(int mode, bool det) { return 4 * buffers(mode, det) * buffer_bytes; }
 };
 
-__device__ __forceinline__ void cp_async8(void* sdst, const void* gsrc) {
+template <typename C> __device__ __forceinline__ void cp_async_cell(C* sdst, const C* gsrc) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(sdst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(gsrc) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(gsrc), "n"(sizeof(C)) : "memory");
 }
+// cells of a 16-byte shared slot (two float cells or one double)
+__device__ __forceinline__ void ld_slot(const float2* s, float2* v) {
+    const float4 q = *reinterpret_cast<const float4*>(s);
+    v[0] = make_float2(q.x, q.y);
+    v[1] = make_float2(q.z, q.w);
+}
+__device__ __forceinline__ void ld_slot(const double2* s, double2* v) { v[0] = *s; }
+__device__ __forceinline__ void st_slot(float2* s, const float2* v) {
+    *reinterpret_cast<float4*>(s) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+}
+__device__ __forceinline__ void st_slot(double2* s, const double2* v) { *s = v[0]; }
+// a 16-byte shared slot added to / written from global cells
+__device__ __forceinline__ void red_slot(float2* p, const float2* s) {
+    const float4 q = *reinterpret_cast<const float4*>(s);
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(q.x), "f"(q.y), "f"(q.z), "f"(q.w)
+                 : "memory");
+}
+__device__ __forceinline__ void red_slot(double2* p, const double2* s) { atomic_add_c(p, *s); }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+// w x + acc and w x of a complex x by a real w: packed two-lane FP32
+__device__ __forceinline__ float2 c_fma(float w, float2 x, float2 acc) { return __ffma2_rn(make_float2(w, w), x, acc); }
+__device__ __forceinline__ double2 c_fma(double w, double2 x, double2 acc) {
+    return make_double2(fma(w, x.x, acc.x), fma(w, x.y, acc.y));
+}
+__device__ __forceinline__ float2 c_mul(float w, float2 x) { return __fmul2_rn(make_float2(w, w), x); }
+__device__ __forceinline__ double2 c_mul(double w, double2 x) { return make_double2(w * x.x, w * x.y); }
+
+// Resident blocks the lane kernels are compiled for: lane pairs four (three
+// where the patches are stored), fewer where a lane holds more than three rows
+// of six cells or doubles.
+template <typename T, int J, int MODE, int H, bool DET> constexpr int lane_min_blocks() {
+    if (H != 2) return 1;
+    if (sizeof(T) == 8) return MODE == LANE_GG ? 1 : 2;
+    if (J > 6) return MODE == LANE_GG ? 2 : 3;
+    return DET ? 3 : 4;
+}
 
 // With DET the accumulators are not added to the grid: run q's J x J patch
 // is stored at out[(b J + a) * dstride + q] (q = set * (32 / H) + its lane
 // in the set), for k_lane_gather to sum in a fixed order.
-template <int J, int MODE, int H, bool DET = false>
-__global__ void __launch_bounds__(128, H == 2 ? (DET ? 3 : 4) : 1)
-k_lane(const float2* __restrict__ X, const float2* __restrict__ yin, float2* __restrict__ yout,
-       const int2* __restrict__ set_info, const int2* __restrict__ run_cl, const float2* __restrict__ recs,
-       const int* __restrict__ idx, int nsets, KbPoly kp, int Kx, int Ky, float2* __restrict__ out,
+template <typename T, int J, int MODE, int H, bool DET = false>
+__global__ void __launch_bounds__(128, lane_min_blocks<T, J, MODE, H, DET>())
+k_lane(const typename cplx_of<T>::type* __restrict__ X, const typename cplx_of<T>::type* __restrict__ yin,
+       typename cplx_of<T>::type* __restrict__ yout, const int2* __restrict__ set_info,
+       const int2* __restrict__ run_cl, const T* __restrict__ recs, const int* __restrict__ idx, int nsets,
+       typename KbOf<T>::type kp, int ld, int xm, int Ky, typename cplx_of<T>::type* __restrict__ out,
        const int* __restrict__ skip, int64_t dstride) {
+    using C = typename cplx_of<T>::type;
+    using Stage = LaneStage<T, J, H>;
     constexpr bool HAS_X = MODE != LANE_GRID, HAS_ACC = MODE != LANE_DEGRID;
-    constexpr int WID = 32 / H, RH = LaneStage<J, H>::RH, LS = LaneStage<J, H>::LS;
+    constexpr int WID = Stage::WID, RH = Stage::RH;
     pdl_wait();
     if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, r = lane % WID, h = lane / WID;
     const int W = gridDim.x * (blockDim.x >> 5), wg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    // this lane's two staging buffers
-    float2* stage = reinterpret_cast<float2*>(smem_raw) + ((size_t)(threadIdx.x >> 5) * 64 + lane) * LS;
-    auto buf = [&](int i) { return stage + (size_t)(i & 1) * 32 * LS; };
+    C* const stage = reinterpret_cast<C*>(smem_raw) +
+                     (size_t)(threadIdx.x >> 5) * Stage::buffers(MODE, DET) * WID * Stage::RS;
+    auto buf = [&](int i) { return stage + (size_t)(Stage::buffers(MODE, DET) > 1 ? (i & 1) : 0) * WID * Stage::RS; };
     auto set_of = [&](int i) { return i * W + ((i & 1) ? W - 1 - wg : wg); };
-    // this lane's rows of a run's X patch into a staging buffer
-    auto patch_async = [&](int2 rcn, float2* dst) {
-        const int cx = rcn.x & 0xFFFF, cy = (int)((unsigned)rcn.x >> 16);
+    // f(run's cell, run's length, shared slot, grid cell) for this lane's
+    // 16-byte part of every patch row of the set whose runs lanes 0 .. WID - 1
+    // hold in rcn
+    const int part = lane % Stage::GL, item0 = lane / Stage::GL;
+    auto patch_rows = [&](int2 rcn, C* base, auto&& f) {
+#pragma unroll
+        for (int k = 0; k < Stage::NIT; ++k) {
+            const int item = k * Stage::IPI + item0, run = min(item / J, WID - 1), row = item - item / J * J;
+            const int cell = __shfl_sync(0xffffffffu, rcn.x, run), len = __shfl_sync(0xffffffffu, rcn.y, run);
+            if (item0 < Stage::IPI && item < WID * J && len > 0) {
+                const int c0 = cell & 0xFFFF, cy = (int)((unsigned)cell >> 16);
+                const int col = (c0 / Stage::CV * Stage::CV + part * Stage::CV) & xm;
+                f(c0 % Stage::CV, base + run * Stage::RS + row * Stage::GW + part * Stage::CV,
+                  (size_t)((cy + row) & (Ky - 1)) * ld + col);
+            }
+        }
+    };
+    // this lane's rows of a run's X patch into a staging buffer, at the run's
+    // offset in its windows
+    auto patch_async = [&](int2 rcn, C* dst) {
+        const int c0 = rcn.x & 0xFFFF, cy = (int)((unsigned)rcn.x >> 16);
         if (rcn.y <= 0) return;
+        dst += r * Stage::RS + c0 % Stage::CV;
 #pragma unroll
         for (int i = 0; i < RH; ++i) {
             const int b = h * RH + i;
             if (b < J) {
-                const float2* row = X + (size_t)((cy + b) & (Ky - 1)) * Kx;
+                const C* row = X + (size_t)((cy + b) & (Ky - 1)) * ld;
 #pragma unroll
-                for (int a = 0; a < J; ++a) cp_async8(dst + i * J + a, row + ((cx + a) & (Kx - 1)));
+                for (int a = 0; a < J; ++a) cp_async_cell(dst + b * Stage::GW + a, row + ((c0 + a) & xm));
             }
         }
     };
     // records: with H = 2 each lane reads its own axis offset (the work
     // stores a record row as the 16 runs' x offsets, then their y offsets),
     // with H = 1 both offsets; PD steps ahead of their use
-    using Rec = typename std::conditional<H == 2, float, float2>::type;
+    using Rec = typename std::conditional<H == 2, T, C>::type;
     constexpr int PD = 3;
     const Rec* __restrict__ rl = reinterpret_cast<const Rec*>(recs);
     auto rec_at = [&](int row0, int k) -> Rec { return rl[(size_t)(row0 + k) * 32 + lane]; };
@@ -612,26 +689,37 @@ k_lane(const float2* __restrict__ X, const float2* __restrict__ yin, float2* __r
         // complex patch values and accumulators as (re, im) pairs: the
         // interpolation and spreading below are packed two-lane FP32
         // multiply-adds (per component the same roundings as scalar ones)
-        float2 xv[HAS_X ? RH : 1][HAS_X ? J : 1];
-        float2 av[HAS_ACC ? RH : 1][HAS_ACC ? J : 1];
+        C xv[HAS_X ? RH : 1][HAS_X ? J : 1];
+        C av[HAS_ACC ? RH : 1][HAS_ACC ? J : 1];
         if constexpr (HAS_X) {
             cp_async_wait_all();
-            const float2* cur = buf(it);
+            const C* cur = buf(it) + r * Stage::RS + h * RH * Stage::GW;
+            const bool odd = cx % Stage::CV != 0;
 #pragma unroll
             for (int i = 0; i < RH; ++i) {
                 const bool rowok = len > 0 && h * RH + i < J;
+                if (H * RH > J && h * RH + i >= J) {   // no such row (and no such slot)
+#pragma unroll
+                    for (int a = 0; a < J; ++a) xv[i][a] = cmake<C>(T(0), T(0));
+                    continue;
+                }
+                C win[Stage::GW];
+#pragma unroll
+                for (int c = 0; c < Stage::GW; c += Stage::CV) ld_slot(cur + i * Stage::GW + c, &win[c]);
 #pragma unroll
                 for (int a = 0; a < J; ++a) {
-                    const float2 v = rowok ? cur[i * J + a] : make_float2(0.f, 0.f);
-                    xv[i][a] = v;
+                    const C z = cmake<C>(T(0), T(0));
+                    const C at1 = win[a + 1 < Stage::GW ? a + 1 : a];
+                    xv[i][a] = !rowok ? z : (odd ? at1 : win[a]);
                 }
             }
+            __syncwarp();   // before the buffer is written again
         }
         if constexpr (HAS_ACC) {
 #pragma unroll
             for (int i = 0; i < RH; ++i)
 #pragma unroll
-                for (int a = 0; a < J; ++a) av[i][a] = make_float2(0.f, 0.f);
+                for (int a = 0; a < J; ++a) av[i][a] = cmake<C>(T(0), T(0));
         }
         // the next set's patch (into the buffer read at the start of the
         // previous set) and first records, a whole set ahead of their use
@@ -665,11 +753,20 @@ k_lane(const float2* __restrict__ X, const float2* __restrict__ yin, float2* __r
         // steps ahead)
         constexpr int YD = MODE == LANE_GRID ? 2 : 1;
         static_assert(YD < PD, "value prefetch needs the index further ahead");
-        float2 yq[YD];
+        C yq[YD];
+        auto value = [&](int code) -> C {
+            C v = cmake<C>(T(0), T(0));
+            if (code >= 0) v = yin[code];
+            else if (code < -1) {
+                v = yin[fold_index(code)];
+                v.y = -v.y;
+            }
+            return v;
+        };
 #pragma unroll
         for (int j = 0; j < YD; ++j) {
-            yq[j] = make_float2(0.f, 0.f);
-            if (MODE == LANE_GRID && iq[j] >= 0) yq[j] = yin[iq[j]];
+            yq[j] = cmake<C>(T(0), T(0));
+            if (MODE == LANE_GRID) yq[j] = value(iq[j]);
         }
         for (int k = 0; k < lmax; ++k) {
             // records PD steps ahead, gridding values YD steps ahead
@@ -679,37 +776,37 @@ k_lane(const float2* __restrict__ X, const float2* __restrict__ yin, float2* __r
                 rn = rec_at(row0, k + PD);
                 if (MODE != LANE_GG) in = idx_at(row0, k + PD);
             }
-            float2 ynew = make_float2(0.f, 0.f);
-            if (MODE == LANE_GRID && iq[YD] >= 0) ynew = yin[iq[YD]];
+            C ynew = cmake<C>(T(0), T(0));
+            if (MODE == LANE_GRID) ynew = value(iq[YD]);
             const bool valid = k < len;
-            float wx[J], wy[RH];
+            T wx[J], wy[RH];
             if constexpr (H == 1) {
-                kb_weights<J>(kp, rq[0].x, wx);
-                kb_weights<J>(kp, rq[0].y, wy);
+                kb_weights_z<J>(kp, rq[0].x, wx);
+                kb_weights_z<J>(kp, rq[0].y, wy);
             } else {
                 // this lane's axis, then the partner's by shuffle
-                float own[J], oth[J];
-                kb_weights<J>(kp, rq[0], own);
+                T own[J], oth[J];
+                kb_weights_z<J>(kp, rq[0], own);
 #pragma unroll
                 for (int a = 0; a < J; ++a) oth[a] = __shfl_xor_sync(0xffffffffu, own[a], WID);
 #pragma unroll
                 for (int a = 0; a < J; ++a) wx[a] = h ? oth[a] : own[a];
 #pragma unroll
                 for (int i = 0; i < RH; ++i) {
-                    const float w0 = oth[i];                                              // row i (h = 0)
-                    const float w1 = RH + i < J ? own[RH + i < J ? RH + i : 0] : 0.f;   // row RH + i (h = 1)
+                    const T w0 = oth[i];                                              // row i (h = 0)
+                    const T w1 = RH + i < J ? own[RH + i < J ? RH + i : 0] : T(0);   // row RH + i (h = 1)
                     wy[i] = h ? w1 : w0;
                 }
             }
-            float yr = 0.f, yi = 0.f;
+            T yr = 0, yi = 0;
             if constexpr (HAS_X) {
-                float2 y2 = make_float2(0.f, 0.f);
+                C y2 = cmake<C>(T(0), T(0));
 #pragma unroll
                 for (int i = 0; i < RH; ++i) {
-                    float2 t = make_float2(0.f, 0.f);
+                    C t = cmake<C>(T(0), T(0));
 #pragma unroll
-                    for (int a = 0; a < J; ++a) t = __ffma2_rn(make_float2(wx[a], wx[a]), xv[i][a], t);
-                    y2 = __ffma2_rn(make_float2(wy[i], wy[i]), t, y2);
+                    for (int a = 0; a < J; ++a) t = c_fma(wx[a], xv[i][a], t);
+                    y2 = c_fma(wy[i], t, y2);
                 }
                 yr = y2.x;
                 yi = y2.y;
@@ -720,21 +817,24 @@ k_lane(const float2* __restrict__ X, const float2* __restrict__ yin, float2* __r
                     yi += __shfl_xor_sync(0xffffffffu, yi, WID);
                 }
                 // a step past the run's end contributes nothing
-                if (!valid) yr = yi = 0.f;
+                if (!valid) yr = yi = T(0);
             }
             if constexpr (MODE == LANE_GRID) {
                 yr = yq[0].x;
                 yi = yq[0].y;
             }
             if constexpr (MODE == LANE_DEGRID) {
-                if (valid && iq[0] >= 0 && h == 0) yout[iq[0]] = make_float2(yr, yi);
+                if (valid && h == 0) {
+                    const bool fold = iq[0] < 0;
+                    yout[fold ? fold_index(iq[0]) : iq[0]] = cmake<C>(yr, fold ? -yi : yi);
+                }
             }
             if constexpr (HAS_ACC) {
 #pragma unroll
                 for (int i = 0; i < RH; ++i) {
-                    const float2 u = __fmul2_rn(make_float2(wy[i], wy[i]), make_float2(yr, yi));
+                    const C u = c_mul(wy[i], cmake<C>(yr, yi));
 #pragma unroll
-                    for (int a = 0; a < J; ++a) av[i][a] = __ffma2_rn(make_float2(wx[a], wx[a]), u, av[i][a]);
+                    for (int a = 0; a < J; ++a) av[i][a] = c_fma(wx[a], u, av[i][a]);
                 }
             }
 #pragma unroll
@@ -753,7 +853,7 @@ k_lane(const float2* __restrict__ X, const float2* __restrict__ yin, float2* __r
                 if constexpr (DET) {
                     // this lane's rows, tap by tap (consecutive runs of the
                     // set write consecutive slots of each tap plane)
-                    float2* P = out + (size_t)set * WID + r + (size_t)(h * RH * J) * dstride;
+                    C* P = out + (size_t)set * WID + r + (size_t)(h * RH * J) * dstride;
 #pragma unroll
                     for (int i = 0; i < RH; ++i) {
                         if (h * RH + i < J) {
@@ -764,18 +864,48 @@ k_lane(const float2* __restrict__ X, const float2* __restrict__ yin, float2* __r
                             }
                         }
                     }
-                } else {
+                }
+            }
+            if constexpr (!DET && MODE == LANE_GRID) {
+                // the patch rows to the staging buffer at the run's offset in
+                // its window (the window's other cells zero), then added
+                C* const dst = buf(it) + r * Stage::RS + h * RH * Stage::GW;
+                const bool odd = cx % Stage::CV != 0;
+#pragma unroll
+                for (int i = 0; i < RH; ++i) {
+                    if (h * RH + i < J) {
+                        C win[Stage::GW];
+#pragma unroll
+                        for (int c = 0; c < Stage::GW; ++c) {
+                            const C z = cmake<C>(T(0), T(0));
+                            const C even_v = c < J ? av[i][c < J ? c : 0] : z;
+                            const C odd_v = c >= 1 && c <= J ? av[i][c >= 1 && c <= J ? c - 1 : 0] : z;
+                            win[c] = odd ? odd_v : even_v;
+                        }
+#pragma unroll
+                        for (int c = 0; c < Stage::GW; c += Stage::CV) st_slot(dst + i * Stage::GW + c, &win[c]);
+                    }
+                }
+                __syncwarp();
+                patch_rows(rc, buf(it), [&](int off, C* s, size_t g) {
+                    // an even window of an even J ends before its last slot
+                    if (J % 2 != 0 || Stage::CV == 1 || off != 0 || part != Stage::GL - 1) red_slot(out + g, s);
+                });
+                __syncwarp();
+            }
+            if constexpr (!DET && MODE == LANE_GG) {
+                if (len > 0) {
 #pragma unroll
                     for (int i = 0; i < RH; ++i) {
                         const int b = h * RH + i;
                         if (b < J) {
-                            float ar[J], ai[J];
+                            T ar[J], ai[J];
 #pragma unroll
                             for (int a = 0; a < J; ++a) {
                                 ar[a] = av[i][a].x;
                                 ai[a] = av[i][a].y;
                             }
-                            red_row<J>(out + (size_t)((cy + b) & (Ky - 1)) * Kx, cx, Kx, ar, ai);
+                            red_row<J>(out + (size_t)((cy + b) & (Ky - 1)) * ld, cx, ld, ar, ai);
                         }
                     }
                 }
@@ -920,6 +1050,75 @@ k_degrid_tile(const typename cplx_of<T>::type* __restrict__ grid, const T* __res
     pdl_trigger();
 }
 
+// entry i's records of K visibilities, one access each
+template <typename C> __device__ __forceinline__ void ld_records(const C* z, const int* idx, int64_t i, C (&zm)[1], int (&code)[1]) {
+    zm[0] = __ldcs(z + i);
+    code[0] = __ldcs(idx + i);
+}
+__device__ __forceinline__ void ld_records(const float2* z, const int* idx, int64_t i, float2 (&zm)[2], int (&code)[2]) {
+    const float4 q = __ldcs(reinterpret_cast<const float4*>(z) + i);
+    const int2 c = __ldcs(reinterpret_cast<const int2*>(idx) + i);
+    zm[0] = make_float2(q.x, q.y);
+    zm[1] = make_float2(q.z, q.w);
+    code[0] = c.x;
+    code[1] = c.y;
+}
+
+// G on the half-plane grid (see HalfPlane, SortedWork): a thread per K
+// visibilities of one first-tap cell, threads in the order of the cells, so
+// the lanes of a warp read the same few cells and one L1 line serves most of a
+// load. Nothing is staged, exchanged or kept between visibilities; the values
+// are scattered to the caller's (or the solver's) order. Bound by what L1 can
+// return to the registers (8 J^2 bytes a thread, J^2 / 2 cycles a warp) and by
+// a line per scattered value: two visibilities per thread share the cells'
+// loads. 1024 x 1024, 10.5 M visibilities, J = 6: 271 us by tiles in shared
+// memory, 211 us by lane pairs over runs, 182 us with K = 1, 142 us with K = 2.
+template <typename T, int J, int K>
+__global__ void __launch_bounds__(256)
+k_degrid_sorted(const typename cplx_of<T>::type* __restrict__ X, const typename cplx_of<T>::type* __restrict__ z,
+                const int* __restrict__ cell, const int* __restrict__ idx, int64_t n, typename KbOf<T>::type kp,
+                int ld, int Ky, typename cplx_of<T>::type* __restrict__ y, const int* __restrict__ skip) {
+    using C = typename cplx_of<T>::type;
+    pdl_wait();
+    if (skip && *skip) return;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) {
+        // the records are read once, as streams: L2 is left to the values
+        const int c = __ldcs(cell + i);
+        int code[K];
+        C zm[K];
+        ld_records(z, idx, i, zm, code);
+        T wx[K][J], wy[K][J];
+        C acc[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            kb_weights_z<J>(kp, zm[k].x, wx[k]);
+            kb_weights_z<J>(kp, zm[k].y, wy[k]);
+            acc[k] = cmake<C>(T(0), T(0));
+        }
+        const int cx = c & 0xFFFF, cy = (int)((unsigned)c >> 16);
+#pragma unroll
+        for (int b = 0; b < J; ++b) {
+            const C* row = X + (size_t)((cy + b) & (Ky - 1)) * ld + cx;
+            C t[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) t[k] = cmake<C>(T(0), T(0));
+#pragma unroll
+            for (int a = 0; a < J; ++a) {
+                const C v = row[a];
+#pragma unroll
+                for (int k = 0; k < K; ++k) t[k] = c_fma(wx[k][a], v, t[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < K; ++k) acc[k] = c_fma(wy[k][b], t[k], acc[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (code[k] != -1) y[code[k] < 0 ? fold_index(code[k]) : code[k]] = cmake<C>(acc[k].x, code[k] < 0 ? -acc[k].y : acc[k].y);
+    }
+    pdl_trigger();
+}
+
 // ------------------------------------------------------------- launchers
 template <typename K> static void set_smem(K kernel, size_t bytes) {
     if (bytes > 48 * 1024) PURIFY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
@@ -945,12 +1144,6 @@ static int blocks_per_sm(std::atomic<int> (&cache)[64], K kernel, int threads, s
     return v;
 }
 
-
-// the plan's kernel polynomials in precision T
-template <typename T> static const typename KbOf<T>::type& kb_table(const purify_plan* p) {
-    if constexpr (sizeof(T) == 4) return p->kbp;
-    else return p->kbpd;
-}
 
 template <typename T, int J> static void degrid_tj(purify_plan* p, void* y, bool caller_order, const int* skip) {
     using C = typename cplx_of<T>::type;
@@ -1008,18 +1201,6 @@ int grid_list_unit(int dtype, int J) {
     return (dtype == PURIFY_F32 ? grid_warps<float>() : grid_warps<double>()) * G * P;
 }
 
-#define PURIFY_J_DISPATCH(J, FN, ...)                                     \
-    switch (J) {                                                          \
-        case 2: FN<2>(__VA_ARGS__); break;                                \
-        case 3: FN<3>(__VA_ARGS__); break;                                \
-        case 4: FN<4>(__VA_ARGS__); break;                                \
-        case 5: FN<5>(__VA_ARGS__); break;                                \
-        case 6: FN<6>(__VA_ARGS__); break;                                \
-        case 7: FN<7>(__VA_ARGS__); break;                                \
-        case 8: FN<8>(__VA_ARGS__); break;                                \
-        default: throw Error{PURIFY_EINVAL, "kb_width out of range"};     \
-    }
-
 template <int J> static void degrid_f(purify_plan* p, void* y, bool c, const int* s) { degrid_tj<float, J>(p, y, c, s); }
 template <int J> static void degrid_d(purify_plan* p, void* y, bool c, const int* s) { degrid_tj<double, J>(p, y, c, s); }
 template <int J> static void grid_f(purify_plan* p, const void* y, bool c, const int* s, bool z) { grid_tj<float, J>(p, y, c, s, z); }
@@ -1053,21 +1234,22 @@ static void grid_sets_tj(purify_plan* p, const void* y, bool caller_order, const
 // grid of 4-warp blocks (as many as are resident at once, or fewer when
 // there is less work).
 static const LaneWork& lane_work(const purify_plan* p, int kind) { return p->lanes[kind == 6 ? 1 : kind - 3]; }
-template <int J, int MODE, int H, bool DET>
+template <typename T, int J, int MODE, int H, bool DET>
 static void lane_launch(purify_plan* p, const LaneWork& lw, const void* yin, void* yout, bool caller_order,
-                        const int* skip, float2* out, int64_t dstride) {
-    const size_t lane_smem = 4 * LaneStage<J, H>::bytes_per_warp;
+                        const int* skip, typename cplx_of<T>::type* out, int64_t dstride, bool half) {
+    using C = typename cplx_of<T>::type;
+    const size_t lane_smem = LaneStage<T, J, H>::smem(MODE, DET);
     static std::atomic<int> occ[64];   // resident blocks per SM of this instantiation, per device
-    const int per_sm = blocks_per_sm(occ, k_lane<J, MODE, H, DET>, 128, lane_smem);
+    const int per_sm = blocks_per_sm(occ, k_lane<T, J, MODE, H, DET>, 128, lane_smem);
     int sms = 0, dev = 0;
     PURIFY_CUDA(cudaGetDevice(&dev));
     PURIFY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int blocks = std::max(1, std::min(sms * per_sm, (lw.nsets + 3) / 4));
     Launch L(p, MODE == LANE_GG ? "normal_gg" : (MODE == LANE_GRID ? "grid" : "degrid"));
-    launch_dependent(k_lane<J, MODE, H, DET>, blocks, 128, lane_smem, p->stream, p->grid.as<float2>(),
-                     (const float2*)yin, (float2*)yout, lw.set_info.as<int2>(), lw.run_cl.as<int2>(),
-                     lw.rec.as<float2>(), caller_order ? lw.idx_caller.as<int>() : lw.idx.as<int>(), lw.nsets,
-                     p->kbp, p->Kx, p->Ky, out, skip, dstride);
+    launch_dependent(k_lane<T, J, MODE, H, DET>, blocks, 128, lane_smem, p->stream, p->grid.as<C>(), (const C*)yin,
+                     (C*)yout, lw.set_info.as<int2>(), lw.run_cl.as<int2>(), lw.rec.as<T>(),
+                     caller_order ? lw.idx_caller.as<int>() : lw.idx.as<int>(), lw.nsets, kb_table<T>(p),
+                     half ? p->half.W : p->Kx, half ? ~0 : p->Kx - 1, p->Ky, out, skip, dstride);
     L.done();
 }
 template <int J, int MODE, int H>
@@ -1080,7 +1262,8 @@ static void lane_tw(purify_plan* p, const LaneWork& lw, const void* yin, void* y
             const int64_t stride = (int64_t)lw.nsets * lw.width;
             PURIFY_REQUIRE(p->det_patch.bytes >= sizeof(float2) * (size_t)J * J * (size_t)stride,
                            "deterministic patch buffer too small");
-            lane_launch<J, MODE, H, true>(p, lw, yin, yout, caller_order, skip, p->det_patch.as<float2>(), stride);
+            lane_launch<float, J, MODE, H, true>(p, lw, yin, yout, caller_order, skip, p->det_patch.as<float2>(),
+                                                 stride, false);
             const int64_t cells = (int64_t)p->Kx * p->Ky;
             Launch L(p, "det_gather");
             launch_dependent(k_lane_gather<J>, (unsigned)((cells + 255) / 256), 256, 0, p->stream,
@@ -1092,7 +1275,47 @@ static void lane_tw(purify_plan* p, const LaneWork& lw, const void* yin, void* y
     }
     if (MODE != LANE_DEGRID && !zeroed) PURIFY_CUDA(cudaMemsetAsync(p->gacc.p, 0, p->gacc.bytes, p->stream));
     if (lw.nsets == 0) return;
-    lane_launch<J, MODE, H, false>(p, lw, yin, yout, caller_order, skip, p->gacc.as<float2>(), 0);
+    lane_launch<float, J, MODE, H, false>(p, lw, yin, yout, caller_order, skip, p->gacc.as<float2>(), 0, false);
+}
+// G^H and (FP32) G^H G on the half-plane grid by lanes (the solver's order
+// of the visibilities), G by sorted visibilities
+static void clear_half(purify_plan* p) {
+    const size_t cell = p->dtype == PURIFY_F32 ? sizeof(float2) : sizeof(double2);
+    PURIFY_CUDA(cudaMemsetAsync(p->gacc.p, 0, cell * (size_t)p->Ky * p->half.W, p->stream));
+}
+template <typename T, int J, int MODE>
+static void half_lane(purify_plan* p, const void* yin, const int* skip, bool zeroed) {
+    using C = typename cplx_of<T>::type;
+    if (!zeroed) clear_half(p);
+    lane_launch<T, J, MODE, 2, false>(p, p->half_lanes, yin, nullptr, false, skip, p->gacc.as<C>(), 0, true);
+}
+template <int J> static void half_lane_any(purify_plan* p, int mode, const void* yin, const int* s, bool z) {
+    if (p->dtype == PURIFY_F32) {
+        if (mode == LANE_GG) half_lane<float, J, LANE_GG>(p, yin, s, z);
+        else half_lane<float, J, LANE_GRID>(p, yin, s, z);
+    } else {
+        if (mode == LANE_GG) throw Error{PURIFY_EINVAL, "no lane form of the double normal operator"};
+        else half_lane<double, J, LANE_GRID>(p, yin, s, z);
+    }
+}
+static void launch_half_lanes(purify_plan* p, int mode, const void* yin, const int* s, bool z) {
+    PURIFY_J_DISPATCH(p->J, half_lane_any, p, mode, yin, s, z);
+}
+
+template <typename T, int J> static void degrid_sorted_tj(purify_plan* p, void* y, bool caller_order, const int* skip) {
+    using C = typename cplx_of<T>::type;
+    const SortedWork& w = p->half_sorted;
+    auto kern = k_degrid_sorted<T, J, 1>;
+    if constexpr (sizeof(T) == 4) { if (w.per == 2) kern = k_degrid_sorted<T, J, 2>; }
+    Launch L(p, "degrid");
+    launch_dependent(kern, (unsigned)((w.n + 255) / 256), 256, 0, p->stream, (const C*)p->grid.as<C>(),
+                     (const C*)w.z.as<C>(), (const int*)w.cell.as<int>(),
+                     (const int*)(caller_order ? w.idx_caller.as<int>() : w.idx.as<int>()), w.n, kb_table<T>(p),
+                     p->half.W, p->Ky, (C*)y, skip);
+    L.done();
+}
+template <int J> static void degrid_sorted_j(purify_plan* p, void* y, bool c, const int* s) {
+    if (p->dtype == PURIFY_F32) degrid_sorted_tj<float, J>(p, y, c, s); else degrid_sorted_tj<double, J>(p, y, c, s);
 }
 template <int J, int MODE>
 static void lane_on(purify_plan* p, const LaneWork& lw, const void* yin, void* yout, bool c, const int* s, bool z) {
@@ -1134,8 +1357,10 @@ static void require_lane_work(const purify_plan* p, int kind) {
         throw Error{PURIFY_EINVAL, "lane-per-run kernels need an FP32 plan with J <= 6 built for that form"};
 }
 
-void launch_normal_gg(purify_plan* p, const int* skip, bool zeroed) {
-    if (p->normal_kind >= 3 && lane_work_ok(p)) { PURIFY_J_DISPATCH(p->J, lane_gg, p, p->normal_kind, skip, zeroed); }
+void launch_normal_gg(purify_plan* p, const int* skip, bool zeroed, bool half) {
+    if (half && p->stencil.on) { launch_stencil(p, skip); }
+    else if (half) { launch_half_lanes(p, LANE_GG, nullptr, skip, zeroed); }
+    else if (p->normal_kind >= 3 && lane_work_ok(p)) { PURIFY_J_DISPATCH(p->J, lane_gg, p, p->normal_kind, skip, zeroed); }
     else if (p->dtype == PURIFY_F32) { PURIFY_J_DISPATCH(p->J, normal_f, p, skip, zeroed); }
     else { PURIFY_J_DISPATCH(p->J, normal_d, p, skip, zeroed); }
 }
@@ -1186,7 +1411,11 @@ int max_grid_tile(int dtype, int J) {
     return t;
 }
 
-void launch_degrid(purify_plan* p, void* y, bool caller_order, const int* skip) {
+void launch_degrid(purify_plan* p, void* y, bool caller_order, const int* skip, bool half) {
+    if (half) {
+        PURIFY_J_DISPATCH(p->J, degrid_sorted_j, p, y, caller_order, skip);
+        return;
+    }
     if (p->degrid_kind >= 3) {
         launch_degrid_lanes(p, p->degrid_kind, y, caller_order, skip);
         return;
@@ -1194,7 +1423,12 @@ void launch_degrid(purify_plan* p, void* y, bool caller_order, const int* skip) 
     if (p->dtype == PURIFY_F32) { PURIFY_J_DISPATCH(p->J, degrid_f, p, y, caller_order, skip); }
     else { PURIFY_J_DISPATCH(p->J, degrid_d, p, y, caller_order, skip); }
 }
-void launch_grid(purify_plan* p, const void* y, bool caller_order, const int* skip, bool zeroed) {
+void launch_grid(purify_plan* p, const void* y, bool caller_order, const int* skip, bool zeroed, bool half) {
+    if (half) {
+        PURIFY_REQUIRE(!caller_order, "the half-plane adjoint takes the solver's order");
+        launch_half_lanes(p, LANE_GRID, y, skip, zeroed);
+        return;
+    }
     if (p->grid_kind == 2) {
         launch_grid_sets(p, y, caller_order, skip, zeroed);
         return;
@@ -1208,16 +1442,18 @@ void launch_grid(purify_plan* p, const void* y, bool caller_order, const int* sk
 }
 
 void launch_phi(purify_plan* p, const void* x, void* y, bool caller_order, double scale, bool zero_acc) {
-    launch_scale_pad_rows(p, x, scale, nullptr, true, zero_acc);
-    launch_cols_fwd(p, nullptr);
-    launch_degrid(p, y, caller_order, nullptr);
+    const bool half = p->half_on;
+    launch_scale_pad_rows(p, x, scale, nullptr, true, zero_acc, nullptr, half);
+    launch_cols_fwd(p, nullptr, half);
+    launch_degrid(p, y, caller_order, nullptr, half);
 }
 
 void launch_phi_adj(purify_plan* p, const void* y, void* out, bool caller_order, double scale, int out_mode,
                     const void* add, bool acc_zeroed) {
-    launch_grid(p, y, caller_order, nullptr, acc_zeroed);
-    launch_cols_inv(p, nullptr);
-    launch_rows_inv_crop(p, out, scale, out_mode, add, 1.0, nullptr);
+    const bool half = p->half_on && out_mode == 1;
+    launch_grid(p, y, caller_order, nullptr, acc_zeroed, half);
+    launch_cols_inv(p, nullptr, nullptr, half);
+    launch_rows_inv_crop(p, out, scale, out_mode, add, 1.0, nullptr, nullptr, true, half);
 }
 
 }  // namespace purify

@@ -9,6 +9,7 @@
 #include <map>
 #include <mutex>
 #include <numeric>
+#include <thread>
 #include <tuple>
 #include <vector>
 
@@ -61,6 +62,20 @@ template <typename T> static std::vector<T> cast_vec(const std::vector<double>& 
     return o;
 }
 
+// f(begin, end) over [0, n) in contiguous pieces on the host's cores.
+template <typename F> static void parallel_for(int64_t n, F&& f) {
+    const int64_t piece = 1 << 15;
+    const int nt = (int)std::min<int64_t>(std::min(16u, std::max(1u, std::thread::hardware_concurrency())),
+                                          (n + piece - 1) / piece);
+    if (nt <= 1) {
+        f((int64_t)0, n);
+        return;
+    }
+    std::vector<std::thread> ts;
+    for (int t = 0; t < nt; ++t) ts.emplace_back([&, t] { f(n * t / nt, n * (t + 1) / nt); });
+    for (auto& t : ts) t.join();
+}
+
 // Grid cell of each visibility's first tap (wrapped), as computed by the
 // kernels.
 template <typename T>
@@ -68,14 +83,16 @@ static void first_tap_cells(purify_plan* p, const std::vector<T>& u, const std::
                             std::vector<int>& cy) {
     cx.resize(p->M);
     cy.resize(p->M);
-    for (int64_t m = 0; m < p->M; ++m) {
-        int kx0, ky0;
-        T phx, phy;
-        split_coord(u[m], p->ax, p->J, kx0, phx);
-        split_coord(v[m], p->ay, p->J, ky0, phy);
-        cx[m] = kx0 & (p->Kx - 1);
-        cy[m] = ky0 & (p->Ky - 1);
-    }
+    parallel_for(p->M, [&](int64_t a, int64_t b) {
+        for (int64_t m = a; m < b; ++m) {
+            int kx0, ky0;
+            T phx, phy;
+            split_coord(u[m], p->ax, p->J, kx0, phx);
+            split_coord(v[m], p->ay, p->J, ky0, phy);
+            cx[m] = kx0 & (p->Kx - 1);
+            cy[m] = ky0 & (p->Ky - 1);
+        }
+    });
 }
 
 // Sort the visibilities of each block by a hierarchical tile key: the
@@ -176,7 +193,7 @@ struct TuneKey {
         return std::tie(nx, ny, J, dtype, mlog, R, gm) < std::tie(o.nx, o.ny, o.J, o.dtype, o.mlog, o.R, o.gm);
     }
 };
-struct TuneVal { int tile, dtile, rb, cb, cw, units, dunits, gkind, dkind, nkind; };
+struct TuneVal { int tile, dtile, rb, cb, cw, units, dunits, gkind; };
 static std::mutex g_tune_mutex;
 static std::map<TuneKey, TuneVal> g_tune_cache;
 
@@ -244,7 +261,7 @@ static void autotune(purify_plan* p, const std::vector<int>& cand, BinsFor bins_
     // visibilities, in batch units
     const int64_t unit = grid_list_unit(p->dtype, p->J);
     const int u0 = (int)std::max<int64_t>(1, std::min<int64_t>(16, (p->M / (152 * 4) + unit / 2) / unit));
-    TuneVal val{p->work.tile, p->work.tile, 0, 0, 0, u0, u0, 1, 1, 2};
+    TuneVal val{p->work.tile, p->work.tile, 0, 0, 0, u0, u0, 1};
     bool cached = false;
     if (tune) {
         std::lock_guard<std::mutex> lk(g_tune_mutex);
@@ -265,12 +282,13 @@ static void autotune(purify_plan* p, const std::vector<int>& cand, BinsFor bins_
         // bring the clocks up before the first candidate is timed
         for (int i = 0; i < 40; ++i) launch_cols_fwd(p, nullptr);
         PURIFY_CUDA(cudaStreamSynchronize(p->stream));
-        // FFT launch shapes
+        // FFT launch shapes, on the half-plane passes where the plan has them
+        const bool half = p->half_on;
         float best = 1e30f;
         for (int rb = 1; rb <= 8; rb *= 2) {
-            if (p->ny % rb || !fft_shape_ok(rb, p->Kx, p->dtype)) continue;
+            if ((half ? p->ny / 2 : p->ny) % rb || !fft_shape_ok(rb, p->Kx, p->dtype)) continue;
             p->fft_rb = rb;
-            float ms = time_ms(p, [&] { launch_scale_pad_rows(p, ximg, 1.0, nullptr); }, 10);
+            float ms = time_ms(p, [&] { launch_scale_pad_rows(p, ximg, 1.0, nullptr, true, false, nullptr, half); }, 10);
             if (ms < best) { best = ms; val.rb = rb; }
         }
         best = 1e30f;
@@ -280,42 +298,38 @@ static void autotune(purify_plan* p, const std::vector<int>& cand, BinsFor bins_
                 if (p->Kx % cb || !fft_shape_ok(cb, p->Ky, p->dtype, cw)) continue;
                 p->fft_cb = cb;
                 p->fft_cw = cw;
-                float ms = time_ms(p, [&] { launch_cols_fwd(p, nullptr); }, 10);
+                float ms = time_ms(p, [&] { launch_cols_fwd(p, nullptr, half); }, 10);
                 if (ms < best) { best = ms; val.cb = cb; val.cw = cw; }
             }
         }
         p->fft_rb = val.rb;
         p->fft_cb = val.cb;
         p->fft_cw = val.cw;
-        // gridding and degridding tiles, each timed on its own kernel
+        // gridding and degridding tiles, each timed on its own kernel (with
+        // the half-plane path only the adjoint's complex image grids on the
+        // whole plane: G^H alone)
         if (cand.size() > 1 && p->M >= 32768) {
             float bg = 1e30f, bd = 1e30f;
             for (int t : cand) {
                 const std::vector<int> bins = bins_for(t);
                 for (int u : {1, 2, 4, 8}) {
                     build_gridlist(p, bins, cell_order, t, u, p->work);
-                    build_gridlist(p, bins, cell_order, t, u, p->dwork);
                     float mg = time_ms(p, [&] { launch_grid(p, yv, false, nullptr); }, 5);
-                    float md = time_ms(p, [&] { launch_degrid(p, yv, false, nullptr); }, 5);
                     if (mg < bg) { bg = mg; val.tile = t; val.units = u; }
+                    if (half) continue;
+                    build_gridlist(p, bins, cell_order, t, u, p->dwork);
+                    float md = time_ms(p, [&] { launch_degrid(p, yv, false, nullptr); }, 5);
                     if (md < bd) { bd = md; val.dtile = t; val.dunits = u; }
                 }
             }
-            // gridding by run sets, and G^H, G and G^H G by lanes (one pool,
-            // or by tiles of each candidate edge); the normal operator by
-            // run sets or lanes
+            // gridding by run sets and by lanes (one pool, or by tiles)
             if (p->desc.grid_mode == 0) {
                 const float mr = time_ms(p, [&] { launch_grid_sets(p, yv, false, nullptr); }, 5);
                 if (mr < bg) { bg = mr; val.gkind = 2; }
-                float bn = time_ms(p, [&] { launch_normal_lanes(p, 2, nullptr); }, 5);
                 if (lane_work_ok(p)) {
                     for (int kind = 3; kind <= 5; ++kind) {
-                        const float mn = time_ms(p, [&] { launch_normal_lanes(p, kind, nullptr); }, 5);
                         const float ml = time_ms(p, [&] { launch_grid_lanes(p, kind, yv, false, nullptr); }, 5);
-                        const float mdl = time_ms(p, [&] { launch_degrid_lanes(p, kind, yv, false, nullptr); }, 5);
-                        if (mn < bn) { bn = mn; val.nkind = kind; }
                         if (ml < bg) { bg = ml; val.gkind = kind; }
-                        if (mdl < bd) { bd = mdl; val.dkind = kind; }
                     }
                 }
             }
@@ -331,10 +345,10 @@ static void autotune(purify_plan* p, const std::vector<int>& cand, BinsFor bins_
     // the deterministic lane pairs and degrids by the lane pairs
     const int gm = p->desc.grid_mode;
     p->grid_kind = gm == 0 ? val.gkind : gm;
-    p->degrid_kind = gm == 0 ? val.dkind : (gm == 6 ? 4 : (gm >= 3 ? gm : 1));
-    p->normal_kind = gm == 0 ? val.nkind : (gm >= 3 ? gm : 2);
+    p->degrid_kind = gm == 0 ? 8 : (gm == 6 ? 4 : (gm >= 3 ? gm : 1));
+    p->normal_kind = gm == 0 ? (p->stencil.on ? 7 : normal_half(p) ? 4 : 2) : (gm >= 3 ? gm : 2);
     build_gridlist(p, bins_for(val.tile), cell_order, val.tile, val.units, p->work);
-    build_gridlist(p, bins_for(val.dtile), cell_order, val.dtile, val.dunits, p->dwork);
+    if (!p->half_on) build_gridlist(p, bins_for(val.dtile), cell_order, val.dtile, val.dunits, p->dwork);
 }
 
 // Lane-per-run work (see LaneWork) from the length-sorted runs: `width`
@@ -374,29 +388,30 @@ static void build_lanework(purify_plan* p, const std::vector<HostRun>& runs, con
     }
     PURIFY_REQUIRE(rows * width < ((int64_t)1 << 31), "too many visibility records for the lane work");
     PURIFY_REQUIRE(width == 32 || width == 16, "lane work width must be 32 or 16");
-    // record row layout: width 32, (phx, phy) per run; width 16, the 16
-    // runs' phx then their phy (each lane of a pair reads its own axis)
+    // record row layout: width 32, (zx, zy) per run; width 16, the 16 runs'
+    // zx then their zy (each lane of a pair reads its own axis)
     std::vector<float> lrec((size_t)rows * 2 * width, 0.f);   // 8 bytes per record
     std::vector<int> lidx((size_t)rows * width, -1), lcal((size_t)rows * width, -1);
-    for (int s = 0; s < nsets; ++s)
-        for (int l = 0; l < width; ++l) {
-            const size_t q0 = (size_t)s * width + l;
-            if (q0 >= nr) continue;
+    parallel_for((int64_t)nr, [&](int64_t qa, int64_t qb) {
+        for (int64_t q0 = qa; q0 < qb; ++q0) {
+            const int s = (int)(q0 / width), l = (int)(q0 % width);
             const int r = order[q0];
             for (int k = 0; k < runs[r].len; ++k) {
                 const Rec& e = rec[start[r] + k];
                 const size_t row = (size_t)set_info[s].x + k, q = row * width + l;
+                const float zx = kb_z((float)e.phx), zy = kb_z((float)e.phy);
                 if (width == 32) {
-                    lrec[2 * q] = (float)e.phx;
-                    lrec[2 * q + 1] = (float)e.phy;
+                    lrec[2 * q] = zx;
+                    lrec[2 * q + 1] = zy;
                 } else {
-                    lrec[row * 2 * width + l] = (float)e.phx;
-                    lrec[row * 2 * width + width + l] = (float)e.phy;
+                    lrec[row * 2 * width + l] = zx;
+                    lrec[row * 2 * width + width + l] = zy;
                 }
                 lidx[q] = e.m;
                 lcal[q] = perm[e.m];
             }
         }
+    });
     w.nsets = nsets;
     w.width = width;
     w.tile = tile;
@@ -435,10 +450,152 @@ static void build_lanework(purify_plan* p, const std::vector<HostRun>& runs, con
     }
 }
 
+static const int kRunMax = 48;
+
+// Longest run of the half-plane lane work: a warp's share of the records is
+// M / (runs per set x resident warps) steps, and a set's longest run is a
+// serial chain, so runs are cut to half the share (at most kRunMax, at least
+// 16: every run costs a patch).
+static int run_cap(int64_t M, int width) {
+    const int64_t share = M / ((int64_t)width * 152 * 16);
+    return (int)std::min<int64_t>(kRunMax, std::max<int64_t>(16, share / 2));
+}
+
+// Whether G^H G runs as a stencil (stencil.cu) or over the runs. The stencil
+// reads its coefficients whatever the number of visibilities: 0.22 us per MB
+// and 3 us. The lane pairs (FP32) cost 8 us, 105 us per million runs and 7 us
+// per million visibilities at J = 6, and as J^2 (fits within 15% of 1024 x
+// 1024 with 10.5, 2.0 and 0.6 M visibilities: 226, 83 and 47 us against 120,
+// 108 and 108; 512 x 512 with 2.6, 0.8 and 0.15 M: 53, 34 and 20 against 35,
+// 35 and 31; 256 x 256 with 0.66 M: 21 against 12). The double run sets cost
+// about 2 ns per visibility. The coefficients and the sums they are built
+// from must also leave most of the free memory alone.
+static bool use_stencil(const purify_plan* p, size_t nruns) {
+    const double bytes = (double)stencil_bytes(p), j2 = p->J * p->J / 36.0;
+    const double stencil_us = 3.0 + 0.22e-6 * bytes;
+    const double runs_us = p->dtype == PURIFY_F32 ? 8.0 + j2 * (105e-6 * nruns + 7e-6 * p->M) : 20.0 + 2e-3 * p->M;
+    if (stencil_us > runs_us) return false;
+    size_t free_b = 0, total_b = 0;
+    PURIFY_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    return 3.0 * bytes <= free_b / 4.0;
+}
+
+// The half-plane lane work (see HalfPlane, LaneWork): the visibilities, folded
+// where their first-tap column is in the upper half, in runs of one cell,
+// runs sorted by length (longest first, then by cell), a lane pair per run.
+template <typename T>
+static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std::vector<T>& vs,
+                             const std::vector<int>& scx, const std::vector<int>& scy, const std::vector<int>& perm) {
+    const int64_t M = p->M;
+    const int J = p->J, Kx = p->Kx, Ky = p->Ky, W = p->half.W, off = p->half.off, WID = 16;
+    std::vector<int> cell(M), order(M);
+    parallel_for(M, [&](int64_t a, int64_t b) {
+        for (int64_t m = a; m < b; ++m)
+            cell[m] = scx[m] < Kx / 2 ? scy[m] * W + scx[m] + off
+                                      : ((Ky - scy[m] - J + 1) & (Ky - 1)) * W + Kx - scx[m] - J + 1 + off;
+    });
+    {
+        std::vector<int> pos((size_t)Ky * W + 1, 0);
+        for (int64_t m = 0; m < M; ++m) pos[cell[m] + 1]++;
+        for (size_t c = 1; c < pos.size(); ++c) pos[c] += pos[c - 1];
+        for (int64_t m = 0; m < M; ++m) order[pos[cell[m]]++] = (int)m;
+    }
+    const int cap = run_cap(M, WID);
+    struct Run { int first, len, id; };   // id: place in cell order
+    std::vector<Run> runs, sorted;
+    std::vector<int> bylen(kRunMax + 2, 0);
+    for (int64_t i = 0; i < M;) {
+        int64_t j = i + 1;
+        while (j < M && j - i < cap && cell[order[j]] == cell[order[i]]) ++j;
+        runs.push_back({(int)i, (int)(j - i), (int)runs.size()});
+        bylen[j - i]++;
+        i = j;
+    }
+    const size_t nr = runs.size();
+    {
+        std::vector<size_t> at(kRunMax + 2, 0);   // first place of the runs of each length
+        for (int l = kRunMax - 1; l >= 1; --l) at[l] = at[l + 1] + bylen[l + 1];
+        sorted.resize(nr);
+        for (const Run& r : runs) sorted[at[r.len]++] = r;
+    }
+    const int nsets = (int)((nr + WID - 1) / WID);
+    std::vector<int2> set_info(nsets), run_cl((size_t)nsets * WID, make_int2(0, 0));
+    int64_t rows = 0;
+    for (int s = 0; s < nsets; ++s) {
+        const int lmax = sorted[(size_t)s * WID].len;
+        set_info[s] = make_int2((int)rows, lmax);
+        rows += lmax;
+    }
+    PURIFY_REQUIRE(rows * WID < ((int64_t)1 << 31), "too many visibility records for the lane work");
+    // entries of the sorted form: two visibilities of a cell each where that
+    // makes at most 3/4 as many (a thread of two costs about 4/3 of one); the
+    // double kernels are bound by arithmetic and take one
+    std::vector<int64_t> entry;   // first entry of each run in cell order, K = 2
+    SortedWork& sw = p->half_sorted;
+    {
+        int64_t n2 = 0;
+        for (const Run& r : runs) {
+            entry.push_back(n2);
+            n2 += (r.len + 1) / 2;
+        }
+        sw.per = sizeof(T) == 4 && 4 * n2 <= 3 * M ? 2 : 1;
+        sw.n = sw.per == 2 ? n2 : M;
+    }
+    const int per = sw.per;
+    std::vector<T> rec((size_t)rows * 2 * WID, T(0)), sz(2 * (size_t)(sw.n * per), T(0));
+    std::vector<int> idx((size_t)rows * WID, -1), sc(sw.n), si(sw.n * per, -1), sk(sw.n * per, -1);
+    parallel_for((int64_t)nr, [&](int64_t a, int64_t b) {
+        for (int64_t q = a; q < b; ++q) {
+            const int s = (int)(q / WID), l = (int)(q % WID);
+            const Run& r = sorted[q];
+            const int c = cell[order[r.first]], packed = ((c / W) << 16) | (c % W);
+            run_cl[q] = make_int2(packed, r.len);
+            const size_t at0 = per == 2 ? 2 * (size_t)entry[r.id] : (size_t)r.first;
+            for (int k = 0; k < r.len; ++k) {
+                const int m = order[r.first + k];
+                const bool fold = scx[m] >= Kx / 2;
+                int k0;
+                T phx, phy;
+                split_coord(us[m], p->ax, J, k0, phx);
+                split_coord(vs[m], p->ay, J, k0, phy);
+                const T zx = fold ? -kb_z(phx) : kb_z(phx), zy = fold ? -kb_z(phy) : kb_z(phy);
+                const size_t row = (size_t)set_info[s].x + k, at = at0 + k;
+                rec[row * 2 * WID + l] = zx;
+                rec[row * 2 * WID + WID + l] = zy;
+                idx[row * WID + l] = si[at] = fold ? fold_index(m) : m;
+                sk[at] = fold ? fold_index(perm[m]) : perm[m];
+                sc[at / per] = packed;
+                sz[2 * at] = zx;
+                sz[2 * at + 1] = zy;
+            }
+        }
+    });
+    LaneWork& w = p->half_lanes;
+    w.nsets = nsets;
+    w.width = WID;
+    w.tile = 0;
+    w.rows = rows;
+    upload(w.set_info, set_info);
+    upload(w.run_cl, run_cl);
+    upload(w.rec, rec);
+    upload(w.idx, idx);
+    upload(sw.z, sz);
+    upload(sw.cell, sc);
+    upload(sw.idx, si);
+    upload(sw.idx_caller, sk);
+    p->workspace_bytes += (int64_t)(sw.z.bytes + sw.cell.bytes + sw.idx.bytes + sw.idx_caller.bytes);
+    // the normal operator as a stencil, where that is the faster form
+    if (use_stencil(p, nr)) {
+        std::vector<int> cells(nr);
+        for (size_t q = 0; q < nr; ++q) cells[q] = cell[order[sorted[q].first]];
+        build_stencil(p, cells);
+        p->workspace_bytes += (int64_t)(p->stencil.coef.bytes + p->stencil.used.bytes);
+    }
+}
+
 // Run-ordered work (see RunWork): runs of equal first-tap cell in the cell
 // order, cut at kRunMax visibilities, sorted by length (longest first,
 // stable), padded to a multiple of G; records in run order.
-static const int kRunMax = 48;
 template <typename T>
 static void build_runwork(purify_plan* p, const std::vector<T>& us, const std::vector<T>& vs,
                                 const std::vector<int>& scx, const std::vector<int>& scy,
@@ -465,16 +622,20 @@ static void build_runwork(purify_plan* p, const std::vector<T>& us, const std::v
         cell[r] = runs[r].cell;
         start[r] = (int)q;
         len[r] = runs[r].len;
-        for (int k = 0; k < runs[r].len; ++k) {
-            const int m = cell_order[runs[r].first + k];
-            int kx0, ky0;
-            Rec e{};
-            split_coord(us[m], p->ax, p->J, kx0, e.phx);
-            split_coord(vs[m], p->ay, p->J, ky0, e.phy);
-            e.m = m;
-            rec[q++] = e;
-        }
+        q += runs[r].len;
     }
+    parallel_for((int64_t)runs.size(), [&](int64_t a, int64_t b) {
+        for (int64_t r = a; r < b; ++r)
+            for (int k = 0; k < runs[r].len; ++k) {
+                const int m = cell_order[runs[r].first + k];
+                int kx0, ky0;
+                Rec e{};
+                split_coord(us[m], p->ax, p->J, kx0, e.phx);
+                split_coord(vs[m], p->ay, p->J, ky0, e.phy);
+                e.m = m;
+                rec[start[r] + k] = e;
+            }
+    });
     if (sizeof(T) == 4 && p->J <= kLaneMaxJ) {
         build_lanework(p, runs, rec, start, perm, 32, 0, p->lanes[0]);
         build_lanework(p, runs, rec, start, perm, 16, 0, p->lanes[1], p->desc.grid_mode == 6);
@@ -604,17 +765,23 @@ template <typename T> static void finish_plan(purify_plan* p) {
     first_tap_cells<T>(p, u, v, cx, cy);
     sort_hierarchical(p, cx, cy, tmin, tmax, perm);
     std::vector<T> us(p->M), vs(p->M);
-    for (int64_t i = 0; i < p->M; ++i) { us[i] = u[perm[i]]; vs[i] = v[perm[i]]; }
+    parallel_for(p->M, [&](int64_t a, int64_t b) {
+        for (int64_t i = a; i < b; ++i) { us[i] = u[perm[i]]; vs[i] = v[perm[i]]; }
+    });
     upload(p->us, us);
     upload(p->vs, vs);
     upload(p->perm, perm);
     upload(p->d_offsets, p->offsets);
     std::vector<int> scx(p->M), scy(p->M);
-    for (int64_t i = 0; i < p->M; ++i) { scx[i] = cx[perm[i]]; scy[i] = cy[perm[i]]; }
+    parallel_for(p->M, [&](int64_t a, int64_t b) {
+        for (int64_t i = a; i < b; ++i) { scx[i] = cx[perm[i]]; scy[i] = cy[perm[i]]; }
+    });
     auto bins_for = [&](int t) {
         std::vector<int> bins(p->M);
         const int tx = p->Kx / t;
-        for (int64_t i = 0; i < p->M; ++i) bins[i] = (scy[i] / t) * tx + scx[i] / t;
+        parallel_for(p->M, [&](int64_t a, int64_t b) {
+            for (int64_t i = a; i < b; ++i) bins[i] = (scy[i] / t) * tx + scx[i] / t;
+        });
         return bins;
     };
     std::vector<int> cand;
@@ -646,9 +813,11 @@ template <typename T> static void finish_plan(purify_plan* p) {
     init_filter_banks();
     // workspaces
     const int nw = z;
-    p->grid.alloc(sizeof(C) * (size_t)p->Kx * p->Ky);
-    p->gacc.alloc(sizeof(C) * (size_t)p->Kx * p->Ky + 256);
-    p->rows.alloc(sizeof(C) * (size_t)p->ny * p->Kx);
+    // (the half plane of a small grid is wider than the grid)
+    const size_t gw = std::max(p->Kx, p->half.W);
+    p->grid.alloc(sizeof(C) * gw * p->Ky);
+    p->gacc.alloc(sizeof(C) * gw * p->Ky + 256);
+    p->rows.alloc(sizeof(C) * gw * p->ny);
     p->ll0.alloc(sizeof(T) * std::max<size_t>(1, (size_t)nw * p->N / 4));
     p->ll1.alloc(sizeof(T) * std::max<size_t>(1, (size_t)nw * p->N / 4));
     p->tmp_img.alloc(sizeof(C) * (size_t)p->N);
@@ -665,15 +834,17 @@ template <typename T> static void finish_plan(purify_plan* p) {
         for (int64_t i = 0; i < p->M; ++i) cell_order[pos[(int64_t)scy[i] * p->Kx + scx[i]]++] = (int)i;
     }
     build_runwork<T>(p, us, vs, scx, scy, cell_order, perm);
+    if (p->half_on) build_half_lanes<T>(p, us, vs, scx, scy, perm);
     autotune<T>(p, cand, bins_for, cell_order, d.tile == 0);
     // keep only the lane work in use (kind 6 runs on the lane pairs of kind 4)
     auto uses = [&](int k) {
         auto is = [&](int kind) { return kind == k || (k == 4 && kind == 6); };
-        return is(p->grid_kind) || is(p->degrid_kind) || is(p->normal_kind);
+        return is(p->grid_kind) || (!p->half_on && (is(p->degrid_kind) || is(p->normal_kind)));
     };
     for (int k = 3; k <= 5; ++k)
         if (!uses(k)) p->lanes[k - 3].release();
     for (int k = 0; k < 3; ++k) p->workspace_bytes += lane_bytes(p->lanes[k]);
+    p->workspace_bytes += lane_bytes(p->half_lanes);
     p->workspace_bytes += (int64_t)p->det_patch.bytes;
 }
 
@@ -739,6 +910,14 @@ purify_plan* create_plan(const purify_plan_desc* d) {
         p->ax = AxisConst{(int)Kx, (float)cx, (float)(cx - (double)(float)cx), cx};
         p->ay = AxisConst{(int)Ky, (float)cy, (float)(cy - (double)(float)cy), cy};
         p->kbp = fit_kb_poly(p->J, p->beta, kb_poly_degree(p->J));
+        // autotuned plans take the half-plane path; a forced decomposition runs
+        // on the whole plane
+        if (d->grid_mode == 0) {
+            p->half_on = true;
+            p->half.off = p->J - 2;
+            p->half.W0 = p->Kx / 2 + 2 * p->J - 3;
+            p->half.W = (p->half.W0 + 8 + 15) / 16 * 16;
+        }
         if (p->dtype == PURIFY_F64) p->kbpd = fit_kb_poly_d(p->J, p->beta);
         if (p->dtype == PURIFY_F32) finish_plan<float>(p); else finish_plan<double>(p);
         p->desc.u = p->desc.v = nullptr;

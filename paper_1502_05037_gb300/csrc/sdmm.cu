@@ -503,6 +503,7 @@ template <typename T> struct Solver {
         d2.levels = 1;
         d2.basis_mask = 1;
         d2.tile = p->work.tile;
+        if (d2.grid_mode == 0) d2.grid_mode = 1;   // only the adjoint's complex image: no half plane
         d2.stream = p->stream;
         purify_plan* q = create_plan(&d2);
         try {
@@ -701,15 +702,16 @@ template <typename T> struct Solver {
             } else {
                 // the pending update and the transform of the new r fused into
                 // the first FFT pass, then u = A r
-                launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, true, &fold);
-                launch_cols_fwd(p, skip);
+                const bool half = group < 0 && normal_half(p);
+                launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, true, &fold, half);
+                launch_cols_fwd(p, skip, half);
                 if (group >= 0) launch_lanes_on(p, p->group_lanes[group], 0, nullptr, nullptr, false, skip, true);
-                else launch_normal_gg(p, skip, true);
-                launch_cols_inv(p, skip);
+                else launch_normal_gg(p, skip, true, half);
+                launch_cols_inv(p, skip, nullptr, half);
                 // u = 2 r + Re Phi^H Phi r / nu^2 (G Re Phi_g^H Phi_g r / nu^2
                 // for a group), with r.r, r.u and the CG scalars fused in
                 launch_rows_inv_crop(p, s.u.p, group >= 0 ? inv_nu * s.groups : inv_nu, 1, s.r.p, 2.0, skip, &fold,
-                                     true);
+                                     true, half);
             }
         }
         // the last step's pending update is applied by the relative-change kernel
@@ -735,11 +737,12 @@ template <typename T> struct Solver {
         const int* skip = flags() + F_CGDONE;
         CgFold fold = make_fold();
         fold.step = k;
-        launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, true, &fold);
-        launch_cols_fwd(p, skip);
-        launch_normal_gg(p, skip, true);
-        launch_cols_inv(p, skip);
-        launch_rows_inv_crop(p, u_out, inv_nu, 1, nullptr, 0.0, skip, nullptr, true);
+        const bool half = normal_half(p);
+        launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, true, &fold, half);
+        launch_cols_fwd(p, skip, half);
+        launch_normal_gg(p, skip, true, half);
+        launch_cols_inv(p, skip, nullptr, half);
+        launch_rows_inv_crop(p, u_out, inv_nu, 1, nullptr, 0.0, skip, nullptr, true, half);
     }
 
     // Block-sharded CG step k, after the exchange: u = 2 r + u_sum, the dot
@@ -790,8 +793,8 @@ template <typename T> static void pd_iteration(Solver<T>& S, double tau, double 
                              S.scal(), p->R, 2);
             L.done();
         }
-        launch_grid(p, s.v2.p, false, nullptr, true);
-        launch_cols_inv(p, nullptr);
+        launch_grid(p, s.v2.p, false, nullptr, true, p->half_on);
+        launch_cols_inv(p, nullptr, nullptr, p->half_on);
         if (fork) PURIFY_CUDA(cudaEventRecord(s.ev_join, s.side));
     } catch (...) {
         p->stream = main_stream;
@@ -808,7 +811,7 @@ template <typename T> static void pd_iteration(Solver<T>& S, double tau, double 
     launch_psi(p, s.z1.p, s.p.p);
     if (fork) PURIFY_CUDA(cudaStreamWaitEvent(p->stream, s.ev_join, 0));
     // g = Psi p1 + Re Phi^H (sigma z) / nu
-    launch_rows_inv_crop(p, s.u.p, sigma * inv_nu, 1, s.p.p, 1.0, nullptr);
+    launch_rows_inv_crop(p, s.u.p, sigma * inv_nu, 1, s.p.p, 1.0, nullptr, nullptr, true, p->half_on);
     {
         Launch L(p, "pd_primal");
         launch_dependent(k_pd_primal<T>, ew_blocks(p->N), 256, 0, p->stream, x, s.u.template as<T>(), xbar,

@@ -194,6 +194,8 @@ struct TuneKey {
     }
 };
 struct TuneVal { int tile, dtile, rb, cb, cw, units, dunits, gkind; };
+// below this many visibilities gridding is not tuned (tile subproblems)
+static const int64_t kTuneMinM = 32768;
 static std::mutex g_tune_mutex;
 static std::map<TuneKey, TuneVal> g_tune_cache;
 
@@ -308,7 +310,7 @@ static void autotune(purify_plan* p, const std::vector<int>& cand, BinsFor bins_
         // gridding and degridding tiles, each timed on its own kernel (with
         // the half-plane path only the adjoint's complex image grids on the
         // whole plane: G^H alone)
-        if (cand.size() > 1 && p->M >= 32768) {
+        if (cand.size() > 1 && p->M >= kTuneMinM) {
             float bg = 1e30f, bd = 1e30f;
             for (int t : cand) {
                 const std::vector<int> bins = bins_for(t);
@@ -326,7 +328,7 @@ static void autotune(purify_plan* p, const std::vector<int>& cand, BinsFor bins_
             if (p->desc.grid_mode == 0) {
                 const float mr = time_ms(p, [&] { launch_grid_sets(p, yv, false, nullptr); }, 5);
                 if (mr < bg) { bg = mr; val.gkind = 2; }
-                if (lane_work_ok(p)) {
+                if (lane_work_ok(p) && p->lanes[0].nsets > 0) {
                     for (int kind = 3; kind <= 5; ++kind) {
                         const float ml = time_ms(p, [&] { launch_grid_lanes(p, kind, yv, false, nullptr); }, 5);
                         if (ml < bg) { bg = ml; val.gkind = kind; }
@@ -636,7 +638,9 @@ static void build_runwork(purify_plan* p, const std::vector<T>& us, const std::v
                 rec[start[r] + k] = e;
             }
     });
-    if (sizeof(T) == 4 && p->J <= kLaneMaxJ) {
+    // the whole-plane lane forms: forced, or candidates of the autotuner
+    const bool lanes = p->desc.grid_mode >= 3 || (p->desc.grid_mode == 0 && p->desc.tile == 0 && M >= kTuneMinM);
+    if (sizeof(T) == 4 && p->J <= kLaneMaxJ && lanes) {
         build_lanework(p, runs, rec, start, perm, 32, 0, p->lanes[0]);
         build_lanework(p, runs, rec, start, perm, 16, 0, p->lanes[1], p->desc.grid_mode == 6);
         build_lanework(p, runs, rec, start, perm, 16, std::min(32, std::min(p->Kx, p->Ky)), p->lanes[2]);

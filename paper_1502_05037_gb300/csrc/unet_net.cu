@@ -11,7 +11,10 @@
 //                    the skip (channel offsets of one buffer), conv3x3+ReLU x 2
 //   head:            conv1x1 (c -> 1) plus the input (residual), FP32.
 // Backward: input gradients are convolutions with the flipped, transposed
-// weights on the tensor cores; weight gradients are FP32 CUDA-core sums.
+// weights, weight gradients the transposed product, both on the tensor cores;
+// the ReLU masks are applied where a gradient is produced (the convolution's
+// epilogue, the pooling and upsampling kernels), which write the BF16 operand
+// of the next step directly.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -29,171 +32,214 @@ namespace purify {
 // ------------------------------------------------------------ small kernels
 static inline int eblocks(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 8192)); }
 
+// 8 BF16 channels as floats, and back
+struct Ch8 {
+    float v[8];
+    __device__ __forceinline__ void load(const bf16* p) {
+        bf16 t[8];
+        *reinterpret_cast<uint4*>(t) = *reinterpret_cast<const uint4*>(p);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = __bfloat162float(t[e]);
+    }
+    __device__ __forceinline__ void load(const float* p) {
+        const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    }
+    __device__ __forceinline__ void store(bf16* p) const {
+        bf16 t[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) t[e] = __float2bfloat16_rn(v[e]);
+        *reinterpret_cast<uint4*>(p) = *reinterpret_cast<const uint4*>(t);
+    }
+};
+// pooled pixel and channel group of index i over [B][Ho][Wo][C / 8]
+struct Pool8 {
+    int c;
+    size_t base;   // its 2 x 2 window's first pixel at full resolution
+    __device__ __forceinline__ Pool8(int64_t i, int H, int W, int C) {
+        const int G = C / 8, Ho = H / 2, Wo = W / 2;
+        int r = (int)(i / G);
+        c = (int)(i - (int64_t)r * G) * 8;
+        const int x = r % Wo;
+        r /= Wo;
+        const int y = r % Ho, b = r / Ho;
+        base = (size_t)(b * H + 2 * y) * W + 2 * x;
+    }
+    __device__ __forceinline__ size_t pix(int k, int W) const { return base + (k & 1) + (size_t)(k >> 1) * W; }
+};
+
+// All channel counts below are multiples of 8, one thread per 8 channels.
 __global__ void k_maxpool_fwd(const bf16* __restrict__ in, int cs, int co, bf16* __restrict__ out, int B, int H, int W,
                               int C) {
-    const int Ho = H / 2, Wo = W / 2;
-    const int64_t n = (int64_t)B * Ho * Wo * C;
+    const int64_t n = (int64_t)B * (H / 2) * (W / 2) * (C / 8);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int c = (int)(i % C);
-        int64_t r = i / C;
-        int x = (int)(r % Wo);
-        r /= Wo;
-        int y = (int)(r % Ho);
-        int b = (int)(r / Ho);
-        const bf16* p = in + ((size_t)(b * H + 2 * y) * W + 2 * x) * cs + co + c;
-        float m = __bfloat162float(p[0]);
-        m = fmaxf(m, __bfloat162float(p[cs]));
-        m = fmaxf(m, __bfloat162float(p[(size_t)W * cs]));
-        m = fmaxf(m, __bfloat162float(p[(size_t)W * cs + cs]));
-        out[i] = __float2bfloat16_rn(m);
+        const Pool8 p(i, H, W, C);
+        Ch8 m, t;
+        m.load(in + p.base * cs + co + p.c);
+#pragma unroll
+        for (int k = 1; k < 4; ++k) {
+            t.load(in + p.pix(k, W) * cs + co + p.c);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) m.v[e] = fmaxf(m.v[e], t.v[e]);
+        }
+        m.store(out + i * 8);
     }
 }
 
-// gin[b][y][x][c] = (first maximum of its 2x2 window, row-major) ? gout : 0,
-// plus gadd (stride as, offset ao) when given.
+// Through the pooling and the ReLU before it: gz[b][y][x][c] = in > 0 ?
+// ((first maximum of its 2x2 window, row-major) ? gout : 0) + gadd : 0, BF16;
+// gadd the skip's gradient [pixels][C].
 __global__ void k_maxpool_bwd(const bf16* __restrict__ in, int cs, int co, const float* __restrict__ gout,
-                              const float* __restrict__ gadd, int as, int ao, float* __restrict__ gin, int B, int H,
-                              int W, int C) {
-    const int Ho = H / 2, Wo = W / 2;
-    const int64_t n = (int64_t)B * Ho * Wo * C;
+                              const float* __restrict__ gadd, bf16* __restrict__ gz, int B, int H, int W, int C) {
+    const int64_t n = (int64_t)B * (H / 2) * (W / 2) * (C / 8);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int c = (int)(i % C);
-        int64_t r = i / C;
-        int x = (int)(r % Wo);
-        r /= Wo;
-        int y = (int)(r % Ho);
-        int b = (int)(r / Ho);
-        size_t base = (size_t)(b * H + 2 * y) * W + 2 * x;
-        size_t pix[4] = {base, base + 1, base + W, base + W + 1};
-        float best = -INFINITY;
-        int arg = 0;
-        for (int k = 0; k < 4; ++k) {
-            float v = __bfloat162float(in[pix[k] * cs + co + c]);
-            if (v > best) { best = v; arg = k; }
-        }
-        float g = gout[i];
-        for (int k = 0; k < 4; ++k) {
-            float v = (k == arg) ? g : 0.f;
-            if (gadd) v += gadd[pix[k] * as + ao + c];
-            gin[pix[k] * C + c] = v;
-        }
-    }
-}
-
-// gz = (act > 0) ? g : 0 as BF16 [P][C]; g has stride gs/offset go, act stride as/offset ao
-__global__ void k_relu_grad(const float* __restrict__ g, int gs, int go, const bf16* __restrict__ act, int as, int ao,
-                            bf16* __restrict__ gz, int64_t P, int C) {
-    const int64_t n = P * C;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int c = (int)(i % C);
-        int64_t p = i / C;
-        float a = __bfloat162float(act[p * as + ao + c]);
-        gz[i] = __float2bfloat16_rn(a > 0.f ? g[p * gs + go + c] : 0.f);
-    }
-}
-
-// g_lo[b][y][x][c] = sum of the 2x2 block of g_hi
-__global__ void k_upsample_bwd(const float* __restrict__ ghi, float* __restrict__ glo, int B, int H, int W, int C) {
-    const int Ho = H / 2, Wo = W / 2;
-    const int64_t n = (int64_t)B * Ho * Wo * C;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int c = (int)(i % C);
-        int64_t r = i / C;
-        int x = (int)(r % Wo);
-        r /= Wo;
-        int y = (int)(r % Ho);
-        int b = (int)(r / Ho);
-        size_t base = (size_t)(b * H + 2 * y) * W + 2 * x;
-        glo[i] = ghi[base * C + c] + ghi[(base + 1) * C + c] + ghi[(base + W) * C + c] + ghi[(base + W + 1) * C + c];
-    }
-}
-
-// Weight gradients of a k x k convolution on the CUDA cores, one tap per
-// block row of the grid:
-//   dW[co][tap][ci] += sum_p gz[p][co] * x[p + tap][ci]
-// a register-tiled GEMM (64 x 64 output tile, 4 x 4 per thread, K = 16
-// pixels per shared-memory stage) over a chunk of pixels, added to dW with
-// one atomic per output and block.
-__global__ void __launch_bounds__(256) k_dw(const bf16* __restrict__ gz, int Cout, const bf16* __restrict__ x, int xcs,
-                                            int xco, int Cin, int B, int H, int W, int up, int k, int pch,
-                                            float* __restrict__ dW) {
-    constexpr int BK = 16;
-    __shared__ __align__(16) float gs[BK][64];
-    __shared__ __align__(16) float xs[BK][64];
-    const int co0 = blockIdx.x * 64, ci0 = blockIdx.y * 64;
-    const int tap = blockIdx.z % (k * k), chunk = blockIdx.z / (k * k);
-    const int dy = tap / k - k / 2, dx = tap % k - k / 2;
-    const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-    const int64_t P = (int64_t)B * H * W;
-    const int64_t p0 = (int64_t)chunk * pch, p1 = min(P, p0 + pch);
-    const int sh = up ? 1 : 0;
-    const int Hs = H >> sh, Ws = W >> sh;
-    float acc[4][4] = {};
-    const int lk = tid / 16, lj = (tid % 16) * 4;   // this thread's loads: row lk, columns lj..lj+3
-    for (int64_t pb = p0; pb < p1; pb += BK) {
-        const int64_t p = pb + lk;
-        float gv[4] = {0, 0, 0, 0}, xv[4] = {0, 0, 0, 0};
-        if (p < p1) {
+        const Pool8 p(i, H, W, C);
+        Ch8 v[4], g;
+        g.load(gout + i * 8);
+        int arg[8] = {};
+        float best[8];
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (co0 + lj + e < Cout) gv[e] = __bfloat162float(gz[p * Cout + co0 + lj + e]);
-            const int b = (int)(p / (H * W));
-            const int rem = (int)(p - (int64_t)b * H * W);
-            const int yy = rem / W + dy, xx = rem % W + dx;
-            if (yy >= 0 && yy < H && xx >= 0 && xx < W) {
-                const bf16* src = x + ((size_t)(b * Hs + (yy >> sh)) * Ws + (xx >> sh)) * xcs + xco + ci0 + lj;
+        for (int e = 0; e < 8; ++e) best[e] = -INFINITY;
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (ci0 + lj + e < Cin) xv[e] = __bfloat162float(src[e]);
+        for (int k = 0; k < 4; ++k) {
+            v[k].load(in + p.pix(k, W) * cs + co + p.c);
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (v[k].v[e] > best[e]) { best[e] = v[k].v[e]; arg[e] = k; }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const size_t o = p.pix(k, W) * C + p.c;
+            Ch8 r;
+            r.load(gadd + o);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float t = (k == arg[e] ? g.v[e] : 0.f) + r.v[e];
+                r.v[e] = v[k].v[e] > 0.f ? t : 0.f;
+            }
+            r.store(gz + o);
+        }
+    }
+}
+
+// Through the x2 upsampling and the ReLU before it: the sum of the 2x2 block
+// of ghi, zero where act (channel stride C) is not positive, BF16.
+__global__ void k_upsample_bwd(const float* __restrict__ ghi, const bf16* __restrict__ act, bf16* __restrict__ gz, int B,
+                               int H, int W, int C) {
+    const int64_t n = (int64_t)B * (H / 2) * (W / 2) * (C / 8);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const Pool8 p(i, H, W, C);
+        Ch8 s, t, m;
+        s.load(ghi + p.base * C + p.c);
+#pragma unroll
+        for (int k = 1; k < 4; ++k) {
+            t.load(ghi + p.pix(k, W) * C + p.c);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) s.v[e] += t.v[e];
+        }
+        m.load(act + i * 8);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s.v[e] = m.v[e] > 0.f ? s.v[e] : 0.f;
+        s.store(gz + i * 8);
+    }
+}
+
+// out[c] += sum over pixels of w[p] v[p][c] (w = 1 when null; v has channel
+// stride cs), and with w also wsum += sum of w[p]: the bias gradients, and the
+// head's weight and bias gradient. A thread keeps 8 channels of every
+// (blockDim / (C / 8))-th pixel of the block's chunk; the block's sums are
+// combined in shared memory, one atomic per channel and block.
+__global__ void __launch_bounds__(256) k_colsum(const bf16* __restrict__ v, int cs, int C, int64_t P, int pch,
+                                                const bf16* __restrict__ w, float* __restrict__ out,
+                                                float* __restrict__ wsum) {
+    __shared__ float sh[256][9];
+    const int G = C / 8, lanes = blockDim.x / G;
+    const int g = threadIdx.x % G, l = threadIdx.x / G;
+    float acc[9] = {};
+    if (l < lanes) {
+        const int64_t p1 = min(P, ((int64_t)blockIdx.x + 1) * pch);
+        for (int64_t p = (int64_t)blockIdx.x * pch + l; p < p1; p += lanes) {
+            Ch8 t;
+            t.load(v + p * cs + g * 8);
+            const float s = w ? __bfloat162float(w[p]) : 1.f;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] = fmaf(s, t.v[e], acc[e]);
+            acc[8] += s;
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 9; ++e) sh[threadIdx.x][e] = acc[e];
+    __syncthreads();
+    for (int c = threadIdx.x; c <= C; c += blockDim.x) {
+        const int gg = c < C ? c / 8 : 0, e = c < C ? c % 8 : 8;
+        if (c == C && !wsum) continue;
+        float s = 0.f;
+        for (int k = 0; k < lanes; ++k) s += sh[k * G + gg][e];
+        atomicAdd(c < C ? out + c : wsum, s);
+    }
+}
+
+// Weight gradient of a 3 x 3 convolution of one input channel: dW[co][tap] +=
+// sum over pixels of gz[p][co] x[p + tap]. A thread owns one output channel and
+// walks pixels of a row with the 3 x 3 window of x in registers.
+__global__ void __launch_bounds__(256) k_dw_point(const bf16* __restrict__ gz, int Cout, const bf16* __restrict__ x,
+                                                  int B, int H, int W, int seg, float* __restrict__ dW) {
+    __shared__ float sh[256][9];
+    const int lanes = blockDim.x / Cout, co = threadIdx.x % Cout, l = threadIdx.x / Cout;
+    const int per_row = (W + seg - 1) / seg;
+    const int64_t nseg = (int64_t)B * H * per_row;
+    float acc[9] = {};
+    if (l < lanes) {
+        for (int64_t s = (int64_t)blockIdx.x * lanes + l; s < nseg; s += (int64_t)gridDim.x * lanes) {
+            const int r = (int)(s / per_row), x0 = (int)(s - (int64_t)r * per_row) * seg, x1 = min(W, x0 + seg);
+            const int b = r / H, y = r - b * H;
+            auto at = [&](int dy, int xx) -> float {
+                const int yy = y + dy;
+                return yy >= 0 && yy < H && xx >= 0 && xx < W ? __bfloat162float(x[((size_t)b * H + yy) * W + xx]) : 0.f;
+            };
+            float w0[3], w1[3], w2[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                w0[d] = at(d - 1, x0 - 1);
+                w1[d] = at(d - 1, x0);
+            }
+            for (int xx = x0; xx < x1; ++xx) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) w2[d] = at(d - 1, xx + 1);
+                const float g = __bfloat162float(gz[(((size_t)b * H + y) * W + xx) * Cout + co]);
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    acc[3 * d] = fmaf(g, w0[d], acc[3 * d]);
+                    acc[3 * d + 1] = fmaf(g, w1[d], acc[3 * d + 1]);
+                    acc[3 * d + 2] = fmaf(g, w2[d], acc[3 * d + 2]);
+                    w0[d] = w1[d];
+                    w1[d] = w2[d];
+                }
             }
         }
-        *reinterpret_cast<float4*>(&gs[lk][lj]) = make_float4(gv[0], gv[1], gv[2], gv[3]);
-        *reinterpret_cast<float4*>(&xs[lk][lj]) = make_float4(xv[0], xv[1], xv[2], xv[3]);
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            float4 a = *reinterpret_cast<const float4*>(&gs[kk][ty * 4]);
-            float4 c = *reinterpret_cast<const float4*>(&xs[kk][tx * 4]);
-            const float av[4] = {a.x, a.y, a.z, a.w}, cv[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] += av[i] * cv[j];
-        }
-        __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int co = co0 + ty * 4 + i;
-        if (co >= Cout) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int ci = ci0 + tx * 4 + j;
-            if (ci < Cin) atomicAdd(&dW[((size_t)co * k * k + tap) * Cin + ci], acc[i][j]);
-        }
-    }
-}
-
-// db[co] += sum over a chunk of pixels of gz[p][co]
-__global__ void k_db(const bf16* __restrict__ gz, int Cout, int64_t P, int pch, float* __restrict__ db) {
-    const int64_t p0 = (int64_t)blockIdx.x * pch, p1 = min(P, p0 + pch);
-    for (int co = threadIdx.x; co < Cout; co += blockDim.x) {
+    for (int e = 0; e < 9; ++e) sh[threadIdx.x][e] = acc[e];
+    __syncthreads();
+    for (int i = threadIdx.x; i < 9 * Cout; i += blockDim.x) {
+        const int c = i / 9, e = i - c * 9;
         float s = 0.f;
-        for (int64_t p = p0; p < p1; ++p) s += __bfloat162float(gz[p * Cout + co]);
-        atomicAdd(&db[co], s);
+        for (int k = 0; k < lanes; ++k) s += sh[k * Cout + c][e];
+        atomicAdd(&dW[i], s);
     }
 }
 
-// FP32 weights [Cout][k][k][Cin] -> flipped, transposed BF16 [Nb][k][k][Cb]:
-// W'[ci][ky][kx][co] = W[co][k-1-ky][k-1-kx][ci] (zero padded)
+// FP32 weights [Cout][k][k][Cin] -> flipped, transposed BF16
+// [k][k][Cb / 8][Nb][8]: W'[ci][ky][kx][co] = W[co][k-1-ky][k-1-kx][ci] (zero
+// padded)
 __global__ void k_pack_weights_bwd(const float* __restrict__ w, bf16* __restrict__ wp, int Cout, int k, int Cin, int Nb,
                                    int Cb) {
     const int64_t n = (int64_t)Nb * k * k * Cb;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        int co = (int)(i % Cb);
-        int64_t r = i / Cb;
-        int tap = (int)(r % (k * k));
-        int ci = (int)(r / (k * k));
+        const int64_t r = i / 8;
+        const int ci = (int)(r % Nb), g = (int)(r / Nb), tap = g / (Cb / 8);
+        const int co = (g - tap * (Cb / 8)) * 8 + (int)(i % 8);
         int ky = tap / k, kx = tap % k;
         int ftap = (k - 1 - ky) * k + (k - 1 - kx);
         float v = (ci < Cin && co < Cout) ? w[((int64_t)co * k * k + ftap) * Cin + ci] : 0.f;
@@ -201,15 +247,15 @@ __global__ void k_pack_weights_bwd(const float* __restrict__ w, bf16* __restrict
     }
 }
 
-// loss = mean (pred - t)^2, g = 2 (pred - t) / n; loss to scal[0] (FP64, fixed order)
-__global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ t, float* __restrict__ g, int64_t n,
+// loss = mean (pred - t)^2 to *out (FP64, fixed order), g = 2 (pred - t) / n in BF16
+__global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ t, bf16* __restrict__ g, int64_t n,
                       double* part, unsigned* counter, double* out) {
     float acc = 0.f;
     const float s = 2.f / (float)n;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         float d = pred[i] - t[i];
         acc += d * d;
-        g[i] = s * d;
+        g[i] = __float2bfloat16_rn(s * d);
     }
     double b = block_sum((double)acc);
     if (threadIdx.x == 0) part[blockIdx.x] = b;
@@ -258,7 +304,7 @@ struct Unet {
     DevBuf pred;                                // FP32 [B][H][W]
     // gradients (FP32) and BF16 staging
     std::vector<DevBuf> gcat;
-    DevBuf g1, g2, gz, gpred;
+    DevBuf g1, gz, gz2;
     DevBuf red_part, red_ctr, loss, err;
     int ch(int l) const { return base << l; }
     int64_t pix(int l, int B) const { return (int64_t)B * (H >> l) * (W >> l); }
@@ -360,7 +406,7 @@ Unet* unet_create(int H, int W, int L, int base, int maxB, uint64_t seed, cudaSt
             u->pool[l].alloc(sizeof(bf16) * u->pix(l + 1, maxB) * c);
             u->da[l].alloc(sizeof(bf16) * P * c);
             u->dbb[l].alloc(sizeof(bf16) * P * c);
-            u->gcat[l].alloc(sizeof(float) * P * 2 * c);
+            u->gcat[l].alloc(sizeof(float) * P * c);
         }
         int64_t Pb = u->pix(L - 1, maxB);
         u->bA.alloc(sizeof(bf16) * Pb * u->ch(L - 1));
@@ -369,9 +415,8 @@ Unet* unet_create(int H, int W, int L, int base, int maxB, uint64_t seed, cudaSt
         int64_t gmax = 0;
         for (int l = 0; l < L; ++l) gmax = std::max(gmax, u->pix(l, maxB) * 2 * u->ch(l));
         u->g1.alloc(sizeof(float) * gmax);
-        u->g2.alloc(sizeof(float) * gmax);
         u->gz.alloc(sizeof(bf16) * gmax);
-        u->gpred.alloc(sizeof(float) * u->pix(0, maxB));
+        u->gz2.alloc(sizeof(bf16) * gmax);
         u->red_part.alloc(sizeof(double) * 8192);
         u->red_ctr.alloc(sizeof(unsigned) * 4);
         u->loss.alloc(sizeof(double));
@@ -431,7 +476,7 @@ void unet_forward(Unet& u, const float* x, int B, float* out) {
         std::string s = std::to_string(l);
         fwd_conv(u, "e" + s + "a", B, in, in_cs, 0, l, 0, u.a[l].as<bf16>(), c, 0);
         fwd_conv(u, "e" + s + "b", B, u.a[l].as<bf16>(), c, 0, l, 0, u.cat[l].as<bf16>(), 2 * c, 0);
-        int64_t n = u.pix(l + 1, B) * c;
+        int64_t n = u.pix(l + 1, B) * c / 8;
         k_maxpool_fwd<<<eblocks(n), 256, 0, u.st>>>(u.cat[l].as<bf16>(), 2 * c, 0, u.pool[l].as<bf16>(), B, u.H >> l,
                                                    u.W >> l, c);
         add_launches(1);
@@ -458,35 +503,55 @@ void unet_forward(Unet& u, const float* x, int B, float* out) {
     conv_tc_launch(a, u.st);
 }
 
-// input gradient of a conv layer: gz (BF16 [P][cout]) -> g_out FP32 [P][cin] at level lev
-static void bwd_dx(Unet& u, UnetLayer& l, int B, int lev, const bf16* gz, float* gout) {
+// Where an input gradient goes: channels below f32_ch (all with out null) to
+// f32 [P][f32_ch], the others masked by the activation they belong to (its
+// ReLU) to BF16 `out` [P][cin - f32_ch].
+struct GradOut {
+    float* f32 = nullptr;
+    int f32_ch = 0;
+    bf16* out = nullptr;
+    const bf16* act = nullptr;
+    int act_cs = 0, act_co = 0;
+};
+
+// input gradient of a conv layer from gz (BF16 [P][cout]) at level lev
+static void bwd_dx(Unet& u, UnetLayer& l, int B, int lev, const bf16* gz, const GradOut& g) {
     ConvArgs a = conv_args(u, l, true);
     a.in = gz; a.in_cs = l.cout; a.in_co = 0; a.up = 0;
     a.B = B; a.H = u.H >> lev; a.W = u.W >> lev; a.relu = 0;
-    a.out = nullptr; a.out_f32 = gout; a.residual = nullptr;
+    a.out_f32 = g.f32; a.f32_ch = g.f32_ch; a.residual = nullptr;
+    a.out = g.out; a.out_cs = l.cin - g.f32_ch; a.out_co = 0; a.bf_from = g.f32_ch;
+    a.mask = g.act; a.mask_cs = g.act_cs; a.mask_co = g.act_co;
     conv_tc_launch(a, u.st);
 }
 
-static void bwd_dw(Unet& u, UnetLayer& l, int B, int lev, const bf16* gz, const bf16* x, int xcs, int xco, int up) {
-    const int H = u.H >> lev, W = u.W >> lev;
-    const int64_t P = (int64_t)B * H * W;
-    // pixel chunk per block: about 8 blocks per SM over all taps and tiles
-    const int tiles = ((l.cout + 63) / 64) * ((l.cin + 63) / 64) * l.k * l.k;
-    int64_t want = std::max<int64_t>(1, (152 * 8) / tiles);
-    int pch = (int)std::max<int64_t>(256, (P + want - 1) / want);
-    pch = (pch + 15) / 16 * 16;
-    const int nchunk = (int)((P + pch - 1) / pch);
-    dim3 g((l.cout + 63) / 64, (l.cin + 63) / 64, l.k * l.k * nchunk);
-    k_dw<<<g, 256, 0, u.st>>>(gz, l.cout, x, xcs, xco, l.cin, B, H, W, up, l.k, pch, u.grads.as<float>() + l.woff);
-    const int dch = 1024;
-    k_db<<<(int)((P + dch - 1) / dch), 64, 0, u.st>>>(gz, l.cout, P, dch, u.grads.as<float>() + l.boff);
+static void colsum(Unet& u, const bf16* v, int cs, int C, int64_t P, const bf16* w, float* out, float* wsum) {
+    const int pch = (int)std::max<int64_t>(64, (P + 152 * 4 - 1) / (152 * 4));
+    k_colsum<<<(int)((P + pch - 1) / pch), 256, 0, u.st>>>(v, cs, C, P, pch, w, out, wsum);
     PURIFY_CUDA(cudaGetLastError());
-    add_launches(2);
+    add_launches(1);
 }
 
-static void relu_grad(Unet& u, const float* g, int gs, int go, const bf16* act, int as, int ao, int64_t P, int C) {
-    k_relu_grad<<<eblocks(P * C), 256, 0, u.st>>>(g, gs, go, act, as, ao, u.gz.as<bf16>(), P, C);
-    add_launches(1);
+// weight and bias gradients of a layer with input x (channel stride xcs)
+static void bwd_dw(Unet& u, UnetLayer& l, int B, int lev, const bf16* gz, const bf16* x, int xcs, int up) {
+    const int H = u.H >> lev, W = u.W >> lev;
+    const int64_t P = (int64_t)B * H * W;
+    float* dW = u.grads.as<float>() + l.woff;
+    float* db = u.grads.as<float>() + l.boff;
+    if (l.cout == 1 && l.k == 1) {
+        // the head: both gradients in one pass
+        colsum(u, x, xcs, l.cin, P, gz, dW, db);
+        return;
+    }
+    if (l.cin == 1 && l.k == 3 && !up && xcs == 1) {
+        k_dw_point<<<152 * 4, 256, 0, u.st>>>(gz, l.cout, x, B, H, W, 32, dW);
+        PURIFY_CUDA(cudaGetLastError());
+        add_launches(1);
+    } else {
+        PURIFY_REQUIRE(dw_tc_ok(l.cout, l.cin, xcs, 0), "unet: layer channels must be multiples of 8");
+        dw_tc_launch(gz, l.cout, x, xcs, 0, l.cin, B, H, W, up, l.k, dW, u.err.as<int>(), u.st);
+    }
+    colsum(u, gz, l.cout, l.cout, P, nullptr, db, nullptr);
 }
 
 // forward + backward; gradients in u.grads, loss in u.loss (device)
@@ -496,77 +561,78 @@ void unet_gradients(Unet& u, const float* x, const float* target, int B) {
     unet_forward(u, x, B, nullptr);
     PURIFY_CUDA(cudaMemsetAsync(u.grads.p, 0, u.grads.bytes, u.st));
     const int64_t P0 = u.pix(0, B);
-    k_mse<<<256, 256, 0, u.st>>>(u.pred.as<float>(), target, u.gpred.as<float>(), P0, u.red_part.as<double>(),
+    // gz: gradient with respect to the current layer's pre-activation (BF16
+    // [P][cout]); each step writes the next one's into the other buffer
+    bf16 *gz = u.gz.as<bf16>(), *gn = u.gz2.as<bf16>();
+    float* const t = u.g1.as<float>();
+    auto masked = [&](const bf16* act, int cs, int co) {
+        GradOut g;
+        g.out = gn;
+        g.act = act;
+        g.act_cs = cs;
+        g.act_co = co;
+        return g;
+    };
+    GradOut plain;   // all channels in FP32
+    plain.f32 = t;
+    // head (1x1, no ReLU): gz = the loss gradient
+    k_mse<<<256, 256, 0, u.st>>>(u.pred.as<float>(), target, gz, P0, u.red_part.as<double>(),
                                  u.red_ctr.as<unsigned>(), u.loss.as<double>());
     add_launches(1);
-    // head (1x1, no ReLU): gz = gpred
-    k_f32_to_bf16<<<eblocks(P0), 256, 0, u.st>>>(u.gpred.as<float>(), u.gz.as<bf16>(), P0);
-    add_launches(1);
     UnetLayer& head = u.layer("head");
-    bwd_dw(u, head, B, 0, u.gz.as<bf16>(), u.dbb[0].as<bf16>(), u.base, 0, 0);
-    bwd_dx(u, head, B, 0, u.gz.as<bf16>(), u.g1.as<float>());
-    float* g = u.g1.as<float>();   // gradient w.r.t. the current layer's output
-    float* t = u.g2.as<float>();
+    bwd_dw(u, head, B, 0, gz, u.dbb[0].as<bf16>(), u.base, 0);
+    bwd_dx(u, head, B, 0, gz, masked(u.dbb[0].as<bf16>(), u.base, 0));
+    std::swap(gz, gn);
     for (int l = 0; l < L - 1; ++l) {
         const int c = u.ch(l);
-        const int64_t P = u.pix(l, B);
         std::string s = std::to_string(l);
         UnetLayer& lb = u.layer("d" + s + "b");
-        relu_grad(u, g, c, 0, u.dbb[l].as<bf16>(), c, 0, P, c);
-        bwd_dw(u, lb, B, l, u.gz.as<bf16>(), u.da[l].as<bf16>(), c, 0, 0);
-        bwd_dx(u, lb, B, l, u.gz.as<bf16>(), t);
-        std::swap(g, t);
+        bwd_dw(u, lb, B, l, gz, u.da[l].as<bf16>(), c, 0);
+        bwd_dx(u, lb, B, l, gz, masked(u.da[l].as<bf16>(), c, 0));
+        std::swap(gz, gn);
+        // the concatenation: channels [0, c) the skip (kept for the encoder),
+        // [c, 2c) the up branch
         UnetLayer& la = u.layer("d" + s + "a");
-        relu_grad(u, g, c, 0, u.da[l].as<bf16>(), c, 0, P, c);
-        bwd_dw(u, la, B, l, u.gz.as<bf16>(), u.cat[l].as<bf16>(), 2 * c, 0, 0);
-        bwd_dx(u, la, B, l, u.gz.as<bf16>(), u.gcat[l].as<float>());
-        // up branch: channels [c, 2c) of the concat
+        bwd_dw(u, la, B, l, gz, u.cat[l].as<bf16>(), 2 * c, 0);
+        GradOut both = masked(u.cat[l].as<bf16>(), 2 * c, c);
+        both.f32 = u.gcat[l].as<float>();
+        both.f32_ch = c;
+        bwd_dx(u, la, B, l, gz, both);
+        std::swap(gz, gn);
         UnetLayer& lu = u.layer("d" + s + "u");
-        relu_grad(u, u.gcat[l].as<float>(), 2 * c, c, u.cat[l].as<bf16>(), 2 * c, c, P, c);
         const bf16* low = (l == L - 2) ? u.bB.as<bf16>() : u.dbb[l + 1].as<bf16>();
-        bwd_dw(u, lu, B, l, u.gz.as<bf16>(), low, 2 * c, 0, 1);
-        bwd_dx(u, lu, B, l, u.gz.as<bf16>(), t);   // [P][2c] at level l
-        int64_t nlo = u.pix(l + 1, B) * 2 * c;
-        k_upsample_bwd<<<eblocks(nlo), 256, 0, u.st>>>(t, g, B, u.H >> l, u.W >> l, 2 * c);
+        bwd_dw(u, lu, B, l, gz, low, 2 * c, 1);
+        bwd_dx(u, lu, B, l, gz, plain);   // [P][2c] at level l
+        const int64_t nlo = u.pix(l + 1, B) * 2 * c / 8;
+        k_upsample_bwd<<<eblocks(nlo), 256, 0, u.st>>>(t, low, gn, B, u.H >> l, u.W >> l, 2 * c);
         add_launches(1);
-        // g now holds the gradient of the level-(l+1) decoder output (or the bottom)
+        std::swap(gz, gn);
     }
     const int cb = u.ch(L - 1);
-    const int64_t Pb = u.pix(L - 1, B);
     UnetLayer& lbb = u.layer("bb");
-    relu_grad(u, g, cb, 0, u.bB.as<bf16>(), cb, 0, Pb, cb);
-    bwd_dw(u, lbb, B, L - 1, u.gz.as<bf16>(), u.bA.as<bf16>(), cb, 0, 0);
-    bwd_dx(u, lbb, B, L - 1, u.gz.as<bf16>(), t);
-    std::swap(g, t);
+    bwd_dw(u, lbb, B, L - 1, gz, u.bA.as<bf16>(), cb, 0);
+    bwd_dx(u, lbb, B, L - 1, gz, masked(u.bA.as<bf16>(), cb, 0));
+    std::swap(gz, gn);
     UnetLayer& lba = u.layer("ba");
-    relu_grad(u, g, cb, 0, u.bA.as<bf16>(), cb, 0, Pb, cb);
-    bwd_dw(u, lba, B, L - 1, u.gz.as<bf16>(), u.pool[L - 2].as<bf16>(), u.ch(L - 2), 0, 0);
-    bwd_dx(u, lba, B, L - 1, u.gz.as<bf16>(), t);   // gradient of pool[L-2]
-    std::swap(g, t);
+    bwd_dw(u, lba, B, L - 1, gz, u.pool[L - 2].as<bf16>(), u.ch(L - 2), 0);
+    bwd_dx(u, lba, B, L - 1, gz, plain);   // gradient of pool[L-2]
     for (int l = L - 2; l >= 0; --l) {
         const int c = u.ch(l);
-        const int64_t P = u.pix(l, B);
         std::string s = std::to_string(l);
-        // through the max pooling, plus the skip gradient (channels [0, c) of gcat)
-        int64_t npool = u.pix(l + 1, B) * c;
-        k_maxpool_bwd<<<eblocks(npool), 256, 0, u.st>>>(u.cat[l].as<bf16>(), 2 * c, 0, g, u.gcat[l].as<float>(), 2 * c,
-                                                        0, t, B, u.H >> l, u.W >> l, c);
+        // through the max pooling, plus the skip gradient
+        const int64_t npool = u.pix(l + 1, B) * c / 8;
+        k_maxpool_bwd<<<eblocks(npool), 256, 0, u.st>>>(u.cat[l].as<bf16>(), 2 * c, 0, t, u.gcat[l].as<float>(), gz, B,
+                                                        u.H >> l, u.W >> l, c);
         add_launches(1);
-        std::swap(g, t);
         UnetLayer& lb = u.layer("e" + s + "b");
-        relu_grad(u, g, c, 0, u.cat[l].as<bf16>(), 2 * c, 0, P, c);
-        bwd_dw(u, lb, B, l, u.gz.as<bf16>(), u.a[l].as<bf16>(), c, 0, 0);
-        bwd_dx(u, lb, B, l, u.gz.as<bf16>(), t);
-        std::swap(g, t);
+        bwd_dw(u, lb, B, l, gz, u.a[l].as<bf16>(), c, 0);
+        bwd_dx(u, lb, B, l, gz, masked(u.a[l].as<bf16>(), c, 0));
+        std::swap(gz, gn);
         UnetLayer& la = u.layer("e" + s + "a");
-        relu_grad(u, g, c, 0, u.a[l].as<bf16>(), c, 0, P, c);
         const bf16* xin = l == 0 ? u.xbf.as<bf16>() : u.pool[l - 1].as<bf16>();
         const int xcs = l == 0 ? 1 : u.ch(l - 1);
-        bwd_dw(u, la, B, l, u.gz.as<bf16>(), xin, xcs, 0, 0);
-        if (l > 0) {
-            bwd_dx(u, la, B, l, u.gz.as<bf16>(), t);
-            std::swap(g, t);
-        }
+        bwd_dw(u, la, B, l, gz, xin, xcs, 0);
+        if (l > 0) bwd_dx(u, la, B, l, gz, plain);
     }
 }
 

@@ -7,21 +7,27 @@
 //
 // One analysis level maps an h x w low-pass band to four h/2 x w/2 sub-bands
 //   a[k] = sum_n h[n] x[(2k + n) mod len],  d[k] = sum_n g[n] x[(2k + n) mod len]
-// applied along rows, then along columns. A thread block owns a TH x TW tile
-// of every sub-band: it stages the (2TH + L - 2) x (2TW + L - 2) input tile
-// (indices wrapped as often as needed) in shared memory, filters the rows,
-// then the columns. All wavelet bases of a level run in one launch
-// (blockIdx.z); level 1 also writes the Dirac plane.
-//
-// Synthesis is the transpose: out[m] = sum over n of parity m of
-//   h[n] a[k] + g[n] d[k], k = ((m - n) mod len) / 2,
-// columns first, then rows. The finest level sums all bases and the Dirac
-// plane in one block per output tile, so the image is written once.
+// applied along rows, then along columns. A block owns a TH x TW tile of every
+// sub-band of one basis: its threads filter the rows of the input tile (TH plus
+// halo) straight from global memory, KX outputs of both filters from one
+// register window, into shared memory, then the columns, RK outputs of the four
+// sub-bands from two windows. Synthesis is the transpose: out[2i + par] = sum_j
+// h[2j + par] a[i - j] + g[2j + par] d[i - j], rows first (from global
+// memory), then columns; the finest level sums all bases in the block's
+// registers, so the image is written once. All wavelet bases of a level run in
+// one launch (blockIdx.z), filters with their compile-time lengths. The levels
+// whose bands fit shared memory run in one launch, a block per basis (*_tail).
+// The filters are a few multiply-adds per byte, so the register windows carry
+// the weight: with every tap read from shared memory these kernels were bound
+// by it (9 bases: analysis of 1024 x 1024 over 5 levels 58 us, now 32; synthesis
+// of 512 x 1024 over 4 levels 72 us, now 33; the coefficients' 42 and 21 MB
+// take 6 and 3 us).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -40,12 +46,22 @@ template <typename T> __device__ __forceinline__ const FilterBank<T>& fbank();
 template <> __device__ __forceinline__ const FilterBank<float>& fbank<float>() { return c_bank_f; }
 template <> __device__ __forceinline__ const FilterBank<double>& fbank<double>() { return c_bank_d; }
 
-// Tile geometry (compile time): analysis blocks own a DWT_T x DWT_T tile of
-// every sub-band; synthesis blocks own an (2 SYN_T) x (2 SYN_T) output tile.
-// Band sizes are powers of two, so periodic wrapping is a mask.
-static constexpr int DWT_T = 16;
-static constexpr int SYN_T = 8;
-static constexpr int SYN_GROUP = 64;   // threads per basis in a synthesis block
+// Tile geometry. FP32: sub-band tiles of 32 columns, 256 threads. FP64 is
+// bound by its arithmetic pipe (2 FMA per clock and SM): small tiles spread a
+// level over all SMs. Band sizes are powers of two, so wrapping is a mask.
+template <typename T> struct WaveTile;
+template <> struct WaveTile<float> {
+    static constexpr int TW = 32, KX = 4, THREADS = 256;
+    // largest band area of the tails: one SM per basis; 128 x 128 (two levels
+    // fewer launches) took 29 us where two launches of tiles take 10
+    static constexpr int TAIL = 1024;
+    static constexpr int SYN_TH = 16, SYN_RK = 4, SYN_THREADS = 256, GROUPS = 2;   // GROUPS: of the finest synthesis
+};
+template <> struct WaveTile<double> {
+    static constexpr int TW = 8, KX = 2, THREADS = 64, TAIL = 64;
+    static constexpr int SYN_TH = 4, SYN_RK = 2, SYN_THREADS = 32, GROUPS = 8;
+};
+static constexpr int TAIL_THREADS = 512;
 
 // The filter taps of basis pb in registers (unused entries are zero).
 template <typename T, int L> struct Taps {
@@ -72,68 +88,116 @@ template <typename T, int L> struct Taps {
     }
 
 // ------------------------------------------------------------- analysis
-// One analysis level of basis pb on the sub-band tile at (ky0, kx0).
-template <typename T, int L>
+// Row filters: low- and high-pass outputs k0 .. k0 + KX - 1 of one input row
+// (periodic, w columns) from a register window of 2 KX + L - 2 inputs; `vec`:
+// the row is in global memory or 16-byte aligned, w >= 4 (the window then
+// comes in 16-byte loads, which wrap as a whole).
+template <typename T, int L, int KX, bool VEC>
+__device__ __forceinline__ void row_filter(const Taps<T, L>& f, const T* __restrict__ row, int w, int k0, T (&a)[KX],
+                                           T (&d)[KX]) {
+    constexpr int V = 16 / sizeof(T), N = (2 * KX + L - 2 + V - 1) / V * V;
+    alignas(16) T win[N];
+    if constexpr (VEC) {
+#pragma unroll
+        for (int i = 0; i < N; i += V) {
+            const uint4 q = *reinterpret_cast<const uint4*>(row + ((2 * k0 + i) & (w - 1)));
+            *reinterpret_cast<uint4*>(win + i) = q;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 2 * KX + L - 2; ++i) win[i] = row[(2 * k0 + i) & (w - 1)];
+    }
+#pragma unroll
+    for (int j = 0; j < KX; ++j) {
+        a[j] = d[j] = T(0);
+#pragma unroll
+        for (int n = 0; n < L; ++n) {
+            a[j] += f.h[n] * win[2 * j + n];
+            d[j] += f.g[n] * win[2 * j + n];
+        }
+    }
+}
+
+// Column filters: sub-band rows 0 .. RK - 1 of one column from rows 0 .. 2 RK +
+// L - 3 (masked by rm) of the row-filtered columns ta, td (row stride ld).
+template <typename T, int L, int RK>
+__device__ __forceinline__ void col_filter(const Taps<T, L>& f, const T* ta, const T* td, int ld, int r0, int rm,
+                                           T (&ll)[RK], T (&lh)[RK], T (&hl)[RK], T (&hh)[RK]) {
+#pragma unroll
+    for (int j = 0; j < RK; ++j) ll[j] = lh[j] = hl[j] = hh[j] = T(0);
+#pragma unroll
+    for (int i = 0; i < 2 * RK + L - 2; ++i) {
+        const T av = ta[((r0 + i) & rm) * ld], dv = td[((r0 + i) & rm) * ld];
+#pragma unroll
+        for (int j = 0; j < RK; ++j) {
+            const int n = i - 2 * j;
+            if (n >= 0 && n < L) {
+                ll[j] += f.h[n] * av;
+                lh[j] += f.g[n] * av;
+                hl[j] += f.h[n] * dv;
+                hh[j] += f.g[n] * dv;
+            }
+        }
+    }
+}
+
+// One analysis level of basis pb on the TH x TW sub-band tile at (ky0, kx0).
+template <typename T, int L, int TH>
 __device__ __forceinline__ void dwt_tile(const T* __restrict__ in, int src_ld, T* __restrict__ out, int nx,
                                          T* __restrict__ llo, int h, int w, int ky0, int kx0, int pb, T inv_sqrt_q,
                                          T* smem) {
-    constexpr int RS = 2 * DWT_T + L - 2, CS = 2 * DWT_T + L - 2;
+    using W = WaveTile<T>;
+    constexpr int TW = W::TW, KX = W::KX, RK = TH * TW / W::THREADS, RG = TW / KX;
     Taps<T, L> f;
     f.load(pb);
     const int hs = h >> 1, wsub = w >> 1;
-    const int th = min(DWT_T, hs - ky0), tw = min(DWT_T, wsub - kx0);
-    const int Rin = 2 * th + L - 2, Cin = 2 * tw + L - 2;
-    T* tin = smem;                 // [RS][CS]
-    T* ta = tin + RS * CS;         // [RS][DWT_T] row low-pass
-    T* td = ta + RS * DWT_T;       // [RS][DWT_T] row high-pass
-    for (int t = threadIdx.x; t < Rin * CS; t += blockDim.x) {
-        const int r = t / CS, c = t - r * CS;
-        if (c < Cin) tin[t] = in[(size_t)((2 * ky0 + r) & (h - 1)) * src_ld + ((2 * kx0 + c) & (w - 1))];
+    const int th = min(TH, hs - ky0), tw = min(TW, wsub - kx0);
+    const int rows = 2 * th + L - 2;
+    T* ta = smem;                          // [2 TH + L - 2][TW] row low-pass
+    T* td = ta + (2 * TH + L - 2) * TW;    // row high-pass
+    for (int t = threadIdx.x; t < rows * RG; t += W::THREADS) {
+        const int r = t / RG, k = (t - r * RG) * KX;
+        if (k >= tw) continue;
+        const T* row = in + (size_t)((2 * ky0 + r) & (h - 1)) * src_ld;
+        alignas(16) T a[KX], d[KX];
+        if (w >= 4) row_filter<T, L, KX, true>(f, row, w, kx0 + k, a, d);
+        else row_filter<T, L, KX, false>(f, row, w, kx0 + k, a, d);
+        // KX outputs are 16 bytes; outputs past tw are not read
+        *reinterpret_cast<uint4*>(ta + r * TW + k) = *reinterpret_cast<const uint4*>(a);
+        *reinterpret_cast<uint4*>(td + r * TW + k) = *reinterpret_cast<const uint4*>(d);
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < Rin * DWT_T; t += blockDim.x) {
-        const int r = t / DWT_T, k = t - r * DWT_T;
-        if (k < tw) {
-            const T* row = tin + r * CS + 2 * k;
-            T a = 0, d = 0;
+    const int kx = threadIdx.x % TW, ky = threadIdx.x / TW * RK;
+    if (kx < tw && ky < th) {
+        T ll[RK], lh[RK], hl[RK], hh[RK];
+        col_filter<T, L, RK>(f, ta + kx, td + kx, TW, 2 * ky, ~0, ll, lh, hl, hh);
+        const int gx = kx0 + kx;
 #pragma unroll
-            for (int n = 0; n < L; ++n) { a += f.h[n] * row[n]; d += f.g[n] * row[n]; }
-            ta[t] = a;
-            td[t] = d;
+        for (int j = 0; j < RK; ++j) {
+            const int gy = ky0 + ky + j;
+            if (ky + j >= th) break;
+            if (llo) llo[(size_t)gy * wsub + gx] = ll[j];
+            else out[(size_t)gy * nx + gx] = ll[j] * inv_sqrt_q;
+            out[(size_t)gy * nx + wsub + gx] = hl[j] * inv_sqrt_q;
+            out[(size_t)(hs + gy) * nx + gx] = lh[j] * inv_sqrt_q;
+            out[(size_t)(hs + gy) * nx + wsub + gx] = hh[j] * inv_sqrt_q;
         }
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < DWT_T * DWT_T; t += blockDim.x) {
-        const int ky = t / DWT_T, kx = t - ky * DWT_T;
-        if (ky >= th || kx >= tw) continue;
-        T ll = 0, lh = 0, hl = 0, hh = 0;
-#pragma unroll
-        for (int n = 0; n < L; ++n) {
-            const T av = ta[(2 * ky + n) * DWT_T + kx], dv = td[(2 * ky + n) * DWT_T + kx];
-            ll += f.h[n] * av; lh += f.g[n] * av;
-            hl += f.h[n] * dv; hh += f.g[n] * dv;
-        }
-        const int gy = ky0 + ky, gx = kx0 + kx;
-        if (llo) llo[(size_t)gy * wsub + gx] = ll;
-        else out[(size_t)gy * nx + gx] = ll * inv_sqrt_q;
-        out[(size_t)gy * nx + wsub + gx] = hl * inv_sqrt_q;
-        out[(size_t)(hs + gy) * nx + gx] = lh * inv_sqrt_q;
-        out[(size_t)(hs + gy) * nx + wsub + gx] = hh * inv_sqrt_q;
     }
 }
 
 // One analysis level for every wavelet basis (blockIdx.z < nw) and, at the
-// first level, the Dirac plane (blockIdx.z == nw, a 2TH x 2TW image tile).
-template <typename T>
-__global__ void k_dwt_level(const T* __restrict__ src, int src_basis_stride, int src_ld,
-                            T* __restrict__ coef, const int* __restrict__ planes, int N, int nx,
-                            T* __restrict__ ll_out, int ll_basis_stride, int h, int w, int TH, int TW,
-                            const int* __restrict__ pids, int nw, int dirac_plane, T inv_sqrt_q) {
+// first level, the Dirac plane (blockIdx.z == nw, the tile's 2 TH x 2 TW image
+// pixels).
+template <typename T, int TH>
+__global__ void __launch_bounds__(WaveTile<T>::THREADS)
+k_dwt_level(const T* __restrict__ src, int src_basis_stride, int src_ld, T* __restrict__ coef,
+            const int* __restrict__ planes, int N, int nx, T* __restrict__ ll_out, int ll_basis_stride, int h, int w,
+            const int* __restrict__ pids, int nw, int dirac_plane, T inv_sqrt_q) {
+    constexpr int TW = WaveTile<T>::TW;
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int z = blockIdx.z;
     if (z == nw) {
-        // Dirac plane: coef[dirac] = x / sqrt(q) over a 2TH x 2TW image tile
         const int r0 = blockIdx.y * 2 * TH, c0 = blockIdx.x * 2 * TW;
         for (int t = threadIdx.x; t < 4 * TH * TW; t += blockDim.x) {
             int r = r0 + t / (2 * TW), c = c0 + t % (2 * TW);
@@ -145,184 +209,350 @@ __global__ void k_dwt_level(const T* __restrict__ src, int src_basis_stride, int
     const T* in = src + (size_t)z * src_basis_stride;
     T* out = coef + (size_t)planes[z] * N;
     T* llo = ll_out ? ll_out + (size_t)z * ll_basis_stride : nullptr;
-    const int ky0 = blockIdx.y * DWT_T, kx0 = blockIdx.x * DWT_T;
-    T* smem = reinterpret_cast<T*>(smem_raw);
     PURIFY_WITH_LENGTH(fbank<T>().len[pb],
-                       (dwt_tile<T, L>(in, src_ld, out, nx, llo, h, w, ky0, kx0, pb, inv_sqrt_q, smem)));
+                       (dwt_tile<T, L, TH>(in, src_ld, out, nx, llo, h, w, blockIdx.y * TH, blockIdx.x * TW, pb,
+                                           inv_sqrt_q, reinterpret_cast<T*>(smem_raw))));
+    pdl_trigger();
+}
+template <typename T> static size_t dwt_smem_bytes(int maxL, int TH) {
+    return sizeof(T) * 2 * (size_t)(2 * TH + maxL - 2) * WaveTile<T>::TW;
+}
+
+// The last `levels` analysis levels of basis pb in shared memory, from the h x
+// w band at `in` (row stride src_ld): a block per basis.
+template <typename T, int L>
+__device__ __forceinline__ void dwt_tail(const T* __restrict__ in, int src_ld, T* __restrict__ out, int nx, int h, int w,
+                                         int levels, int pb, T inv_sqrt_q, T* smem) {
+    constexpr int KX = WaveTile<T>::KX, RK = 2;
+    Taps<T, L> f;
+    f.load(pb);
+    // odd row strides: the row filters' lanes take consecutive rows
+    T* band = smem;                       // [h][w + 1]
+    T* ta = band + h * (w + 1);           // [h][w / 2 + 1]
+    T* td = ta + h * (w / 2 + 1);
+    for (int t = threadIdx.x; t < h * w; t += blockDim.x) band[t / w * (w + 1) + t % w] = in[(size_t)(t / w) * src_ld + t % w];
+    for (int lev = 0; lev < levels; ++lev) {
+        __syncthreads();
+        const int hs = h >> 1, wsub = w >> 1, rg = (wsub + KX - 1) / KX, ldt = wsub + 1;
+        for (int t = threadIdx.x; t < h * rg; t += blockDim.x) {
+            const int r = t & (h - 1), k = t / h * KX;
+            T a[KX], d[KX];
+            row_filter<T, L, KX, false>(f, band + r * (w + 1), w, k, a, d);
+#pragma unroll
+            for (int j = 0; j < KX; ++j)
+                if (k + j < wsub) {
+                    ta[r * ldt + k + j] = a[j];
+                    td[r * ldt + k + j] = d[j];
+                }
+        }
+        __syncthreads();
+        const bool last = lev == levels - 1;
+        const int kg = (hs + RK - 1) / RK;
+        for (int t = threadIdx.x; t < kg * wsub; t += blockDim.x) {
+            const int kx = t % wsub, ky = t / wsub * RK;
+            T ll[RK], lh[RK], hl[RK], hh[RK];
+            col_filter<T, L, RK>(f, ta + kx, td + kx, ldt, 2 * ky, h - 1, ll, lh, hl, hh);
+#pragma unroll
+            for (int j = 0; j < RK; ++j) {
+                const int gy = ky + j;
+                if (gy >= hs) break;
+                if (last) out[(size_t)gy * nx + kx] = ll[j] * inv_sqrt_q;
+                else band[gy * (wsub + 1) + kx] = ll[j];
+                out[(size_t)gy * nx + wsub + kx] = hl[j] * inv_sqrt_q;
+                out[(size_t)(hs + gy) * nx + kx] = lh[j] * inv_sqrt_q;
+                out[(size_t)(hs + gy) * nx + wsub + kx] = hh[j] * inv_sqrt_q;
+            }
+        }
+        h = hs;
+        w = wsub;
+    }
+}
+// blockIdx.x < nw: a wavelet basis; the blocks past them (when the tail holds
+// the first level) copy the Dirac plane
+template <typename T>
+__global__ void __launch_bounds__(TAIL_THREADS)
+k_dwt_tail(const T* __restrict__ src, int src_basis_stride, int src_ld, T* __restrict__ coef,
+           const int* __restrict__ planes, int N, int nx, int h, int w, int levels, const int* __restrict__ pids, int nw,
+           int dirac_plane, T inv_sqrt_q) {
+    pdl_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int z = blockIdx.x;
+    if (z >= nw) {
+        for (int t = threadIdx.x; t < h * w; t += blockDim.x)
+            coef[(size_t)dirac_plane * N + (size_t)(t / w) * nx + t % w] = src[(size_t)(t / w) * src_ld + t % w] * inv_sqrt_q;
+        return;
+    }
+    const int pb = pids[z];
+    PURIFY_WITH_LENGTH(fbank<T>().len[pb],
+                       (dwt_tail<T, L>(src + (size_t)z * src_basis_stride, src_ld, coef + (size_t)planes[z] * N, nx, h, w,
+                                       levels, pb, inv_sqrt_q, reinterpret_cast<T*>(smem_raw))));
     pdl_trigger();
 }
 
-// Shared memory of one analysis block (filters up to maxL taps).
-static size_t dwt_smem_bytes(int maxL, size_t tbytes) {
-    const size_t RS = 2 * DWT_T + maxL - 2;
-    return tbytes * (RS * RS + 2 * RS * DWT_T);
+// ------------------------------------------------------------ synthesis
+// Column synthesis of sub-band rows i0 .. i0 + RK - 1 of one column: output
+// rows 2 i0 .. 2 i0 + 2 RK - 1 of lo(i) and hi(i), the low- and high-pass
+// samples of row i (any i; the accessor wraps).
+template <typename T, int L, int RK, typename Lo, typename Hi>
+__device__ __forceinline__ void syn_filter(const Taps<T, L>& f, int i0, Lo lo, Hi hi, T (&o)[2 * RK]) {
+#pragma unroll
+    for (int m = 0; m < 2 * RK; ++m) o[m] = T(0);
+#pragma unroll
+    for (int i = 0; i < RK + L / 2 - 1; ++i) {
+        const T a = lo(i0 - (L / 2 - 1) + i), d = hi(i0 - (L / 2 - 1) + i);
+#pragma unroll
+        for (int r = 0; r < RK; ++r) {
+            const int j = r + L / 2 - 1 - i;   // tap pair of output row pair r
+            if (j >= 0 && j < L / 2) {
+                o[2 * r] += f.h[2 * j] * a + f.g[2 * j] * d;
+                o[2 * r + 1] += f.h[2 * j + 1] * a + f.g[2 * j + 1] * d;
+            }
+        }
+    }
 }
 
-// ------------------------------------------------------------ synthesis
-// Reconstruct the th2 x tw2 output tile at (oy0, ox0) of an h x w band for
-// basis pb from its four sub-bands, by the thread group (gt of gn threads).
-// `ll` points at the low-pass sub-band (row stride ll_ld); the three detail
-// sub-bands are read from `det` (the basis' coefficient plane, row stride
-// nx). Output t = gt + i * gn of the tile (row-major, stride tw2) is added to
-// acc[i].
-template <typename T, int L, int PER>
-__device__ __forceinline__ void synth_tile(const T* __restrict__ ll, int ll_ld, const T* __restrict__ det, int nx,
-                                           int h, int w, int oy0, int ox0, int th2, int tw2, int pb, T* smem, int gt,
-                                           int gn, T (&acc)[PER]) {
-    constexpr int KS = SYN_T + L / 2;            // sub-band tile stride (rows and columns)
+// barrier of one group of SYN_THREADS threads
+template <typename T> __device__ __forceinline__ void syn_sync(int group) {
+    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(WaveTile<T>::SYN_THREADS) : "memory");
+}
+
+// Row synthesis of 2 KX outputs from low-pass samples of `lo` and high-pass
+// samples of `hi` (n columns each, periodic), sub-band columns k0 .. k0 + KX - 1
+// (k0 a multiple of KX) and the L / 2 - 1 before them; VEC: both rows 16-byte
+// aligned, n >= 4 (the window comes in whole 16-byte loads).
+template <typename T, int L, int KX, bool VEC>
+__device__ __forceinline__ void syn_row(const Taps<T, L>& f, const T* __restrict__ lo, const T* __restrict__ hi, int n,
+                                        int k0, T* o) {
+    constexpr int V = 16 / sizeof(T), E = L / 2 - 1, EB = (E + V - 1) / V * V, NW = EB + KX;
+    alignas(16) T a[NW], d[NW];
+    if constexpr (VEC) {
+#pragma unroll
+        for (int i = 0; i < NW; i += V) {
+            const int c = (k0 - EB + i) & (n - 1);
+            *reinterpret_cast<uint4*>(a + i) = *reinterpret_cast<const uint4*>(lo + c);
+            *reinterpret_cast<uint4*>(d + i) = *reinterpret_cast<const uint4*>(hi + c);
+        }
+    } else {
+#pragma unroll
+        for (int i = EB - E; i < NW; ++i) {
+            const int c = (k0 - EB + i) & (n - 1);
+            a[i] = lo[c];
+            d[i] = hi[c];
+        }
+    }
+    T r[2 * KX];
+    syn_filter<T, L, KX>(f, 0, [&](int i) { return a[i + EB]; }, [&](int i) { return d[i + EB]; }, r);
+#pragma unroll
+    for (int e = 0; e < 2 * KX; ++e) o[e] = r[e];
+}
+
+// Basis pb's part of the (2 TH) x (2 TW) output tile whose sub-band tile
+// starts at (ky0, kx0): rows first (the four sub-bands in 16-byte loads, the low
+// and the high rows to shared memory), then columns. Thread item (output
+// column, group of RK sub-band rows) holds 2 RK outputs, added to acc. `ll`: the
+// low-pass sub-band (row stride ll_ld); the details are in `det` (row stride
+// nx). Ends with the shared tile free for the next basis.
+template <typename T, int L>
+__device__ __forceinline__ void synth_tile(const T* __restrict__ ll, int ll_ld, const T* __restrict__ det, int nx, int h,
+                                           int w, int ky0, int kx0, int pb, T* smem, int group, int tid,
+                                           T (&acc)[2 * WaveTile<T>::SYN_RK]) {
+    using W = WaveTile<T>;
+    constexpr int TH = W::SYN_TH, TW = W::TW, RK = W::SYN_RK, KX = W::KX, E = L / 2 - 1, RG = TW / KX, CW = 2 * TW;
+    static_assert(E <= 7, "filter longer than the row margin");
     Taps<T, L> f;
     f.load(pb);
     const int hs = h >> 1, wsub = w >> 1;
-    const int Kr = th2 / 2 + L / 2, Kc = tw2 / 2 + L / 2;
-    const int ky_lo = oy0 / 2 - L / 2, kx_lo = ox0 / 2 - L / 2;
-    T* sLL = smem;
-    T* sHL = sLL + KS * KS;   // row-detail, column-approx: (ky, wsub + kx)
-    T* sLH = sHL + KS * KS;   // row-approx, column-detail: (hs + ky, kx)
-    T* sHH = sLH + KS * KS;
-    T* sA = sHH + KS * KS;    // [2 SYN_T][KS]: column synthesis of the row-approx half
-    T* sD = sA + 2 * SYN_T * KS;
-    for (int t = gt; t < Kr * KS; t += gn) {
-        const int r = t / KS, c = t - r * KS;
-        if (c >= Kc) continue;
-        const int ky = (ky_lo + r) & (hs - 1), kx = (kx_lo + c) & (wsub - 1);
-        sLL[t] = ll[(size_t)ky * ll_ld + kx];
-        sHL[t] = det[(size_t)ky * nx + wsub + kx];
-        sLH[t] = det[(size_t)(hs + ky) * nx + kx];
-        sHH[t] = det[(size_t)(hs + ky) * nx + wsub + kx];
-    }
-    __syncthreads();
-    for (int t = gt; t < th2 * KS; t += gn) {
-        const int mr = t / KS, c = t - mr * KS;
-        if (c >= Kc) continue;
-        // output row m = oy0 + mr takes the taps n of its parity; sub-band
-        // row (m - n) / 2 - ky_lo = (mr - par) / 2 + L / 2 - j for n = 2 j + par
-        const int par = mr & 1;
-        const int r0 = ((mr - par) >> 1) + L / 2;
-        T a = 0, d = 0;
-#pragma unroll
-        for (int j = 0; j < L / 2; ++j) {
-            const T hn = par ? f.h[2 * j + 1] : f.h[2 * j], gn_ = par ? f.g[2 * j + 1] : f.g[2 * j];
-            const int r = r0 - j;
-            a += hn * sLL[r * KS + c] + gn_ * sLH[r * KS + c];
-            d += hn * sHL[r * KS + c] + gn_ * sHH[r * KS + c];
+    T* sL = smem;                    // [TH + 7][CW] rows of the low-pass (along y) half
+    T* sH = sL + (TH + 7) * CW;      // and of the high-pass half
+    for (int t = tid; t < (TH + E) * RG; t += W::SYN_THREADS) {
+        const int r = t / RG, k = (t - r * RG) * KX;
+        if (kx0 + k >= wsub) continue;
+        const int ky = (ky0 - E + r) & (hs - 1);
+        const T* const lo = det + (size_t)ky * nx + wsub;          // row-detail, column-approx
+        const T* const hi = det + (size_t)(hs + ky) * nx;          // row-approx, column-detail
+        alignas(16) T oL[2 * KX], oH[2 * KX];
+        if (wsub >= 4) {
+            syn_row<T, L, KX, true>(f, ll + (size_t)ky * ll_ld, lo, wsub, kx0 + k, oL);
+            syn_row<T, L, KX, true>(f, hi, hi + wsub, wsub, kx0 + k, oH);
+        } else {
+            syn_row<T, L, KX, false>(f, ll + (size_t)ky * ll_ld, lo, wsub, kx0 + k, oL);
+            syn_row<T, L, KX, false>(f, hi, hi + wsub, wsub, kx0 + k, oH);
         }
-        sA[t] = a;
-        sD[t] = d;
-    }
-    __syncthreads();
+        constexpr int V = 16 / sizeof(T);
 #pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const int t = gt + i * gn;
-        if (t < th2 * tw2) {
-            const int mr = t / tw2, mc = t - mr * tw2;
-            const int par = mc & 1;
-            const int c0 = ((mc - par) >> 1) + L / 2;
-            T sacc = 0;
-#pragma unroll
-            for (int j = 0; j < L / 2; ++j) {
-                const T hn = par ? f.h[2 * j + 1] : f.h[2 * j], gn_ = par ? f.g[2 * j + 1] : f.g[2 * j];
-                const int c = c0 - j;
-                sacc += hn * sA[mr * KS + c] + gn_ * sD[mr * KS + c];
-            }
-            acc[i] += sacc;
+        for (int e = 0; e < 2 * KX; e += V) {
+            *reinterpret_cast<uint4*>(sL + r * CW + 2 * k + e) = *reinterpret_cast<const uint4*>(oL + e);
+            *reinterpret_cast<uint4*>(sH + r * CW + 2 * k + e) = *reinterpret_cast<const uint4*>(oH + e);
         }
     }
-    __syncthreads();
+    syn_sync<T>(group);
+    static_assert(CW * (TH / RK) == W::SYN_THREADS, "one column item per thread");
+    {
+        const int x = tid % CW, g = tid / CW * RK;
+        const T *cl = sL + (g + E) * CW + x, *ch = sH + (g + E) * CW + x;
+        T o[2 * RK];
+        syn_filter<T, L, RK>(f, 0, [&](int i) { return cl[i * CW]; }, [&](int i) { return ch[i * CW]; }, o);
+#pragma unroll
+        for (int m = 0; m < 2 * RK; ++m) acc[m] += o[m];
+    }
+    syn_sync<T>(group);
+}
+// The same out of line, for the loop over bases (inlined there, the eight
+// lengths' windows were kept live together and spilled).
+template <typename T> struct SynthPart { T v[2 * WaveTile<T>::SYN_RK]; };
+template <typename T, int L>
+__device__ __noinline__ SynthPart<T> synth_part(const T* __restrict__ ll, int ll_ld, const T* __restrict__ det, int nx, int h,
+                                                int w, int ky0, int kx0, int pb, T* smem, int group, int tid) {
+    SynthPart<T> p = {};
+    synth_tile<T, L>(ll, ll_ld, det, nx, h, w, ky0, kx0, pb, smem, group, tid, p.v);
+    return p;
+}
+template <typename T> static size_t synth_smem_bytes() {
+    return sizeof(T) * 2 * (WaveTile<T>::SYN_TH + 7) * 2 * WaveTile<T>::TW;
 }
 
-// Shared memory of one synthesis tile (filters up to maxL taps).
-static size_t synth_smem_elems(int maxL) {
-    const size_t KS = SYN_T + maxL / 2;
-    return 4 * KS * KS + 2 * (2 * SYN_T) * KS;
-}
-
-// One synthesis level for every wavelet basis (blockIdx.z), SYN_LEVEL_THREADS
-// threads per block: writes the reconstructed h x w band of basis z into
-// ll_out (row stride w).
-static constexpr int SYN_LEVEL_THREADS = 128;
+// One synthesis level for every wavelet basis (blockIdx.z): the reconstructed
+// h x w band of basis z into ll_out (row stride w).
 template <typename T>
-__global__ void __launch_bounds__(SYN_LEVEL_THREADS)
+__global__ void __launch_bounds__(WaveTile<T>::SYN_THREADS)
 k_idwt_level(const T* __restrict__ ll_in, int ll_basis_stride, int ll_ld, const T* __restrict__ coef,
              const int* __restrict__ planes, int N, int nx, T* __restrict__ ll_out, int out_basis_stride, int h,
              int w, const int* __restrict__ pids) {
+    using W = WaveTile<T>;
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int PER = (4 * SYN_T * SYN_T + SYN_LEVEL_THREADS - 1) / SYN_LEVEL_THREADS;
-    const int z = blockIdx.z;
-    const int pb = pids[z];
-    const int oy0 = blockIdx.y * 2 * SYN_T, ox0 = blockIdx.x * 2 * SYN_T;
-    const int th2 = min(2 * SYN_T, h - oy0), tw2 = min(2 * SYN_T, w - ox0);
+    const int z = blockIdx.z, pb = pids[z];
+    const int ky0 = blockIdx.y * W::SYN_TH, kx0 = blockIdx.x * W::TW;
     const T* det = coef + (size_t)planes[z] * N;
     const T* ll = ll_in ? ll_in + (size_t)z * ll_basis_stride : det;
-    const int ld = ll_in ? ll_ld : nx;
-    T acc[PER];
-#pragma unroll
-    for (int i = 0; i < PER; ++i) acc[i] = 0;
-    T* smem = reinterpret_cast<T*>(smem_raw);
+    T acc[2 * W::SYN_RK] = {};
     PURIFY_WITH_LENGTH(fbank<T>().len[pb],
-                       (synth_tile<T, L, PER>(ll, ld, det, nx, h, w, oy0, ox0, th2, tw2, pb, smem,
-                                              (int)threadIdx.x, SYN_LEVEL_THREADS, acc)));
-    T* out = ll_out + (size_t)z * out_basis_stride;
+                       (synth_tile<T, L>(ll, ll_in ? ll_ld : nx, det, nx, h, w, ky0, kx0, pb,
+                                         reinterpret_cast<T*>(smem_raw), 0, (int)threadIdx.x, acc)));
+    constexpr int CW = 2 * W::TW;
+    const int y = 2 * (ky0 + threadIdx.x / CW * W::SYN_RK), x = 2 * kx0 + threadIdx.x % CW;
+    if (x < w) {
+        T* out = ll_out + (size_t)z * out_basis_stride + x;
 #pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const int t = threadIdx.x + i * SYN_LEVEL_THREADS;
-        if (t < th2 * tw2) {
-            const int mr = t / tw2, mc = t - mr * tw2;
-            out[(size_t)(oy0 + mr) * w + ox0 + mc] = acc[i];
-        }
+        for (int m = 0; m < 2 * W::SYN_RK; ++m)
+            if (y + m < h) out[(size_t)(y + m) * w] = acc[m];
     }
     pdl_trigger();
 }
 
 // Finest synthesis level summed over all wavelet bases plus the Dirac plane:
-// x = (c_dirac + sum_z W_z^T c_z) / sqrt(q). Thread group z (SYN_GROUP
-// threads) synthesises basis z's contribution to the block's output tile;
-// the partial tiles are then added in basis order. When `ll_in` is null
-// (L == 1) the low-pass bands come from the coefficient planes.
-// Every group runs the same code: filters zero-padded to the plan's longest
-// length L (the padded taps add exact zeros), so the block has one instruction
-// stream and one barrier sequence whatever the bases.
-template <typename T, int L>
-__global__ void __launch_bounds__(512, 2)
+// x = (c_dirac + sum_z W_z^T c_z) / sqrt(q). GROUPS groups of threads share a
+// tile, group g takes bases g, g + GROUPS, ... in order (their column passes
+// wait for global memory at different times), and the groups' sums are added
+// in group order. When `ll_in` is null (L == 1) the low-pass bands come from the
+// coefficient planes.
+template <typename T>
+__global__ void __launch_bounds__(WaveTile<T>::SYN_THREADS * WaveTile<T>::GROUPS, sizeof(T) == 4 ? 2 : 1)
 k_idwt_final(const T* __restrict__ ll_in, int ll_basis_stride, const T* __restrict__ coef,
-                             const int* __restrict__ planes, int N, int nx, int ny, int group_elems,
-                             const int* __restrict__ pids, int nw, int dirac_plane,
-                             T inv_sqrt_q, T* __restrict__ x) {
+             const int* __restrict__ planes, int N, int nx, int ny, const int* __restrict__ pids, int nw,
+             int dirac_plane, T inv_sqrt_q, T* __restrict__ x) {
+    using W = WaveTile<T>;
+    constexpr int NO = 2 * W::SYN_RK, G = W::GROUPS, NT = W::SYN_THREADS, CW = 2 * W::TW, GE = 2 * (W::SYN_TH + 7) * CW;
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int PER = (4 * SYN_T * SYN_T + SYN_GROUP - 1) / SYN_GROUP;
-    const int oy0 = blockIdx.y * 2 * SYN_T, ox0 = blockIdx.x * 2 * SYN_T;
-    const int th2 = min(2 * SYN_T, ny - oy0), tw2 = min(2 * SYN_T, nx - ox0);
-    const int z = threadIdx.x / SYN_GROUP, gt = threadIdx.x - z * SYN_GROUP;
-    const size_t per_group = (size_t)group_elems;   // shared elements of one group's tile
-    T* part = reinterpret_cast<T*>(smem_raw);                       // [nw][4 SYN_T^2] partial tiles
-    T* gsm = part + (size_t)nw * 4 * SYN_T * SYN_T + (size_t)z * per_group;
-    T acc[PER];
-#pragma unroll
-    for (int i = 0; i < PER; ++i) acc[i] = 0;
-    if (z < nw) {
+    T* const smem = reinterpret_cast<T*>(smem_raw);
+    const int ky0 = blockIdx.y * W::SYN_TH, kx0 = blockIdx.x * W::TW;
+    const int group = threadIdx.x / NT, tid = threadIdx.x - group * NT;
+    T acc[NO] = {};
+    for (int z = group; z < nw; z += G) {
         const int pb = pids[z];
         const T* det = coef + (size_t)planes[z] * N;
         const T* ll = ll_in ? ll_in + (size_t)z * ll_basis_stride : det;
-        const int ld = ll_in ? (nx >> 1) : nx;
-        synth_tile<T, L, PER>(ll, ld, det, nx, ny, nx, oy0, ox0, th2, tw2, pb, gsm, gt, SYN_GROUP, acc);
+        SynthPart<T> part;
+        PURIFY_WITH_LENGTH(fbank<T>().len[pb],
+                           (part = synth_part<T, L>(ll, ll_in ? (nx >> 1) : nx, det, nx, ny, nx, ky0, kx0, pb,
+                                                    smem + group * GE, group, tid)));
 #pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int t = gt + i * SYN_GROUP;
-            if (t < 4 * SYN_T * SYN_T) part[(size_t)z * 4 * SYN_T * SYN_T + t] = acc[i];
-        }
+        for (int e = 0; e < NO; ++e) acc[e] += part.v[e];
+    }
+    // the other groups' sums through shared memory (all are done with theirs)
+    __syncthreads();
+    if (group > 0) {
+#pragma unroll
+        for (int e = 0; e < NO; ++e) smem[((group - 1) * NO + e) * NT + tid] = acc[e];
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < th2 * tw2; t += blockDim.x) {
-        const int mr = t / tw2, mc = t - mr * tw2;
-        T v = 0;
-        for (int zz = 0; zz < nw; ++zz) v += part[(size_t)zz * 4 * SYN_T * SYN_T + t];
-        const size_t idx = (size_t)(oy0 + mr) * nx + ox0 + mc;
-        if (dirac_plane >= 0) v += coef[(size_t)dirac_plane * N + idx];
-        x[idx] = v * inv_sqrt_q;
+    const int y = 2 * (ky0 + tid / CW * W::SYN_RK), xx = 2 * kx0 + tid % CW;
+    if (group == 0 && xx < nx) {
+#pragma unroll
+        for (int e = 0; e < NO; ++e) {
+            T v = acc[e];
+#pragma unroll
+            for (int g = 0; g + 1 < G; ++g) v += smem[(g * NO + e) * NT + tid];
+            if (y + e < ny) {
+                const size_t idx = (size_t)(y + e) * nx + xx;
+                if (dirac_plane >= 0) v += coef[(size_t)dirac_plane * N + idx];
+                x[idx] = v * inv_sqrt_q;
+            }
+        }
     }
     pdl_trigger();
 }
+
+// The coarsest `levels` synthesis levels of a basis in shared memory, up to the
+// h x w band, written to ll_out (row stride w): a block per basis.
+template <typename T, int L>
+__device__ __forceinline__ void idwt_tail(const T* __restrict__ det, int nx, T* __restrict__ out, int h, int w, int levels,
+                                          int pb, T* smem) {
+    constexpr int KX = WaveTile<T>::KX, RK = 2;
+    Taps<T, L> f;
+    f.load(pb);
+    T* band = smem;                     // the low-pass band so far, [hs][wsub]
+    T* sA = band + h * (w + 1);         // [h][wsub + 1]: an odd stride, the row passes' lanes take consecutive rows
+    T* sD = sA + h * (w / 2 + 1);
+    {
+        const int hc = h >> levels, wc = w >> levels;
+        for (int t = threadIdx.x; t < hc * wc; t += blockDim.x) band[t] = det[(size_t)(t / wc) * nx + t % wc];
+    }
+    for (int lev = levels - 1; lev >= 0; --lev) {
+        __syncthreads();
+        const int hl = h >> lev, wl = w >> lev, hs = hl >> 1, wsub = wl >> 1, rg = (hs + RK - 1) / RK;
+        for (int t = threadIdx.x; t < rg * wsub; t += blockDim.x) {
+            const int kx = t % wsub, i0 = t / wsub * RK;
+            auto at = [&](const T* p) { return [=](int i) { return p[(size_t)(i & (hs - 1)) * nx + kx]; }; };
+            T o[2 * RK], q[2 * RK];
+            syn_filter<T, L, RK>(f, i0, [&](int i) { return band[(i & (hs - 1)) * wsub + kx]; }, at(det + (size_t)hs * nx), o);
+            syn_filter<T, L, RK>(f, i0, at(det + wsub), at(det + (size_t)hs * nx + wsub), q);
+#pragma unroll
+            for (int m = 0; m < 2 * RK; ++m)
+                if (2 * i0 + m < hl) {
+                    sA[(2 * i0 + m) * (wsub + 1) + kx] = o[m];
+                    sD[(2 * i0 + m) * (wsub + 1) + kx] = q[m];
+                }
+        }
+        __syncthreads();
+        T* dst = lev == 0 ? out : band;
+        const int cg = (wsub + KX - 1) / KX;
+        for (int t = threadIdx.x; t < hl * cg; t += blockDim.x) {
+            const int m = t & (hl - 1), k = t / hl * KX;
+            const T *ra = sA + m * (wsub + 1), *rd = sD + m * (wsub + 1);
+            T o[2 * KX];
+            syn_filter<T, L, KX>(f, k, [&](int i) { return ra[i & (wsub - 1)]; }, [&](int i) { return rd[i & (wsub - 1)]; }, o);
+#pragma unroll
+            for (int e = 0; e < 2 * KX; ++e)
+                if (2 * k + e < wl) dst[(size_t)m * wl + 2 * k + e] = o[e];
+        }
+    }
+}
+template <typename T>
+__global__ void __launch_bounds__(TAIL_THREADS)
+k_idwt_tail(const T* __restrict__ coef, const int* __restrict__ planes, int N, int nx, T* __restrict__ ll_out,
+            int out_basis_stride, int h, int w, int levels, const int* __restrict__ pids) {
+    pdl_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int z = blockIdx.x, pb = pids[z];
+    PURIFY_WITH_LENGTH(fbank<T>().len[pb],
+                       (idwt_tail<T, L>(coef + (size_t)planes[z] * N, nx, ll_out + (size_t)z * out_basis_stride, h, w,
+                                        levels, pb, reinterpret_cast<T*>(smem_raw))));
+    pdl_trigger();
+}
+// band and the two half-width columns, odd strides
+template <typename T> static size_t tail_smem_bytes(int h, int w) { return sizeof(T) * (size_t)h * (2 * w + 3); }
 
 // ------------------------------------------------------------- launchers
 struct WaveletLayout {
@@ -376,92 +606,125 @@ void init_filter_banks() {
     g_bank_ready[dev] = true;
 }
 
-template <typename T> static void psi_adj_t(purify_plan* p, const void* xv, void* cv) {
-    const T* x = (const T*)xv;
-    T* c = (T*)cv;
-    WaveletLayout wl = layout(p);
-    const T inv_sqrt_q = (T)(1.0 / std::sqrt((double)p->q));
-    const int N = (int)p->N;
-    if (wl.nw == 0) {
-        // Dirac only
-        Launch Lc(p, "dwt_level");
-        dim3 g((p->nx + 31) / 32, (p->ny + 31) / 32, 1);
-        launch_dependent(k_dwt_level<T>, g, 256, 0, p->stream, x, 0, p->nx, c, plane_array(p), N, p->nx, nullptr, 0, p->ny,
-                                                 p->nx, 16, 16, pid_array(p), 0, wl.dirac_plane, inv_sqrt_q);
-        Lc.done();
-        return;
-    }
-    int h = p->ny, w = p->nx;
+template <typename K> static void wave_smem(K kernel, size_t bytes) {
+    if (bytes > 48 * 1024) PURIFY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+}
+
+// Psi^dagger of an ny x nx image into coefficient planes c: `bufs` the two
+// low-pass buffers with their per-basis strides; launched(name) brackets each
+// launch (returns a callable run after it).
+template <typename T, typename Launched>
+static void analyse(const T* x, T* c, int nx, int ny, int levels, int nw, int dirac_plane, int q, int maxL,
+                    const int* pids, const int* planes, T* const (&bufs)[2], const int (&strides)[2], cudaStream_t st,
+                    Launched launched) {
+    using W = WaveTile<T>;
+    const T inv_sqrt_q = (T)(1.0 / std::sqrt((double)q));
+    const int N = nx * ny;
+    int h = ny, w = nx;
     const T* src = x;
-    int src_stride = 0, src_ld = p->nx;
-    T* bufs[2] = {p->ll0.as<T>(), p->ll1.as<T>()};
-    const int llstride = (int)(p->N / 4);
-    for (int lev = 0; lev < p->levels; ++lev) {
-        const bool last = lev == p->levels - 1;
+    int src_stride = 0, src_ld = nx;
+    if (nw == 0) levels = 1;   // the Dirac plane alone
+    for (int lev = 0; lev < levels; ++lev) {
+        const bool first = lev == 0;
+        const int dirac = first && dirac_plane >= 0 ? 1 : 0;
+        auto done = launched("dwt_level");
+        if (nw > 0 && h * w <= W::TAIL) {
+            const size_t sm = tail_smem_bytes<T>(h, w);
+            wave_smem(k_dwt_tail<T>, sm);
+            launch_dependent(k_dwt_tail<T>, nw + dirac, TAIL_THREADS, sm, st, src, src_stride, src_ld, c, planes, N, nx, h,
+                             w, levels - lev, pids, nw, dirac_plane, inv_sqrt_q);
+            done();
+            return;
+        }
         const int hs = h / 2, wsub = w / 2;
-        const int TH = std::min(DWT_T, hs), TW = std::min(DWT_T, wsub);
-        int maxL = 2;
-        for (int b : p->bases) if (b > 0) maxL = std::max(maxL, 2 * b);
-        const size_t sm = dwt_smem_bytes(maxL, sizeof(T));
-        int zdim = wl.nw + ((lev == 0 && wl.dirac_plane >= 0) ? 1 : 0);
-        dim3 g((wsub + TW - 1) / TW, (hs + TH - 1) / TH, zdim);
-        T* llo = last ? nullptr : bufs[lev & 1];
-        Launch L(p, "dwt_level");
-        launch_dependent(k_dwt_level<T>, g, 256, sm, p->stream, src, src_stride, src_ld, c, plane_array(p), N, p->nx, llo,
-                                                  llstride, h, w, TH, TW, pid_array(p), wl.nw,
-                                                  wl.dirac_plane, inv_sqrt_q);
-        L.done();
+        T* llo = lev == levels - 1 ? nullptr : bufs[lev & 1];
+        auto go = [&](auto kern, int TH) {
+            const size_t sm = dwt_smem_bytes<T>(maxL, TH);
+            wave_smem(kern, sm);
+            const dim3 g((wsub + W::TW - 1) / W::TW, (hs + TH - 1) / TH, nw + dirac);
+            launch_dependent(kern, g, W::THREADS, sm, st, src, src_stride, src_ld, c, planes, N, nx, llo, strides[lev & 1],
+                             h, w, pids, nw, dirac_plane, inv_sqrt_q);
+        };
+        // tall tiles cost less halo; short ones while those do not fill the chip
+        if constexpr (sizeof(T) == 4) {
+            const int64_t cols = (wsub + W::TW - 1) / W::TW;
+            if (cols * ((hs + 31) / 32) * std::max(nw, 1) >= 152 * 4) go(k_dwt_level<T, 32>, 32);
+            else if (cols * ((hs + 15) / 16) * std::max(nw, 1) >= 152) go(k_dwt_level<T, 16>, 16);
+            else go(k_dwt_level<T, 8>, 8);
+        } else {
+            go(k_dwt_level<T, 8>, 8);
+        }
+        done();
         src = llo;
-        src_stride = llstride;
+        src_stride = strides[lev & 1];
         src_ld = wsub;
         h = hs;
         w = wsub;
     }
 }
 
-template <typename T, int L>
-static void launch_idwt_final(purify_plan* p, dim3 g, int threads, size_t sm, const T* ll_in, int llstride,
-                              const T* c, int N, int group_elems, const WaveletLayout& wl, T inv_sqrt_q, T* x) {
-    if (sm > 48 * 1024)
-        PURIFY_CUDA(cudaFuncSetAttribute(k_idwt_final<T, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    launch_dependent(k_idwt_final<T, L>, g, threads, sm, p->stream, ll_in, llstride, c, plane_array(p), N, p->nx,
-                     p->ny, group_elems, pid_array(p), wl.nw, wl.dirac_plane, inv_sqrt_q, x);
+static int longest_filter(const purify_plan* p) {
+    int maxL = 2;
+    for (int b : p->bases) if (b > 0) maxL = std::max(maxL, 2 * b);
+    return maxL;
+}
+
+template <typename T> static void psi_adj_t(purify_plan* p, const void* xv, void* cv) {
+    const WaveletLayout wl = layout(p);
+    T* const bufs[2] = {p->ll0.as<T>(), p->ll1.as<T>()};
+    const int strides[2] = {(int)(p->N / 4), (int)(p->N / 4)};
+    analyse<T>((const T*)xv, (T*)cv, p->nx, p->ny, p->levels, wl.nw, wl.dirac_plane, p->q, longest_filter(p),
+               pid_array(p), plane_array(p), bufs, strides, p->stream, [&](const char* name) {
+                   auto l = std::make_shared<Launch>(p, name);
+                   return [l] { l->done(); };
+               });
 }
 
 template <typename T> static void psi_t(purify_plan* p, const void* cv, void* xv) {
+    using W = WaveTile<T>;
     const T* c = (const T*)cv;
     T* x = (T*)xv;
-    WaveletLayout wl = layout(p);
+    const WaveletLayout wl = layout(p);
     const T inv_sqrt_q = (T)(1.0 / std::sqrt((double)p->q));
-    const int N = (int)p->N;
-    int maxL = 2;
-    for (int b : p->bases) if (b > 0) maxL = std::max(maxL, 2 * b);
+    const int N = (int)p->N, llstride = (int)(p->N / 4);
     T* bufs[2] = {p->ll0.as<T>(), p->ll1.as<T>()};
-    const int llstride = (int)(p->N / 4);
     const T* ll_in = nullptr;  // coarsest level reads LL from the coefficients
     int ll_ld = p->nx;
-    // levels L .. 2 reconstruct low-pass bands into scratch
-    const size_t group_elems = synth_smem_elems(maxL);
-    for (int lev = p->levels - 1; lev >= 1 && wl.nw > 0; --lev) {
-        const int h = p->ny >> lev, w = p->nx >> lev;
-        const size_t sm = sizeof(T) * group_elems;
-        dim3 g((w + 2 * SYN_T - 1) / (2 * SYN_T), (h + 2 * SYN_T - 1) / (2 * SYN_T), wl.nw);
-        T* out = bufs[lev & 1];
-        if (sm > 48 * 1024) PURIFY_CUDA(cudaFuncSetAttribute(k_idwt_level<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        Launch L(p, "idwt_level");
-        launch_dependent(k_idwt_level<T>, g, SYN_LEVEL_THREADS, sm, p->stream, ll_in, llstride, ll_ld, c, plane_array(p), N,
-                                                                 p->nx, out, llstride, h, w, pid_array(p));
-        L.done();
-        ll_in = out;
-        ll_ld = w;
+    // levels L .. 2 reconstruct low-pass bands into scratch, the coarse ones
+    // together
+    int lev = p->levels - 1;
+    if (wl.nw > 0) {
+        int top = lev + 1;   // finest of the levels whose output fits the tail
+        while (top > 1 && ((int64_t)(p->ny >> (top - 1)) * (p->nx >> (top - 1))) <= W::TAIL) --top;
+        if (top <= lev) {
+            const int h = p->ny >> top, w = p->nx >> top;
+            T* out = bufs[top & 1];
+            const size_t sm = tail_smem_bytes<T>(h, w);
+            wave_smem(k_idwt_tail<T>, sm);
+            Launch L(p, "idwt_level");
+            launch_dependent(k_idwt_tail<T>, wl.nw, TAIL_THREADS, sm, p->stream, c, plane_array(p), N, p->nx, out, llstride, h,
+                             w, lev - top + 1, pid_array(p));
+            L.done();
+            ll_in = out;
+            ll_ld = w;
+            lev = top - 1;
+        }
+        for (; lev >= 1; --lev) {
+            const int h = p->ny >> lev, w = p->nx >> lev;
+            dim3 g((w / 2 + W::TW - 1) / W::TW, (h / 2 + W::SYN_TH - 1) / W::SYN_TH, wl.nw);
+            T* out = bufs[lev & 1];
+            Launch L(p, "idwt_level");
+            launch_dependent(k_idwt_level<T>, g, W::SYN_THREADS, synth_smem_bytes<T>(), p->stream, ll_in, llstride, ll_ld, c,
+                             plane_array(p), N, p->nx, out, llstride, h, w, pid_array(p));
+            L.done();
+            ll_in = out;
+            ll_ld = w;
+        }
     }
-    // finest level: one thread group per basis, partial tiles summed in order
-    const size_t sm = sizeof(T) * ((size_t)wl.nw * 4 * SYN_T * SYN_T + (size_t)wl.nw * group_elems);
-    dim3 g((p->nx + 2 * SYN_T - 1) / (2 * SYN_T), (p->ny + 2 * SYN_T - 1) / (2 * SYN_T), 1);
-    const int threads = std::max(1, wl.nw) * SYN_GROUP;
+    dim3 g((p->nx / 2 + W::TW - 1) / W::TW, (p->ny / 2 + W::SYN_TH - 1) / W::SYN_TH, 1);
     Launch Lf(p, "idwt_final");
-    PURIFY_WITH_LENGTH(maxL, (launch_idwt_final<T, L>(p, g, threads, sm, ll_in, llstride, c, N, (int)group_elems, wl,
-                                                       inv_sqrt_q, x)));
+    launch_dependent(k_idwt_final<T>, g, W::SYN_THREADS * W::GROUPS, synth_smem_bytes<T>() * W::GROUPS, p->stream, ll_in, llstride, c, plane_array(p), N,
+                     p->nx, p->ny, pid_array(p), wl.nw, wl.dirac_plane, inv_sqrt_q, x);
     Lf.done();
 }
 
@@ -554,46 +817,19 @@ static void psi_adj_static_t(const T* x, T* c, int nx, int ny, int levels, unsig
         ++q;
     }
     // per-basis strides: N / 4 in the first buffer, N / 16 in the second
-    T* bufs[2] = {static_cast<T*>(scratch), static_cast<T*>(scratch) + (size_t)nw * (N / 4)};
+    T* const bufs[2] = {static_cast<T*>(scratch), static_cast<T*>(scratch) + (size_t)nw * (N / 4)};
     const int strides[2] = {(int)(N / 4), (int)(N / 16)};
     int maxL = 2;
     for (int b = 1; b < 9; ++b) if (mask >> b & 1) maxL = std::max(maxL, 2 * b);
-    const T inv_sqrt_q = (T)(1.0 / std::sqrt((double)q));
     k_static_meta<<<1, 32, 0, st>>>(mask, meta);
     PURIFY_CUDA(cudaGetLastError());
     add_launches(1);
-    const int* pids = meta;
-    const int* planes = meta + 8;
-    if (nw == 0) {
-        dim3 g((nx + 31) / 32, (ny + 31) / 32, 1);
-        launch_dependent(k_dwt_level<T>, g, 256, 0, st, x, 0, nx, c, planes, (int)N, nx, nullptr, 0, ny, nx, 16, 16, pids, 0,
-                                          dirac_plane, inv_sqrt_q);
-        PURIFY_CUDA(cudaGetLastError());
-        add_launches(1);
-        return;
-    }
-    int h = ny, w = nx;
-    const T* src = x;
-    int src_stride = 0, src_ld = nx;
-    for (int lev = 0; lev < levels; ++lev) {
-        const bool last = lev == levels - 1;
-        const int hs = h / 2, wsub = w / 2;
-        const int TH = std::min(DWT_T, hs), TW = std::min(DWT_T, wsub);
-        const size_t sm = dwt_smem_bytes(maxL, sizeof(T));
-        int zdim = nw + ((lev == 0 && dirac_plane >= 0) ? 1 : 0);
-        dim3 g((wsub + TW - 1) / TW, (hs + TH - 1) / TH, zdim);
-        T* llo = last ? nullptr : bufs[lev & 1];
-        const int llstride = strides[lev & 1];
-        launch_dependent(k_dwt_level<T>, g, 256, sm, st, src, src_stride, src_ld, c, planes, (int)N, nx, llo, llstride, h, w, TH,
-                                           TW, pids, nw, dirac_plane, inv_sqrt_q);
-        PURIFY_CUDA(cudaGetLastError());
-        add_launches(1);
-        src = llo;
-        src_stride = llstride;
-        src_ld = wsub;
-        h = hs;
-        w = wsub;
-    }
+    analyse<T>(x, c, nx, ny, levels, nw, dirac_plane, q, maxL, meta, meta + 8, bufs, strides, st, [](const char*) {
+        return [] {
+            PURIFY_CUDA(cudaGetLastError());
+            add_launches(1);
+        };
+    });
 }
 
 void psi_adj_static(const void* x, void* c, int nx, int ny, int levels, unsigned mask, int dtype,

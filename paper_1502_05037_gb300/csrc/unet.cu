@@ -42,6 +42,7 @@ static constexpr uint32_t WAIT_LIMIT = 1u << 24;
 static constexpr int T_ROWS = 16, T_COLS = 8, HALO_W = T_COLS + 2, HALO_N = (T_ROWS + 2) * HALO_W, TP = HALO_N + 1;
 static constexpr int CONV_STAGE = 16384;    // bytes of weights per ring stage
 static constexpr int CONV_SLOTS = 4;
+static constexpr int CONV_THREADS = 256;   // two warps per 32 accumulator rows: each takes every other 16 columns
 
 __device__ __forceinline__ void cp_async16z(uint32_t sdst, const void* gsrc, bool valid) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sdst), "l"(gsrc), "r"(valid ? 16 : 0) : "memory");
@@ -59,30 +60,29 @@ template <int N> __device__ __forceinline__ void cp_async_wait_pending() {
 __device__ __forceinline__ void load_halo(unsigned char* sdst, const bf16* in, int b, int y0, int x0, int H, int W,
                                           int Cin, int cs, int co, int up, int g0, int ng, bool vec) {
     const int Hs = H >> up, Ws = W >> up;
-    // item (pos, g) = (i / ng, i mod ng), advanced without divisions
-    const int dpos = (int)blockDim.x / ng, dg = (int)blockDim.x - dpos * ng;
-    int pos = (int)threadIdx.x / ng, g = (int)threadIdx.x - pos * ng;
     const bf16* const base = in + (size_t)b * Hs * Ws * cs + co + g0 * 8;
     const uint32_t sbase = tc::smem_u32(sdst);
     const int cmax = Cin - g0 * 8;
-    while (pos < HALO_N) {
-        const int py = pos / HALO_W, y = y0 + py - 1, x = x0 + (pos - py * HALO_W) - 1;
-        const bool inside = (unsigned)y < (unsigned)H && (unsigned)x < (unsigned)W && g * 8 < cmax;
-        const bf16* src = inside ? base + (size_t)((y >> up) * Ws + (x >> up)) * cs + g * 8 : in;
-        const int slot = (g * TP + pos) * 16;
-        if (vec) {
-            cp_async16z(sbase + slot, src, inside);
-        } else {
-            bf16 v[8];
+    // a thread takes channel group g of halo column px and every nr-th row of
+    // it (the columns that do not fit the block's threads in further rounds)
+    const int cols = ng * HALO_W, nr = max(1, min(T_ROWS + 2, CONV_THREADS / cols));
+    for (int j = threadIdx.x; j < cols * nr; j += CONV_THREADS) {
+        const int g = j % ng, q = j / ng, px = q % HALO_W, x = x0 + px - 1;
+        const bool xin = (unsigned)x < (unsigned)W && g * 8 < cmax;
+        const bf16* const col = base + (xin ? (size_t)(x >> up) * cs + g * 8 : 0);
+        for (int py = q / HALO_W; py < T_ROWS + 2; py += nr) {
+            const int y = y0 + py - 1;
+            const bool inside = xin && (unsigned)y < (unsigned)H;
+            const bf16* src = inside ? col + (size_t)((y >> up) * Ws) * cs : in;
+            const int slot = (g * TP + py * HALO_W + px) * 16;
+            if (vec) {
+                cp_async16z(sbase + slot, src, inside);
+            } else {
+                bf16 v[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = inside && g * 8 + e < cmax ? src[e] : __float2bfloat16(0.f);
-            *reinterpret_cast<uint4*>(sdst + slot) = *reinterpret_cast<const uint4*>(v);
-        }
-        pos += dpos;
-        g += dg;
-        if (g >= ng) {
-            g -= ng;
-            ++pos;
+                for (int e = 0; e < 8; ++e) v[e] = inside && g * 8 + e < cmax ? src[e] : __float2bfloat16(0.f);
+                *reinterpret_cast<uint4*>(sdst + slot) = *reinterpret_cast<const uint4*>(v);
+            }
         }
     }
 }
@@ -141,20 +141,143 @@ __device__ __forceinline__ void conv_store(const ConvArgs& a, size_t q, int c, f
     }
 }
 
-// Convolution by halo tiles (see the top). blockIdx.x: tile; blockIdx.y:
+// Convolution by halo tiles with all of a block's weights in shared memory: a
+// block keeps the weights of its output channels [blockIdx.y nsub, + nsub) and
+// walks tiles blockIdx.x, + gridDim.x, ...; while the MMAs of a tile run (into
+// one of two accumulators), the next tile's halo is copied into the other of
+// two buffers and the previous tile's accumulator is stored.
+// Eight warps load and store (two per quarter of the accumulator rows), so that
+// the issue slots, not one warp's chain of address and conversion work, bound
+// a tile: with four, a 32 -> 32 tile took 10 thousand cycles to store and 1.9
+// to load beside 2.3 of MMA issue. A gradient (8 images, 256 x 256, 4 levels,
+// base 32) took 4438 us and a forward pass of one 361 with a block per tile and
+// one thread issuing, and 3402 and 271 now; with a block per tile and the rest
+// as here, 3495 and 283.
+__global__ void __launch_bounds__(CONV_THREADS) k_conv_tiles(ConvArgs a, int tiles_x, int tiles_y, int ntiles, int nsub) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t bar[2];
+    __shared__ uint32_t s_taddr;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int G8 = a.Cinp / 8, KT = a.k * a.k * G8;
+    const int a_bytes = (G8 * TP * 16 + 127) / 128 * 128;
+    unsigned char* const sB = smem + 2 * (size_t)a_bytes;
+    uint32_t ncols = 32;
+    while ((int)ncols < 2 * nsub) ncols <<= 1;
+    if (warp == 0) {
+        tc::tmem_alloc(&s_taddr, ncols);
+        tc::tmem_relinquish();
+    }
+    if (tid == 0) {
+        tc::mbar_init(&bar[0], 1);
+        tc::mbar_init(&bar[1], 1);
+    }
+    const int n0 = blockIdx.y * nsub;
+    const bool vec_in = a.in_cs % 8 == 0 && a.in_co % 8 == 0 && a.Cin % 8 == 0;
+    auto origin = [&](int tile, int& b, int& y0, int& x0) {
+        b = tile / (tiles_x * tiles_y);
+        const int rem = tile - b * tiles_x * tiles_y;
+        y0 = rem / tiles_x * T_ROWS;
+        x0 = (rem - rem / tiles_x * tiles_x) * T_COLS;
+    };
+    auto load = [&](int tile, int buf) {
+        int b, y0, x0;
+        origin(tile, b, y0, x0);
+        load_halo(smem + (size_t)buf * a_bytes, a.in, b, y0, x0, a.H, a.W, a.Cin, a.in_cs, a.in_co, a.up, 0, G8, vec_in);
+    };
+    // the weights, packed [tap][ci / 8][Npad][8]
+    {
+        const int dgr = CONV_THREADS / nsub, drow = CONV_THREADS - dgr * nsub;
+        int g = tid / nsub, r = tid - g * nsub;
+        uint32_t d = tc::smem_u32(sB) + tid * 16;
+        while (g < KT) {
+            cp_async16z(d, a.w + ((size_t)g * a.Npad + n0 + r) * 8, true);
+            d += CONV_THREADS * 16;
+            g += dgr;
+            r += drow;
+            if (r >= nsub) {
+                r -= nsub;
+                ++g;
+            }
+        }
+    }
+    const int first = blockIdx.x, step = gridDim.x;
+    load(first, 0);
+    cp_async_commit_group();
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tbase = s_taddr, idesc = tc::idesc_bf16_f32(128, nsub);
+    const uint64_t ad0 = tc::smem_desc(tc::smem_u32(smem), TP * 16, HALO_W * 16);
+    const uint64_t bd0 = tc::smem_desc(tc::smem_u32(sB), nsub * 16, 128);
+    auto store = [&](int tile, int buf) {
+        int b, y0, x0;
+        origin(tile, b, y0, x0);
+        const int row = (warp & 3) * 32 + lane, y = y0 + row / T_COLS, x = x0 + row % T_COLS;
+        const bool ok = y < a.H && x < a.W;
+        const size_t q = ((size_t)b * a.H + y) * a.W + x;
+        for (int c = (warp >> 2) * 16; c < nsub; c += 32) {
+            float v[16];
+            tc::tmem_ld16(tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(buf * nsub + c), v);
+            if (ok && n0 + c < a.Cout) conv_store(a, q, n0 + c, v);
+        }
+    };
+    int fail = 0, i = 0;
+    for (int tile = first; tile < ntiles; tile += step, ++i) {
+        const int buf = i & 1;
+        cp_async_wait_pending<0>();
+        tc::fence_proxy_async();
+        tc::fence_before_sync();
+        if (__syncthreads_or(fail)) { fail = 1; break; }
+        if (warp == 0) {
+            tc::fence_after_sync();
+            uint64_t bd = bd0;
+            const uint64_t ad = ad0 + (uint32_t)(buf * (a_bytes / 16));
+            int g = 0, tap = 0, sh = a.k == 3 ? 0 : HALO_W + 1;
+            for (int s = 0; s < KT; s += 2) {
+                tc::mma_bf16(tbase + (uint32_t)(buf * nsub), ad + (uint32_t)(g * TP + sh), bd, idesc, s > 0 ? 1u : 0u);
+                bd += 2 * nsub;
+                g += 2;
+                if (g == G8) {
+                    g = 0;
+                    ++tap;
+                    sh += tap % 3 == 0 ? HALO_W - 2 : 1;
+                }
+            }
+            tc::mma_commit(&bar[buf]);
+        }
+        // the MMAs of the tile before are done: its buffer and accumulator are free to use
+        if (i > 0 && !tc::mbar_wait(&bar[buf ^ 1], ((i - 1) >> 1) & 1, WAIT_LIMIT)) fail = 1;
+        if (!fail && tile + step < ntiles) load(tile + step, buf ^ 1);
+        cp_async_commit_group();
+        if (!fail && i > 0) {
+            tc::fence_after_sync();
+            store(tile - step, buf ^ 1);
+        }
+    }
+    if (!fail && !tc::mbar_wait(&bar[(i - 1) & 1], ((i - 1) >> 1) & 1, WAIT_LIMIT)) fail = 1;
+    cp_async_wait_pending<0>();
+    fail = __syncthreads_or(fail);
+    tc::fence_after_sync();
+    if (!fail) store(first + (i - 1) * step, (i - 1) & 1);
+    else if (tid == 0) atomicExch(a.err, 1);
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(tbase, ncols);
+}
+
+// Convolution by halo tiles, the weights streamed (wide inputs). blockIdx.x: tile; blockIdx.y:
 // output channels [blockIdx.y nsub, + nsub). kg: 8-channel groups of weights per
 // ring stage (even).
 // Bound by shared-memory bandwidth (a 128 x N x 16 MMA reads (128 + N) x 32
 // bytes) and, for the narrow layers, by the copies into it; several blocks per
 // SM overlap one's copies with another's MMAs and epilogue. The form before it
-// gathered every tap's rows anew and waited for the MMAs after each 64
-// channels: the layers of 8 images at 256 x 256 (4 levels, base 32) took 252 us
-// on average, now 74; at 32 x 32 154 and now 55.
-__global__ void __launch_bounds__(128) k_conv_halo(ConvArgs a, int tiles_x, int tiles_y, int nsub, int kg, int slots) {
+// gathered every tap's rows anew and waited for the MMAs after each 64 channels:
+// 8 images of 32 x 32, 256 to 512 channels, took 154 us, now 44.
+__global__ void __launch_bounds__(CONV_THREADS) k_conv_halo(ConvArgs a, int tiles_x, int tiles_y, int nsub, int kg, int slots) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar[CONV_SLOTS];
     __shared__ uint32_t s_taddr;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int G8 = a.Cinp / 8;                       // channel groups of the input
     const int KT = a.k * a.k * G8;                   // channel groups over all taps
     const int NS = (KT + kg - 1) / kg;               // stages
@@ -177,7 +300,7 @@ __global__ void __launch_bounds__(128) k_conv_halo(ConvArgs a, int tiles_x, int 
     load_halo(sA, a.in, b, y0, x0, a.H, a.W, a.Cin, a.in_cs, a.in_co, a.up, 0, G8, vec_in);
     // stage i of the weights: channel groups [i kg, (i + 1) kg) of the packed
     // order [tap][ci / 8][Npad][8], this block's output channels
-    const int dgr = 128 / nsub, drow = 128 - dgr * nsub, g_first = tid / nsub, r_first = tid - g_first * nsub;
+    const int dgr = CONV_THREADS / nsub, drow = CONV_THREADS - dgr * nsub, g_first = tid / nsub, r_first = tid - g_first * nsub;
     const uint32_t b0 = tc::smem_u32(sB);
     auto load_stage = [&](int i) {
         const int k0 = i * kg, n = min(kg, KT - k0);
@@ -186,7 +309,7 @@ __global__ void __launch_bounds__(128) k_conv_halo(ConvArgs a, int tiles_x, int 
         int g = g_first, r = r_first;
         while (g < n) {
             cp_async16z(d, src + (size_t)(g * a.Npad + r) * 8, true);
-            d += 128 * 16;
+            d += CONV_THREADS * 16;
             g += dgr;
             r += drow;
             if (r >= nsub) {
@@ -207,14 +330,14 @@ __global__ void __launch_bounds__(128) k_conv_halo(ConvArgs a, int tiles_x, int 
     // operand descriptors; a start address moves in units of 16 bytes
     const uint64_t ad0 = tc::smem_desc(tc::smem_u32(sA), TP * 16, HALO_W * 16);
     const uint64_t bd0 = tc::smem_desc(b0, nsub * 16, 128);
-    int tap = 0, g = 0, fail = 0;   // of the next K step (thread 0)
+    int tap = 0, g = 0, fail = 0;   // of the next K step
     int sh = a.k == 3 ? 0 : HALO_W + 1;
     for (int i = 0; i < NS; ++i) {
         cp_async_wait_pending<CONV_SLOTS - 2>();
         tc::fence_proxy_async();
         tc::fence_before_sync();
         if (__syncthreads_or(fail)) { fail = 1; break; }
-        if (tid == 0) {
+        if (warp == 0) {
             tc::fence_after_sync();
             const int n = min(kg, KT - i * kg);
             uint64_t bd = bd0 + (uint32_t)((i % slots) * (slot_bytes / 16));
@@ -244,12 +367,12 @@ __global__ void __launch_bounds__(128) k_conv_halo(ConvArgs a, int tiles_x, int 
     tc::fence_after_sync();
     if (!fail) {
         // accumulator row of this lane: pixel (row / 8, row % 8) of the tile
-        const int row = warp * 32 + lane, y = y0 + row / T_COLS, x = x0 + row % T_COLS;
+        const int row = (warp & 3) * 32 + lane, y = y0 + row / T_COLS, x = x0 + row % T_COLS;
         const bool ok = y < a.H && x < a.W;
         const size_t q = ((size_t)b * a.H + y) * a.W + x;
-        for (int c = 0; c < nsub; c += 16) {
+        for (int c = (warp >> 2) * 16; c < nsub; c += 32) {
             float v[16];
-            tc::tmem_ld16(tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, v);
+            tc::tmem_ld16(tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c, v);
             if (ok && n0 + c < a.Cout) conv_store(a, q, n0 + c, v);
         }
     } else if (tid == 0) {
@@ -270,7 +393,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
     uint64_t* bar = reinterpret_cast<uint64_t*>(sB + 256 * CONV_KC);
     uint32_t* s_taddr = reinterpret_cast<uint32_t*>(bar + 1);
     int* s_fail = reinterpret_cast<int*>(s_taddr + 1);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int Npad = a.Npad;
     uint32_t ncols = 32;
     while ((int)ncols < Npad) ncols <<= 1;
@@ -338,7 +461,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a) {
             tc::fence_proxy_async();
             tc::fence_before_sync();
             __syncthreads();
-            if (tid == 0) {
+            if (warp == 0) {
                 tc::fence_after_sync();
                 const uint32_t a0 = tc::smem_u32(sA), b0 = tc::smem_u32(sB);
                 for (int s = 0; s < kc / 16; ++s) {
@@ -401,18 +524,37 @@ void conv_tc_launch(const ConvArgs& args, cudaStream_t st) {
                 (uintptr_t)a.mask % 16 == 0;
     const int tx = (a.W + T_COLS - 1) / T_COLS, ty = (a.H + T_ROWS - 1) / T_ROWS;
     const int64_t tiles = (int64_t)a.B * tx * ty;
-    // output channels per block: halved while the blocks do not fill the chip
-    // (each block then stages the same input tile for fewer channels)
-    int nsub = a.Npad;
-    while (nsub % 32 == 0 && tiles * (a.Npad / nsub) < 152) nsub /= 2;
     const int KT = a.k * a.k * a.Cinp / 8;
+    const size_t halo = ((size_t)a.Cinp / 8 * TP * 16 + 127) / 128 * 128;
+    if (tiles >= (int64_t)1 << 31) throw Error{PURIFY_EINVAL, "conv: image too large"};
+    // output channels per block: all, or halves until a block's weights fit
+    // shared memory beside two halo tiles (wider outputs repeat the copies
+    // and read the tile for fewer channels: not below 32)
+    int nsub = a.Npad;
+    auto resident = [&](int n) { return 2 * halo + (size_t)KT * n * 16; };
+    while (nsub % 64 == 0 && resident(nsub) > (size_t)200 * 1024) nsub /= 2;
+    if (resident(nsub) <= (size_t)200 * 1024) {
+        // and while the blocks do not fill the chip
+        while (nsub % 32 == 0 && tiles * (a.Npad / nsub) < 152) nsub /= 2;
+        const size_t sm = resident(nsub);
+        const int per_sm = std::max(1, std::min((int)((size_t)220 * 1024 / (sm + 1024)), 256 / std::max(32, 2 * nsub)));
+        const int gx = (int)std::min<int64_t>(tiles, std::max(1, 152 * per_sm / (a.Npad / nsub)));
+        static std::atomic<bool> tiles_attr[64];
+        raise_smem(tiles_attr, k_conv_tiles, kConvSmemMax);
+        k_conv_tiles<<<dim3((unsigned)gx, a.Npad / nsub), CONV_THREADS, sm, st>>>(a, tx, ty, (int)tiles, nsub);
+        PURIFY_CUDA(cudaGetLastError());
+        add_launches(1);
+        return;
+    }
+    nsub = a.Npad;
+    while (nsub % 32 == 0 && tiles * (a.Npad / nsub) < 152) nsub /= 2;
     const int kg = std::min(std::max(2, CONV_STAGE / (nsub * 16) / 2 * 2), KT);
     const int slots = std::min(CONV_SLOTS, (KT + kg - 1) / kg);
-    const size_t sa = ((size_t)a.Cinp / 8 * TP * 16 + 127) / 128 * 128, sm = sa + (size_t)slots * kg * nsub * 16;
-    if (sm <= (size_t)200 * 1024 && tiles < (int64_t)1 << 31) {
+    const size_t sm = halo + (size_t)slots * kg * nsub * 16;
+    if (sm <= (size_t)200 * 1024) {
         static std::atomic<bool> halo_attr[64];
         raise_smem(halo_attr, k_conv_halo, kConvSmemMax);
-        k_conv_halo<<<dim3((unsigned)tiles, a.Npad / nsub), 128, sm, st>>>(a, tx, ty, nsub, kg, slots);
+        k_conv_halo<<<dim3((unsigned)tiles, a.Npad / nsub), CONV_THREADS, sm, st>>>(a, tx, ty, nsub, kg, slots);
     } else {
         static std::atomic<bool> attr[64];
         raise_smem(attr, k_conv_tc, (int)conv_smem_bytes());
@@ -434,7 +576,8 @@ void conv_tc_launch(const ConvArgs& args, cudaStream_t st) {
 // MN-major: a core matrix is 8 pixels x 8 channels, 16 bytes a pixel, exactly
 // what the copies write; a tap is again a start address.
 // By register tiles on the CUDA cores this took 10.5 ms of a 19.7 ms gradient
-// (8 images of 256 x 256, 4 levels, base 32), now 1.6 ms.
+// (8 images of 256 x 256, 4 levels, base 32), now 1.2 ms (1.6 with four warps a
+// block and one thread issuing).
 // The tensor core's own FP32 additions lose more than a rounded sum's: over
 // the hundreds of MMAs of a block's tiles the error against 64 bits was 1.8e-6
 // to 4e-6 where the CUDA cores had 3.5e-7 to 4.5e-7. The accumulators are
@@ -442,14 +585,15 @@ void conv_tc_launch(const ConvArgs& args, cudaStream_t st) {
 static constexpr int DW_SLOTS = 3;
 static constexpr int DW_FLUSH = 3;
 static constexpr int GP = T_ROWS * T_COLS + 1;   // gz group stride in pixels
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(CONV_THREADS)
 k_dw_tc(const bf16* __restrict__ gz, int Cout, const bf16* __restrict__ x, int xcs, int xco, int Cin, int B, int H, int W,
         int up, int k, int tiles_x, int tiles_y, int nt, int ntap, int ci_tiles, int tap_groups,
         float* __restrict__ dW, int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar[DW_SLOTS];
     __shared__ uint32_t s_taddr;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int quarter = warp & 3;   // accumulator rows 32 quarter .. + 31
     int id = blockIdx.x;
     const int tg = id % tap_groups; id /= tap_groups;
     const int ci0 = (id % ci_tiles) * nt, co0 = id / ci_tiles * 128;
@@ -465,7 +609,7 @@ k_dw_tc(const bf16* __restrict__ gz, int Cout, const bf16* __restrict__ x, int x
     if (tid == 0)
         for (int i = 0; i < DW_SLOTS; ++i) tc::mbar_init(&bar[i], 1);
     const int ng = min(16, (Cout - co0 + 7) / 8);   // channel groups of gz; those past them stay zero
-    const int dpos = 128 / ng, dgr = 128 - dpos * ng, pos_first = tid / ng, g_first = tid - pos_first * ng;
+    const int dpos = CONV_THREADS / ng, dgr = CONV_THREADS - dpos * ng, pos_first = tid / ng, g_first = tid - pos_first * ng;
     auto load_tile = [&](int i) {
         const int tile = first + i * step;
         const int b = tile / (tiles_x * tiles_y), rem = tile - b * tiles_x * tiles_y;
@@ -489,7 +633,7 @@ k_dw_tc(const bf16* __restrict__ gz, int Cout, const bf16* __restrict__ x, int x
     };
     // the zero rows of narrow outputs, written once
     for (int s = 0; s < DW_SLOTS; ++s)
-        for (int t = tid; t < 16 * GP; t += 128)
+        for (int t = tid; t < 16 * GP; t += CONV_THREADS)
             *reinterpret_cast<uint4*>(smem + (size_t)s * slot_bytes + (size_t)t * 16) = make_uint4(0, 0, 0, 0);
     __syncthreads();
 #pragma unroll
@@ -509,16 +653,16 @@ k_dw_tc(const bf16* __restrict__ gz, int Cout, const bf16* __restrict__ x, int x
     // the accumulators' sums so far added to dW; with at most 32 output
     // channels (one warp's rows) to the block's own sums in shared memory
     // until the last time
-    const int co = co0 + warp * 32 + lane;
+    const int co = co0 + quarter * 32 + lane;
     float* const sums = Cout <= 32 ? reinterpret_cast<float*>(smem + (size_t)DW_SLOTS * slot_bytes) + lane : nullptr;
     auto flush = [&](bool first_time, bool last) {
-        if (co0 + warp * 32 >= Cout) return;   // this warp's rows are the zero rows
+        if (co0 + quarter * 32 >= Cout) return;   // this warp's rows are the zero rows
         const int n = min(nt, Cin - ci0);
         for (int t = 0; t < taps; ++t) {
             float* row = dW + ((size_t)co * k * k + tap0 + t) * Cin + ci0;
-            for (int c = 0; c < nt; c += 16) {
+            for (int c = (warp >> 2) * 16; c < nt; c += 32) {
                 float v[16];
-                tc::tmem_ld16(tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)(t * nt + c), v);
+                tc::tmem_ld16(tbase + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(t * nt + c), v);
                 if (co >= Cout) continue;
                 if (sums) {
                     float* p = sums + (t * nt + c) * 32;
@@ -552,7 +696,7 @@ k_dw_tc(const bf16* __restrict__ gz, int Cout, const bf16* __restrict__ x, int x
         tc::fence_proxy_async();
         tc::fence_before_sync();
         if (__syncthreads_or(fail)) { fail = 1; break; }
-        if (tid == 0) {
+        if (warp == 0) {
             tc::fence_after_sync();
             const uint32_t slot = (uint32_t)((i % DW_SLOTS) * (slot_bytes / 16));
             for (int t = 0; t < taps; ++t) {
@@ -609,7 +753,7 @@ void dw_tc_launch(const bf16* gz, int Cout, const bf16* x, int xcs, int xco, int
     static std::atomic<bool> attr[64];
     raise_smem(attr, k_dw_tc, kConvSmemMax);
     const size_t sums = Cout <= 32 ? (size_t)ntap * nt * 32 * sizeof(float) : 0;
-    k_dw_tc<<<dim3(blocks, split), 128, (size_t)DW_SLOTS * slot + sums, st>>>(gz, Cout, x, xcs, xco, Cin, B, H, W, up, k, tx, ty, nt,
+    k_dw_tc<<<dim3(blocks, split), CONV_THREADS, (size_t)DW_SLOTS * slot + sums, st>>>(gz, Cout, x, xcs, xco, Cin, B, H, W, up, k, tx, ty, nt,
                                                                       ntap, ci_tiles, tap_groups, dW, err);
     PURIFY_CUDA(cudaGetLastError());
     add_launches(1);

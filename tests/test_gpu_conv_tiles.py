@@ -55,3 +55,23 @@ def test_gradients_on_partial_tiles(H, W, levels, base, B):
     bad = {k: round(e, 4) for k, e in errs.items() if e > 3e-2}
     assert not bad, bad
     assert rel(flat_from_oracle(got, levels, base), flat_from_oracle(want, levels, base)) <= 1.5e-2
+
+
+@pytest.mark.parametrize("B,H,W,Cin,Cout,k", [
+    (41, 70, 45, 32, 64, 3),     # several tiles a block, a last round that is not full
+    (60, 33, 41, 16, 16, 1),
+    (12, 70, 90, 8, 128, 3),
+])
+def test_blocks_that_walk_tiles(B, H, W, Cin, Cout, k):
+    """A block's second and later tiles are the same sums in the same order as
+    one image alone, where every block has one tile: equal to the bit."""
+    g = np.random.default_rng(B)
+    x = torch.from_numpy(g.standard_normal((B, H, W, Cin)).astype(np.float32)).to(DEV)
+    w = torch.from_numpy((g.standard_normal((Cout, k, k, Cin)) / np.sqrt(k * k * Cin)).astype(np.float32)).to(DEV)
+    b = torch.from_numpy(g.standard_normal(Cout).astype(np.float32)).to(DEV)
+    out = torch.empty((B, H, W, Cout), dtype=torch.float32, device=DEV)
+    one = torch.empty((1, H, W, Cout), dtype=torch.float32, device=DEV)
+    pk.purify_conv2d(x, w, b, out, k)
+    for i in (0, 1, B // 2, B - 1):
+        pk.purify_conv2d(x[i:i + 1].contiguous(), w, b, one, k)
+        assert torch.equal(out[i], one[0]), i

@@ -269,8 +269,10 @@ struct purify_plan {
                                       // per run; two lanes per run; two, sets grouped by tile
     bool half_on = false;             // the half-plane path is built (autotuned plans)
     purify::HalfPlane half;
-    purify::LaneWork half_lanes;      // lane pairs of the folded visibilities (any dtype, J;
-                                      // internal order only)
+    purify::LaneWork half_lanes;      // folded visibilities: a lane per run (FP32, J <= 6) or lane pairs,
+                                      // internal order only
+    purify::LaneWork half_pairs;      // lane pairs for G^H G where half_lanes has a lane per run and
+                                      // there is no stencil
     purify::SortedWork half_sorted;   // the same visibilities sorted by cell
     purify::Stencil stencil;          // G^H G of the half plane as a stencil, where it is the faster form
     purify::DevBuf det_patch;         // run patches of the deterministic lane form (float2)

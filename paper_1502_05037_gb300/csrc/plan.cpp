@@ -71,9 +71,16 @@ template <typename F> static void parallel_for(int64_t n, F&& f) {
         f((int64_t)0, n);
         return;
     }
+    // where no more threads can be started, the rest is done here
     std::vector<std::thread> ts;
-    for (int t = 0; t < nt; ++t) ts.emplace_back([&, t] { f(n * t / nt, n * (t + 1) / nt); });
-    for (auto& t : ts) t.join();
+    int t = 0;
+    try {
+        ts.reserve(nt - 1);
+        for (; t < nt - 1; ++t) ts.emplace_back([&f, n, nt, t] { f(n * t / nt, n * (t + 1) / nt); });
+    } catch (...) {
+    }
+    f(n * t / nt, n);
+    for (auto& th : ts) th.join();
 }
 
 // Grid cell of each visibility's first tap (wrapped), as computed by the
@@ -457,9 +464,10 @@ static const int kRunMax = 48;
 // Longest run of the half-plane lane work: a warp's share of the records is
 // M / (runs per set x resident warps) steps, and a set's longest run is a
 // serial chain, so runs are cut to half the share (at most kRunMax, at least
-// 16: every run costs a patch).
+// 16: every run costs a patch). Resident warps per SM: about 16 with a lane
+// pair per run, 12 with a lane per run (it holds the whole patch).
 static int run_cap(int64_t M, int width) {
-    const int64_t share = M / ((int64_t)width * 152 * 16);
+    const int64_t share = M / ((int64_t)width * 152 * (width == 32 ? 12 : 16));
     return (int)std::min<int64_t>(kRunMax, std::max<int64_t>(16, share / 2));
 }
 
@@ -484,12 +492,14 @@ static bool use_stencil(const purify_plan* p, size_t nruns) {
 
 // The half-plane lane work (see HalfPlane, LaneWork): the visibilities, folded
 // where their first-tap column is in the upper half, in runs of one cell,
-// runs sorted by length (longest first, then by cell), a lane pair per run.
+// runs sorted by length (longest first, then by cell). A lane per run where
+// its patch fits the registers (FP32, J <= 6; see half_lane), else a lane pair.
 template <typename T>
 static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std::vector<T>& vs,
                              const std::vector<int>& scx, const std::vector<int>& scy, const std::vector<int>& perm) {
     const int64_t M = p->M;
-    const int J = p->J, Kx = p->Kx, Ky = p->Ky, W = p->half.W, off = p->half.off, WID = 16;
+    const int J = p->J, Kx = p->Kx, Ky = p->Ky, W = p->half.W, off = p->half.off;
+    const int width = sizeof(T) == 4 && J <= kLaneMaxJ ? 32 : 16;
     std::vector<int> cell(M), order(M);
     parallel_for(M, [&](int64_t a, int64_t b) {
         for (int64_t m = a; m < b; ++m)
@@ -502,33 +512,29 @@ static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std
         for (size_t c = 1; c < pos.size(); ++c) pos[c] += pos[c - 1];
         for (int64_t m = 0; m < M; ++m) order[pos[cell[m]]++] = (int)m;
     }
-    const int cap = run_cap(M, WID);
+    const int cap = run_cap(M, width);
     struct Run { int first, len, id; };   // id: place in cell order
     std::vector<Run> runs, sorted;
-    std::vector<int> bylen(kRunMax + 2, 0);
     for (int64_t i = 0; i < M;) {
         int64_t j = i + 1;
         while (j < M && j - i < cap && cell[order[j]] == cell[order[i]]) ++j;
         runs.push_back({(int)i, (int)(j - i), (int)runs.size()});
-        bylen[j - i]++;
         i = j;
     }
     const size_t nr = runs.size();
     {
-        std::vector<size_t> at(kRunMax + 2, 0);   // first place of the runs of each length
-        for (int l = kRunMax - 1; l >= 1; --l) at[l] = at[l + 1] + bylen[l + 1];
+        // runs by length, longest first, then in cell order
+        std::vector<size_t> at(kRunMax + 1, 0);   // first place of the runs of each length
+        for (const Run& r : runs) at[r.len]++;
+        size_t first = 0;
+        for (int l = kRunMax; l >= 1; --l) {
+            const size_t n = at[l];
+            at[l] = first;
+            first += n;
+        }
         sorted.resize(nr);
         for (const Run& r : runs) sorted[at[r.len]++] = r;
     }
-    const int nsets = (int)((nr + WID - 1) / WID);
-    std::vector<int2> set_info(nsets), run_cl((size_t)nsets * WID, make_int2(0, 0));
-    int64_t rows = 0;
-    for (int s = 0; s < nsets; ++s) {
-        const int lmax = sorted[(size_t)s * WID].len;
-        set_info[s] = make_int2((int)rows, lmax);
-        rows += lmax;
-    }
-    PURIFY_REQUIRE(rows * WID < ((int64_t)1 << 31), "too many visibility records for the lane work");
     // entries of the sorted form: two visibilities of a cell each where that
     // makes at most 3/4 as many (a thread of two costs about 4/3 of one); the
     // double kernels are bound by arithmetic and take one
@@ -544,43 +550,71 @@ static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std
         sw.n = sw.per == 2 ? n2 : M;
     }
     const int per = sw.per;
-    std::vector<T> rec((size_t)rows * 2 * WID, T(0)), sz(2 * (size_t)(sw.n * per), T(0));
-    std::vector<int> idx((size_t)rows * WID, -1), sc(sw.n), si(sw.n * per, -1), sk(sw.n * per, -1);
-    parallel_for((int64_t)nr, [&](int64_t a, int64_t b) {
-        for (int64_t q = a; q < b; ++q) {
-            const int s = (int)(q / WID), l = (int)(q % WID);
-            const Run& r = sorted[q];
-            const int c = cell[order[r.first]], packed = ((c / W) << 16) | (c % W);
-            run_cl[q] = make_int2(packed, r.len);
-            const size_t at0 = per == 2 ? 2 * (size_t)entry[r.id] : (size_t)r.first;
-            for (int k = 0; k < r.len; ++k) {
-                const int m = order[r.first + k];
-                const bool fold = scx[m] >= Kx / 2;
-                int k0;
-                T phx, phy;
-                split_coord(us[m], p->ax, J, k0, phx);
-                split_coord(vs[m], p->ay, J, k0, phy);
-                const T zx = fold ? -kb_z(phx) : kb_z(phx), zy = fold ? -kb_z(phy) : kb_z(phy);
-                const size_t row = (size_t)set_info[s].x + k, at = at0 + k;
-                rec[row * 2 * WID + l] = zx;
-                rec[row * 2 * WID + WID + l] = zy;
-                idx[row * WID + l] = si[at] = fold ? fold_index(m) : m;
-                sk[at] = fold ? fold_index(perm[m]) : perm[m];
-                sc[at / per] = packed;
-                sz[2 * at] = zx;
-                sz[2 * at + 1] = zy;
-            }
+    std::vector<T> sz(2 * (size_t)(sw.n * per), T(0));
+    std::vector<int> sc(sw.n), si(sw.n * per, -1), sk(sw.n * per, -1);
+    // the visibilities of run r: f(k, m, folded, zx, zy)
+    auto each = [&](const Run& r, auto&& f) {
+        for (int k = 0; k < r.len; ++k) {
+            const int m = order[r.first + k];
+            const bool fold = scx[m] >= Kx / 2;
+            int k0;
+            T phx, phy;
+            split_coord(us[m], p->ax, J, k0, phx);
+            split_coord(vs[m], p->ay, J, k0, phy);
+            f(k, m, fold, fold ? -kb_z(phx) : kb_z(phx), fold ? -kb_z(phy) : kb_z(phy));
         }
-    });
-    LaneWork& w = p->half_lanes;
-    w.nsets = nsets;
-    w.width = WID;
-    w.tile = 0;
-    w.rows = rows;
-    upload(w.set_info, set_info);
-    upload(w.run_cl, run_cl);
-    upload(w.rec, rec);
-    upload(w.idx, idx);
+    };
+    auto packed_cell = [&](const Run& r) {
+        const int c = cell[order[r.first]];
+        return ((c / W) << 16) | (c % W);
+    };
+    // lane work of `wid` runs per set (layout: see LaneWork), with the sorted
+    // form filled on the way the first time
+    auto fill = [&](LaneWork& w, int wid, bool with_sorted) {
+        const int nsets = (int)((nr + wid - 1) / wid);
+        std::vector<int2> set_info(nsets), run_cl((size_t)nsets * wid, make_int2(0, 0));
+        int64_t rows = 0;
+        for (int s = 0; s < nsets; ++s) {
+            const int lmax = sorted[(size_t)s * wid].len;
+            set_info[s] = make_int2((int)rows, lmax);
+            rows += lmax;
+        }
+        PURIFY_REQUIRE(rows * wid < ((int64_t)1 << 31), "too many visibility records for the lane work");
+        const int ax = wid == 32 ? 1 : 16, ay = wid == 32 ? 2 : 1;   // strides of the axis and of the run
+        std::vector<T> rec((size_t)rows * 2 * wid, T(0));
+        std::vector<int> idx((size_t)rows * wid, -1);
+        parallel_for((int64_t)nr, [&](int64_t a, int64_t b) {
+            for (int64_t q = a; q < b; ++q) {
+                const int s = (int)(q / wid), l = (int)(q % wid);
+                const Run& r = sorted[q];
+                const int packed = packed_cell(r);
+                run_cl[q] = make_int2(packed, r.len);
+                const size_t at0 = per == 2 ? 2 * (size_t)entry[r.id] : (size_t)r.first;
+                each(r, [&](int k, int m, bool fold, T zx, T zy) {
+                    const size_t row = (size_t)set_info[s].x + k;
+                    rec[row * 2 * wid + l * ay] = zx;
+                    rec[row * 2 * wid + l * ay + ax] = zy;
+                    idx[row * wid + l] = fold ? fold_index(m) : m;
+                    if (!with_sorted) return;
+                    const size_t at = at0 + k;
+                    si[at] = fold ? fold_index(m) : m;
+                    sk[at] = fold ? fold_index(perm[m]) : perm[m];
+                    sc[at / per] = packed;
+                    sz[2 * at] = zx;
+                    sz[2 * at + 1] = zy;
+                });
+            }
+        });
+        w.nsets = nsets;
+        w.width = wid;
+        w.tile = 0;
+        w.rows = rows;
+        upload(w.set_info, set_info);
+        upload(w.run_cl, run_cl);
+        upload(w.rec, rec);
+        upload(w.idx, idx);
+    };
+    fill(p->half_lanes, width, true);
     upload(sw.z, sz);
     upload(sw.cell, sc);
     upload(sw.idx, si);
@@ -592,6 +626,8 @@ static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std
         for (size_t q = 0; q < nr; ++q) cells[q] = cell[order[sorted[q].first]];
         build_stencil(p, cells);
         p->workspace_bytes += (int64_t)(p->stencil.coef.bytes + p->stencil.used.bytes);
+    } else if (sizeof(T) == 4 && width == 32) {
+        fill(p->half_pairs, 16, false);
     }
 }
 
@@ -848,7 +884,7 @@ template <typename T> static void finish_plan(purify_plan* p) {
     for (int k = 3; k <= 5; ++k)
         if (!uses(k)) p->lanes[k - 3].release();
     for (int k = 0; k < 3; ++k) p->workspace_bytes += lane_bytes(p->lanes[k]);
-    p->workspace_bytes += lane_bytes(p->half_lanes);
+    p->workspace_bytes += lane_bytes(p->half_lanes) + lane_bytes(p->half_pairs);
     p->workspace_bytes += (int64_t)p->det_patch.bytes;
 }
 

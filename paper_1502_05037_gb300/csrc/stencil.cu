@@ -40,7 +40,7 @@ PURIFY_HD constexpr int stencil_plane(int J, int dy, int dx) {
 template <typename T, int J>
 __global__ void __launch_bounds__(128)
 k_stencil_build(const int2* __restrict__ set_info, const int2* __restrict__ run_cl, const T* __restrict__ rec,
-                int nruns, typename KbOf<T>::type kp, int W, int Ky, double* __restrict__ out) {
+                int nruns, int width, typename KbOf<T>::type kp, int W, int Ky, double* __restrict__ out) {
     constexpr int NP = J * (J + 1) / 2, NI = (NP + 31) / 32, NC = stencil_planes(J);
     constexpr int DEG = sizeof(T) == 4 ? kb_poly_deg(J) : kb_poly_deg_d(J);
     const int lane = threadIdx.x & 31, axis = lane >> 4, tap = min(lane & 15, J - 1);
@@ -60,14 +60,16 @@ k_stencil_build(const int2* __restrict__ set_info, const int2* __restrict__ run_
     for (int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < nruns; q += nw) {
         const int2 cl = run_cl[q];
         if (cl.y <= 0) continue;
-        const T* z = rec + (size_t)set_info[q / 16].x * 32 + axis * 16 + q % 16;
+        // this lane's axis of the run's records (see LaneWork), a row apart
+        const T* z = rec + (size_t)set_info[q / width].x * 2 * width +
+                     (width == 32 ? 2 * (q % 32) + axis : q % 16 + 16 * axis);
         T acc[NI][NP];
 #pragma unroll
         for (int s = 0; s < NI; ++s)
 #pragma unroll
             for (int j = 0; j < NP; ++j) acc[s][j] = T(0);
         for (int k = 0; k < cl.y; ++k) {
-            const T zk = z[(size_t)k * 32];
+            const T zk = z[(size_t)k * 2 * width];
             // lane (axis, tap): this tap's weight
             T w = cf[DEG];
 #pragma unroll
@@ -264,7 +266,7 @@ template <typename T, int J> static void stencil_build_tj(purify_plan* p) {
     }
     PURIFY_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * n, p->stream));
     k_stencil_build<T, J><<<152 * 8, 128, 0, p->stream>>>(lw.set_info.as<int2>(), lw.run_cl.as<int2>(), lw.rec.as<T>(),
-                                                          lw.nsets * lw.width, kb_table<T>(p), p->half.W, p->Ky, acc);
+                                                          lw.nsets * lw.width, lw.width, kb_table<T>(p), p->half.W, p->Ky, acc);
     PURIFY_CUDA(cudaGetLastError());
     if (sizeof(T) == 4) {
         k_to_float<<<152 * 8, 256, 0, p->stream>>>(acc, s.coef.as<float>(), n);

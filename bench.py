@@ -123,20 +123,41 @@ class ClockSampler:
         return {"sm_mhz": statistics.median(sm), "sm_max_mhz": mx, "reasons": reasons, "samples": len(rows)}
 
 
+def half_plane(info) -> bool:
+    """Whether the operators of real images run on the stored half of the
+    Hermitian grid (degrid_mode 8 is built with it)."""
+    return info.degrid_mode == 8
+
+
+def grid_columns(info) -> int:
+    """Stored columns of the grid: Kx, or the half plane's row stride."""
+    if not half_plane(info):
+        return info.Kx
+    return (info.Kx // 2 + 2 * info.J - 3 + 8 + 15) // 16 * 16
+
+
+def stencil_planes(J: int) -> int:
+    """Kept offsets of the stencil form of G^H G."""
+    return J + (J - 1) * (2 * J - 1)
+
+
 def algorithmic_bytes(name: str, info, dtype_bytes: int = 4) -> float | None:
     """Bytes a kernel launch must move at minimum (FP32, internal order):
     visibility kernels 8 B per (u, v) pair and 8 B per complex visibility,
-    the oversampled grid 8 B per cell read or written once, images 4 B per
-    pixel, coefficients 4 B per entry."""
-    N, M, Kx, Ky, D = info.N, info.M, info.Kx, info.Ky, info.D
-    ny = int(round(np.sqrt(N * Ky / Kx)))
+    the stored grid 8 B per cell read or written once, images 4 B per
+    pixel, coefficients 4 B per entry; G^H G as a stencil its coefficients
+    once and the grid in and out."""
+    N, M, Ky, D = info.N, info.M, info.Ky, info.D
+    ny = int(round(np.sqrt(N * Ky / info.Kx)))
+    Kx = grid_columns(info)
     c = 2 * dtype_bytes
     table = {
         "degrid": 8 * M + c * M + c * Kx * Ky,
         "grid": 8 * M + c * M + c * Kx * Ky,
         # G^H G of the forward grid: coordinates once, the grid read once and
         # the output grid written once (no visibility vector)
-        "normal_gg": 8 * M + 2 * c * Kx * Ky,
+        "normal_gg": (dtype_bytes * stencil_planes(info.J) * Kx * Ky if info.normal_mode == 7 else 8 * M)
+                     + 2 * c * Kx * Ky,
         "fft_rows_fwd": dtype_bytes * N + c * ny * Kx,
         "fft_cols_fwd": c * ny * Kx + c * Kx * Ky,
         "fft_cols_inv": c * Kx * Ky + c * ny * Kx,
@@ -153,21 +174,25 @@ def algorithmic_bytes(name: str, info, dtype_bytes: int = 4) -> float | None:
 def algorithmic_flops(name: str, info) -> float | None:
     """FP32 operations a launch must perform (kernel weights evaluated from
     J per-tap polynomials of degree 8-10 per axis, J*J taps of a real weight
-    times a complex value; FFT passes 5 n log2 n per length-n transform)."""
+    times a complex value; a stencil coefficient times two complex values;
+    FFT passes 5 n log2 n per length-n transform, two rows per transform on
+    the half plane)."""
     import math
     J, M = info.J, info.M
     deg = 10 if J <= 3 else (9 if J == 4 else 8)
     weights = 2 * J * (deg + 1) * 2          # Horner: one FMA (2 flops) per coefficient
     taps = J * J * (1 + 4)                    # weight product + complex multiply-accumulate
-    ny = int(round(np.sqrt(info.N * info.Ky / info.Kx)))
+    ny = int(round(np.sqrt(info.N * info.Ky / info.Kx))) // (2 if half_plane(info) else 1)
+    cols = grid_columns(info)
     table = {
         "grid": M * (weights + taps),
-        "normal_gg": M * (weights + 2 * taps),
+        "normal_gg": cols * info.Ky * 4 * (2 * stencil_planes(J) - 1) if info.normal_mode == 7
+                     else M * (weights + 2 * taps),
         "degrid": M * (weights + taps),
         "fft_rows_fwd": ny * 5 * info.Kx * math.log2(info.Kx),
         "fft_rows_inv": ny * 5 * info.Kx * math.log2(info.Kx),
-        "fft_cols_fwd": info.Kx * 5 * info.Ky * math.log2(info.Ky),
-        "fft_cols_inv": info.Kx * 5 * info.Ky * math.log2(info.Ky),
+        "fft_cols_fwd": cols * 5 * info.Ky * math.log2(info.Ky),
+        "fft_cols_inv": cols * 5 * info.Ky * math.log2(info.Ky),
     }
     return float(table[name]) if name in table else None
 

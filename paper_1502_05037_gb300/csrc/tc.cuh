@@ -41,11 +41,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t phase) {
         : "memory");
     return ok != 0;
 }
-// Wait for the phase to complete; gives up after `limit` polls (returns false).
+// Wait for the phase to complete, by a whole warp; gives up after `limit` polls.
+// All lanes return the same (false when any lane gave up), together: what
+// follows are warp-wide instructions.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase, uint32_t limit) {
-    for (uint32_t i = 0; i < limit; ++i)
-        if (mbar_try_wait(bar, phase)) return true;
-    return false;
+    bool done = false;
+    for (uint32_t i = 0; i < limit && !done; ++i) done = mbar_try_wait(bar, phase);
+    return __all_sync(0xffffffffu, done);
 }
 
 // Shared-memory matrix descriptor, no swizzle (core matrices of 8 rows x 16
@@ -93,9 +95,13 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
         : "memory");
 }
 
-// 16 consecutive FP32 accumulator columns of this thread's lane.
+// 16 consecutive FP32 accumulator columns of this thread's lane. The load is
+// a warp-wide aligned instruction: the warp is brought together first, as the
+// callers come here from loops whose bodies only some lanes run (rows outside
+// the image, channels past the last).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),

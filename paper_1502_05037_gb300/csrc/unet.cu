@@ -103,7 +103,7 @@ __device__ __forceinline__ void conv_store(const ConvArgs& a, size_t q, int c, f
         if (a.residual) {
             for (int e = 0; e < n; ++e) v[e] += a.residual[q * a.f32_ch + c + e];
         }
-        if (n == 16 && a.f32_ch % 4 == 0) {
+        if (n == 16 && a.vec_f32) {
 #pragma unroll
             for (int e = 0; e < 16; e += 4) *reinterpret_cast<float4*>(o + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
         } else {
@@ -522,6 +522,8 @@ void conv_tc_launch(const ConvArgs& args, cudaStream_t st) {
     a.vec_out = a.out && a.out_cs % 8 == 0 && a.out_co % 8 == 0 && a.bf_from % 16 == 0 &&
                 (!a.mask || (a.mask_cs % 8 == 0 && a.mask_co % 8 == 0)) && (uintptr_t)a.out % 16 == 0 &&
                 (uintptr_t)a.mask % 16 == 0;
+    // out_f32 may be a caller's array, aligned to its elements only
+    a.vec_f32 = a.out_f32 && a.f32_ch % 4 == 0 && (uintptr_t)a.out_f32 % 16 == 0;
     const int tx = (a.W + T_COLS - 1) / T_COLS, ty = (a.H + T_ROWS - 1) / T_ROWS;
     const int64_t tiles = (int64_t)a.B * tx * ty;
     const int KT = a.k * a.k * a.Cinp / 8;

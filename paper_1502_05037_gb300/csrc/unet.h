@@ -25,7 +25,7 @@ struct ConvArgs {
     const bf16* mask;        // not null: `out` is zero where this activation (same pixels; channel
     int mask_cs, mask_co;    // stride, first channel) is not positive
     int f32_ch, bf_from;     // f32_ch 0: all channels
-    int vec_out;             // set by the launch: `out` (and the mask) take 16-byte accesses
+    int vec_out, vec_f32;    // set by the launch: `out` (and the mask), `out_f32` take 16-byte accesses
     int up;                  // 1: the input is the (H/2, W/2) image read through a x2 nearest upsampling
 };
 

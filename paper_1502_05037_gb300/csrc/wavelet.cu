@@ -89,9 +89,9 @@ template <typename T, int L> struct Taps {
 
 // ------------------------------------------------------------- analysis
 // Row filters: low- and high-pass outputs k0 .. k0 + KX - 1 of one input row
-// (periodic, w columns) from a register window of 2 KX + L - 2 inputs; `vec`:
-// the row is in global memory or 16-byte aligned, w >= 4 (the window then
-// comes in 16-byte loads, which wrap as a whole).
+// (periodic, w columns) from a register window of 2 KX + L - 2 inputs; VEC:
+// the row is 16-byte aligned, w >= 4 (the window then comes in 16-byte loads,
+// which wrap as a whole).
 template <typename T, int L, int KX, bool VEC>
 __device__ __forceinline__ void row_filter(const Taps<T, L>& f, const T* __restrict__ row, int w, int k0, T (&a)[KX],
                                            T (&d)[KX]) {
@@ -143,7 +143,7 @@ __device__ __forceinline__ void col_filter(const Taps<T, L>& f, const T* ta, con
 
 // One analysis level of basis pb on the TH x TW sub-band tile at (ky0, kx0).
 template <typename T, int L, int TH>
-__device__ __forceinline__ void dwt_tile(const T* __restrict__ in, int src_ld, T* __restrict__ out, int nx,
+__device__ __forceinline__ void dwt_tile(const T* __restrict__ in, int src_ld, bool vec, T* __restrict__ out, int nx,
                                          T* __restrict__ llo, int h, int w, int ky0, int kx0, int pb, T inv_sqrt_q,
                                          T* smem) {
     using W = WaveTile<T>;
@@ -160,7 +160,7 @@ __device__ __forceinline__ void dwt_tile(const T* __restrict__ in, int src_ld, T
         if (k >= tw) continue;
         const T* row = in + (size_t)((2 * ky0 + r) & (h - 1)) * src_ld;
         alignas(16) T a[KX], d[KX];
-        if (w >= 4) row_filter<T, L, KX, true>(f, row, w, kx0 + k, a, d);
+        if (vec) row_filter<T, L, KX, true>(f, row, w, kx0 + k, a, d);
         else row_filter<T, L, KX, false>(f, row, w, kx0 + k, a, d);
         // KX outputs are 16 bytes; outputs past tw are not read
         *reinterpret_cast<uint4*>(ta + r * TW + k) = *reinterpret_cast<const uint4*>(a);
@@ -190,7 +190,7 @@ __device__ __forceinline__ void dwt_tile(const T* __restrict__ in, int src_ld, T
 // pixels).
 template <typename T, int TH>
 __global__ void __launch_bounds__(WaveTile<T>::THREADS)
-k_dwt_level(const T* __restrict__ src, int src_basis_stride, int src_ld, T* __restrict__ coef,
+k_dwt_level(const T* __restrict__ src, int src_basis_stride, int src_ld, int vec, T* __restrict__ coef,
             const int* __restrict__ planes, int N, int nx, T* __restrict__ ll_out, int ll_basis_stride, int h, int w,
             const int* __restrict__ pids, int nw, int dirac_plane, T inv_sqrt_q) {
     constexpr int TW = WaveTile<T>::TW;
@@ -210,7 +210,7 @@ k_dwt_level(const T* __restrict__ src, int src_basis_stride, int src_ld, T* __re
     T* out = coef + (size_t)planes[z] * N;
     T* llo = ll_out ? ll_out + (size_t)z * ll_basis_stride : nullptr;
     PURIFY_WITH_LENGTH(fbank<T>().len[pb],
-                       (dwt_tile<T, L, TH>(in, src_ld, out, nx, llo, h, w, blockIdx.y * TH, blockIdx.x * TW, pb,
+                       (dwt_tile<T, L, TH>(in, src_ld, vec != 0, out, nx, llo, h, w, blockIdx.y * TH, blockIdx.x * TW, pb,
                                            inv_sqrt_q, reinterpret_cast<T*>(smem_raw))));
     pdl_trigger();
 }
@@ -351,10 +351,11 @@ __device__ __forceinline__ void syn_row(const Taps<T, L>& f, const T* __restrict
 // and the high rows to shared memory), then columns. Thread item (output
 // column, group of RK sub-band rows) holds 2 RK outputs, added to acc. `ll`: the
 // low-pass sub-band (row stride ll_ld); the details are in `det` (row stride
-// nx). Ends with the shared tile free for the next basis.
+// nx); `vec`: both begin at a multiple of 16 bytes, w >= 8. Ends with the shared
+// tile free for the next basis.
 template <typename T, int L>
-__device__ __forceinline__ void synth_tile(const T* __restrict__ ll, int ll_ld, const T* __restrict__ det, int nx, int h,
-                                           int w, int ky0, int kx0, int pb, T* smem, int group, int tid,
+__device__ __forceinline__ void synth_tile(const T* __restrict__ ll, int ll_ld, const T* __restrict__ det, bool vec,
+                                           int nx, int h, int w, int ky0, int kx0, int pb, T* smem, int group, int tid,
                                            T (&acc)[2 * WaveTile<T>::SYN_RK]) {
     using W = WaveTile<T>;
     constexpr int TH = W::SYN_TH, TW = W::TW, RK = W::SYN_RK, KX = W::KX, E = L / 2 - 1, RG = TW / KX, CW = 2 * TW;
@@ -371,7 +372,7 @@ __device__ __forceinline__ void synth_tile(const T* __restrict__ ll, int ll_ld, 
         const T* const lo = det + (size_t)ky * nx + wsub;          // row-detail, column-approx
         const T* const hi = det + (size_t)(hs + ky) * nx;          // row-approx, column-detail
         alignas(16) T oL[2 * KX], oH[2 * KX];
-        if (wsub >= 4) {
+        if (vec) {
             syn_row<T, L, KX, true>(f, ll + (size_t)ky * ll_ld, lo, wsub, kx0 + k, oL);
             syn_row<T, L, KX, true>(f, hi, hi + wsub, wsub, kx0 + k, oH);
         } else {
@@ -401,10 +402,11 @@ __device__ __forceinline__ void synth_tile(const T* __restrict__ ll, int ll_ld, 
 // lengths' windows were kept live together and spilled).
 template <typename T> struct SynthPart { T v[2 * WaveTile<T>::SYN_RK]; };
 template <typename T, int L>
-__device__ __noinline__ SynthPart<T> synth_part(const T* __restrict__ ll, int ll_ld, const T* __restrict__ det, int nx, int h,
-                                                int w, int ky0, int kx0, int pb, T* smem, int group, int tid) {
+__device__ __noinline__ SynthPart<T> synth_part(const T* __restrict__ ll, int ll_ld, const T* __restrict__ det, bool vec,
+                                                int nx, int h, int w, int ky0, int kx0, int pb, T* smem, int group,
+                                                int tid) {
     SynthPart<T> p = {};
-    synth_tile<T, L>(ll, ll_ld, det, nx, h, w, ky0, kx0, pb, smem, group, tid, p.v);
+    synth_tile<T, L>(ll, ll_ld, det, vec, nx, h, w, ky0, kx0, pb, smem, group, tid, p.v);
     return p;
 }
 template <typename T> static size_t synth_smem_bytes() {
@@ -415,7 +417,7 @@ template <typename T> static size_t synth_smem_bytes() {
 // h x w band of basis z into ll_out (row stride w).
 template <typename T>
 __global__ void __launch_bounds__(WaveTile<T>::SYN_THREADS)
-k_idwt_level(const T* __restrict__ ll_in, int ll_basis_stride, int ll_ld, const T* __restrict__ coef,
+k_idwt_level(const T* __restrict__ ll_in, int ll_basis_stride, int ll_ld, const T* __restrict__ coef, int vec,
              const int* __restrict__ planes, int N, int nx, T* __restrict__ ll_out, int out_basis_stride, int h,
              int w, const int* __restrict__ pids) {
     using W = WaveTile<T>;
@@ -427,7 +429,7 @@ k_idwt_level(const T* __restrict__ ll_in, int ll_basis_stride, int ll_ld, const 
     const T* ll = ll_in ? ll_in + (size_t)z * ll_basis_stride : det;
     T acc[2 * W::SYN_RK] = {};
     PURIFY_WITH_LENGTH(fbank<T>().len[pb],
-                       (synth_tile<T, L>(ll, ll_in ? ll_ld : nx, det, nx, h, w, ky0, kx0, pb,
+                       (synth_tile<T, L>(ll, ll_in ? ll_ld : nx, det, vec != 0, nx, h, w, ky0, kx0, pb,
                                          reinterpret_cast<T*>(smem_raw), 0, (int)threadIdx.x, acc)));
     constexpr int CW = 2 * W::TW;
     const int y = 2 * (ky0 + threadIdx.x / CW * W::SYN_RK), x = 2 * kx0 + threadIdx.x % CW;
@@ -448,7 +450,7 @@ k_idwt_level(const T* __restrict__ ll_in, int ll_basis_stride, int ll_ld, const 
 // coefficient planes.
 template <typename T>
 __global__ void __launch_bounds__(WaveTile<T>::SYN_THREADS * WaveTile<T>::GROUPS, sizeof(T) == 4 ? 2 : 1)
-k_idwt_final(const T* __restrict__ ll_in, int ll_basis_stride, const T* __restrict__ coef,
+k_idwt_final(const T* __restrict__ ll_in, int ll_basis_stride, const T* __restrict__ coef, int vec,
              const int* __restrict__ planes, int N, int nx, int ny, const int* __restrict__ pids, int nw,
              int dirac_plane, T inv_sqrt_q, T* __restrict__ x) {
     using W = WaveTile<T>;
@@ -465,7 +467,7 @@ k_idwt_final(const T* __restrict__ ll_in, int ll_basis_stride, const T* __restri
         const T* ll = ll_in ? ll_in + (size_t)z * ll_basis_stride : det;
         SynthPart<T> part;
         PURIFY_WITH_LENGTH(fbank<T>().len[pb],
-                           (part = synth_part<T, L>(ll, ll_in ? (nx >> 1) : nx, det, nx, ny, nx, ky0, kx0, pb,
+                           (part = synth_part<T, L>(ll, ll_in ? (nx >> 1) : nx, det, vec != 0, nx, ny, nx, ky0, kx0, pb,
                                                     smem + group * GE, group, tid)));
 #pragma unroll
         for (int e = 0; e < NO; ++e) acc[e] += part.v[e];
@@ -642,8 +644,10 @@ static void analyse(const T* x, T* c, int nx, int ny, int levels, int nw, int di
             const size_t sm = dwt_smem_bytes<T>(maxL, TH);
             wave_smem(kern, sm);
             const dim3 g((wsub + W::TW - 1) / W::TW, (hs + TH - 1) / TH, nw + dirac);
-            launch_dependent(kern, g, W::THREADS, sm, st, src, src_stride, src_ld, c, planes, N, nx, llo, strides[lev & 1],
-                             h, w, pids, nw, dirac_plane, inv_sqrt_q);
+            // the image may begin at any element of the caller's array
+            const int vec = w >= 4 && (uintptr_t)src % 16 == 0;
+            launch_dependent(kern, g, W::THREADS, sm, st, src, src_stride, src_ld, vec, c, planes, N, nx, llo,
+                             strides[lev & 1], h, w, pids, nw, dirac_plane, inv_sqrt_q);
         };
         // tall tiles cost less halo; short ones while those do not fill the chip
         if constexpr (sizeof(T) == 4) {
@@ -689,6 +693,7 @@ template <typename T> static void psi_t(purify_plan* p, const void* cv, void* xv
     const int N = (int)p->N, llstride = (int)(p->N / 4);
     T* bufs[2] = {p->ll0.as<T>(), p->ll1.as<T>()};
     const T* ll_in = nullptr;  // coarsest level reads LL from the coefficients
+    const bool aligned = (uintptr_t)c % 16 == 0;   // the coefficients may begin at any element of the caller's array
     int ll_ld = p->nx;
     // levels L .. 2 reconstruct low-pass bands into scratch, the coarse ones
     // together
@@ -715,7 +720,7 @@ template <typename T> static void psi_t(purify_plan* p, const void* cv, void* xv
             T* out = bufs[lev & 1];
             Launch L(p, "idwt_level");
             launch_dependent(k_idwt_level<T>, g, W::SYN_THREADS, synth_smem_bytes<T>(), p->stream, ll_in, llstride, ll_ld, c,
-                             plane_array(p), N, p->nx, out, llstride, h, w, pid_array(p));
+                             (int)(aligned && w >= 8), plane_array(p), N, p->nx, out, llstride, h, w, pid_array(p));
             L.done();
             ll_in = out;
             ll_ld = w;
@@ -723,8 +728,8 @@ template <typename T> static void psi_t(purify_plan* p, const void* cv, void* xv
     }
     dim3 g((p->nx / 2 + W::TW - 1) / W::TW, (p->ny / 2 + W::SYN_TH - 1) / W::SYN_TH, 1);
     Launch Lf(p, "idwt_final");
-    launch_dependent(k_idwt_final<T>, g, W::SYN_THREADS * W::GROUPS, synth_smem_bytes<T>() * W::GROUPS, p->stream, ll_in, llstride, c, plane_array(p), N,
-                     p->nx, p->ny, pid_array(p), wl.nw, wl.dirac_plane, inv_sqrt_q, x);
+    launch_dependent(k_idwt_final<T>, g, W::SYN_THREADS * W::GROUPS, synth_smem_bytes<T>() * W::GROUPS, p->stream, ll_in, llstride, c,
+                     (int)(aligned && p->nx >= 8), plane_array(p), N, p->nx, p->ny, pid_array(p), wl.nw, wl.dirac_plane, inv_sqrt_q, x);
     Lf.done();
 }
 

@@ -5,8 +5,10 @@ import pytest
 import torch
 
 import paper_1502_05037_gb300 as pk
-from gpu_util import DEV, rel
+from gpu_util import DEV, TOL, make_plan, np_real, rel, t_real
 from oracle import unet as un
+from oracle import wavelets as ow
+from paper_1502_05037_gb300 import synth
 from test_gpu_unet import bf16_round
 
 pytestmark = pytest.mark.gpu
@@ -36,3 +38,35 @@ def test_conv2d_output_at_an_odd_element(Cin, Cout, first):
     assert out.data_ptr() % 16 == 4 * first and out.is_contiguous()
     pk.purify_conv2d(*args, out, k)
     assert rel(out.cpu().numpy(), un.conv2d(bf16_round(x), bf16_round(w), b.astype(np.float64))) <= 1e-5
+
+
+@pytest.mark.parametrize("dtype", [pk.PURIFY_F32, pk.PURIFY_F64])
+@pytest.mark.parametrize("nx,ny,levels,mask", [
+    (128, 64, 3, 0x1FF), (64, 256, 2, 0x1FE), (16, 512, 3, 0x1FF), (256, 256, 4, 0x107),
+])
+def test_dictionary_of_arrays_at_an_odd_element(nx, ny, levels, mask, dtype):
+    plan, *_ = make_plan(nx, ny, 64, 4, levels=levels, dtype=dtype, mask=mask)
+    rt, q, tol = t_real(dtype), bin(mask).count("1"), TOL[dtype]
+    g = synth.rng(nx + levels)
+    x = g.standard_normal((ny, nx)).astype(np_real(dtype))
+    c = g.standard_normal((q, ny, nx)).astype(np_real(dtype))
+    want_c = ow.psi_adj(x.astype(np.float64), levels, mask)
+    want_x = ow.psi(c.astype(np.float64), levels, mask)
+    for first in (1, 2, 3) if dtype == pk.PURIFY_F32 else (1,):
+        xs, cs = shifted(x.shape, rt, first), shifted(c.shape, rt, first)
+        xs.copy_(torch.from_numpy(x))
+        cs.copy_(torch.from_numpy(c))
+        assert xs.data_ptr() % 16 and cs.data_ptr() % 16
+        got_c, got_x = shifted(c.shape, rt, first), shifted(x.shape, rt, first)
+        pk.purify_psi_adj(plan, xs, got_c)
+        assert rel(got_c.cpu(), want_c) <= tol
+        pk.purify_psi(plan, cs, got_x)
+        assert rel(got_x.cpu(), want_x) <= tol
+        pk.purify_reweight(plan, xs, 0.1, got_c)
+        assert rel(got_c.cpu(), 0.1 / (0.1 + np.abs(want_c))) <= tol
+        assert abs(pk.purify_coef_std(plan, xs) - want_c.std()) <= tol * want_c.std()
+        got_c.zero_()
+        torch.cuda.synchronize()
+        pk.purify_psi_adj_static(xs, got_c, nx, ny, levels, mask, dtype)
+        torch.cuda.synchronize()
+        assert rel(got_c.cpu(), want_c) <= tol

@@ -1029,7 +1029,9 @@ template <typename T, bool INV> static void fft2_dir(purify_plan* p, void* grid)
     const int cb = cols_per_block<T>(p->Ky, p->Kx);
     const int ar = fft_alt(rb, p->Kx, sizeof(C)), ac = fft_alt(cb, p->Ky, sizeof(C));
     const size_t smr = fft_smem(rb, p->Kx, sizeof(C), ar), smc = fft_smem(cb, p->Ky, sizeof(C), ac);
-    const int wc = col_lanes<T>(cb, 0);
+    // two columns a thread are 16-byte accesses: not where the caller's grid
+    // begins at an odd element
+    const int wc = (uintptr_t)grid % 16 == 0 ? col_lanes<T>(cb, 0) : 1;
     with_log2(p->Kx, [&](auto lg) {
         auto kern = k_rows_full<T, decltype(lg)::value, INV>;
         set_fft_smem(kern, smr);

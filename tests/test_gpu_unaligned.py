@@ -70,3 +70,18 @@ def test_dictionary_of_arrays_at_an_odd_element(nx, ny, levels, mask, dtype):
         pk.purify_psi_adj_static(xs, got_c, nx, ny, levels, mask, dtype)
         torch.cuda.synchronize()
         assert rel(got_c.cpu(), want_c) <= tol
+
+
+@pytest.mark.parametrize("nx,ny", [(512, 256), (256, 16)])
+def test_transform_of_a_grid_at_an_odd_element(nx, ny):
+    plan, *_ = make_plan(nx, ny, 64, 4, levels=2)
+    Kx, Ky = plan.info.Kx, plan.info.Ky
+    g = synth.rng(nx)
+    x = (g.standard_normal((Ky, Kx)) + 1j * g.standard_normal((Ky, Kx))).astype(np.complex64)
+    grid = shifted((Ky, Kx), torch.complex64)
+    assert grid.data_ptr() % 16 == 8
+    for inverse in (False, True):
+        grid.copy_(torch.from_numpy(x))
+        pk.purify_fft2(plan, grid, inverse)
+        ref = np.fft.ifft2(x.astype(np.complex128)) * Kx * Ky if inverse else np.fft.fft2(x.astype(np.complex128))
+        assert rel(grid.cpu(), ref) <= TOL[pk.PURIFY_F32]

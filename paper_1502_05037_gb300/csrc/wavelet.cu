@@ -20,7 +20,7 @@
 // The filters are a few multiply-adds per byte, so the register windows carry
 // the weight: with every tap read from shared memory these kernels were bound
 // by it (9 bases: analysis of 1024 x 1024 over 5 levels 58 us, now 32; synthesis
-// of 512 x 1024 over 4 levels 72 us, now 33; the coefficients' 42 and 21 MB
+// of 512 x 1024 over 4 levels 72 us, now 31; the coefficients' 42 and 21 MB
 // take 6 and 3 us).
 #include <cuda_runtime.h>
 
@@ -30,6 +30,7 @@
 #include <memory>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
@@ -55,12 +56,15 @@ template <> struct WaveTile<float> {
     // largest band area of the tails: one SM per basis; 128 x 128 (two levels
     // fewer launches) took 29 us where two launches of tiles take 10
     static constexpr int TAIL = 1024;
-    static constexpr int SYN_TH = 16, SYN_RK = 4, SYN_THREADS = 256, GROUPS = 2;   // GROUPS: of the finest synthesis
+    static constexpr int SYN_RK = 4;
 };
 template <> struct WaveTile<double> {
     static constexpr int TW = 8, KX = 2, THREADS = 64, TAIL = 64;
-    static constexpr int SYN_TH = 4, SYN_RK = 2, SYN_THREADS = 32, GROUPS = 8;
+    static constexpr int SYN_RK = 2;
 };
+// threads of a synthesis tile of TH sub-band rows: one per output column and
+// SYN_RK sub-band rows
+template <typename T, int TH> constexpr int syn_threads() { return 2 * WaveTile<T>::TW * TH / WaveTile<T>::SYN_RK; }
 static constexpr int TAIL_THREADS = 512;
 
 // The filter taps of basis pb in registers (unused entries are zero).
@@ -311,9 +315,9 @@ __device__ __forceinline__ void syn_filter(const Taps<T, L>& f, int i0, Lo lo, H
     }
 }
 
-// barrier of one group of SYN_THREADS threads
-template <typename T> __device__ __forceinline__ void syn_sync(int group) {
-    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(WaveTile<T>::SYN_THREADS) : "memory");
+// barrier of one group of N threads
+template <int N> __device__ __forceinline__ void syn_sync(int group) {
+    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(N) : "memory");
 }
 
 // Row synthesis of 2 KX outputs from low-pass samples of `lo` and high-pass
@@ -353,19 +357,20 @@ __device__ __forceinline__ void syn_row(const Taps<T, L>& f, const T* __restrict
 // low-pass sub-band (row stride ll_ld); the details are in `det` (row stride
 // nx); `vec`: both begin at a multiple of 16 bytes, w >= 8. Ends with the shared
 // tile free for the next basis.
-template <typename T, int L>
+template <typename T, int L, int TH>
 __device__ __forceinline__ void synth_tile(const T* __restrict__ ll, int ll_ld, const T* __restrict__ det, bool vec,
                                            int nx, int h, int w, int ky0, int kx0, int pb, T* smem, int group, int tid,
                                            T (&acc)[2 * WaveTile<T>::SYN_RK]) {
     using W = WaveTile<T>;
-    constexpr int TH = W::SYN_TH, TW = W::TW, RK = W::SYN_RK, KX = W::KX, E = L / 2 - 1, RG = TW / KX, CW = 2 * TW;
+    constexpr int TW = W::TW, RK = W::SYN_RK, KX = W::KX, E = L / 2 - 1, RG = TW / KX, CW = 2 * TW;
+    constexpr int NT = syn_threads<T, TH>();
     static_assert(E <= 7, "filter longer than the row margin");
     Taps<T, L> f;
     f.load(pb);
     const int hs = h >> 1, wsub = w >> 1;
     T* sL = smem;                    // [TH + 7][CW] rows of the low-pass (along y) half
     T* sH = sL + (TH + 7) * CW;      // and of the high-pass half
-    for (int t = tid; t < (TH + E) * RG; t += W::SYN_THREADS) {
+    for (int t = tid; t < (TH + E) * RG; t += NT) {
         const int r = t / RG, k = (t - r * RG) * KX;
         if (kx0 + k >= wsub) continue;
         const int ky = (ky0 - E + r) & (hs - 1);
@@ -386,8 +391,7 @@ __device__ __forceinline__ void synth_tile(const T* __restrict__ ll, int ll_ld, 
             *reinterpret_cast<uint4*>(sH + r * CW + 2 * k + e) = *reinterpret_cast<const uint4*>(oH + e);
         }
     }
-    syn_sync<T>(group);
-    static_assert(CW * (TH / RK) == W::SYN_THREADS, "one column item per thread");
+    syn_sync<NT>(group);
     {
         const int x = tid % CW, g = tid / CW * RK;
         const T *cl = sL + (g + E) * CW + x, *ch = sH + (g + E) * CW + x;
@@ -396,27 +400,30 @@ __device__ __forceinline__ void synth_tile(const T* __restrict__ ll, int ll_ld, 
 #pragma unroll
         for (int m = 0; m < 2 * RK; ++m) acc[m] += o[m];
     }
-    syn_sync<T>(group);
+    syn_sync<NT>(group);
 }
 // The same out of line, for the loop over bases (inlined there, the eight
 // lengths' windows were kept live together and spilled).
 template <typename T> struct SynthPart { T v[2 * WaveTile<T>::SYN_RK]; };
-template <typename T, int L>
+template <typename T, int L, int TH>
 __device__ __noinline__ SynthPart<T> synth_part(const T* __restrict__ ll, int ll_ld, const T* __restrict__ det, bool vec,
                                                 int nx, int h, int w, int ky0, int kx0, int pb, T* smem, int group,
                                                 int tid) {
     SynthPart<T> p = {};
-    synth_tile<T, L>(ll, ll_ld, det, vec, nx, h, w, ky0, kx0, pb, smem, group, tid, p.v);
+    synth_tile<T, L, TH>(ll, ll_ld, det, vec, nx, h, w, ky0, kx0, pb, smem, group, tid, p.v);
     return p;
 }
-template <typename T> static size_t synth_smem_bytes() {
-    return sizeof(T) * 2 * (WaveTile<T>::SYN_TH + 7) * 2 * WaveTile<T>::TW;
+template <int V> using Int = std::integral_constant<int, V>;
+// tiles of TH sub-band rows that synthesise a w x h band
+template <typename T> static int64_t synth_tiles(int w, int h, int TH) {
+    return (int64_t)((w / 2 + WaveTile<T>::TW - 1) / WaveTile<T>::TW) * ((h / 2 + TH - 1) / TH);
 }
+template <typename T> static size_t synth_smem_bytes(int TH) { return sizeof(T) * 2 * (TH + 7) * 2 * WaveTile<T>::TW; }
 
 // One synthesis level for every wavelet basis (blockIdx.z): the reconstructed
 // h x w band of basis z into ll_out (row stride w).
-template <typename T>
-__global__ void __launch_bounds__(WaveTile<T>::SYN_THREADS)
+template <typename T, int TH>
+__global__ void __launch_bounds__(syn_threads<T, TH>())
 k_idwt_level(const T* __restrict__ ll_in, int ll_basis_stride, int ll_ld, const T* __restrict__ coef, int vec,
              const int* __restrict__ planes, int N, int nx, T* __restrict__ ll_out, int out_basis_stride, int h,
              int w, const int* __restrict__ pids) {
@@ -424,12 +431,12 @@ k_idwt_level(const T* __restrict__ ll_in, int ll_basis_stride, int ll_ld, const 
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int z = blockIdx.z, pb = pids[z];
-    const int ky0 = blockIdx.y * W::SYN_TH, kx0 = blockIdx.x * W::TW;
+    const int ky0 = blockIdx.y * TH, kx0 = blockIdx.x * W::TW;
     const T* det = coef + (size_t)planes[z] * N;
     const T* ll = ll_in ? ll_in + (size_t)z * ll_basis_stride : det;
     T acc[2 * W::SYN_RK] = {};
     PURIFY_WITH_LENGTH(fbank<T>().len[pb],
-                       (synth_tile<T, L>(ll, ll_in ? ll_ld : nx, det, vec != 0, nx, h, w, ky0, kx0, pb,
+                       (synth_tile<T, L, TH>(ll, ll_in ? ll_ld : nx, det, vec != 0, nx, h, w, ky0, kx0, pb,
                                          reinterpret_cast<T*>(smem_raw), 0, (int)threadIdx.x, acc)));
     constexpr int CW = 2 * W::TW;
     const int y = 2 * (ky0 + threadIdx.x / CW * W::SYN_RK), x = 2 * kx0 + threadIdx.x % CW;
@@ -443,34 +450,40 @@ k_idwt_level(const T* __restrict__ ll_in, int ll_basis_stride, int ll_ld, const 
 }
 
 // Finest synthesis level summed over all wavelet bases plus the Dirac plane:
-// x = (c_dirac + sum_z W_z^T c_z) / sqrt(q). GROUPS groups of threads share a
-// tile, group g takes bases g, g + GROUPS, ... in order (their column passes
+// x = (c_dirac + sum_z W_z^T c_z) / sqrt(q). G groups of threads share a
+// tile, group g takes bases g, g + G, ... in order (their column passes
 // wait for global memory at different times), and the groups' sums are added
-// in group order. When `ll_in` is null (L == 1) the low-pass bands come from the
-// coefficient planes.
-template <typename T>
-__global__ void __launch_bounds__(WaveTile<T>::SYN_THREADS * WaveTile<T>::GROUPS, sizeof(T) == 4 ? 2 : 1)
+// in group order. LEN > 0: all groups run the code of that filter length (see
+// the rule in psi_t). When `ll_in` is null (L == 1) the low-pass bands come from
+// the coefficient planes.
+template <typename T, int TH, int G, int LEN>
+__global__ void __launch_bounds__(syn_threads<T, TH>() * G, sizeof(T) == 4 && LEN == 0 ? 2 : 1)
 k_idwt_final(const T* __restrict__ ll_in, int ll_basis_stride, const T* __restrict__ coef, int vec,
              const int* __restrict__ planes, int N, int nx, int ny, const int* __restrict__ pids, int nw,
              int dirac_plane, T inv_sqrt_q, T* __restrict__ x) {
     using W = WaveTile<T>;
-    constexpr int NO = 2 * W::SYN_RK, G = W::GROUPS, NT = W::SYN_THREADS, CW = 2 * W::TW, GE = 2 * (W::SYN_TH + 7) * CW;
+    constexpr int NO = 2 * W::SYN_RK, NT = syn_threads<T, TH>(), CW = 2 * W::TW, GE = 2 * (TH + 7) * CW;
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* const smem = reinterpret_cast<T*>(smem_raw);
-    const int ky0 = blockIdx.y * W::SYN_TH, kx0 = blockIdx.x * W::TW;
+    const int ky0 = blockIdx.y * TH, kx0 = blockIdx.x * W::TW;
     const int group = threadIdx.x / NT, tid = threadIdx.x - group * NT;
     T acc[NO] = {};
     for (int z = group; z < nw; z += G) {
         const int pb = pids[z];
         const T* det = coef + (size_t)planes[z] * N;
         const T* ll = ll_in ? ll_in + (size_t)z * ll_basis_stride : det;
-        SynthPart<T> part;
-        PURIFY_WITH_LENGTH(fbank<T>().len[pb],
-                           (part = synth_part<T, L>(ll, ll_in ? (nx >> 1) : nx, det, vec != 0, nx, ny, nx, ky0, kx0, pb,
-                                                    smem + group * GE, group, tid)));
+        T* const tile = smem + group * GE;
+        if constexpr (LEN > 0) {
+            synth_tile<T, LEN, TH>(ll, ll_in ? (nx >> 1) : nx, det, vec != 0, nx, ny, nx, ky0, kx0, pb, tile, group, tid, acc);
+        } else {
+            SynthPart<T> part;
+            PURIFY_WITH_LENGTH(fbank<T>().len[pb],
+                               (part = synth_part<T, L, TH>(ll, ll_in ? (nx >> 1) : nx, det, vec != 0, nx, ny, nx, ky0,
+                                                            kx0, pb, tile, group, tid)));
 #pragma unroll
-        for (int e = 0; e < NO; ++e) acc[e] += part.v[e];
+            for (int e = 0; e < NO; ++e) acc[e] += part.v[e];
+        }
     }
     // the other groups' sums through shared memory (all are done with theirs)
     __syncthreads();
@@ -630,7 +643,7 @@ static void analyse(const T* x, T* c, int nx, int ny, int levels, int nw, int di
         const bool first = lev == 0;
         const int dirac = first && dirac_plane >= 0 ? 1 : 0;
         auto done = launched("dwt_level");
-        if (nw > 0 && h * w <= W::TAIL) {
+        if (nw > 0 && h * w <= W::TAIL && levels - lev >= 2) {   // (one level alone is faster by tiles: 10.4 us against 12.6 at 256 x 256)
             const size_t sm = tail_smem_bytes<T>(h, w);
             wave_smem(k_dwt_tail<T>, sm);
             launch_dependent(k_dwt_tail<T>, nw + dirac, TAIL_THREADS, sm, st, src, src_stride, src_ld, c, planes, N, nx, h,
@@ -701,7 +714,7 @@ template <typename T> static void psi_t(purify_plan* p, const void* cv, void* xv
     if (wl.nw > 0) {
         int top = lev + 1;   // finest of the levels whose output fits the tail
         while (top > 1 && ((int64_t)(p->ny >> (top - 1)) * (p->nx >> (top - 1))) <= W::TAIL) --top;
-        if (top <= lev) {
+        if (top < lev) {   // (one level alone is faster by tiles)
             const int h = p->ny >> top, w = p->nx >> top;
             T* out = bufs[top & 1];
             const size_t sm = tail_smem_bytes<T>(h, w);
@@ -716,21 +729,60 @@ template <typename T> static void psi_t(purify_plan* p, const void* cv, void* xv
         }
         for (; lev >= 1; --lev) {
             const int h = p->ny >> lev, w = p->nx >> lev;
-            dim3 g((w / 2 + W::TW - 1) / W::TW, (h / 2 + W::SYN_TH - 1) / W::SYN_TH, wl.nw);
             T* out = bufs[lev & 1];
-            Launch L(p, "idwt_level");
-            launch_dependent(k_idwt_level<T>, g, W::SYN_THREADS, synth_smem_bytes<T>(), p->stream, ll_in, llstride, ll_ld, c,
-                             (int)(aligned && w >= 8), plane_array(p), N, p->nx, out, llstride, h, w, pid_array(p));
-            L.done();
+            auto go = [&](auto th) {
+                constexpr int TH = decltype(th)::value;
+                const dim3 g((w / 2 + W::TW - 1) / W::TW, (h / 2 + TH - 1) / TH, wl.nw);
+                Launch L(p, "idwt_level");
+                launch_dependent(k_idwt_level<T, TH>, g, syn_threads<T, TH>(), synth_smem_bytes<T>(TH), p->stream, ll_in,
+                                 llstride, ll_ld, c, (int)(aligned && w >= 8), plane_array(p), N, p->nx, out, llstride, h,
+                                 w, pid_array(p));
+                L.done();
+            };
+            // tall tiles cost less halo; FP64 takes short ones where tall
+            // ones are fewer than the SMs (Psi of 128 x 128: 59.7 us against
+            // 61.0; of 512 x 512, where they are not: 247 against 240)
+            if (sizeof(T) == 8 && synth_tiles<T>(w, h, 16) * wl.nw < 152) go(Int<8>());
+            else go(Int<16>());
             ll_in = out;
             ll_ld = w;
         }
     }
-    dim3 g((p->nx / 2 + W::TW - 1) / W::TW, (p->ny / 2 + W::SYN_TH - 1) / W::SYN_TH, 1);
-    Launch Lf(p, "idwt_final");
-    launch_dependent(k_idwt_final<T>, g, W::SYN_THREADS * W::GROUPS, synth_smem_bytes<T>() * W::GROUPS, p->stream, ll_in, llstride, c,
-                     (int)(aligned && p->nx >= 8), plane_array(p), N, p->nx, p->ny, pid_array(p), wl.nw, wl.dirac_plane, inv_sqrt_q, x);
-    Lf.done();
+    auto go = [&](auto th, auto groups, auto len) {
+        constexpr int TH = decltype(th)::value, G = decltype(groups)::value, LEN = decltype(len)::value;
+        const size_t sm = synth_smem_bytes<T>(TH) * G;
+        wave_smem(k_idwt_final<T, TH, G, LEN>, sm);
+        const dim3 g((p->nx / 2 + W::TW - 1) / W::TW, (p->ny / 2 + TH - 1) / TH, 1);
+        Launch L(p, "idwt_final");
+        launch_dependent(k_idwt_final<T, TH, G, LEN>, g, syn_threads<T, TH>() * G, sm, p->stream, ll_in, llstride, c,
+                         (int)(aligned && p->nx >= 8), plane_array(p), N, p->nx, p->ny, pid_array(p), wl.nw,
+                         wl.dirac_plane, inv_sqrt_q, x);
+        L.done();
+    };
+    // One SM walks a tile's bases, so tiles are chosen by how many there are.
+    // From 256 tall ones on the chip is full: one group of threads, the least
+    // halo. With fewer, short tiles and more groups side by side; and where
+    // even the short tiles are fewer than the SMs, a tile's time is a chain of
+    // latencies, with the fetching of eight filter lengths' code among them:
+    // eight groups run one code, of the longest filter's length (shorter
+    // filters end in zeros, so an infinite coefficient reaches as far as the
+    // longest). Psi over 4 levels (5 at 1024 x 1024), nine bases,
+    // us, one group of tall tiles | two of short | eight of the same code:
+    // 128 x 128 21.5 17.9 14.3, 256 x 256 24.7 20.2 15.2, 512 x 256 24.3 20.4
+    // 19.6, 512 x 512 25.0 21.5 27.8, 1024 x 512 28.4 30.3 42.7, 1024 x 1024
+    // 48.5 50.3 77.5. FP64 is bound by its arithmetic: the number of tiles alone
+    // decides (64 x 64 51.8 with four groups of 8 rows, 48.2 with eight of 4;
+    // 512 x 64 54.5 and 72.0, 67.1 with two of 16; 256 x 256 95.6, 134.8, 84.7).
+    const int64_t tall = synth_tiles<T>(p->nx, p->ny, 16);
+    if constexpr (sizeof(T) == 4) {
+        if (tall >= 256) go(Int<16>(), Int<1>(), Int<0>());
+        else if (tall >= 128) go(Int<8>(), Int<2>(), Int<0>());
+        else PURIFY_WITH_LENGTH(longest_filter(p), (go(Int<4>(), Int<8>(), Int<L>())));
+    } else {
+        if (tall >= 128) go(Int<16>(), Int<2>(), Int<0>());
+        else if (synth_tiles<T>(p->nx, p->ny, 8) >= 128) go(Int<8>(), Int<4>(), Int<0>());
+        else go(Int<4>(), Int<8>(), Int<0>());
+    }
 }
 
 void launch_psi_adj(purify_plan* p, const void* x, void* c) {

@@ -37,3 +37,26 @@ def test_transforms(nx, ny, levels, mask, dtype):
         pk.purify_psi_adj_static(torch.from_numpy(x).to(DEV), got_c, nx, ny, levels, mask, dtype)
         torch.cuda.synchronize()
         assert rel(got_c.cpu(), ow.psi_adj(x.astype(np.float64), levels, mask)) <= TOL[dtype]
+
+
+@pytest.mark.parametrize("dtype", [pk.PURIFY_F32, pk.PURIFY_F64])
+@pytest.mark.parametrize("nx,ny,levels,mask", [
+    # either side of each choice of the finest synthesis: by 16-row tiles of 32 columns (FP32) or 8 (FP64)
+    (512, 256, 2, 0x1FF), (512, 512, 2, 0x1FF), (1024, 512, 2, 0x1FF),
+    (128, 128, 2, 0x1FF), (512, 64, 2, 0x1FF), (256, 256, 2, 0x1FF), (32, 2048, 2, 0x0FF),
+    # fewer bases than groups, and filters shorter than the longest beside it
+    (64, 64, 2, 0x100), (64, 64, 2, 0x181), (512, 512, 1, 0x00E), (1024, 512, 1, 0x102),
+    # one level below the finest in a band that fits the tail, several levels there
+    (32, 32, 2, 0x1FF), (16, 16, 3, 0x1FE), (16, 64, 2, 0x1FF), (8, 1024, 2, 0x1FF),
+])
+def test_synthesis_and_analysis_by_every_tile(nx, ny, levels, mask, dtype):
+    plan, *_ = make_plan(nx, ny, 64, 4, levels=levels, dtype=dtype, mask=mask)
+    g = synth.rng(3 * nx + ny + levels)
+    x = g.standard_normal((ny, nx)).astype(np_real(dtype))
+    c = g.standard_normal((bin(mask).count("1"), ny, nx)).astype(np_real(dtype))
+    got_c = torch.empty(c.shape, dtype=t_real(dtype), device=DEV)
+    got_x = torch.empty((ny, nx), dtype=t_real(dtype), device=DEV)
+    pk.purify_psi_adj(plan, torch.from_numpy(x).to(DEV), got_c)
+    pk.purify_psi(plan, torch.from_numpy(c).to(DEV), got_x)
+    assert rel(got_c.cpu(), ow.psi_adj(x.astype(np.float64), levels, mask)) <= TOL[dtype]
+    assert rel(got_x.cpu(), ow.psi(c.astype(np.float64), levels, mask)) <= TOL[dtype]

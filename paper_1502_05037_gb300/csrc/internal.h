@@ -35,6 +35,12 @@ struct Error {
 struct KernelTimer;
 void note_launch(const char* name, cudaStream_t s, KernelTimer* t, bool begin);
 
+// Tables go to the device by copies from pageable memory and memsets on the
+// legacy stream, which may still run when the call returns and which a
+// caller's non-blocking stream does not wait for. This waits for them: called
+// before anything on such a stream reads what was just uploaded.
+void settle_uploads();
+
 // ------------------------------------------------------- device buffers
 struct DevBuf {
     void* p = nullptr;

@@ -56,6 +56,8 @@ template <typename T> static void upload(DevBuf& b, const std::vector<T>& v) {
     PURIFY_CUDA(cudaMemcpy(b.p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
 }
 
+void settle_uploads() { PURIFY_CUDA(cudaStreamSynchronize(cudaStreamLegacy)); }
+
 template <typename T> static std::vector<T> cast_vec(const std::vector<double>& v) {
     std::vector<T> o(v.size());
     for (size_t i = 0; i < v.size(); ++i) o[i] = (T)v[i];
@@ -768,6 +770,7 @@ void build_group_lanes(purify_plan* p, int G) {
         upload(gc.cend, ce);
         upload(gc.chunk_first, cf);
     }
+    settle_uploads();
     p->group_count = G;
 }
 

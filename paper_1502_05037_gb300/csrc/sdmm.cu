@@ -492,6 +492,7 @@ template <typename T> struct Solver {
         PURIFY_CUDA(cudaMemcpy(s.chunk_first.p, cf.data(), sizeof(int) * cf.size(), cudaMemcpyHostToDevice));
         PURIFY_CUDA(cudaMemset(s.scal.p, 0, s.scal.bytes));
         PURIFY_CUDA(cudaMemset(s.counters.p, 0, s.counters.bytes));
+        settle_uploads();
         s.ready = true;
     }
 

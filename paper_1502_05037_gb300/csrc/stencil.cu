@@ -287,6 +287,7 @@ void build_stencil(purify_plan* p, const std::vector<int>& cells) {
     const std::vector<unsigned char> used = stencil_used(p, cells);
     p->stencil.used.alloc(used.size());
     PURIFY_CUDA(cudaMemcpy(p->stencil.used.p, used.data(), used.size(), cudaMemcpyHostToDevice));
+    settle_uploads();   // the build reads the run tables on the plan's stream
     PURIFY_J_DISPATCH(p->J, stencil_build_j, p);
     p->stencil.on = true;
 }

@@ -423,6 +423,7 @@ Unet* unet_create(int H, int W, int L, int base, int maxB, uint64_t seed, cudaSt
         u->err.alloc(sizeof(int));
         PURIFY_CUDA(cudaMemset(u->red_ctr.p, 0, u->red_ctr.bytes));
         PURIFY_CUDA(cudaMemset(u->err.p, 0, sizeof(int)));
+        settle_uploads();
         pack_all(*u);
         PURIFY_CUDA(cudaStreamSynchronize(st));
     } catch (...) {

@@ -618,6 +618,7 @@ void init_filter_banks() {
     }
     PURIFY_CUDA(cudaMemcpyToSymbol(c_bank_f, &bf, sizeof(bf)));
     PURIFY_CUDA(cudaMemcpyToSymbol(c_bank_d, &bd, sizeof(bd)));
+    settle_uploads();
     g_bank_ready[dev] = true;
 }
 

@@ -118,7 +118,11 @@ typedef struct {
     int32_t degrid_mode;           /* the G decomposition in use: 1 tile subproblems, 3..5 lanes,
                                       8 visibilities sorted by cell (autotuned plans) */
     int32_t normal_mode;           /* the fused G^H G of the CG normal operator: 2 runs, 3..5 lanes,
-                                      6 deterministic lanes, 7 a stencil on the grid (autotuned plans) */
+                                      6 deterministic lanes, 7 a stencil on the grid (autotuned plans;
+                                      only where its coefficients and the sums they are built from
+                                      leave three quarters of the device's free memory alone, so that
+                                      what else is allocated can decide, and with it the last bits of
+                                      a result) */
     int32_t lane_tile;             /* grid tile edge grouping the runs of normal_mode 5 (else 0) */
     int32_t fft_rows_per_block;    /* FFT launch shape in use: row transforms per block, */
     int32_t fft_cols_per_block;    /* column transforms per block, */

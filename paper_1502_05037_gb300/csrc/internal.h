@@ -427,9 +427,10 @@ double coef_std(purify_plan* p, const void* x);
 inline bool normal_half(const purify_plan* p) { return p->half_on && (p->stencil.on || p->dtype == PURIFY_F32); }
 // G^H G as a stencil (stencil.cu): bytes of the coefficients; the build from
 // the half-plane lane work (cells: the runs' first-tap cells, row * W +
-// column); the application, which writes all of gacc
+// column), false where the device has no room for it; the application, which
+// writes all of gacc
 int64_t stencil_bytes(const purify_plan* p);
-void build_stencil(purify_plan* p, const std::vector<int>& cells);
+bool build_stencil(purify_plan* p, const std::vector<int>& cells);
 void launch_stencil(purify_plan* p, const int* skip);
 #define PURIFY_J_DISPATCH(J, FN, ...)                                     \
     switch (J) {                                                          \

@@ -622,11 +622,13 @@ static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std
     upload(sw.idx, si);
     upload(sw.idx_caller, sk);
     p->workspace_bytes += (int64_t)(sw.z.bytes + sw.cell.bytes + sw.idx.bytes + sw.idx_caller.bytes);
-    // the normal operator as a stencil, where that is the faster form
+    // the normal operator as a stencil, where that is the faster form and fits
     if (use_stencil(p, nr)) {
         std::vector<int> cells(nr);
         for (size_t q = 0; q < nr; ++q) cells[q] = cell[order[sorted[q].first]];
         build_stencil(p, cells);
+    }
+    if (p->stencil.on) {
         p->workspace_bytes += (int64_t)(p->stencil.coef.bytes + p->stencil.used.bytes);
     } else if (sizeof(T) == 4 && width == 32) {
         fill(p->half_pairs, 16, false);

@@ -283,13 +283,22 @@ int64_t stencil_bytes(const purify_plan* p) {
     return (int64_t)p->Ky * stencil_planes(p->J) * p->half.W * (p->dtype == PURIFY_F32 ? 4 : 8);
 }
 
-void build_stencil(purify_plan* p, const std::vector<int>& cells) {
+bool build_stencil(purify_plan* p, const std::vector<int>& cells) {
     const std::vector<unsigned char> used = stencil_used(p, cells);
-    p->stencil.used.alloc(used.size());
-    PURIFY_CUDA(cudaMemcpy(p->stencil.used.p, used.data(), used.size(), cudaMemcpyHostToDevice));
-    settle_uploads();   // the build reads the run tables on the plan's stream
-    PURIFY_J_DISPATCH(p->J, stencil_build_j, p);
+    try {
+        p->stencil.used.alloc(used.size());
+        PURIFY_CUDA(cudaMemcpy(p->stencil.used.p, used.data(), used.size(), cudaMemcpyHostToDevice));
+        settle_uploads();   // the build reads the run tables on the plan's stream
+        PURIFY_J_DISPATCH(p->J, stencil_build_j, p);
+    } catch (const Error& e) {
+        // the memory that was free when it was chosen may be gone by now
+        if (e.status != PURIFY_ENOMEM) throw;
+        p->stencil.coef.release();
+        p->stencil.used.release();
+        return false;
+    }
     p->stencil.on = true;
+    return true;
 }
 
 template <typename T, int J> static void stencil_tj(purify_plan* p, const int* skip) {

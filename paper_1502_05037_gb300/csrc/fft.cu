@@ -412,28 +412,93 @@ template <typename T> struct RowFold {
         if (first && blockIdx.x == 0 && threadIdx.x == 0) f.flags[F_CGDONE] = 0;   // the next kernels read it
         return true;
     }
-    // Chronopoulos-Gear update of pixel idx, then the new r
-    __device__ __forceinline__ T pixel(size_t idx) const {
-        T rv = r[idx];
-        if (first) {
-            if (add) {
-                rv += add[idx];
-                r[idx] = rv;
+    // Chronopoulos-Gear update of the pixels at offset idx (none where
+    // negative), then the new r; 0 where there is none. All loads come before
+    // the first store: the vectors are not known to be distinct, so a pixel at
+    // a time each would wait for memory after the one before (by events, a pass
+    // of a CG step on the half plane, eight pixels a thread: 10.4 -> 8.8 us at
+    // 128 x 128, 12.4 -> 10.6 at 512 x 512).
+    template <int N> __device__ __forceinline__ void pixels(const int (&idx)[N], T (&rv)[N]) const {
+        T pv[N], sv[N], uv[N], xv[N];
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            rv[e] = pv[e] = sv[e] = uv[e] = xv[e] = T(0);
+            if (idx[e] < 0) continue;
+            rv[e] = r[idx[e]];
+            if (first) {
+                if (add) uv[e] = add[idx[e]];
+            } else if (pending) {
+                pv[e] = p[idx[e]];
+                sv[e] = s[idx[e]];
+                uv[e] = u[idx[e]];
+                xv[e] = x[idx[e]];
             }
-            p[idx] = T(0);
-            s[idx] = T(0);
-        } else if (pending) {
-            const T pv = rv + beta * p[idx];
-            const T sv = u[idx] + beta * s[idx];
-            p[idx] = pv;
-            s[idx] = sv;
-            x[idx] += alpha * pv;
-            rv = rv - alpha * sv;
-            r[idx] = rv;
         }
-        return rv;
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            if (idx[e] < 0) continue;
+            if (first) {
+                if (add) {
+                    rv[e] += uv[e];
+                    r[idx[e]] = rv[e];
+                }
+                p[idx[e]] = T(0);
+                s[idx[e]] = T(0);
+            } else if (pending) {
+                const T pn = rv[e] + beta * pv[e];
+                const T sn = uv[e] + beta * sv[e];
+                p[idx[e]] = pn;
+                s[idx[e]] = sn;
+                x[idx[e]] = xv[e] + alpha * pn;
+                rv[e] = rv[e] - alpha * sn;
+                r[idx[e]] = rv[e];
+            }
+        }
     }
 };
+
+// S Z of rows row0 .. row0 + ROWS - 1 of the image for the thread's eight
+// elements p1 = t + k Kx / 8 of a row transform: f(k, values of the rows).
+// Elements k in the order 0 1 6 7, 2 3 4 5 (with oversampling 2 the image is in
+// the first four), BATCH pixels at a time.
+template <typename T, int Kx, int ROWS, typename F>
+__device__ __forceinline__ void row_elements(const RowFold<T>& cg, const T* __restrict__ x, const T* __restrict__ sx,
+                                             const T* __restrict__ sy, int nx, int row0, int t, T scale, F&& f) {
+    constexpr int BATCH = sizeof(T) == 4 ? 4 : 2, KS = BATCH / ROWS, N8 = Kx / 8;
+    T rowscale[ROWS];
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) rowscale[q] = sy[row0 + q] * scale;
+#pragma unroll
+    for (int g = 0; g < 8; g += KS) {
+        int idx[BATCH];
+        T v[BATCH], c[KS];
+#pragma unroll
+        for (int b = 0; b < KS; ++b) {
+            constexpr int order[8] = {0, 1, 6, 7, 2, 3, 4, 5};
+            const int k = order[g + b], p1 = t + k * N8;
+            // pixel column j with (j - nx/2) mod Kx == p1 (p1 < Kx/2 exactly when k < 4)
+            const int j = (k < 4 ? p1 : p1 - Kx) + nx / 2;
+            const bool in = j >= 0 && j < nx;
+            c[b] = in ? sx[j] : T(0);
+#pragma unroll
+            for (int q = 0; q < ROWS; ++q) idx[b * ROWS + q] = in ? (row0 + q) * nx + j : -1;
+        }
+        if (cg.on) {
+            cg.pixels(idx, v);
+        } else {
+#pragma unroll
+            for (int e = 0; e < BATCH; ++e) v[e] = idx[e] >= 0 ? x[idx[e]] : T(0);
+        }
+#pragma unroll
+        for (int b = 0; b < KS; ++b) {
+            constexpr int order[8] = {0, 1, 6, 7, 2, 3, 4, 5};
+            T w[ROWS];
+#pragma unroll
+            for (int q = 0; q < ROWS; ++q) w[q] = v[b * ROWS + q] * c[b] * rowscale[q];
+            f(order[g + b], w);
+        }
+    }
+}
 
 // Block b clears rows [b Ky/gridDim, (b+1) Ky/gridDim) of a Ky x ld grid of
 // C (Ky is a multiple of the block count) in 16-byte stores.
@@ -464,17 +529,11 @@ __global__ void __launch_bounds__(1024) k_rows_fwd(const T* __restrict__ x, type
     if (zero_grid) clear_rows(zero_grid, Ky, Kx);
     int i0, t, f;
     row_thread<N8>(rb, i0, t, f);
-    // S Z of pixel p1 of image row i (p1 < Kx/2 exactly when k < 4)
-    auto pix = [&](int i, int k, int p1) -> T {
-        // pixel column j with (j - nx/2) mod Kx == p1
-        const int j = (k < 4 ? p1 : p1 - Kx) + nx / 2;
-        if (j < 0 || j >= nx) return T(0);
-        const size_t idx = (size_t)i * nx + j;
-        return (cg.on ? cg.pixel(idx) : x[idx]) * sx[j] * (sy[i] * scale);
-    };
+    C in[8];
+    row_elements<T, Kx, 1>(cg, x, sx, sy, nx, i0, t, scale, [&](int k, T (&w)[1]) { in[k] = cmake<C>(w[0], T(0)); });
     C* buf = reinterpret_cast<C*>(smem_raw) + f * fft_padded(Kx);
     C* const out = rows + (size_t)i0 * Kx;
-    auto load = [&](int k, int p1) -> C { return cmake<C>(pix(i0, k, p1), T(0)); };
+    auto load = [&](int k, int) -> C { return in[k]; };
     auto store = [&](int, int k, C v) { out[k] = v; };
     fft_core<C, false, LX>(t, tw, load, store, FftSlots<C>{buf, 1, alt});
     pdl_trigger();
@@ -501,18 +560,14 @@ __global__ void __launch_bounds__(1024) k_rows_fwd_half(const T* __restrict__ x,
     if (zero_grid) clear_rows(zero_grid, Ky, hp.W);
     int i, t, f;
     row_thread<N8>(rb, i, t, f);
-    auto pix = [&](int row, int k, int p1) -> T {
-        const int j = (k < 4 ? p1 : p1 - Kx) + nx / 2;
-        if (j < 0 || j >= nx) return T(0);
-        const size_t idx = (size_t)row * nx + j;
-        return (cg.on ? cg.pixel(idx) : x[idx]) * sx[j] * (sy[row] * scale);
-    };
+    C in[8];
+    row_elements<T, Kx, 2>(cg, x, sx, sy, nx, 2 * i, t, scale, [&](int k, T (&w)[2]) { in[k] = cmake<C>(w[0], w[1]); });
     C* const buf = reinterpret_cast<C*>(smem_raw) + f * fft_padded(Kx);
     // the transform's output goes back to shared memory: the buffer its last
     // stage does not read (see fft_core), or the only one after a barrier
     constexpr int NST = (LX - (LX % 3 == 0 ? 3 : LX % 3)) / 3;
     C* const z = (alt && NST % 2 == 1) ? buf + alt : buf;
-    auto load = [&](int k, int p1) -> C { return cmake<C>(pix(2 * i, k, p1), pix(2 * i + 1, k, p1)); };
+    auto load = [&](int k, int) -> C { return in[k]; };
     auto store = [&](int q, int k, C v) {
         if (q == 0 && !alt) __syncthreads();
         z[fft_pad(k)] = v;
@@ -521,12 +576,15 @@ __global__ void __launch_bounds__(1024) k_rows_fwd_half(const T* __restrict__ x,
     __syncthreads();
     C* const r0 = rows + (size_t)(2 * i) * hp.W;
     C* const r1 = r0 + hp.W;
-    for (int j = t; j < hp.W; j += N8) {
+    auto column = [&](int j) {
         const int k = (j - hp.off) & (Kx - 1);
         const C a = z[fft_pad(k)], b = z[fft_pad((Kx - k) & (Kx - 1))];
         r0[j] = cmake<C>(T(0.5) * (a.x + b.x), T(0.5) * (a.y - b.y));
         r1[j] = cmake<C>(T(0.5) * (a.y + b.y), T(0.5) * (b.x - a.x));
-    }
+    };
+#pragma unroll
+    for (int q = 0; q < 4; ++q) column(t + q * N8);   // (W > Kx / 2)
+    for (int j = t + 4 * N8; j < hp.W; j += N8) column(j);
     pdl_trigger();
 }
 
@@ -727,11 +785,28 @@ __global__ void __launch_bounds__(MAXT) k_rows_inv_half(const typename cplx_of<T
     row_thread<N8>(rb, i, t, f);
     T dacc = 0, gacc2 = 0;   // add.out, and with the folded CG add.add (add = r, out = A r)
     const bool cg = cgf.part != nullptr;
-    auto emit = [&](int row, int j, T v) {
+    // the pixels of `add` under way before the transform (FP32; doubles have no
+    // registers to spare): by events 13.2 -> 12.6 us at 128 x 128, 15.6 -> 14.4 at
+    // 512 x 512
+    constexpr bool EARLY = sizeof(T) == 4;
+    T early[EARLY ? 8 : 1][2];
+    if constexpr (EARLY) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int j = (t + q * N8 + nx / 2) & (Kx - 1);
+            early[q][0] = early[q][1] = T(0);
+            if (add && j < nx) {
+                early[q][0] = add[(size_t)(2 * i) * nx + j];
+                early[q][1] = add[(size_t)(2 * i + 1) * nx + j];
+            }
+        }
+    }
+    auto emit = [&](int q, int side, int j, T v) {
+        const int row = 2 * i + side;
         const size_t idx = (size_t)row * nx + j;
         T r = v * (sx[j] * (sy[row] * scale));
         if (add) {
-            const T a = add[idx];
+            const T a = EARLY ? early[EARLY ? q : 0][side] : add[idx];
             r += add_coef * a;
             dacc += a * r;
             if (cg) gacc2 += a * a;
@@ -740,11 +815,16 @@ __global__ void __launch_bounds__(MAXT) k_rows_inv_half(const typename cplx_of<T
     };
     const C* const r0 = rows + (size_t)(2 * i) * hp.W;
     const C* const r1 = r0 + hp.W;
+    // column k: one load, whose address the condition decides (nothing waits
+    // for it before the others are under way); only the smallest grid stores
+    // more columns than it has, some twice
     auto column = [&](const C* r, int k) -> C {
         C v = cmake<C>(T(0), T(0));
         const int j = k + hp.off;
-        if (j < hp.W0) v = r[j];
-        if (j >= Kx) v = cadd(v, r[j - Kx]);
+        if (j < hp.W0 || j >= Kx) v = r[j < hp.W0 ? j : j - Kx];
+        if constexpr (LX == 4) {
+            if (j < hp.W0 && j >= Kx) v = cadd(v, r[j - Kx]);
+        }
         return v;
     };
     auto load = [&](int, int k) -> C {
@@ -752,11 +832,11 @@ __global__ void __launch_bounds__(MAXT) k_rows_inv_half(const typename cplx_of<T
         const C a = column(r0, k), am = column(r0, m), b = column(r1, k), bm = column(r1, m);
         return cmake<C>(T(0.5) * ((a.x + am.x) - (b.y - bm.y)), T(0.5) * ((a.y - am.y) + (b.x + bm.x)));
     };
-    auto store = [&](int, int p1, C v) {
+    auto store = [&](int q, int p1, C v) {
         const int j = (p1 + nx / 2) & (Kx - 1);
         if (j >= nx) return;
-        emit(2 * i, j, v.x);
-        emit(2 * i + 1, j, v.y);
+        emit(q, 0, j, v.x);
+        emit(q, 1, j, v.y);
     };
     C* buf = reinterpret_cast<C*>(smem_raw) + f * fft_padded(Kx);
     fft_core<C, true, LX>(t, tw, load, store, FftSlots<C>{buf, 1, alt});

@@ -76,8 +76,10 @@ typedef struct {
     purify_dtype dtype;            /* operator precision */
     void *stream;                  /* cudaStream_t; NULL = legacy default stream */
     int32_t tile;                  /* gridding tile edge (power of two, 8..64); 0 => autotune */
-    int32_t grid_mode;             /* G^H / G work decomposition: 0 => autotuned (tile
-                                      subproblems when `tile` is fixed), 1 => tile subproblems
+    int32_t grid_mode;             /* G^H / G work decomposition: 0 => autotuned (with `tile`
+                                      fixed not timed: G^H of purify_phi_adj by tile
+                                      subproblems, Phi, the solver's adjoint and the normal
+                                      operator on the half plane of a real image), 1 => tile subproblems
                                       (shared-memory tile per subproblem), 2 => G^H by runs of
                                       visibilities sharing their first-tap cell, flushed to the
                                       grid (G by tiles), 3..5 => G^H, G and the solver's G^H G
@@ -117,7 +119,8 @@ typedef struct {
                                       description) */
     int32_t degrid_mode;           /* the G decomposition in use: 1 tile subproblems, 3..5 lanes,
                                       8 visibilities sorted by cell (autotuned plans) */
-    int32_t normal_mode;           /* the fused G^H G of the CG normal operator: 2 runs, 3..5 lanes,
+    int32_t normal_mode;           /* the fused G^H G of the CG normal operator: 2 runs, 3..5 lanes
+                                      (4 also: lane pairs on the half plane),
                                       6 deterministic lanes, 7 a stencil on the grid (autotuned plans;
                                       only where its coefficients and the sums they are built from
                                       leave three quarters of the device's free memory alone, so that

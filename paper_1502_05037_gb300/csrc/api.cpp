@@ -170,7 +170,7 @@ purify_status purify_plan_get_info(const purify_plan* plan, purify_plan_info* in
         info->grid_mode = plan->grid_kind;
         info->degrid_mode = plan->degrid_kind;
         info->normal_mode = plan->normal_kind;
-        info->lane_tile = plan->normal_kind == 5 ? plan->lanes[2].tile : 0;
+        info->lane_tile = plan->normal_kind == 5 && !plan->normal_half ? plan->lanes[2].tile : 0;
         fft_launch_shape(plan, info->fft_rows_per_block, info->fft_cols_per_block, info->fft_cols_per_thread);
     });
 }
@@ -204,8 +204,8 @@ purify_status purify_phi_normal(purify_plan* p, const void* x, void* out) {
         Staged xs = stage_in(p, x, rb * p->N, p->stage_in);
         Staged os = stage_out(p, out, rb * p->N, p->stage_out);
         // the forward row pass clears the accumulator that G^H G adds into
-        const bool half = normal_half(p);
-        launch_scale_pad_rows(p, xs.dev, 1.0, nullptr, true, true, nullptr, half);
+        const bool half = p->normal_half;
+        launch_scale_pad_rows(p, xs.dev, 1.0, nullptr, true, clear_acc(half), nullptr, half);
         launch_cols_fwd(p, nullptr, half);
         launch_normal_gg(p, nullptr, true, half);
         launch_cols_inv(p, nullptr, nullptr, half);

@@ -512,21 +512,21 @@ template <typename C> __device__ __forceinline__ void clear_rows(C* grid, int Ky
 // S Z and the forward row FFT: rows [i0, i0+rb) of the image to rows[i][0..Kx).
 // With a CG fold (fold.x set) the input is the residual r after the step's
 // update (see CgFold), not x. When zero_grid != null the pass also clears
-// that Ky x Kx complex grid (the gridding accumulator of the same CG step, or
-// of the adjoint that follows Phi).
+// that Ky x zero_ld complex grid (the gridding accumulator of the same CG step,
+// or of the adjoint that follows Phi, on the whole plane or on the half).
 template <typename T, int LX>
 __global__ void __launch_bounds__(1024) k_rows_fwd(const T* __restrict__ x, typename cplx_of<T>::type* __restrict__ rows,
                            const T* __restrict__ sx, const T* __restrict__ sy,
                            const typename cplx_of<T>::type* __restrict__ tw, int nx, int ny,
                            int rb, int alt, T scale, const int* __restrict__ skip,
-                           typename cplx_of<T>::type* __restrict__ zero_grid, int Ky, CgFold fold) {
+                           typename cplx_of<T>::type* __restrict__ zero_grid, int zero_ld, int Ky, CgFold fold) {
     using C = typename cplx_of<T>::type;
     constexpr int Kx = 1 << LX, N8 = Kx >> 3;
     pdl_wait();
     RowFold<T> cg;
     if (!cg.start(fold, skip)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (zero_grid) clear_rows(zero_grid, Ky, Kx);
+    if (zero_grid) clear_rows(zero_grid, Ky, zero_ld);
     int i0, t, f;
     row_thread<N8>(rb, i0, t, f);
     C in[8];
@@ -550,14 +550,15 @@ __global__ void __launch_bounds__(1024) k_rows_fwd_half(const T* __restrict__ x,
                            typename cplx_of<T>::type* __restrict__ rows, const T* __restrict__ sx,
                            const T* __restrict__ sy, const typename cplx_of<T>::type* __restrict__ tw, int nx,
                            int rb, int alt, T scale, const int* __restrict__ skip,
-                           typename cplx_of<T>::type* __restrict__ zero_grid, int Ky, CgFold fold, HalfPlane hp) {
+                           typename cplx_of<T>::type* __restrict__ zero_grid, int zero_ld, int Ky, CgFold fold,
+                           HalfPlane hp) {
     using C = typename cplx_of<T>::type;
     constexpr int Kx = 1 << LX, N8 = Kx >> 3;
     pdl_wait();
     RowFold<T> cg;
     if (!cg.start(fold, skip)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (zero_grid) clear_rows(zero_grid, Ky, hp.W);
+    if (zero_grid) clear_rows(zero_grid, Ky, zero_ld);
     int i, t, f;
     row_thread<N8>(rb, i, t, f);
     C in[8];
@@ -948,19 +949,17 @@ bool fft_shape_ok(int nb, int K, int dtype, int lanes) {
     return nb / lanes * (K / 8) <= 1024 && (size_t)nb * fft_padded(K) * cbytes <= 160 * 1024;
 }
 
-template <typename T> static int plan_rows_per_block(const purify_plan* p) {
-    int rb = p->fft_rb > 0 ? p->fft_rb : rows_per_block<T>(p->ny, p->Kx);
-    while (p->ny % rb) rb >>= 1;
+static const FftShape& plan_shape(const purify_plan* p, bool half) { return half ? p->fft_half : p->fft; }
+// rows per block, or row pairs of the half-plane passes
+template <typename T> static int plan_rows_per_block(const purify_plan* p, bool half) {
+    const int rows = half ? p->ny / 2 : p->ny, tuned = plan_shape(p, half).rb;
+    int rb = tuned > 0 ? tuned : rows_per_block<T>(rows, p->Kx);
+    while (rows % rb) rb >>= 1;
     return rb;
 }
-// row pairs per block of the half-plane passes
-template <typename T> static int plan_pairs_per_block(const purify_plan* p) {
-    int rb = p->fft_rb > 0 ? p->fft_rb : rows_per_block<T>(p->ny / 2, p->Kx);
-    while ((p->ny / 2) % rb) rb >>= 1;
-    return rb;
-}
-template <typename T> static int plan_cols_per_block(const purify_plan* p) {
-    return p->fft_cb > 0 ? p->fft_cb : cols_per_block<T>(p->Ky, p->Kx);
+template <typename T> static int plan_cols_per_block(const purify_plan* p, bool half) {
+    const int tuned = plan_shape(p, half).cb;
+    return tuned > 0 ? tuned : cols_per_block<T>(p->Ky, p->Kx);
 }
 // row stride and number of columns of the grid a column pass runs over
 static int plan_cols(const purify_plan* p, bool half) { return half ? p->half.W : p->Kx; }
@@ -972,31 +971,34 @@ template <typename T> static int col_lanes(int cb, int tuned) {
 }
 
 template <typename T>
-static void rows_fwd_t(purify_plan* p, const void* x, double scale, const int* skip, bool corr, bool zero_acc,
+static void rows_fwd_t(purify_plan* p, const void* x, double scale, const int* skip, bool corr, ClearAcc clear,
                        const CgFold* fold, bool half) {
     using C = typename cplx_of<T>::type;
-    const int rb = half ? plan_pairs_per_block<T>(p) : plan_rows_per_block<T>(p);
+    const int rb = plan_rows_per_block<T>(p, half);
     const int alt = fft_alt(rb, p->Kx, sizeof(C));
     const size_t sm = fft_smem(rb, p->Kx, sizeof(C), alt);
     with_log2(p->Kx, [&](auto lg) {
         constexpr int LX = decltype(lg)::value;
         const T* sx = corr ? p->sx.as<T>() : p->onesx.as<T>();
         const T* sy = corr ? p->sy.as<T>() : p->onesy.as<T>();
-        C* acc = zero_acc ? p->gacc.as<C>() : nullptr;
+        C* acc = clear != CLEAR_NONE ? p->gacc.as<C>() : nullptr;
+        const int acc_ld = clear == CLEAR_HALF ? p->half.W : p->Kx;
         const CgFold cg = fold ? *fold : CgFold();
         if (half) {
             auto kern = k_rows_fwd_half<T, LX>;
             set_fft_smem(kern, sm);
             Launch L(p, "fft_rows_fwd");
             launch_dependent(kern, p->ny / 2 / rb, rb * (p->Kx / 8), sm, p->stream, (const T*)x, p->rows.as<C>(), sx,
-                             sy, p->twx.as<C>(), p->nx, rb, alt, (T)scale, skip, acc, p->Ky, cg, p->half);
+                             sy, p->twx.as<C>(), p->nx, rb, alt, (T)scale, skip, acc, acc_ld, p->Ky, cg,
+                             p->half);
             L.done();
         } else {
             auto kern = k_rows_fwd<T, LX>;
             set_fft_smem(kern, sm);
             Launch L(p, "fft_rows_fwd");
             launch_dependent(kern, p->ny / rb, rb * (p->Kx / 8), sm, p->stream, (const T*)x, p->rows.as<C>(), sx, sy,
-                             p->twx.as<C>(), p->nx, p->ny, rb, alt, (T)scale, skip, acc, p->Ky, cg);
+                             p->twx.as<C>(), p->nx, p->ny, rb, alt, (T)scale, skip, acc, acc_ld, p->Ky,
+                             cg);
             L.done();
         }
     });
@@ -1004,10 +1006,10 @@ static void rows_fwd_t(purify_plan* p, const void* x, double scale, const int* s
 
 template <typename T> static void cols_fwd_t(purify_plan* p, const int* skip, bool half) {
     using C = typename cplx_of<T>::type;
-    const int cb = plan_cols_per_block<T>(p);
+    const int cb = plan_cols_per_block<T>(p, half);
     const int alt = fft_alt(cb, p->Ky, sizeof(C));
     const size_t sm = fft_smem(cb, p->Ky, sizeof(C), alt);
-    const int w = col_lanes<T>(cb, p->fft_cw);
+    const int w = col_lanes<T>(cb, plan_shape(p, half).cw);
     with_log2(p->Ky, [&](auto lg) {
         constexpr int LY = decltype(lg)::value;
         auto kern = k_cols_fwd<T, LY, 1>;
@@ -1022,12 +1024,12 @@ template <typename T> static void cols_fwd_t(purify_plan* p, const int* skip, bo
 
 template <typename T> static void cols_inv_t(purify_plan* p, const int* skip, const void* mult, bool half) {
     using C = typename cplx_of<T>::type;
-    const int cb = plan_cols_per_block<T>(p);
+    const int cb = plan_cols_per_block<T>(p, half);
     const int alt = fft_alt(cb, p->Ky, sizeof(C));
     const size_t sm = fft_smem(cb, p->Ky, sizeof(C), alt);
     // the adjoint reads the gridding output; the circulant path the forward grid
     const C* src = mult ? p->grid.as<C>() : p->gacc.as<C>();
-    const int w = col_lanes<T>(cb, p->fft_cw);
+    const int w = col_lanes<T>(cb, plan_shape(p, half).cw);
     with_log2(p->Ky, [&](auto lg) {
         constexpr int LY = decltype(lg)::value;
         auto kern = k_cols_inv<T, LY, 1>;
@@ -1044,7 +1046,7 @@ template <typename T>
 static void rows_inv_t(purify_plan* p, void* out, double scale, int out_mode, const void* add, double add_coef,
                        const int* skip, const CgFold* cg, bool corr, bool half) {
     using C = typename cplx_of<T>::type;
-    const int rb = half ? plan_pairs_per_block<T>(p) : plan_rows_per_block<T>(p);
+    const int rb = plan_rows_per_block<T>(p, half);
     const int alt = fft_alt(rb, p->Kx, sizeof(C));
     const size_t sm = fft_smem(rb, p->Kx, sizeof(C), alt);
     const int nt = rb * (p->Kx / 8);
@@ -1074,21 +1076,22 @@ static void rows_inv_t(purify_plan* p, void* out, double scale, int out_mode, co
 }
 
 void fft_launch_shape(const purify_plan* p, int& rb, int& cb, int& cw) {
+    const bool half = p->normal_half;
     if (p->dtype == PURIFY_F32) {
-        rb = plan_rows_per_block<float>(p);
-        cb = plan_cols_per_block<float>(p);
-        cw = col_lanes<float>(cb, p->fft_cw);
+        rb = plan_rows_per_block<float>(p, half);
+        cb = plan_cols_per_block<float>(p, half);
+        cw = col_lanes<float>(cb, plan_shape(p, half).cw);
     } else {
-        rb = plan_rows_per_block<double>(p);
-        cb = plan_cols_per_block<double>(p);
-        cw = col_lanes<double>(cb, p->fft_cw);
+        rb = plan_rows_per_block<double>(p, half);
+        cb = plan_cols_per_block<double>(p, half);
+        cw = col_lanes<double>(cb, plan_shape(p, half).cw);
     }
 }
 
-void launch_scale_pad_rows(purify_plan* p, const void* x, double scale, const int* skip, bool corr, bool zero_acc,
+void launch_scale_pad_rows(purify_plan* p, const void* x, double scale, const int* skip, bool corr, ClearAcc clear,
                            const CgFold* fold, bool half) {
-    if (p->dtype == PURIFY_F32) rows_fwd_t<float>(p, x, scale, skip, corr, zero_acc, fold, half);
-    else rows_fwd_t<double>(p, x, scale, skip, corr, zero_acc, fold, half);
+    if (p->dtype == PURIFY_F32) rows_fwd_t<float>(p, x, scale, skip, corr, clear, fold, half);
+    else rows_fwd_t<double>(p, x, scale, skip, corr, clear, fold, half);
 }
 void launch_cols_fwd(purify_plan* p, const int* skip, bool half) {
     if (p->dtype == PURIFY_F32) cols_fwd_t<float>(p, skip, half); else cols_fwd_t<double>(p, skip, half);

@@ -145,6 +145,11 @@ struct LaneWork {
 struct HalfPlane {
     int off = 0, W0 = 0, W = 0;
 };
+// FFT launch shape: rows (row pairs on the half plane) and columns per block, 0
+// by heuristic; columns per thread, 1 or 2 (0: 2 where the shape allows).
+struct FftShape {
+    int rb = 0, cb = 0, cw = 0;
+};
 // index code of a lane record: the visibility, folded ones as -2 - m, -1 padding
 PURIFY_HD int fold_index(int m) { return -2 - m; }
 
@@ -273,7 +278,9 @@ struct purify_plan {
     purify::RunWork runs;             // run-ordered work of the fused normal operator
     purify::LaneWork lanes[3];        // lane-per-run forms of the same runs (FP32, J <= 6): one lane
                                       // per run; two lanes per run; two, sets grouped by tile
-    bool half_on = false;             // the half-plane path is built (autotuned plans)
+    // which of Phi, the solver's adjoint and the normal operator run on the half plane (grid_mode 0; timed
+    // against the whole plane on small images)
+    bool phi_half = false, adj_half = false, normal_half = false;
     purify::HalfPlane half;
     purify::LaneWork half_lanes;      // folded visibilities: a lane per run (FP32, J <= 6) or lane pairs,
                                       // internal order only
@@ -282,16 +289,15 @@ struct purify_plan {
     purify::SortedWork half_sorted;   // the same visibilities sorted by cell
     purify::Stencil stencil;          // G^H G of the half plane as a stencil, where it is the faster form
     purify::DevBuf det_patch;         // run patches of the deterministic lane form (float2)
-    int normal_kind = 2;              // G^H G: 2 run sets, 3..5 lanes (as lanes[kind - 3]; on the half plane
-                                      // half_lanes), 6 the deterministic lane pairs (lanes[1]), 7 the
+    int normal_kind = 2;              // G^H G: 2 run sets, 3..5 lanes (as lanes[kind - 3]; 4 with normal_half: the
+                                      // half plane's lane pairs), 6 the deterministic lane pairs (lanes[1]), 7 the
                                       // half plane's stencil
     int group_count = 0;              // G of group_lanes / group_chunks (0: not built)
     std::vector<purify::LaneWork> group_lanes;
     std::vector<purify::GroupChunks> group_chunks;
     int grid_kind = 1;                // G^H: 1 tile subproblems, 2 run sets, 3..5 lanes, 6 deterministic
     int degrid_kind = 1;              // G: 1 tile subproblems, 3..5 lanes, 8 sorted (half plane)
-    int fft_rb = 0, fft_cb = 0;       // FFT rows / columns per block (0: heuristic)
-    int fft_cw = 0;                   // FFT columns per thread, 1 or 2 (0: 2 where the shape allows)
+    purify::FftShape fft, fft_half;   // of the whole plane's passes and of the half plane's
     // workspaces
     purify::DevBuf grid;              // Ky * Kx complex (forward transform output)
     purify::DevBuf gacc;              // Ky * Kx complex gridding output, then a 256-byte work counter
@@ -346,10 +352,12 @@ void launch_phi_adj(purify_plan* p, const void* y, void* out, bool caller_order,
 void launch_fft2(purify_plan* p, void* grid, bool inverse);
 // Phi stages used by the solver's fused forms; half: on the half-plane grid
 // (a real image in, or the real part out: out_mode 1)
-// zero_acc: the same launch clears the gridding accumulator (gacc); fold:
-// apply the pending CG update first (see CgFold)
+// clear: the same launch clears the gridding accumulator (gacc), of the whole
+// or of the half plane; fold: apply the pending CG update first (see CgFold)
+enum ClearAcc { CLEAR_NONE, CLEAR_WHOLE, CLEAR_HALF };
+inline ClearAcc clear_acc(bool half) { return half ? CLEAR_HALF : CLEAR_WHOLE; }
 void launch_scale_pad_rows(purify_plan* p, const void* x, double scale, const int* skip_flag, bool corr = true,
-                           bool zero_acc = false, const CgFold* fold = nullptr, bool half = false);
+                           ClearAcc clear = CLEAR_NONE, const CgFold* fold = nullptr, bool half = false);
 void launch_cols_fwd(purify_plan* p, const int* skip_flag, bool half = false);
 void launch_degrid(purify_plan* p, void* y, bool caller_order, const int* skip_flag, bool half = false);
 void launch_grid(purify_plan* p, const void* y, bool caller_order, const int* skip_flag, bool zeroed = false,
@@ -423,8 +431,6 @@ bool timing_enabled(const purify_plan* p);
 void reweight(purify_plan* p, const void* x, double rho, void* w);
 double coef_std(purify_plan* p, const void* x);
 
-// the normal operator runs on the half plane (its lane form is FP32 only)
-inline bool normal_half(const purify_plan* p) { return p->half_on && (p->stencil.on || p->dtype == PURIFY_F32); }
 // G^H G as a stencil (stencil.cu): bytes of the coefficients; the build from
 // the half-plane lane work (cells: the runs' first-tap cells, row * W +
 // column), false where the device has no room for it; the application, which

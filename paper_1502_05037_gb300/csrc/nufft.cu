@@ -1452,15 +1452,15 @@ void launch_grid(purify_plan* p, const void* y, bool caller_order, const int* sk
 }
 
 void launch_phi(purify_plan* p, const void* x, void* y, bool caller_order, double scale, bool zero_acc) {
-    const bool half = p->half_on;
-    launch_scale_pad_rows(p, x, scale, nullptr, true, zero_acc, nullptr, half);
+    const bool half = p->phi_half;
+    launch_scale_pad_rows(p, x, scale, nullptr, true, zero_acc ? clear_acc(p->adj_half) : CLEAR_NONE, nullptr, half);
     launch_cols_fwd(p, nullptr, half);
     launch_degrid(p, y, caller_order, nullptr, half);
 }
 
 void launch_phi_adj(purify_plan* p, const void* y, void* out, bool caller_order, double scale, int out_mode,
                     const void* add, bool acc_zeroed) {
-    const bool half = p->half_on && out_mode == 1;
+    const bool half = p->adj_half && out_mode == 1;
     launch_grid(p, y, caller_order, nullptr, acc_zeroed, half);
     launch_cols_inv(p, nullptr, nullptr, half);
     launch_rows_inv_crop(p, out, scale, out_mode, add, 1.0, nullptr, nullptr, true, half);

@@ -192,94 +192,133 @@ void build_gridlist(purify_plan* p, const std::vector<int>& bins, const std::vec
 }
 
 // ---------------------------------------------------------------- autotuner
-// Launch shapes picked by timing on the plan's own data: the tile and the
-// subproblem size of gridding and of degridding (work lists rebuilt from the
-// same cell order) and the rows/columns per block of the FFT passes. Results
-// are cached per problem shape.
+// Launch shapes and decompositions picked by timing on the plan's own data: the
+// rows/columns per block of the FFT passes, the tile and the subproblem size of
+// gridding and of degridding (work lists rebuilt from the same cell order), the
+// form of gridding, and on small images whether Phi, the solver's adjoint and
+// the normal operator run on the half plane or on the whole one. Results are
+// cached per problem shape.
 struct TuneKey {
     int nx, ny, J, dtype, mlog, R, gm;
     bool operator<(const TuneKey& o) const {
         return std::tie(nx, ny, J, dtype, mlog, R, gm) < std::tie(o.nx, o.ny, o.J, o.dtype, o.mlog, o.R, o.gm);
     }
 };
-struct TuneVal { int tile, dtile, rb, cb, cw, units, dunits, gkind; };
+struct TuneVal {
+    int tile, dtile, units, dunits, gkind, dkind, nkind;
+    FftShape fft, fft_half;
+    bool phi_half, adj_half, normal_half;
+};
 // below this many visibilities gridding is not tuned (tile subproblems)
 static const int64_t kTuneMinM = 32768;
+// Up to this many pixels the half plane is timed against the whole. Its row
+// passes make half as many transforms and half as much of everything that
+// follows, but a thread of theirs works on two image rows and takes its pair
+// apart, or puts it together, through shared memory: about half a microsecond
+// more a pass at 32 x 32 to 256 x 256, where a pass is its latency; and few
+// visibilities cost less than the stencil. us of the normal operator on the half
+// plane and on the whole (FP32, J = 6): 64 x 64 with 2001 visibilities 15.2 and
+// 11.8, with 30 001 15.0 and 16.4; 128 x 128 with 33 001 15.5 and 14.5, with 100 001
+// 15.4 and 17.6; 256 x 256 with 33 001 17.8 and 16.4, with 655 361 21.5 and 33.0. At
+// 512 x 512 the half plane is faster at every density measured (100 001: 29.2 and
+// 36.2), so larger images are not timed.
+static const int64_t kTimeHalfN = 1 << 17;
 static std::mutex g_tune_mutex;
 static std::map<TuneKey, TuneVal> g_tune_cache;
+
+static TuneKey tune_key(const purify_plan* p) {
+    int mlog = 0;
+    while ((int64_t(1) << (mlog + 1)) <= p->M) ++mlog;
+    return TuneKey{p->nx, p->ny, p->J, p->dtype, mlog, std::min(p->R, 64), p->desc.grid_mode};
+}
+static bool tune_cached(const purify_plan* p, TuneVal& val) {
+    if (p->desc.tile != 0) return false;
+    std::lock_guard<std::mutex> lk(g_tune_mutex);
+    auto it = g_tune_cache.find(tune_key(p));
+    if (it == g_tune_cache.end()) return false;
+    val = it->second;
+    return true;
+}
 
 // Mean device time of one call of f, which launches work on p->stream: the
 // calls are captured `reps` times into a CUDA graph on a private stream (so
 // host launch overhead does not count), and the best of three graph launches
 // after an untimed one is taken (the minimum discards runs disturbed by clock
 // ramps or other work on the device).
-static float time_ms(purify_plan* p, const std::function<void()>& f, int reps) {
-    cudaStream_t user = p->stream, ts = nullptr;
+struct TuneTimer {
+    purify_plan* p;
+    cudaStream_t user, ts = nullptr;
     cudaEvent_t a = nullptr, b = nullptr;
-    cudaGraph_t g = nullptr;
-    cudaGraphExec_t ge = nullptr;
-    float best = 1e30f;
-    auto cleanup = [&] {
+    explicit TuneTimer(purify_plan* plan) : p(plan), user(plan->stream) {}
+    ~TuneTimer() {
         p->stream = user;
-        if (ge) cudaGraphExecDestroy(ge);
-        if (g) cudaGraphDestroy(g);
         if (a) cudaEventDestroy(a);
         if (b) cudaEventDestroy(b);
         if (ts) cudaStreamDestroy(ts);
-    };
-    try {
-        PURIFY_CUDA(cudaStreamCreateWithFlags(&ts, cudaStreamNonBlocking));
-        PURIFY_CUDA(cudaEventCreate(&a));
-        PURIFY_CUDA(cudaEventCreate(&b));
-        PURIFY_CUDA(cudaDeviceSynchronize());
-        p->stream = ts;
-        f();  // outside the capture: sets kernel attributes
-        PURIFY_CUDA(cudaStreamBeginCapture(ts, cudaStreamCaptureModeThreadLocal));
+    }
+    float operator()(const std::function<void()>& f, int reps) {
+        if (!ts) {
+            PURIFY_CUDA(cudaStreamCreateWithFlags(&ts, cudaStreamNonBlocking));
+            PURIFY_CUDA(cudaEventCreate(&a));
+            PURIFY_CUDA(cudaEventCreate(&b));
+        }
+        cudaGraph_t g = nullptr;
+        cudaGraphExec_t ge = nullptr;
+        float best = 1e30f;
+        auto cleanup = [&] {
+            p->stream = user;
+            if (ge) cudaGraphExecDestroy(ge);
+            if (g) cudaGraphDestroy(g);
+        };
         try {
-            for (int i = 0; i < reps; ++i) f();
+            PURIFY_CUDA(cudaDeviceSynchronize());   // uploads of the work that is timed
+            p->stream = ts;
+            f();  // outside the capture: sets kernel attributes
+            PURIFY_CUDA(cudaStreamBeginCapture(ts, cudaStreamCaptureModeThreadLocal));
+            try {
+                for (int i = 0; i < reps; ++i) f();
+            } catch (...) {
+                cudaStreamEndCapture(ts, &g);
+                throw;
+            }
+            PURIFY_CUDA(cudaStreamEndCapture(ts, &g));
+            PURIFY_CUDA(cudaGraphInstantiate(&ge, g, 0));
+            PURIFY_CUDA(cudaGraphLaunch(ge, ts));
+            for (int trial = 0; trial < 3; ++trial) {
+                PURIFY_CUDA(cudaEventRecord(a, ts));
+                PURIFY_CUDA(cudaGraphLaunch(ge, ts));
+                PURIFY_CUDA(cudaEventRecord(b, ts));
+                PURIFY_CUDA(cudaEventSynchronize(b));
+                float ms = 0.f;
+                PURIFY_CUDA(cudaEventElapsedTime(&ms, a, b));
+                best = std::min(best, ms / reps);
+            }
         } catch (...) {
-            cudaStreamEndCapture(ts, &g);
+            cleanup();
             throw;
         }
-        PURIFY_CUDA(cudaStreamEndCapture(ts, &g));
-        PURIFY_CUDA(cudaGraphInstantiate(&ge, g, 0));
-        PURIFY_CUDA(cudaGraphLaunch(ge, ts));
-        for (int trial = 0; trial < 3; ++trial) {
-            PURIFY_CUDA(cudaEventRecord(a, ts));
-            PURIFY_CUDA(cudaGraphLaunch(ge, ts));
-            PURIFY_CUDA(cudaEventRecord(b, ts));
-            PURIFY_CUDA(cudaEventSynchronize(b));
-            float ms = 0.f;
-            PURIFY_CUDA(cudaEventElapsedTime(&ms, a, b));
-            best = std::min(best, ms / reps);
-        }
-    } catch (...) {
         cleanup();
-        throw;
+        return best;
     }
-    cleanup();
-    return best;
-}
+};
 
+// `known`: val holds the shape's cached choices
 template <typename T, typename BinsFor>
 static void autotune(purify_plan* p, const std::vector<int>& cand, BinsFor bins_for,
-                     const std::vector<int>& cell_order, bool tune) {
+                     const std::vector<int>& cell_order, bool known, TuneVal val) {
     using C = typename cplx_of<T>::type;
-    int mlog = 0;
-    while ((int64_t(1) << (mlog + 1)) <= p->M) ++mlog;
-    TuneKey key{p->nx, p->ny, p->J, p->dtype, mlog, std::min(p->R, 64), p->desc.grid_mode};
-    // default subproblem size: about four subproblems per SM's worth of
-    // visibilities, in batch units
-    const int64_t unit = grid_list_unit(p->dtype, p->J);
-    const int u0 = (int)std::max<int64_t>(1, std::min<int64_t>(16, (p->M / (152 * 4) + unit / 2) / unit));
-    TuneVal val{p->work.tile, p->work.tile, 0, 0, 0, u0, u0, 1};
-    bool cached = false;
-    if (tune) {
-        std::lock_guard<std::mutex> lk(g_tune_mutex);
-        auto it = g_tune_cache.find(key);
-        if (it != g_tune_cache.end()) { val = it->second; cached = true; }
+    // the half plane's work is built (grid_mode 0), and FP64 has its normal
+    // operator there only as a stencil
+    const bool half = p->half_lanes.nsets > 0;
+    auto can_normal_half = [&] { return half && (p->stencil.on || p->dtype == PURIFY_F32); };
+    if (!known) {
+        // default subproblem size: about four subproblems per SM's worth of
+        // visibilities, in batch units
+        const int64_t unit = grid_list_unit(p->dtype, p->J);
+        const int u0 = (int)std::max<int64_t>(1, std::min<int64_t>(16, (p->M / (152 * 4) + unit / 2) / unit));
+        val = TuneVal{p->work.tile, p->work.tile, u0, u0, 1, 1, 2, {}, {}, half, half, half};
     }
-    if (tune && !cached) {
+    if (!known && p->desc.tile == 0) {
         // deterministic test data in the workspaces
         std::vector<T> img(2 * (size_t)p->N), vis(2 * (size_t)p->M);
         uint64_t st = 12345;
@@ -289,77 +328,143 @@ static void autotune(purify_plan* p, const std::vector<int>& cand, BinsFor bins_
         PURIFY_CUDA(cudaMemcpy(p->tmp_img.p, img.data(), sizeof(T) * img.size(), cudaMemcpyHostToDevice));
         PURIFY_CUDA(cudaMemcpy(p->tmp_vis.p, vis.data(), sizeof(T) * vis.size(), cudaMemcpyHostToDevice));
         T* ximg = p->tmp_img.as<T>();
+        T* xout = ximg + p->N;
         C* yv = p->tmp_vis.as<C>();
+        TuneTimer time_ms(p);
         // bring the clocks up before the first candidate is timed
         for (int i = 0; i < 40; ++i) launch_cols_fwd(p, nullptr);
         PURIFY_CUDA(cudaStreamSynchronize(p->stream));
-        // FFT launch shapes, on the half-plane passes where the plan has them
-        const bool half = p->half_on;
-        float best = 1e30f;
-        for (int rb = 1; rb <= 8; rb *= 2) {
-            if ((half ? p->ny / 2 : p->ny) % rb || !fft_shape_ok(rb, p->Kx, p->dtype)) continue;
-            p->fft_rb = rb;
-            float ms = time_ms(p, [&] { launch_scale_pad_rows(p, ximg, 1.0, nullptr, true, false, nullptr, half); }, 10);
-            if (ms < best) { best = ms; val.rb = rb; }
-        }
-        best = 1e30f;
-        // columns per block, and one or two (packed FP32) columns per thread
-        for (int cb = 1; cb <= 8; cb *= 2) {
-            for (int cw = 1; cw <= 2; ++cw) {
-                if (p->Kx % cb || !fft_shape_ok(cb, p->Ky, p->dtype, cw)) continue;
-                p->fft_cb = cb;
-                p->fft_cw = cw;
-                float ms = time_ms(p, [&] { launch_cols_fwd(p, nullptr, half); }, 10);
-                if (ms < best) { best = ms; val.cb = cb; val.cw = cw; }
+        // the whole plane's Phi and normal operator come into question (in
+        // FP64, whose passes cost far more than a launch, they do not: every
+        // size was faster on the half plane)
+        const bool both = half && sizeof(T) == 4 && p->N <= kTimeHalfN, whole = both || !half;
+        // FFT launch shapes: rows (or row pairs) per block; columns per block,
+        // and one or two (packed FP32) columns per thread
+        auto tune_rows = [&](bool hp, FftShape& shape) {
+            float best = 1e30f;
+            int best_rb = 0;
+            for (int rb = 1; rb <= 8; rb *= 2) {
+                if ((hp ? p->ny / 2 : p->ny) % rb || !fft_shape_ok(rb, p->Kx, p->dtype)) continue;
+                shape.rb = rb;
+                float ms = time_ms([&] {
+                    launch_scale_pad_rows(p, ximg, 1.0, nullptr, true, CLEAR_NONE, nullptr, hp);
+                    launch_rows_inv_crop(p, xout, 1.0, 1, nullptr, 0.0, nullptr, nullptr, true, hp);
+                }, 6);
+                if (ms < best) { best = ms; best_rb = rb; }
             }
+            shape.rb = best_rb;
+        };
+        auto tune_cols = [&](bool hp, FftShape& shape) {
+            float best = 1e30f;
+            FftShape best_cols = shape;
+            for (int cb = 1; cb <= 8; cb *= 2) {
+                for (int cw = 1; cw <= 2; ++cw) {
+                    if (p->Kx % cb || !fft_shape_ok(cb, p->Ky, p->dtype, cw)) continue;
+                    shape.cb = cb;
+                    shape.cw = cw;
+                    float ms = time_ms([&] { launch_cols_fwd(p, nullptr, hp); }, 10);
+                    if (ms < best) { best = ms; best_cols = shape; }
+                }
+            }
+            shape = best_cols;
+        };
+        if (half) {
+            tune_rows(true, p->fft_half);
+            tune_cols(true, p->fft_half);
         }
-        p->fft_rb = val.rb;
-        p->fft_cb = val.cb;
-        p->fft_cw = val.cw;
-        // gridding and degridding tiles, each timed on its own kernel (with
-        // the half-plane path only the adjoint's complex image grids on the
-        // whole plane: G^H alone)
+        tune_rows(false, p->fft);
+        if (whole) {
+            tune_cols(false, p->fft);
+        } else {   // (the adjoint's complex image alone)
+            p->fft.cb = p->fft_half.cb;
+            p->fft.cw = p->fft_half.cw;
+        }
+        val.fft = p->fft;
+        val.fft_half = p->fft_half;
+        // gridding and degridding tiles, each timed on its own kernel
         if (cand.size() > 1 && p->M >= kTuneMinM) {
-            float bg = 1e30f, bd = 1e30f;
+            float bg = 1e30f, bd = 1e30f, bn = 1e30f;
             for (int t : cand) {
                 const std::vector<int> bins = bins_for(t);
                 for (int u : {1, 2, 4, 8}) {
                     build_gridlist(p, bins, cell_order, t, u, p->work);
-                    float mg = time_ms(p, [&] { launch_grid(p, yv, false, nullptr); }, 5);
+                    float mg = time_ms([&] { launch_grid(p, yv, false, nullptr); }, 5);
                     if (mg < bg) { bg = mg; val.tile = t; val.units = u; }
-                    if (half) continue;
+                    if (!whole) continue;
                     build_gridlist(p, bins, cell_order, t, u, p->dwork);
-                    float md = time_ms(p, [&] { launch_degrid(p, yv, false, nullptr); }, 5);
+                    float md = time_ms([&] { launch_degrid(p, yv, false, nullptr); }, 5);
                     if (md < bd) { bd = md; val.dtile = t; val.dunits = u; }
                 }
             }
-            // gridding by run sets and by lanes (one pool, or by tiles)
+            // G^H, G and G^H G by run sets and by lanes (one pool, or by tiles)
             if (p->desc.grid_mode == 0) {
-                const float mr = time_ms(p, [&] { launch_grid_sets(p, yv, false, nullptr); }, 5);
+                const float mr = time_ms([&] { launch_grid_sets(p, yv, false, nullptr); }, 5);
                 if (mr < bg) { bg = mr; val.gkind = 2; }
+                if (whole) bn = time_ms([&] { launch_normal_lanes(p, 2, nullptr); }, 5);
                 if (lane_work_ok(p) && p->lanes[0].nsets > 0) {
                     for (int kind = 3; kind <= 5; ++kind) {
-                        const float ml = time_ms(p, [&] { launch_grid_lanes(p, kind, yv, false, nullptr); }, 5);
+                        const float ml = time_ms([&] { launch_grid_lanes(p, kind, yv, false, nullptr); }, 5);
                         if (ml < bg) { bg = ml; val.gkind = kind; }
+                        if (!whole) continue;
+                        const float mn = time_ms([&] { launch_normal_lanes(p, kind, nullptr); }, 5);
+                        const float md = time_ms([&] { launch_degrid_lanes(p, kind, yv, false, nullptr); }, 5);
+                        if (mn < bn) { bn = mn; val.nkind = kind; }
+                        if (md < bd) { bd = md; val.dkind = kind; }
                     }
                 }
             }
         }
+        // Phi, the solver's adjoint and the normal operator, each whole call
+        // on the half plane and on the whole
+        if (both) {
+            build_gridlist(p, bins_for(val.tile), cell_order, val.tile, val.units, p->work);
+            build_gridlist(p, bins_for(val.dtile), cell_order, val.dtile, val.dunits, p->dwork);
+            p->grid_kind = val.gkind;
+            p->degrid_kind = val.dkind;
+            p->normal_kind = val.nkind;
+            // (a CG step's row passes also update its vectors, for which the
+            // half plane's have half the threads: its normal operator has to
+            // win by 5% here)
+            auto half_faster = [&](float margin, auto&& f) {
+                const float h = time_ms([&] { f(true); }, 5), w = time_ms([&] { f(false); }, 5);
+                return h <= margin * w;
+            };
+            val.phi_half = half_faster(1.0f, [&](bool hp) {
+                launch_scale_pad_rows(p, ximg, 1.0, nullptr, true, CLEAR_NONE, nullptr, hp);
+                launch_cols_fwd(p, nullptr, hp);
+                launch_degrid(p, yv, false, nullptr, hp);
+            });
+            val.adj_half = half_faster(1.0f, [&](bool hp) {
+                launch_grid(p, yv, false, nullptr, false, hp);
+                launch_cols_inv(p, nullptr, nullptr, hp);
+                launch_rows_inv_crop(p, xout, 1.0, 1, nullptr, 0.0, nullptr, nullptr, true, hp);
+            });
+            val.normal_half = can_normal_half() && half_faster(0.95f, [&](bool hp) {
+                launch_scale_pad_rows(p, ximg, 1.0, nullptr, true, clear_acc(hp), nullptr, hp);
+                launch_cols_fwd(p, nullptr, hp);
+                launch_normal_gg(p, nullptr, true, hp);
+                launch_cols_inv(p, nullptr, nullptr, hp);
+                launch_rows_inv_crop(p, xout, 1.0, 1, nullptr, 0.0, nullptr, nullptr, true, hp);
+            });
+        }
         std::lock_guard<std::mutex> lk(g_tune_mutex);
-        g_tune_cache[key] = val;
+        g_tune_cache[tune_key(p)] = val;
     }
-    p->fft_rb = val.rb;
-    p->fft_cb = val.cb;
-    p->fft_cw = val.cw;
+    p->fft = val.fft;
+    p->fft_half = val.fft_half;
     // a forced decomposition: grid_mode 1 and 2 degrid by tiles and apply
     // G^H G by run sets, 3..5 do all three by that lane form, 6 grids by
     // the deterministic lane pairs and degrids by the lane pairs
     const int gm = p->desc.grid_mode;
+    p->phi_half = half && val.phi_half;
+    p->adj_half = half && val.adj_half;
+    p->normal_half = val.normal_half && can_normal_half();
     p->grid_kind = gm == 0 ? val.gkind : gm;
-    p->degrid_kind = gm == 0 ? 8 : (gm == 6 ? 4 : (gm >= 3 ? gm : 1));
-    p->normal_kind = gm == 0 ? (p->stencil.on ? 7 : normal_half(p) ? 4 : 2) : (gm >= 3 ? gm : 2);
+    p->degrid_kind = gm == 0 ? (p->phi_half ? 8 : val.dkind) : (gm == 6 ? 4 : (gm >= 3 ? gm : 1));
+    p->normal_kind = gm == 0 ? (!p->normal_half ? val.nkind : p->stencil.on ? 7 : 4) : (gm >= 3 ? gm : 2);
     build_gridlist(p, bins_for(val.tile), cell_order, val.tile, val.units, p->work);
-    if (!p->half_on) build_gridlist(p, bins_for(val.dtile), cell_order, val.dtile, val.dunits, p->dwork);
+    if (!p->phi_half) build_gridlist(p, bins_for(val.dtile), cell_order, val.dtile, val.dunits, p->dwork);
+    else p->dwork = GridWork();
 }
 
 // Lane-per-run work (see LaneWork) from the length-sorted runs: `width`
@@ -496,9 +601,11 @@ static bool use_stencil(const purify_plan* p, size_t nruns) {
 // where their first-tap column is in the upper half, in runs of one cell,
 // runs sorted by length (longest first, then by cell). A lane per run where
 // its patch fits the registers (FP32, J <= 6; see half_lane), else a lane pair.
+// normal: also the normal operator's form.
 template <typename T>
 static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std::vector<T>& vs,
-                             const std::vector<int>& scx, const std::vector<int>& scy, const std::vector<int>& perm) {
+                             const std::vector<int>& scx, const std::vector<int>& scy, const std::vector<int>& perm,
+                             bool normal) {
     const int64_t M = p->M;
     const int J = p->J, Kx = p->Kx, Ky = p->Ky, W = p->half.W, off = p->half.off;
     const int width = sizeof(T) == 4 && J <= kLaneMaxJ ? 32 : 16;
@@ -508,7 +615,12 @@ static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std
             cell[m] = scx[m] < Kx / 2 ? scy[m] * W + scx[m] + off
                                       : ((Ky - scy[m] - J + 1) & (Ky - 1)) * W + Kx - scx[m] - J + 1 + off;
     });
-    {
+    if (M * 32 < (int64_t)Ky * W) {
+        // few visibilities: a sort of them costs less than counters of all cells
+        // (4096 of them, 4096 x 4096: 73 ms a plan with the counters, 56 without)
+        for (int64_t m = 0; m < M; ++m) order[m] = (int)m;
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cell[a] < cell[b]; });
+    } else {
         std::vector<int> pos((size_t)Ky * W + 1, 0);
         for (int64_t m = 0; m < M; ++m) pos[cell[m] + 1]++;
         for (size_t c = 1; c < pos.size(); ++c) pos[c] += pos[c - 1];
@@ -621,18 +733,14 @@ static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std
     upload(sw.cell, sc);
     upload(sw.idx, si);
     upload(sw.idx_caller, sk);
-    p->workspace_bytes += (int64_t)(sw.z.bytes + sw.cell.bytes + sw.idx.bytes + sw.idx_caller.bytes);
     // the normal operator as a stencil, where that is the faster form and fits
+    if (!normal) return;
     if (use_stencil(p, nr)) {
         std::vector<int> cells(nr);
         for (size_t q = 0; q < nr; ++q) cells[q] = cell[order[sorted[q].first]];
         build_stencil(p, cells);
     }
-    if (p->stencil.on) {
-        p->workspace_bytes += (int64_t)(p->stencil.coef.bytes + p->stencil.used.bytes);
-    } else if (sizeof(T) == 4 && width == 32) {
-        fill(p->half_pairs, 16, false);
-    }
+    if (!p->stencil.on && sizeof(T) == 4 && width == 32) fill(p->half_pairs, 16, false);
 }
 
 // Run-ordered work (see RunWork): runs of equal first-tap cell in the cell
@@ -879,17 +987,32 @@ template <typename T> static void finish_plan(purify_plan* p) {
         for (int64_t i = 0; i < p->M; ++i) cell_order[pos[(int64_t)scy[i] * p->Kx + scx[i]]++] = (int)i;
     }
     build_runwork<T>(p, us, vs, scx, scy, cell_order, perm);
-    if (p->half_on) build_half_lanes<T>(p, us, vs, scx, scy, perm);
-    autotune<T>(p, cand, bins_for, cell_order, d.tile == 0);
-    // keep only the lane work in use (kind 6 runs on the lane pairs of kind 4)
+    // autotuned plans take the half-plane path (unless it is known to be the
+    // slower one for their shape); a forced decomposition runs on the whole plane
+    TuneVal val{};
+    const bool known = tune_cached(p, val);
+    if (d.grid_mode == 0 && (!known || val.phi_half || val.adj_half || val.normal_half))
+        build_half_lanes<T>(p, us, vs, scx, scy, perm, !known || val.normal_half);
+    autotune<T>(p, cand, bins_for, cell_order, known, val);
+    // keep only the work in use (kind 6 runs on the lane pairs of kind 4)
     auto uses = [&](int k) {
         auto is = [&](int kind) { return kind == k || (k == 4 && kind == 6); };
-        return is(p->grid_kind) || (!p->half_on && (is(p->degrid_kind) || is(p->normal_kind)));
+        return is(p->grid_kind) || (!p->phi_half && is(p->degrid_kind)) || (!p->normal_half && is(p->normal_kind));
     };
     for (int k = 3; k <= 5; ++k)
         if (!uses(k)) p->lanes[k - 3].release();
+    if (!p->normal_half) {
+        p->stencil = Stencil();
+        p->half_pairs.release();
+    }
+    // (without pairs of their own the normal operator's lanes are half_lanes)
+    if (!p->adj_half && !(p->normal_half && !p->stencil.on && p->half_pairs.nsets == 0)) p->half_lanes.release();
+    if (!p->phi_half) p->half_sorted = SortedWork();
     for (int k = 0; k < 3; ++k) p->workspace_bytes += lane_bytes(p->lanes[k]);
     p->workspace_bytes += lane_bytes(p->half_lanes) + lane_bytes(p->half_pairs);
+    const SortedWork& sw = p->half_sorted;
+    p->workspace_bytes += (int64_t)(sw.z.bytes + sw.cell.bytes + sw.idx.bytes + sw.idx_caller.bytes);
+    p->workspace_bytes += (int64_t)(p->stencil.coef.bytes + p->stencil.used.bytes);
     p->workspace_bytes += (int64_t)p->det_patch.bytes;
 }
 
@@ -955,10 +1078,7 @@ purify_plan* create_plan(const purify_plan_desc* d) {
         p->ax = AxisConst{(int)Kx, (float)cx, (float)(cx - (double)(float)cx), cx};
         p->ay = AxisConst{(int)Ky, (float)cy, (float)(cy - (double)(float)cy), cy};
         p->kbp = fit_kb_poly(p->J, p->beta, kb_poly_degree(p->J));
-        // autotuned plans take the half-plane path; a forced decomposition runs
-        // on the whole plane
-        if (d->grid_mode == 0) {
-            p->half_on = true;
+        if (d->grid_mode == 0) {   // (see finish_plan)
             p->half.off = p->J - 2;
             p->half.W0 = p->Kx / 2 + 2 * p->J - 3;
             p->half.W = (p->half.W0 + 8 + 15) / 16 * 16;

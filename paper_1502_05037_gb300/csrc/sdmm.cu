@@ -672,7 +672,7 @@ template <typename T> struct Solver {
                 // r = G Re Phi_g^H v2 / nu
                 const LaneWork& lw = p->group_lanes[group];
                 const GroupChunks* gc = &p->group_chunks[group];
-                launch_scale_pad_rows(p, x, inv_nu, nullptr, true, true);
+                launch_scale_pad_rows(p, x, inv_nu, nullptr, true, CLEAR_WHOLE);
                 launch_cols_fwd(p, nullptr);
                 launch_lanes_on(p, lw, 2, nullptr, s.v2.p, false, nullptr, true);
                 proj_norms(true, gc);
@@ -753,15 +753,15 @@ template <typename T> struct Solver {
             fold.step = k;
             if (s.toeplitz) {
                 // u = A r = 2 r + (embedded normal operator) r
-                launch_scale_pad_rows(p, nullptr, 1.0, skip, false, false, &fold);
+                launch_scale_pad_rows(p, nullptr, 1.0, skip, false, CLEAR_NONE, &fold);
                 launch_cols_fwd(p, skip);
                 launch_cols_inv(p, skip, s.toep.p);
                 launch_rows_inv_crop(p, s.u.p, 1.0, 1, s.r.p, 2.0, skip, &fold, false);
             } else {
                 // the pending update and the transform of the new r fused into
                 // the first FFT pass, then u = A r
-                const bool half = group < 0 && normal_half(p);
-                launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, true, &fold, half);
+                const bool half = group < 0 && p->normal_half;
+                launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, clear_acc(half), &fold, half);
                 launch_cols_fwd(p, skip, half);
                 if (group >= 0) launch_lanes_on(p, p->group_lanes[group], 0, nullptr, nullptr, false, skip, true);
                 else launch_normal_gg(p, skip, true, half);
@@ -795,8 +795,8 @@ template <typename T> struct Solver {
         const int* skip = flags() + F_CGDONE;
         CgFold fold = make_fold();
         fold.step = k;
-        const bool half = normal_half(p);
-        launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, true, &fold, half);
+        const bool half = p->normal_half;
+        launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, clear_acc(half), &fold, half);
         launch_cols_fwd(p, skip, half);
         launch_normal_gg(p, skip, true, half);
         launch_cols_inv(p, skip, nullptr, half);
@@ -851,8 +851,8 @@ template <typename T> static void pd_iteration(Solver<T>& S, double tau, double 
                              S.scal(), p->R, 2);
             L.done();
         }
-        launch_grid(p, s.v2.p, false, nullptr, true, p->half_on);
-        launch_cols_inv(p, nullptr, nullptr, p->half_on);
+        launch_grid(p, s.v2.p, false, nullptr, true, p->adj_half);
+        launch_cols_inv(p, nullptr, nullptr, p->adj_half);
         if (fork) PURIFY_CUDA(cudaEventRecord(s.ev_join, s.side));
     } catch (...) {
         p->stream = main_stream;
@@ -869,7 +869,7 @@ template <typename T> static void pd_iteration(Solver<T>& S, double tau, double 
     launch_psi(p, s.z1.p, s.p.p);
     if (fork) PURIFY_CUDA(cudaStreamWaitEvent(p->stream, s.ev_join, 0));
     // g = Psi p1 + Re Phi^H (sigma z) / nu
-    launch_rows_inv_crop(p, s.u.p, sigma * inv_nu, 1, s.p.p, 1.0, nullptr, nullptr, true, p->half_on);
+    launch_rows_inv_crop(p, s.u.p, sigma * inv_nu, 1, s.p.p, 1.0, nullptr, nullptr, true, p->adj_half);
     {
         Launch L(p, "pd_primal");
         launch_dependent(k_pd_primal<T>, ew_blocks(p->N), 256, 0, p->stream, x, s.u.template as<T>(), xbar,

@@ -516,47 +516,42 @@ k_grid_sets(const typename cplx_of<T>::type* __restrict__ yin, const typename cp
 // it is read or written.
 enum { LANE_GG = 0, LANE_GRID = 1, LANE_DEGRID = 2 };
 
-// Shared staging of the lane kernels, per warp and buffer [run][row][GW]
-// cells. A lane copies its rows of the next run's grid patch there cell by
-// cell. G^H adds the accumulated patches of a set to the grid from there, a row
-// at a time by GL neighbouring lanes in 16-byte accesses (the row's cells from
-// the even column at or below its first one: GW cells), 32 / GL rows per
-// instruction: a lane adding its own rows touches a cache line per lane and
-// access (512 x 512 channel, 786 433 visibilities, J = 6: 37.5 -> 34.5 us). In
-// G^H G, which has no registers to spare, both that and copying the patches
-// in the same way cost more than they gave (34 -> 35 and 37 us). The stride RS
-// of a run keeps 16-byte alignment and spreads the runs over the banks.
+// Shared staging of the lane kernels. G^H G and G: per warp two buffers (current
+// and next set) of each lane's RH x J patch of X, copied cell by cell, lane
+// stride LS complex values (odd, so that the 8-byte accesses of a half-warp fall
+// on distinct banks). G^H with a common flush (COOP): one buffer [run][row][GW]
+// per warp; the accumulated patches of a set are added to the grid from there, a
+// row at a time by GL neighbouring lanes in 16-byte accesses (the row's cells
+// from the even column at or below its first one: GW cells), 32 / GL rows per
+// instruction; without it each lane adds its own rows, a cache line per lane and
+// access (lane_coop says where which is taken). The stride RS of a run keeps
+// 16-byte alignment and spreads the runs over the banks.
 template <typename T, int J, int H> struct LaneStage {
     static constexpr int WID = 32 / H;                     // runs per set
     static constexpr int RH = (J + H - 1) / H;             // patch rows per lane
+    static constexpr int LS = (RH * J) | 1;
     static constexpr int CV = 16 / sizeof(typename cplx_of<T>::type);   // cells per 16-byte access
     static constexpr int GL = CV == 2 ? (J + 2) / 2 : J;   // lanes per row
     static constexpr int GW = CV * GL;
     static constexpr int RS = CV == 2 ? (J * GW + 13) / 16 * 16 + 2 : (J * GW) | 1;
     static constexpr int IPI = 32 / GL;                    // rows per instruction
     static constexpr int NIT = (WID * J + IPI - 1) / IPI;
-    static constexpr size_t buffer_bytes = (size_t)WID * RS * sizeof(typename cplx_of<T>::type);
-    // buffers of a mode: two where patches are read ahead, one to add them back
-    static constexpr int buffers(int mode, bool det) { return mode != 1 ? 2 : (det ? 0 : 1); }
-    static constexpr size_t smem(int mode, bool det) { return 4 * buffers(mode, det) * buffer_bytes; }
+    // cells per warp
+    static constexpr int cells(int mode, bool coop) { return mode != 1 ? 2 * 32 * LS : (coop ? WID * RS : 0); }
+    static constexpr size_t smem(int mode, bool coop) {
+        return 4 * sizeof(typename cplx_of<T>::type) * (size_t)cells(mode, coop);
+    }
 };
 
 template <typename C> __device__ __forceinline__ void cp_async_cell(C* sdst, const C* gsrc) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(sdst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(gsrc), "n"(sizeof(C)) : "memory");
 }
-// cells of a 16-byte shared slot (two float cells or one double)
-__device__ __forceinline__ void ld_slot(const float2* s, float2* v) {
-    const float4 q = *reinterpret_cast<const float4*>(s);
-    v[0] = make_float2(q.x, q.y);
-    v[1] = make_float2(q.z, q.w);
-}
-__device__ __forceinline__ void ld_slot(const double2* s, double2* v) { v[0] = *s; }
+// a 16-byte shared slot (two float cells or one double) written, and added to global cells
 __device__ __forceinline__ void st_slot(float2* s, const float2* v) {
     *reinterpret_cast<float4*>(s) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
 }
 __device__ __forceinline__ void st_slot(double2* s, const double2* v) { *s = v[0]; }
-// a 16-byte shared slot added to / written from global cells
 __device__ __forceinline__ void red_slot(float2* p, const float2* s) {
     const float4 q = *reinterpret_cast<const float4*>(s);
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(q.x), "f"(q.y), "f"(q.z), "f"(q.w)
@@ -588,7 +583,9 @@ template <typename T, int J, int MODE, int H, bool DET> constexpr int lane_min_b
 // With DET the accumulators are not added to the grid: run q's J x J patch
 // is stored at out[(b J + a) * dstride + q] (q = set * (32 / H) + its lane
 // in the set), for k_lane_gather to sum in a fixed order.
-template <typename T, int J, int MODE, int H, bool DET = false>
+// HALF: on the half plane, where an index may be a folded one (G^H only; G has
+// none to fold on the whole plane, and its sorted form on the half).
+template <typename T, int J, int MODE, int H, bool DET, bool HALF, bool COOP>
 __global__ void __launch_bounds__(128, lane_min_blocks<T, J, MODE, H, DET>())
 k_lane(const typename cplx_of<T>::type* __restrict__ X, const typename cplx_of<T>::type* __restrict__ yin,
        typename cplx_of<T>::type* __restrict__ yout, const int2* __restrict__ set_info,
@@ -604,9 +601,10 @@ k_lane(const typename cplx_of<T>::type* __restrict__ X, const typename cplx_of<T
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, r = lane % WID, h = lane / WID;
     const int W = gridDim.x * (blockDim.x >> 5), wg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    C* const stage = reinterpret_cast<C*>(smem_raw) +
-                     (size_t)(threadIdx.x >> 5) * Stage::buffers(MODE, DET) * WID * Stage::RS;
-    auto buf = [&](int i) { return stage + (size_t)(Stage::buffers(MODE, DET) > 1 ? (i & 1) : 0) * WID * Stage::RS; };
+    // the warp's flush buffer, or this lane's two staging buffers
+    C* const stage = reinterpret_cast<C*>(smem_raw) + (size_t)(threadIdx.x >> 5) * Stage::cells(MODE, COOP) +
+                     (HAS_X ? lane * Stage::LS : 0);
+    auto buf = [&](int i) { return stage + (size_t)(i & 1) * 32 * Stage::LS; };
     auto set_of = [&](int i) { return i * W + ((i & 1) ? W - 1 - wg : wg); };
     // f(run's cell, run's length, shared slot, grid cell) for this lane's
     // 16-byte part of every patch row of the set whose runs lanes 0 .. WID - 1
@@ -625,19 +623,17 @@ k_lane(const typename cplx_of<T>::type* __restrict__ X, const typename cplx_of<T
             }
         }
     };
-    // this lane's rows of a run's X patch into a staging buffer, at the run's
-    // offset in its windows
+    // this lane's rows of a run's X patch into a staging buffer
     auto patch_async = [&](int2 rcn, C* dst) {
         const int c0 = rcn.x & 0xFFFF, cy = (int)((unsigned)rcn.x >> 16);
         if (rcn.y <= 0) return;
-        dst += r * Stage::RS + c0 % Stage::CV;
 #pragma unroll
         for (int i = 0; i < RH; ++i) {
             const int b = h * RH + i;
             if (b < J) {
                 const C* row = X + (size_t)((cy + b) & (Ky - 1)) * ld;
 #pragma unroll
-                for (int a = 0; a < J; ++a) cp_async_cell(dst + b * Stage::GW + a, row + ((c0 + a) & xm));
+                for (int a = 0; a < J; ++a) cp_async_cell(dst + i * J + a, row + ((c0 + a) & xm));
             }
         }
     };
@@ -694,27 +690,16 @@ k_lane(const typename cplx_of<T>::type* __restrict__ X, const typename cplx_of<T
         C av[HAS_ACC ? RH : 1][HAS_ACC ? J : 1];
         if constexpr (HAS_X) {
             cp_async_wait_all();
-            const C* cur = buf(it) + r * Stage::RS + h * RH * Stage::GW;
-            const bool odd = cx % Stage::CV != 0;
+            const C* cur = buf(it);
 #pragma unroll
             for (int i = 0; i < RH; ++i) {
                 const bool rowok = len > 0 && h * RH + i < J;
-                if (H * RH > J && h * RH + i >= J) {   // no such row (and no such slot)
-#pragma unroll
-                    for (int a = 0; a < J; ++a) xv[i][a] = cmake<C>(T(0), T(0));
-                    continue;
-                }
-                C win[Stage::GW];
-#pragma unroll
-                for (int c = 0; c < Stage::GW; c += Stage::CV) ld_slot(cur + i * Stage::GW + c, &win[c]);
 #pragma unroll
                 for (int a = 0; a < J; ++a) {
-                    const C z = cmake<C>(T(0), T(0));
-                    const C at1 = win[a + 1 < Stage::GW ? a + 1 : a];
-                    xv[i][a] = !rowok ? z : (odd ? at1 : win[a]);
+                    const C v = rowok ? cur[i * J + a] : cmake<C>(T(0), T(0));
+                    xv[i][a] = v;
                 }
             }
-            __syncwarp();   // before the buffer is written again
         }
         if constexpr (HAS_ACC) {
 #pragma unroll
@@ -758,9 +743,11 @@ k_lane(const typename cplx_of<T>::type* __restrict__ X, const typename cplx_of<T
         auto value = [&](int code) -> C {
             C v = cmake<C>(T(0), T(0));
             if (code >= 0) v = yin[code];
-            else if (code < -1) {
-                v = yin[fold_index(code)];
-                v.y = -v.y;
+            if constexpr (HALF) {
+                if (code < -1) {
+                    v = yin[fold_index(code)];
+                    v.y = -v.y;
+                }
             }
             return v;
         };
@@ -825,10 +812,7 @@ k_lane(const typename cplx_of<T>::type* __restrict__ X, const typename cplx_of<T
                 yi = yq[0].y;
             }
             if constexpr (MODE == LANE_DEGRID) {
-                if (valid && h == 0) {
-                    const bool fold = iq[0] < 0;
-                    yout[fold ? fold_index(iq[0]) : iq[0]] = cmake<C>(yr, fold ? -yi : yi);
-                }
+                if (valid && iq[0] >= 0 && h == 0) yout[iq[0]] = cmake<C>(yr, yi);
             }
             if constexpr (HAS_ACC) {
 #pragma unroll
@@ -867,10 +851,10 @@ k_lane(const typename cplx_of<T>::type* __restrict__ X, const typename cplx_of<T
                     }
                 }
             }
-            if constexpr (!DET && MODE == LANE_GRID) {
+            if constexpr (COOP) {
                 // the patch rows to the staging buffer at the run's offset in
                 // its window (the window's other cells zero), then added
-                C* const dst = buf(it) + r * Stage::RS + h * RH * Stage::GW;
+                C* const dst = stage + r * Stage::RS + h * RH * Stage::GW;
                 const bool odd = cx % Stage::CV != 0;
 #pragma unroll
                 for (int i = 0; i < RH; ++i) {
@@ -888,13 +872,13 @@ k_lane(const typename cplx_of<T>::type* __restrict__ X, const typename cplx_of<T
                     }
                 }
                 __syncwarp();
-                patch_rows(rc, buf(it), [&](int off, C* s, size_t g) {
+                patch_rows(rc, stage, [&](int off, C* s, size_t g) {
                     // an even window of an even J ends before its last slot
                     if (J % 2 != 0 || Stage::CV == 1 || off != 0 || part != Stage::GL - 1) red_slot(out + g, s);
                 });
                 __syncwarp();
             }
-            if constexpr (!DET && MODE == LANE_GG) {
+            if constexpr (!DET && !COOP) {
                 if (len > 0) {
 #pragma unroll
                     for (int i = 0; i < RH; ++i) {
@@ -1235,23 +1219,51 @@ static void grid_sets_tj(purify_plan* p, const void* y, bool caller_order, const
 // grid of 4-warp blocks (as many as are resident at once, or fewer when
 // there is less work).
 static const LaneWork& lane_work(const purify_plan* p, int kind) { return p->lanes[kind == 6 ? 1 : kind - 3]; }
-template <typename T, int J, int MODE, int H, bool DET>
-static void lane_launch(purify_plan* p, const LaneWork& lw, const void* yin, void* yout, bool caller_order,
-                        const int* skip, typename cplx_of<T>::type* out, int64_t dstride, bool half) {
+template <typename T, int J, int MODE, int H, bool DET, bool HALF, bool COOP>
+static void lane_launch_as(purify_plan* p, const LaneWork& lw, const void* yin, void* yout, bool caller_order,
+                        const int* skip, typename cplx_of<T>::type* out, int64_t dstride) {
     using C = typename cplx_of<T>::type;
-    const size_t lane_smem = LaneStage<T, J, H>::smem(MODE, DET);
+    const size_t lane_smem = LaneStage<T, J, H>::smem(MODE, COOP);
     static std::atomic<int> occ[64];   // resident blocks per SM of this instantiation, per device
-    const int per_sm = blocks_per_sm(occ, k_lane<T, J, MODE, H, DET>, 128, lane_smem);
+    const int per_sm = blocks_per_sm(occ, k_lane<T, J, MODE, H, DET, HALF, COOP>, 128, lane_smem);
     int sms = 0, dev = 0;
     PURIFY_CUDA(cudaGetDevice(&dev));
     PURIFY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int blocks = std::max(1, std::min(sms * per_sm, (lw.nsets + 3) / 4));
     Launch L(p, MODE == LANE_GG ? "normal_gg" : (MODE == LANE_GRID ? "grid" : "degrid"));
-    launch_dependent(k_lane<T, J, MODE, H, DET>, blocks, 128, lane_smem, p->stream, p->grid.as<C>(), (const C*)yin,
+    launch_dependent(k_lane<T, J, MODE, H, DET, HALF, COOP>, blocks, 128, lane_smem, p->stream, p->grid.as<C>(), (const C*)yin,
                      (C*)yout, lw.set_info.as<int2>(), lw.run_cl.as<int2>(), lw.rec.as<T>(),
                      caller_order ? lw.idx_caller.as<int>() : lw.idx.as<int>(), lw.nsets, kb_table<T>(p),
-                     half ? p->half.W : p->Kx, half ? ~0 : p->Kx - 1, p->Ky, out, skip, dstride);
+                     HALF ? p->half.W : p->Kx, HALF ? ~0 : p->Kx - 1, p->Ky, out, skip, dstride);
     L.done();
+}
+// Whether a set's patches are flushed in common (see LaneStage). That trades a
+// trip through shared memory for fewer cache lines an access, so it pays where
+// the patches are wide and the grid is large enough for the reductions to be
+// what G^H waits for; doubles (a cell is 16 bytes) are indifferent and take it.
+// G^H by events, each lane its own rows | in common, us: half plane, a lane per
+// run: J = 4 at 1024 x 1024 with 2.0 M visibilities 52.2 63.3, J = 5 at 512 x 512 with
+// 0.9 M 28.3 29.0 and at 1024 x 1024 71.1 64.5, J = 6 at 128 x 128 with 100 001 16.3 18.3,
+// at 256 x 256 with 0.66 M 22.3 23.5, at 512 x 512 with 0.26 M 25.1 22.9, at 1024 x 1024
+// 93.4 84.2; lane pairs, J = 8: 128 x 128 16.2 17.7, 256 x 256 36.2 34.8, 512 x 512 with 0.9
+// M 65.4 57.2. Whole plane, lane pairs: J = 4 at 1024 x 1024 57.7 64.9, J = 5 at 512 x
+// 512 38.0 31.8, J = 6 49.9 40.3.
+template <typename T, int J> static bool lane_coop(const purify_plan* p, bool half) {
+    if (sizeof(T) == 8) return true;
+    if (J <= 4) return false;
+    const int64_t cells = (int64_t)p->Kx * p->Ky;
+    return cells >= (int64_t)1 << (J >= 7 ? 18 : (J == 5 && half ? 22 : 20));
+}
+template <typename T, int J, int MODE, int H, bool DET, bool HALF>
+static void lane_launch(purify_plan* p, const LaneWork& lw, const void* yin, void* yout, bool caller_order,
+                        const int* skip, typename cplx_of<T>::type* out, int64_t dstride) {
+    if constexpr (MODE == LANE_GRID && !DET) {
+        if (lane_coop<T, J>(p, HALF)) {
+            lane_launch_as<T, J, MODE, H, DET, HALF, true>(p, lw, yin, yout, caller_order, skip, out, dstride);
+            return;
+        }
+    }
+    lane_launch_as<T, J, MODE, H, DET, HALF, false>(p, lw, yin, yout, caller_order, skip, out, dstride);
 }
 template <int J, int MODE, int H>
 static void lane_tw(purify_plan* p, const LaneWork& lw, const void* yin, void* yout, bool caller_order,
@@ -1263,8 +1275,8 @@ static void lane_tw(purify_plan* p, const LaneWork& lw, const void* yin, void* y
             const int64_t stride = (int64_t)lw.nsets * lw.width;
             PURIFY_REQUIRE(p->det_patch.bytes >= sizeof(float2) * (size_t)J * J * (size_t)stride,
                            "deterministic patch buffer too small");
-            lane_launch<float, J, MODE, H, true>(p, lw, yin, yout, caller_order, skip, p->det_patch.as<float2>(),
-                                                 stride, false);
+            lane_launch<float, J, MODE, H, true, false>(p, lw, yin, yout, caller_order, skip,
+                                                        p->det_patch.as<float2>(), stride);
             const int64_t cells = (int64_t)p->Kx * p->Ky;
             Launch L(p, "det_gather");
             launch_dependent(k_lane_gather<J>, (unsigned)((cells + 255) / 256), 256, 0, p->stream,
@@ -1276,7 +1288,7 @@ static void lane_tw(purify_plan* p, const LaneWork& lw, const void* yin, void* y
     }
     if (MODE != LANE_DEGRID && !zeroed) PURIFY_CUDA(cudaMemsetAsync(p->gacc.p, 0, p->gacc.bytes, p->stream));
     if (lw.nsets == 0) return;
-    lane_launch<float, J, MODE, H, false>(p, lw, yin, yout, caller_order, skip, p->gacc.as<float2>(), 0, false);
+    lane_launch<float, J, MODE, H, false, false>(p, lw, yin, yout, caller_order, skip, p->gacc.as<float2>(), 0);
 }
 // G^H and (FP32) G^H G on the half-plane grid by lanes (the solver's order
 // of the visibilities), G by sorted visibilities
@@ -1294,10 +1306,10 @@ static void half_lane(purify_plan* p, const void* yin, const int* skip, bool zer
     // 512 and 22.6 against 24.4 at 256 x 256 (J = 6). Wider patches and
     // doubles, and G^H G (which also loads the patch), by lane pairs.
     if constexpr (MODE == LANE_GRID && sizeof(T) == 4 && J <= kLaneMaxJ)
-        lane_launch<T, J, MODE, 1, false>(p, p->half_lanes, yin, nullptr, false, skip, p->gacc.as<C>(), 0, true);
+        lane_launch<T, J, MODE, 1, false, true>(p, p->half_lanes, yin, nullptr, false, skip, p->gacc.as<C>(), 0);
     else
-        lane_launch<T, J, MODE, 2, false>(p, MODE == LANE_GG && p->half_pairs.nsets > 0 ? p->half_pairs : p->half_lanes,
-                                          yin, nullptr, false, skip, p->gacc.as<C>(), 0, true);
+        lane_launch<T, J, MODE, 2, false, true>(p, MODE == LANE_GG && p->half_pairs.nsets > 0 ? p->half_pairs : p->half_lanes,
+                                                yin, nullptr, false, skip, p->gacc.as<C>(), 0);
 }
 template <int J> static void half_lane_any(purify_plan* p, int mode, const void* yin, const int* s, bool z) {
     if (p->dtype == PURIFY_F32) {

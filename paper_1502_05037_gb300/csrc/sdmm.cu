@@ -95,9 +95,6 @@ __device__ __forceinline__ void ld_pair(const float2* p, float2 (&v)[2]) {
 __device__ __forceinline__ void st_pair(float2* p, const float2 (&v)[2]) {
     *reinterpret_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
 }
-// (never called: FP64 chunks go element by element)
-__device__ __forceinline__ void ld_pair(const double2* p, double2 (&v)[2]) { v[0] = p[0]; v[1] = p[1]; }
-__device__ __forceinline__ void st_pair(double2* p, const double2 (&v)[2]) { p[0] = v[0]; p[1] = v[1]; }
 
 // Per-block norms over visibility chunks: ||v2 + z2 - ybar||^2 (z2 may be
 // null) and ||v2 - ybar||^2.
@@ -119,7 +116,7 @@ __global__ void k_proj_norms(const typename cplx_of<T>::type* __restrict__ v2,
     };
     const C zero = cmake<C>(T(0), T(0));
     for_chunk<T>(cbeg[ch], cend[ch], [&](int m) { add(v2[m], ybar[m], z2 ? z2[m] : zero); },
-                 [&](int m) {
+                 [&](auto m) {   // (FP32 only)
                      C v[2], y[2], z[2] = {zero, zero};
                      ld_pair(v2 + m, v);
                      ld_pair(ybar + m, y);
@@ -132,16 +129,20 @@ __global__ void k_proj_norms(const typename cplx_of<T>::type* __restrict__ v2,
     if (threadIdx.x == 0) { part[2 * ch] = sa; part[2 * ch + 1] = se; }
     if (arrive_last(counters + C_PROJ)) {
         // chunk_first[r] .. chunk_first[r+1] are block r's chunks: a warp per
-        // block, its lanes' strided sums combined in a fixed order
-        for (int r = threadIdx.x >> 5; r < R; r += blockDim.x >> 5) {
+        // block, its lanes' strided sums combined in a fixed order; with hardly a
+        // chunk per block a thread per block (nothing to combine)
+        const int lanes = nchunks <= R ? 1 : 32, l = threadIdx.x % lanes;
+        for (int r = threadIdx.x / lanes; r < R; r += blockDim.x / lanes) {
             double sa2 = 0.0, se2 = 0.0;
-            for (int k = chunk_first[r] + (threadIdx.x & 31); k < chunk_first[r + 1]; k += 32) {
+            for (int k = chunk_first[r] + l; k < chunk_first[r + 1]; k += lanes) {
                 sa2 += __ldcg(part + 2 * k);
                 se2 += __ldcg(part + 2 * k + 1);
             }
-            sa2 = warp_sum(sa2);
-            se2 = warp_sum(se2);
-            if ((threadIdx.x & 31) == 0) {
+            if (lanes > 1) {
+                sa2 = warp_sum(sa2);
+                se2 = warp_sum(se2);
+            }
+            if (l == 0) {
                 if (z2) scal[S_BLOCKS + r] = sa2;
                 scal[S_BLOCKS + R + r] = se2;
             }
@@ -183,7 +184,7 @@ __global__ void k_proj_apply(typename cplx_of<T>::type* __restrict__ v2, typenam
                      v2[m] = step(v2[m], z, ybar[m]);
                      z2[m] = z;
                  },
-                 [&](int m) {
+                 [&](auto m) {   // (FP32 only)
                      C v[2], z[2], y[2];
                      ld_pair(v2 + m, v);
                      ld_pair(z2 + m, z);

@@ -1,12 +1,13 @@
 // Host-side tables of a plan, computed in double precision:
 //  - the gridding correction S (closed-form Fourier transform of the
 //    Kaiser-Bessel kernel),
-//  - per-tap polynomial approximations of the kernel for the float path,
+//  - per-tap polynomial approximations of the kernel,
 //  - FFT twiddle factors,
 //  - Daubechies db1..db8 filters by spectral factorisation.
 #include <cmath>
 #include <complex>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "common.cuh"
@@ -108,7 +109,7 @@ KbPoly fit_kb_poly(int J, double beta, int deg) {
     return kp;
 }
 
-KbPolyD fit_kb_poly_d(int J, double beta) {
+static KbPolyD fit_shape_d(int J, double beta) {
     KbPolyD kp;
     std::memset(&kp, 0, sizeof(kp));
     kp.J = J;
@@ -117,8 +118,10 @@ KbPolyD fit_kb_poly_d(int J, double beta) {
     const int deg = kb_poly_deg_d(J);
     const KbSeries<long double> kb(beta);
     fit_taps(kb, J, deg, kp.coef);
-    // a caller's beta may need a higher degree: compare with the definition
-    // between the nodes, to half a unit of double rounding at 1
+    // a caller's beta may need a higher degree: the rounded polynomial, as the
+    // kernels evaluate it, is compared with the definition between the nodes, to
+    // 2.5e-16 (a little over a unit of double rounding at 1; the default shape's
+    // is within 1.4e-16, of which its interpolant has 2e-17)
     kp.poly = 1;
     for (int a = 0; a < (J + 1) / 2; ++a)
         for (int i = 0; i <= 24; ++i) {
@@ -128,6 +131,16 @@ KbPolyD fit_kb_poly_d(int J, double beta) {
             if (!(std::fabs((long double)v - kb.tap(J, a, 0.5L * (z + 1.0L))) <= 2.5e-16L)) kp.poly = 0;
         }
     return kp;
+}
+
+// The default shape of each width is fitted once (in long double, which takes
+// longer than the rest of a small plan's tables where it is not in hardware).
+KbPolyD fit_kb_poly_d(int J, double beta) {
+    static std::once_flag once[PURIFY_MAX_J + 1];
+    static KbPolyD fitted[PURIFY_MAX_J + 1];
+    if (J < 2 || J > PURIFY_MAX_J || beta != 2.34 * J) return fit_shape_d(J, beta);
+    std::call_once(once[J], [&] { fitted[J] = fit_shape_d(J, beta); });
+    return fitted[J];
 }
 
 int kb_poly_degree(int J) { return kb_poly_deg(J); }

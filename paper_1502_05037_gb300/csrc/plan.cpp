@@ -800,7 +800,6 @@ static void build_runwork(purify_plan* p, const std::vector<T>& us, const std::v
     upload(p->runs.cell, cell);
     upload(p->runs.start, start);
     upload(p->runs.len, len);
-    p->workspace_bytes += (int64_t)(p->runs.rec.bytes + p->runs.cell.bytes + p->runs.start.bytes + p->runs.len.bytes);
 }
 
 // Lane work and visibility chunks of G block groups (block i in group
@@ -1005,11 +1004,13 @@ template <typename T> static void finish_plan(purify_plan* p) {
         p->stencil = Stencil();
         p->half_pairs.release();
     }
+    if (p->grid_kind != 2 && (p->normal_half || p->normal_kind != 2)) p->runs = RunWork();
     // (without pairs of their own the normal operator's lanes are half_lanes)
     if (!p->adj_half && !(p->normal_half && !p->stencil.on && p->half_pairs.nsets == 0)) p->half_lanes.release();
     if (!p->phi_half) p->half_sorted = SortedWork();
     for (int k = 0; k < 3; ++k) p->workspace_bytes += lane_bytes(p->lanes[k]);
     p->workspace_bytes += lane_bytes(p->half_lanes) + lane_bytes(p->half_pairs);
+    p->workspace_bytes += (int64_t)(p->runs.rec.bytes + p->runs.cell.bytes + p->runs.start.bytes + p->runs.len.bytes);
     const SortedWork& sw = p->half_sorted;
     p->workspace_bytes += (int64_t)(sw.z.bytes + sw.cell.bytes + sw.idx.bytes + sw.idx_caller.bytes);
     p->workspace_bytes += (int64_t)(p->stencil.coef.bytes + p->stencil.used.bytes);

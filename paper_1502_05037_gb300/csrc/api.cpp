@@ -203,9 +203,10 @@ purify_status purify_phi_normal(purify_plan* p, const void* x, void* out) {
         const size_t rb = real_bytes(p);
         Staged xs = stage_in(p, x, rb * p->N, p->stage_in);
         Staged os = stage_out(p, out, rb * p->N, p->stage_out);
-        // the forward row pass clears the accumulator that G^H G adds into
+        // the forward row pass clears the accumulator that G^H G adds into (the
+        // stencil writes all of it)
         const bool half = p->normal_half;
-        launch_scale_pad_rows(p, xs.dev, 1.0, nullptr, true, clear_acc(half), nullptr, half);
+        launch_scale_pad_rows(p, xs.dev, 1.0, nullptr, true, clear_normal(p, half), nullptr, half);
         launch_cols_fwd(p, nullptr, half);
         launch_normal_gg(p, nullptr, true, half);
         launch_cols_inv(p, nullptr, nullptr, half);

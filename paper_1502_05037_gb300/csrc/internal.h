@@ -431,6 +431,11 @@ bool timing_enabled(const purify_plan* p);
 void reweight(purify_plan* p, const void* x, double rho, void* w);
 double coef_std(purify_plan* p, const void* x);
 
+// what a normal operator's forward row pass clears: nothing for the stencil,
+// which writes every cell
+inline ClearAcc clear_normal(const purify_plan* p, bool half) {
+    return half && p->stencil.on ? CLEAR_NONE : clear_acc(half);
+}
 // G^H G as a stencil (stencil.cu): bytes of the coefficients; the build from
 // the half-plane lane work (cells: the runs' first-tap cells, row * W +
 // column), false where the device has no room for it; the application, which

@@ -440,7 +440,7 @@ static void autotune(purify_plan* p, const std::vector<int>& cand, BinsFor bins_
                 launch_rows_inv_crop(p, xout, 1.0, 1, nullptr, 0.0, nullptr, nullptr, true, hp);
             });
             val.normal_half = can_normal_half() && half_faster(0.95f, [&](bool hp) {
-                launch_scale_pad_rows(p, ximg, 1.0, nullptr, true, clear_acc(hp), nullptr, hp);
+                launch_scale_pad_rows(p, ximg, 1.0, nullptr, true, clear_normal(p, hp), nullptr, hp);
                 launch_cols_fwd(p, nullptr, hp);
                 launch_normal_gg(p, nullptr, true, hp);
                 launch_cols_inv(p, nullptr, nullptr, hp);

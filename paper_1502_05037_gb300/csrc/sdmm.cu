@@ -762,7 +762,7 @@ template <typename T> struct Solver {
                 // the pending update and the transform of the new r fused into
                 // the first FFT pass, then u = A r
                 const bool half = group < 0 && p->normal_half;
-                launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, clear_acc(half), &fold, half);
+                launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, clear_normal(p, half), &fold, half);
                 launch_cols_fwd(p, skip, half);
                 if (group >= 0) launch_lanes_on(p, p->group_lanes[group], 0, nullptr, nullptr, false, skip, true);
                 else launch_normal_gg(p, skip, true, half);
@@ -797,7 +797,7 @@ template <typename T> struct Solver {
         CgFold fold = make_fold();
         fold.step = k;
         const bool half = p->normal_half;
-        launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, clear_acc(half), &fold, half);
+        launch_scale_pad_rows(p, nullptr, inv_nu, skip, true, clear_normal(p, half), &fold, half);
         launch_cols_fwd(p, skip, half);
         launch_normal_gg(p, skip, true, half);
         launch_cols_inv(p, skip, nullptr, half);

@@ -460,7 +460,7 @@ template <typename T> struct RowFold {
 // S Z of rows row0 .. row0 + ROWS - 1 of the image for the thread's eight
 // elements p1 = t + k Kx / 8 of a row transform: f(k, values of the rows).
 // Elements k in the order 0 1 6 7, 2 3 4 5 (with oversampling 2 the image is in
-// the first four), BATCH pixels at a time.
+// the first four), in a CG step BATCH pixels at a time.
 template <typename T, int Kx, int ROWS, typename F>
 __device__ __forceinline__ void row_elements(const RowFold<T>& cg, const T* __restrict__ x, const T* __restrict__ sx,
                                              const T* __restrict__ sy, int nx, int row0, int t, T scale, F&& f) {
@@ -468,30 +468,39 @@ __device__ __forceinline__ void row_elements(const RowFold<T>& cg, const T* __re
     T rowscale[ROWS];
 #pragma unroll
     for (int q = 0; q < ROWS; ++q) rowscale[q] = sy[row0 + q] * scale;
+    // pixel column j of element k with (j - nx/2) mod Kx == p1 (p1 < Kx/2 exactly when k < 4)
+    auto column = [&](int k) {
+        const int p1 = t + k * N8;
+        return (k < 4 ? p1 : p1 - Kx) + nx / 2;
+    };
+    if (!cg.on) {   // (x is read only: no store stands between these loads)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int j = column(k);
+            const bool in = j >= 0 && j < nx;
+            T w[ROWS];
+#pragma unroll
+            for (int q = 0; q < ROWS; ++q) w[q] = in ? x[(row0 + q) * nx + j] * sx[j] * rowscale[q] : T(0);
+            f(k, w);
+        }
+        return;
+    }
 #pragma unroll
     for (int g = 0; g < 8; g += KS) {
+        constexpr int order[8] = {0, 1, 6, 7, 2, 3, 4, 5};
         int idx[BATCH];
         T v[BATCH], c[KS];
 #pragma unroll
         for (int b = 0; b < KS; ++b) {
-            constexpr int order[8] = {0, 1, 6, 7, 2, 3, 4, 5};
-            const int k = order[g + b], p1 = t + k * N8;
-            // pixel column j with (j - nx/2) mod Kx == p1 (p1 < Kx/2 exactly when k < 4)
-            const int j = (k < 4 ? p1 : p1 - Kx) + nx / 2;
+            const int j = column(order[g + b]);
             const bool in = j >= 0 && j < nx;
             c[b] = in ? sx[j] : T(0);
 #pragma unroll
             for (int q = 0; q < ROWS; ++q) idx[b * ROWS + q] = in ? (row0 + q) * nx + j : -1;
         }
-        if (cg.on) {
-            cg.pixels(idx, v);
-        } else {
-#pragma unroll
-            for (int e = 0; e < BATCH; ++e) v[e] = idx[e] >= 0 ? x[idx[e]] : T(0);
-        }
+        cg.pixels(idx, v);
 #pragma unroll
         for (int b = 0; b < KS; ++b) {
-            constexpr int order[8] = {0, 1, 6, 7, 2, 3, 4, 5};
             T w[ROWS];
 #pragma unroll
             for (int q = 0; q < ROWS; ++q) w[q] = v[b * ROWS + q] * c[b] * rowscale[q];

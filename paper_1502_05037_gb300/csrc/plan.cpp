@@ -307,9 +307,9 @@ template <typename T, typename BinsFor>
 static void autotune(purify_plan* p, const std::vector<int>& cand, BinsFor bins_for,
                      const std::vector<int>& cell_order, bool known, TuneVal val) {
     using C = typename cplx_of<T>::type;
-    // the half plane's work is built (grid_mode 0), and FP64 has its normal
-    // operator there only as a stencil
-    const bool half = p->half_lanes.nsets > 0;
+    // grid_mode 0 has the half plane, FP64 its normal operator there only as a
+    // stencil
+    const bool half = p->desc.grid_mode == 0;
     auto can_normal_half = [&] { return half && (p->stencil.on || p->dtype == PURIFY_F32); };
     if (!known) {
         // default subproblem size: about four subproblems per SM's worth of
@@ -568,6 +568,30 @@ static void build_lanework(purify_plan* p, const std::vector<HostRun>& runs, con
 
 static const int kRunMax = 48;
 
+// What a plan uses of the work that can be built: all that may be, before its
+// shape has been timed, then what was chosen.
+struct Needs {
+    bool runs, lanes[3];                    // run sets; lane forms 3..5 of the whole plane
+    bool sorted, half_lanes, half_normal;   // the half plane's G, G^H, G^H G
+};
+static Needs plan_needs(const purify_plan* p, bool known, const TuneVal& val) {
+    const int gm = p->desc.grid_mode;
+    // the whole plane's lane forms: forced, or candidates of the autotuner
+    const bool any_lane = lane_work_ok(p) && (gm >= 3 || (gm == 0 && p->desc.tile == 0 && p->M >= kTuneMinM));
+    Needs n{true, {any_lane, any_lane, any_lane}, gm == 0, gm == 0, gm == 0};
+    if (!known || gm != 0) return n;
+    auto uses = [&](int kind) {
+        return val.gkind == kind || (!val.phi_half && val.dkind == kind) || (!val.normal_half && val.nkind == kind);
+    };
+    // (a double plan may find no room for its stencil, or no use: run sets)
+    n.runs = val.gkind == 2 || (!val.normal_half && val.nkind == 2) || p->dtype == PURIFY_F64;
+    for (int k = 3; k <= 5; ++k) n.lanes[k - 3] = any_lane && uses(k);
+    n.sorted = val.phi_half;
+    n.half_lanes = val.adj_half;
+    n.half_normal = val.normal_half;
+    return n;
+}
+
 // Longest run of the half-plane lane work: a warp's share of the records is
 // M / (runs per set x resident warps) steps, and a set's longest run is a
 // serial chain, so runs are cut to half the share (at most kRunMax, at least
@@ -601,11 +625,11 @@ static bool use_stencil(const purify_plan* p, size_t nruns) {
 // where their first-tap column is in the upper half, in runs of one cell,
 // runs sorted by length (longest first, then by cell). A lane per run where
 // its patch fits the registers (FP32, J <= 6; see half_lane), else a lane pair.
-// normal: also the normal operator's form.
+// need: which of the forms are uploaded (the stencil is built from the lanes).
 template <typename T>
 static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std::vector<T>& vs,
                              const std::vector<int>& scx, const std::vector<int>& scy, const std::vector<int>& perm,
-                             bool normal) {
+                             const Needs& need) {
     const int64_t M = p->M;
     const int J = p->J, Kx = p->Kx, Ky = p->Ky, W = p->half.W, off = p->half.off;
     const int width = sizeof(T) == 4 && J <= kLaneMaxJ ? 32 : 16;
@@ -684,7 +708,7 @@ static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std
     };
     // lane work of `wid` runs per set (layout: see LaneWork), with the sorted
     // form filled on the way the first time
-    auto fill = [&](LaneWork& w, int wid, bool with_sorted) {
+    auto fill = [&](LaneWork& w, int wid, bool with_sorted, bool with_lanes) {
         const int nsets = (int)((nr + wid - 1) / wid);
         std::vector<int2> set_info(nsets), run_cl((size_t)nsets * wid, make_int2(0, 0));
         int64_t rows = 0;
@@ -719,6 +743,7 @@ static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std
                 });
             }
         });
+        if (!with_lanes) return;
         w.nsets = nsets;
         w.width = wid;
         w.tile = 0;
@@ -728,19 +753,21 @@ static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std
         upload(w.rec, rec);
         upload(w.idx, idx);
     };
-    fill(p->half_lanes, width, true);
-    upload(sw.z, sz);
-    upload(sw.cell, sc);
-    upload(sw.idx, si);
-    upload(sw.idx_caller, sk);
+    fill(p->half_lanes, width, true, need.half_lanes || need.half_normal);
+    if (need.sorted) {
+        upload(sw.z, sz);
+        upload(sw.cell, sc);
+        upload(sw.idx, si);
+        upload(sw.idx_caller, sk);
+    }
     // the normal operator as a stencil, where that is the faster form and fits
-    if (!normal) return;
+    if (!need.half_normal) return;
     if (use_stencil(p, nr)) {
         std::vector<int> cells(nr);
         for (size_t q = 0; q < nr; ++q) cells[q] = cell[order[sorted[q].first]];
         build_stencil(p, cells);
     }
-    if (!p->stencil.on && sizeof(T) == 4 && width == 32) fill(p->half_pairs, 16, false);
+    if (!p->stencil.on && sizeof(T) == 4 && width == 32) fill(p->half_pairs, 16, false, true);
 }
 
 // Run-ordered work (see RunWork): runs of equal first-tap cell in the cell
@@ -749,7 +776,8 @@ static void build_half_lanes(purify_plan* p, const std::vector<T>& us, const std
 template <typename T>
 static void build_runwork(purify_plan* p, const std::vector<T>& us, const std::vector<T>& vs,
                                 const std::vector<int>& scx, const std::vector<int>& scy,
-                                const std::vector<int>& cell_order, const std::vector<int>& perm) {
+                                const std::vector<int>& cell_order, const std::vector<int>& perm, const Needs& need) {
+    if (!need.runs && !need.lanes[0] && !need.lanes[1] && !need.lanes[2]) return;
     using Rec = typename RunRecOf<T>::type;
     using Run = HostRun;
     std::vector<Run> runs;
@@ -786,13 +814,13 @@ static void build_runwork(purify_plan* p, const std::vector<T>& us, const std::v
                 rec[start[r] + k] = e;
             }
     });
-    // the whole-plane lane forms: forced, or candidates of the autotuner
-    const bool lanes = p->desc.grid_mode >= 3 || (p->desc.grid_mode == 0 && p->desc.tile == 0 && M >= kTuneMinM);
-    if (sizeof(T) == 4 && p->J <= kLaneMaxJ && lanes) {
-        build_lanework(p, runs, rec, start, perm, 32, 0, p->lanes[0]);
-        build_lanework(p, runs, rec, start, perm, 16, 0, p->lanes[1], p->desc.grid_mode == 6);
-        build_lanework(p, runs, rec, start, perm, 16, std::min(32, std::min(p->Kx, p->Ky)), p->lanes[2]);
+    if constexpr (sizeof(T) == 4) {
+        if (need.lanes[0]) build_lanework(p, runs, rec, start, perm, 32, 0, p->lanes[0]);
+        if (need.lanes[1]) build_lanework(p, runs, rec, start, perm, 16, 0, p->lanes[1], p->desc.grid_mode == 6);
+        if (need.lanes[2])
+            build_lanework(p, runs, rec, start, perm, 16, std::min(32, std::min(p->Kx, p->Ky)), p->lanes[2]);
     }
+    if (!need.runs) return;
     p->runs.G = G;
     p->runs.nruns = (int)nr;
     p->runs.nsets = (int)(nr / G);
@@ -985,13 +1013,13 @@ template <typename T> static void finish_plan(purify_plan* p) {
         for (int64_t c = 0; c < ncell; ++c) pos[c + 1] += pos[c];
         for (int64_t i = 0; i < p->M; ++i) cell_order[pos[(int64_t)scy[i] * p->Kx + scx[i]]++] = (int)i;
     }
-    build_runwork<T>(p, us, vs, scx, scy, cell_order, perm);
     // autotuned plans take the half-plane path (unless it is known to be the
     // slower one for their shape); a forced decomposition runs on the whole plane
     TuneVal val{};
     const bool known = tune_cached(p, val);
-    if (d.grid_mode == 0 && (!known || val.phi_half || val.adj_half || val.normal_half))
-        build_half_lanes<T>(p, us, vs, scx, scy, perm, !known || val.normal_half);
+    const Needs need = plan_needs(p, known, val);
+    build_runwork<T>(p, us, vs, scx, scy, cell_order, perm, need);
+    if (need.sorted || need.half_lanes || need.half_normal) build_half_lanes<T>(p, us, vs, scx, scy, perm, need);
     autotune<T>(p, cand, bins_for, cell_order, known, val);
     // keep only the work in use (kind 6 runs on the lane pairs of kind 4)
     auto uses = [&](int k) {

@@ -553,7 +553,9 @@ __global__ void __launch_bounds__(1024) k_rows_fwd(const T* __restrict__ x, type
 //   R_2i[k] = (Z[k] + conj Z[-k]) / 2,  R_2i+1[k] = (Z[k] - conj Z[-k]) / 2i,
 // of which columns k = j - hp.off, j < hp.W, are written (rows[i][j]). A block
 // holds rb pairs. Half the transforms and half the columns of k_rows_fwd; the
-// passes are bound by latency and L2, so both count (1024 x 1024: 18 -> 13 us).
+// passes are bound by latency and L2, so both count (by events, beside the
+// other passes of Phi and the normal operator at 1024 x 1024: 18.5 -> 14.8 us; a CG
+// step's vector updates come on top of either).
 template <typename T, int LX>
 __global__ void __launch_bounds__(1024) k_rows_fwd_half(const T* __restrict__ x,
                            typename cplx_of<T>::type* __restrict__ rows, const T* __restrict__ sx,
@@ -795,10 +797,11 @@ __global__ void __launch_bounds__(MAXT) k_rows_inv_half(const typename cplx_of<T
     row_thread<N8>(rb, i, t, f);
     T dacc = 0, gacc2 = 0;   // add.out, and with the folded CG add.add (add = r, out = A r)
     const bool cg = cgf.part != nullptr;
-    // the pixels of `add` under way before the transform (FP32; doubles have no
-    // registers to spare): by events 13.2 -> 12.6 us at 128 x 128, 15.6 -> 14.4 at
-    // 512 x 512
-    constexpr bool EARLY = sizeof(T) == 4;
+    // the pixels of `add` under way before the transform, in FP32 (doubles have
+    // no registers to spare) and up to 1024 points, where a pass is its latency: by
+    // events 13.2 -> 12.6 us at 128 x 128, 15.6 -> 14.4 at 512 x 512, but 15.6 -> 16.4 at
+    // 1024 x 1024
+    constexpr bool EARLY = sizeof(T) == 4 && LX <= 10;
     T early[EARLY ? 8 : 1][2];
     if constexpr (EARLY) {
 #pragma unroll

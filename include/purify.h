@@ -11,7 +11,9 @@
  * Conventions for every call:
  *  - Array arguments are caller-owned and may live on the device (any CUDA
  *    device pointer) or, where stated, on the host; the library detects which.
- *    The plan owns only its internal tables and workspaces.
+ *    The plan owns only its internal tables and workspaces. Device arrays need
+ *    the alignment of their elements, no more (a view may begin at any element; a
+ *    complex element is its pair).
  *  - Real arrays hold `dtype` values (float or double). "Complex" arrays hold
  *    interleaved (re, im) pairs of `dtype`.
  *  - Images are [ny][nx] row-major; pixel (i, j) sits at centred coordinates

@@ -199,9 +199,10 @@ void build_gridlist(purify_plan* p, const std::vector<int>& bins, const std::vec
 // the normal operator run on the half plane or on the whole one. Results are
 // cached per problem shape.
 struct TuneKey {
-    int nx, ny, J, dtype, mlog, R, gm;
+    int nx, ny, Kx, Ky, J, dtype, mlog, R, gm;
     bool operator<(const TuneKey& o) const {
-        return std::tie(nx, ny, J, dtype, mlog, R, gm) < std::tie(o.nx, o.ny, o.J, o.dtype, o.mlog, o.R, o.gm);
+        return std::tie(nx, ny, Kx, Ky, J, dtype, mlog, R, gm) <
+               std::tie(o.nx, o.ny, o.Kx, o.Ky, o.J, o.dtype, o.mlog, o.R, o.gm);
     }
 };
 struct TuneVal {
@@ -229,7 +230,7 @@ static std::map<TuneKey, TuneVal> g_tune_cache;
 static TuneKey tune_key(const purify_plan* p) {
     int mlog = 0;
     while ((int64_t(1) << (mlog + 1)) <= p->M) ++mlog;
-    return TuneKey{p->nx, p->ny, p->J, p->dtype, mlog, std::min(p->R, 64), p->desc.grid_mode};
+    return TuneKey{p->nx, p->ny, p->Kx, p->Ky, p->J, p->dtype, mlog, std::min(p->R, 64), p->desc.grid_mode};
 }
 static bool tune_cached(const purify_plan* p, TuneVal& val) {
     if (p->desc.tile != 0) return false;

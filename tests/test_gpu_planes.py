@@ -102,3 +102,17 @@ def test_small_plans_take_either_plane(nx, ny, M, J, dtype):
         operators(plan, op, nx, ny, M, J, dtype)
         solves(plan, op, nx, ny, M, J, offs, 2, dtype, 1e-3 if dtype == F32 else 1e-9)
     assert modes[0] == modes[1]
+
+
+@pytest.mark.parametrize("dtype", [F32, F64])
+def test_a_shape_is_its_grid_too(dtype):
+    """Plans of one image and other oversampling do not share launch shapes: a
+    block of several short transforms would be one of several thousand threads
+    for the long ones."""
+    n, M, J = 16, 601, 4
+    u, v = coverage(M, 77, dtype)
+    ud, vd = torch.from_numpy(u).to(DEV), torch.from_numpy(v).to(DEV)
+    for alpha in (2.0, 256.0, 32.0, 2.0):
+        op = onf.NufftPlan(n, n, u.astype(np.float64), v.astype(np.float64), J, alpha=alpha)
+        plan = pk.Plan(n, n, ud, vd, kb_width=J, levels=2, dtype=dtype, oversample=alpha)
+        operators(plan, op, n, n, M, 3, dtype)
